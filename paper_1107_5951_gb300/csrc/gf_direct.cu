@@ -2,9 +2,9 @@
 // its N-body form (Eq. 7): every observer against every voxel quadrature
 // point.  Used as the exact path ("direct mode") and its transpose.
 //
-// Layout: one thread per output (observer, or voxel for the transpose); a
-// block stages a tile of 256 inputs in shared memory and every thread of the
-// block sweeps it, so each staged input is read from HBM once per block.
+// Layout: forward, tiles of up to 64 observers whose sources are shared by
+// the warps of a thread-block cluster (gf_pair.cuh); transpose, one thread per
+// voxel, a block staging tiles of 256 observers in shared memory.
 // FP64 path: source coordinates are formed with explicitly rounded
 // operations in the same order as the plain definition, so coincidence
 // decisions (r == x) are exact.  Mixed path: coordinates are carried as
@@ -16,8 +16,11 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "gf_internal.cuh"
+#include "gf_pair.cuh"
+#include "gf_simd.cuh"
 
 namespace gf {
 namespace {
@@ -64,148 +67,342 @@ __device__ __forceinline__ double node_coord(double o, double h, int64_t i, doub
     return __dadd_rn(c, __dmul_rn(__dmul_rn(0.5, h), xi));
 }
 
-__global__ void __launch_bounds__(kTile)
-direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict__ rho,
-               int rho_f32, GridArgs ga, const QuadRule *__restrict__ qr, double G,
-               double *__restrict__ g, double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ double sx[kTile], sy[kTile], sz[kTile], sm[kTile];
-    const int b = blockIdx.y;
-    const int64_t j = (int64_t)blockIdx.x * kTile + threadIdx.x;
-    const bool active = j < M;
-    const double rx = active ? obs[3 * j + 0] : 0.0;
-    const double ry = active ? obs[3 * j + 1] : 0.0;
-    const double rz = active ? obs[3 * j + 2] : 0.0;
-    const int nq = qr->nq;
-    const int64_t N = ga.nvox * nq;
-    const void *rho_b = rho_f32 ? (const void *)((const float *)rho + b * ga.nvox)
-                                : (const void *)((const double *)rho + b * ga.nvox);
-    double s0 = 0, c0 = 0, s1 = 0, c1 = 0, s2 = 0, c2 = 0;
-    bool bad = false;   // a non-finite density (reported through status[0])
-    for (int64_t t0 = 0; t0 < N; t0 += kTile) {
-        const int64_t s = t0 + threadIdx.x;
-        __syncthreads();
-        if (s < N) {
-            const int64_t v = s / nq;
-            const int q = (int)(s - v * nq);
-            const int64_t i = v % ga.nx, jj = (v / ga.nx) % ga.ny, k = v / (ga.nx * ga.ny);
-            sx[threadIdx.x] = node_coord(ga.ox, ga.hx, i, qr->xi[q][0]);
-            sy[threadIdx.x] = node_coord(ga.oy, ga.hy, jj, qr->xi[q][1]);
-            sz[threadIdx.x] = node_coord(ga.oz, ga.hz, k, qr->xi[q][2]);
-            const double rv = load_rho(rho_b, rho_f32, v);
-            bad |= !isfinite(rv);
-            sm[threadIdx.x] = __dmul_rn(__dmul_rn(rv, ga.vol), qr->wn[q]);
-        } else {
-            sx[threadIdx.x] = 0.0;
-            sy[threadIdx.x] = 0.0;
-            sz[threadIdx.x] = 0.0;
-            sm[threadIdx.x] = 0.0;
-        }
-        __syncthreads();
-        const int cnt = (N - t0) < kTile ? (int)(N - t0) : kTile;
-        double px = 0, py = 0, pz = 0;
-#pragma unroll 4
-        for (int u = 0; u < cnt; ++u) {
-            const double dx = rx - sx[u], dy = ry - sy[u], dz = rz - sz[u];
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double ri = rsqrt(r2);
-            const double k3 = (r2 > 0.0) ? sm[u] * (ri * ri * ri) : 0.0;
-            px = fma(k3, dx, px);
-            py = fma(k3, dy, py);
-            pz = fma(k3, dz, pz);
-        }
-        neumaier(s0, c0, px);
-        neumaier(s1, c1, py);
-        neumaier(s2, c2, pz);
+// Work units of the forward sums: the sources of one grid row (fixed j, k
+// and rule node q) share y and z, so a row is cut into pieces of at most
+// kRow voxels and a warp takes every W-th piece (W warps in the cluster).
+// Within a piece only x moves: a pair costs one difference, one square
+// (on top of the row's dy^2 + dz^2), the kernel value and two sums (of k and
+// of k dx); the y and z components are the row's sum of k times dy, dz.
+constexpr int kRow = 30;   // lanes 30 and 31 form the row's y and z
+
+struct RowSplit {
+    int clen, nch;   // voxels per piece, pieces per row
+};
+
+inline RowSplit row_split(int64_t nx) {
+    RowSplit r;
+    r.nch = (int)((nx + kRow - 1) / kRow);
+    r.clen = (int)((nx + r.nch - 1) / r.nch);
+    return r;
+}
+
+// Piece (ch, q, j, k) of the flat index u = ((k ny + j) nq + q) nch + ch,
+// advanced by a fixed step without divisions.
+struct RowIter {
+    int ch, q, j, k;
+    int dch, dq, dj, dk;
+    int nch, nq, ny;
+    __device__ static void split(int64_t u, int nch, int nq, int ny, int &ch, int &q, int &j, int &k) {
+        ch = (int)(u % nch);
+        u /= nch;
+        q = (int)(u % nq);
+        u /= nq;
+        j = (int)(u % ny);
+        k = (int)(u / ny);
     }
-    if (bad && status && blockIdx.x == 0) atomicOr(status, 1);
-    if (active) {
-        const double vx = G * (s0 + c0), vy = G * (s1 + c1), vz = G * (s2 + c2);
-        if (g) {
-            double *o = g + ((int64_t)b * M + j) * 3;
-            o[0] = vx;
-            o[1] = vy;
-            o[2] = vz;
+    __device__ RowIter(int64_t u0, int64_t step, int nch_, int nq_, int ny_) : nch(nch_), nq(nq_), ny(ny_) {
+        split(u0, nch, nq, ny, ch, q, j, k);
+        split(step, nch, nq, ny, dch, dq, dj, dk);
+    }
+    __device__ void next() {
+        ch += dch;
+        q += dq;
+        j += dj;
+        k += dk;
+        if (ch >= nch) {
+            ch -= nch;
+            ++q;
         }
-        if (gz) gz[(int64_t)b * M + j] = vz;
+        if (q >= nq) {
+            q -= nq;
+            ++j;
+        }
+        if (j >= ny) {
+            j -= ny;
+            ++k;
+        }
+    }
+};
+
+__device__ __forceinline__ const void *rho_of(const void *rho, int f32, int64_t off) {
+    return f32 ? (const void *)((const float *)rho + off) : (const void *)((const double *)rho + off);
+}
+
+// Bound by the FP64 pipe: 11 instructions a pair and about 20 a piece of
+// R x 16 pairs.  16^3 voxels, 2x2x2 rule, 4096 stations (134 M pairs):
+// 41.6 -> 4.07 ms (16 blocks of 256 threads before; 3.0 ms at two FP64
+// instructions a clock and SM).
+template <int R>
+__global__ void __launch_bounds__(kPairThreads)
+direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict__ rho, int rho_f32, GridArgs ga,
+               RowSplit rs, const QuadRule *__restrict__ qr, double G, double *__restrict__ g,
+               double *__restrict__ gz, int *__restrict__ status) {
+    __shared__ double2 red[(kPairWarps + 1) * 3 * R * 32];
+    __shared__ __align__(16) double2 row_s[kPairWarps][32];   // (x, mass) of the piece; entries 30, 31: y, z
+    const int C = (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.y;
+    const int64_t tile = blockIdx.x / C;
+    double rx[R], ry[R], rz[R];
+    double s[3 * R], c[3 * R], a[3 * R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+        const int64_t j = (tile * R + u) * 32 + lane;
+        rx[u] = j < M ? obs[3 * j + 0] : 0.0;
+        ry[u] = j < M ? obs[3 * j + 1] : 0.0;
+        rz[u] = j < M ? obs[3 * j + 2] : 0.0;
+    }
+#pragma unroll
+    for (int v = 0; v < 3 * R; ++v) s[v] = c[v] = a[v] = 0.0;
+    const void *rho_b = rho_of(rho, rho_f32, b * ga.nvox);
+    double2 *row = row_s[warp];
+    bool bad = false;   // a non-finite density (reported through status[0])
+    RowIter it(rank * kPairWarps + warp, (int64_t)C * kPairWarps, rs.nch, qr->nq, (int)ga.ny);
+    auto fetch = [&](double &rv) {
+        const int64_t i = (int64_t)it.ch * rs.clen + lane;
+        rv = 0.0;
+        if (it.k < ga.nz && lane < rs.clen && i < ga.nx)
+            rv = load_rho(rho_b, rho_f32, ((int64_t)it.k * ga.ny + it.j) * ga.nx + i);
+    };
+    double rv;
+    fetch(rv);
+    int since = 0;   // sources summed since the last merge into (s, c)
+    while (it.k < ga.nz) {
+        const int i0 = it.ch * rs.clen;
+        const int cnt = min(rs.clen, (int)ga.nx - i0);
+        // one node coordinate per lane: x of the piece's voxels, y (lane 30), z (lane 31)
+        const int ax = lane < kRow ? 0 : lane - (kRow - 1);
+        const double co = ax == 0 ? ga.ox : ax == 1 ? ga.oy : ga.oz, ch = ax == 0 ? ga.hx : ax == 1 ? ga.hy : ga.hz;
+        const int ci = ax == 0 ? i0 + lane : ax == 1 ? it.j : it.k;
+        const double x = node_coord(co, ch, ci, qr->xi[it.q][ax]);
+        bad |= !isfinite(rv);
+        const double m = __dmul_rn(__dmul_rn(rv, ga.vol), qr->wn[it.q]);
+        __syncwarp();
+        row[lane] = make_double2(x, m);
+        it.next();
+        fetch(rv);   // the next piece's densities, in flight during this one
+        __syncwarp();
+        const double y = row[kRow].x, z = row[kRow + 1].x;
+        double dy[R], dz[R], yz[R], S[R], SX[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            dy[u] = ry[u] - y;
+            dz[u] = rz[u] - z;
+            yz[u] = fma(dy[u], dy[u], dz[u] * dz[u]);
+            S[u] = SX[u] = 0.0;
+        }
+#pragma unroll 2
+        for (int e = 0; e < cnt; ++e) {
+            const double2 v = row[e];
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const double dx = rx[u] - v.x;
+                const double k3 = inv_r3(fma(dx, dx, yz[u]), v.y);
+                S[u] += k3;
+                SX[u] = fma(k3, dx, SX[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            a[3 * u + 0] += SX[u];
+            a[3 * u + 1] = fma(S[u], dy[u], a[3 * u + 1]);
+            a[3 * u + 2] = fma(S[u], dz[u], a[3 * u + 2]);
+        }
+        since += cnt;
+        if (since >= 240) {
+            since = 0;
+#pragma unroll
+            for (int v = 0; v < 3 * R; ++v) {
+                two_sum_d(s[v], c[v], a[v]);
+                a[v] = 0.0;
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 3 * R; ++v) two_sum_d(s[v], c[v], a[v]);
+    if (bad && status && tile == 0) atomicOr(status, 1);
+    const double tot = cluster_total<3 * R>(s, c, red);
+    const int t = threadIdx.x;
+    if (rank == 0 && t < 3 * R * 32) {
+        const int v = t >> 5, u = v / 3, d = v - 3 * u;
+        const int64_t j = (tile * R + u) * 32 + (t & 31);
+        if (j < M) {
+            if (g) g[((int64_t)b * M + j) * 3 + d] = G * tot;
+            if (gz && d == 2) gz[(int64_t)b * M + j] = G * tot;
+        }
     }
 }
 
 // Mixed precision: positions in voxel units split into an integer part
 // (held exactly in FP32, |i| < 2^24) and a fraction; the pair separation is
-// (ri - si) + (rf - sf), exact integer difference plus one rounding.
-__global__ void __launch_bounds__(kTile)
+// (ri - si) + (rf - sf), exact integer difference plus one rounding.  A lane's
+// two observers form one packed pair (f32x2), the masses are staged as
+// duplicated pairs, and the integer difference steps by one along the row:
+// 9 packed instructions and two reciprocal square roots for two pairs.  A
+// piece's FP32 sums are scaled by the rule's weight and merged into a
+// compensated FP32 pair about every 240 sources (the FP64 pipe is too slow
+// for a merge per piece); the pairs' sums, the factors G and the voxel volume
+// are FP64.  Bound by the special-function unit and the issue slots; at a few
+// hundred stations by latency.  40 x 40 x 32 voxels, 2x2x2 rule, 6000 stations
+// (2.5e9 pairs): 29.3 -> 1.33 ms; 12 x 10 x 9 voxels, 300 stations: 625 -> 46 us,
+// most of it the host.
+__global__ void __launch_bounds__(kPairThreads)
 direct_fwd_mixed(const float *__restrict__ obs_i, const float *__restrict__ obs_f, int64_t M,
-                 const void *__restrict__ rho, int rho_f32, GridArgs ga,
-                 const QuadRule *__restrict__ qr, double G, double *__restrict__ g,
-                 double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ float si[kTile][3], sf[kTile][3], sm[kTile];
+                 const void *__restrict__ rho, int rho_f32, GridArgs ga, RowSplit rs,
+                 const QuadRule *__restrict__ qr, double G, double *__restrict__ g, double *__restrict__ gz,
+                 int *__restrict__ status) {
+    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
+    __shared__ __align__(16) float2 row_s[kPairWarps][32];   // masses as duplicated pairs
+    const int C = (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
-    const int64_t j = (int64_t)blockIdx.x * kTile + threadIdx.x;
-    const bool active = j < M;
-    float ri[3] = {0.f, 0.f, 0.f}, rf[3] = {0.f, 0.f, 0.f};
-    if (active) {
-        for (int a = 0; a < 3; ++a) {
-            ri[a] = obs_i[3 * j + a];
-            rf[a] = obs_f[3 * j + a];
+    const int64_t tile = blockIdx.x / C;
+    uint64_t RI[3], RF[3];
+    {
+        const int64_t j0 = tile * 64 + lane, j1 = j0 + 32;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            RI[d] = pk2(j0 < M ? obs_i[3 * j0 + d] : 0.f, j1 < M ? obs_i[3 * j1 + d] : 0.f);
+            RF[d] = pk2(j0 < M ? obs_f[3 * j0 + d] : 0.f, j1 < M ? obs_f[3 * j1 + d] : 0.f);
         }
     }
-    const float hx = (float)ga.hx, hy = (float)ga.hy, hz = (float)ga.hz;
-    const int nq = qr->nq;
-    const int64_t N = ga.nvox * nq;
-    const void *rho_b = rho_f32 ? (const void *)((const float *)rho + b * ga.nvox)
-                                : (const void *)((const double *)rho + b * ga.nvox);
-    double ax = 0, ay = 0, az = 0;
+    const float fx = (float)ga.hx, fy = (float)ga.hy, fz = (float)ga.hz;
+    const uint64_t HX = pk2(fx, fx), HY = pk2(fy, fy), HZ = pk2(fz, fz), NEG1 = pk2(-1.f, -1.f);
+    const void *rho_b = rho_of(rho, rho_f32, b * ga.nvox);
+    float2 *row = row_s[warp];
+    uint64_t A[3] = {0, 0, 0}, H[3] = {0, 0, 0}, L[3] = {0, 0, 0};
     bool bad = false;   // a non-finite density (reported through status[0])
-    for (int64_t t0 = 0; t0 < N; t0 += kTile) {
-        const int64_t s = t0 + threadIdx.x;
-        __syncthreads();
-        if (s < N) {
-            const int64_t v = s / nq;
-            const int q = (int)(s - v * nq);
-            si[threadIdx.x][0] = (float)(v % ga.nx);
-            si[threadIdx.x][1] = (float)((v / ga.nx) % ga.ny);
-            si[threadIdx.x][2] = (float)(v / (ga.nx * ga.ny));
-            sf[threadIdx.x][0] = qr->offf[q][0];
-            sf[threadIdx.x][1] = qr->offf[q][1];
-            sf[threadIdx.x][2] = qr->offf[q][2];
-            const double rv = load_rho(rho_b, rho_f32, v);
-            bad |= !isfinite(rv);
-            sm[threadIdx.x] = (float)(rv * ga.vol * qr->wn[q]);
-        } else {
-            si[threadIdx.x][0] = si[threadIdx.x][1] = si[threadIdx.x][2] = 0.f;
-            sf[threadIdx.x][0] = sf[threadIdx.x][1] = sf[threadIdx.x][2] = 0.f;
-            sm[threadIdx.x] = 0.f;
+    RowIter it(rank * kPairWarps + warp, (int64_t)C * kPairWarps, rs.nch, qr->nq, (int)ga.ny);
+    auto fetch = [&]() -> float {
+        const int64_t i = (int64_t)it.ch * rs.clen + lane;
+        if (it.k < ga.nz && lane < rs.clen && i < ga.nx) {
+            const int64_t idx = ((int64_t)it.k * ga.ny + it.j) * ga.nx + i;
+            if (rho_f32) {
+                const float v = __ldg((const float *)rho_b + idx);
+                bad |= !isfinite(v);
+                return v;
+            }
+            const double v = __ldg((const double *)rho_b + idx);
+            bad |= !isfinite(v);
+            return (float)v;
         }
-        __syncthreads();
-        const int cnt = (N - t0) < kTile ? (int)(N - t0) : kTile;
-        float px = 0.f, py = 0.f, pz = 0.f;
+        return 0.f;
+    };
+    auto merge = [&]() {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const uint64_t s = add2(H[d], A[d]);
+            const uint64_t bp = sub2(s, H[d]);
+            L[d] = add2(L[d], add2(sub2(H[d], sub2(s, bp)), sub2(A[d], bp)));
+            H[d] = s;
+            A[d] = 0;
+        }
+    };
+    float rv = fetch();
+    int since = 0;   // sources summed since the last merge
+    while (it.k < ga.nz) {
+        const int i0 = it.ch * rs.clen;
+        const int cnt = min(rs.clen, (int)ga.nx - i0);
+        const float *of = qr->offf[it.q];
+        const float sx = of[0], sy = of[1], sz = of[2], wq = qr->wnf[it.q];
+        const float cj = (float)it.j, ck = (float)it.k, ci = (float)(i0 - 1);
+        __syncwarp();
+        row[lane] = make_float2(rv, rv);
+        it.next();
+        rv = fetch();   // the next piece's densities, in flight during this one
+        __syncwarp();
+        const uint64_t FX = sub2(RF[0], pk2(sx, sx));
+        const uint64_t DY = mul2(HY, add2(sub2(RI[1], pk2(cj, cj)), sub2(RF[1], pk2(sy, sy))));
+        const uint64_t DZ = mul2(HZ, add2(sub2(RI[2], pk2(ck, ck)), sub2(RF[2], pk2(sz, sz))));
+        const uint64_t YZ = fma2(DY, DY, mul2(DZ, DZ));
+        uint64_t D = sub2(RI[0], pk2(ci, ci)), S = 0, SX = 0;
+        auto sweep = [&](auto guarded) {
+            constexpr bool kGuard = decltype(guarded)::value;
 #pragma unroll 4
-        for (int u = 0; u < cnt; ++u) {
-            const float dx = hx * ((ri[0] - si[u][0]) + (rf[0] - sf[u][0]));
-            const float dy = hy * ((ri[1] - si[u][1]) + (rf[1] - sf[u][1]));
-            const float dz = hz * ((ri[2] - si[u][2]) + (rf[2] - sf[u][2]));
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            const float rinv = rsqrtf(r2);
-            const float k3 = (r2 > 0.f) ? sm[u] * (rinv * rinv * rinv) : 0.f;
-            px = fmaf(k3, dx, px);
-            py = fmaf(k3, dy, py);
-            pz = fmaf(k3, dz, pz);
+            for (int e = 0; e < cnt; ++e) {
+                const uint64_t m2 = *reinterpret_cast<const uint64_t *>(row + e);
+                D = add2(D, NEG1);
+                const uint64_t E = mul2(add2(D, FX), HX);
+                const uint64_t R2 = fma2(E, E, YZ);
+                float r0, r1;
+                up2(R2, r0, r1);
+                const uint64_t Q = pk2(rsqrt_ftz(r0), rsqrt_ftz(r1));
+                uint64_t K = mul2(mul2(Q, Q), mul2(Q, m2));
+                if constexpr (kGuard) {   // a source on the observer contributes nothing
+                    float k0, k1;
+                    up2(K, k0, k1);
+                    K = pk2(r0 > 1e-37f ? k0 : 0.f, r1 > 1e-37f ? k1 : 0.f);
+                }
+                S = add2(S, K);
+                SX = fma2(K, E, SX);
+            }
+        };
+        float y0, y1;
+        up2(YZ, y0, y1);
+        // only a row through an observer can hold a source at its position
+        if (__any_sync(0xffffffffu, !(y0 > 1e-30f) || !(y1 > 1e-30f)))
+            sweep(std::true_type{});
+        else
+            sweep(std::false_type{});
+        const uint64_t W = pk2(wq, wq), SW = mul2(S, W);
+        A[0] = fma2(SX, W, A[0]);
+        A[1] = fma2(SW, DY, A[1]);
+        A[2] = fma2(SW, DZ, A[2]);
+        since += cnt;
+        if (since >= 240) {
+            since = 0;
+            merge();
         }
-        ax += (double)px;
-        ay += (double)py;
-        az += (double)pz;
     }
-    if (bad && status && blockIdx.x == 0) atomicOr(status, 1);
-    if (active) {
-        const double vx = G * ax, vy = G * ay, vz = G * az;
-        if (g) {
-            double *o = g + ((int64_t)b * M + j) * 3;
-            o[0] = vx;
-            o[1] = vy;
-            o[2] = vz;
+    merge();
+    if (bad && status && tile == 0) atomicOr(status, 1);
+    double s[6], c[6];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        float h0, h1, l0, l1;
+        up2(H[d], h0, h1);
+        up2(L[d], l0, l1);
+        s[d] = (double)h0;
+        c[d] = (double)l0;
+        s[3 + d] = (double)h1;
+        c[3 + d] = (double)l1;
+    }
+    const double tot = cluster_total<6>(s, c, red);
+    const double scale = G * ga.vol;
+    const int t = threadIdx.x;
+    if (rank == 0 && t < 6 * 32) {
+        const int v = t >> 5, u = v / 3, d = v - 3 * u;
+        const int64_t j = tile * 64 + u * 32 + (t & 31);
+        if (j < M) {
+            if (g) g[((int64_t)b * M + j) * 3 + d] = scale * tot;
+            if (gz && d == 2) gz[(int64_t)b * M + j] = scale * tot;
         }
-        if (gz) gz[(int64_t)b * M + j] = vz;
     }
+}
+
+// Tiles of 64 observers (two per lane), or of 32 when there are no more.
+gf_status launch_fwd_f64(const double *obs, int64_t M, const void *rho, int rho_f32, const GridArgs &ga, int nq,
+                         const QuadRule *qr, int B, double G, double *g, double *gz, int *status, cudaStream_t st) {
+    const RowSplit rs = row_split(ga.nx);
+    const int64_t units = (int64_t)rs.nch * nq * ga.ny * ga.nz;
+    if (M <= 32) {
+        const int c = pair_cluster(B, units);
+        return pair_launch(direct_fwd_f64<1>, 1, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+    }
+    const int64_t tiles = (M + 63) / 64;
+    const int c = pair_cluster(tiles * B, units);
+    return pair_launch(direct_fwd_f64<2>, tiles, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+}
+
+gf_status launch_fwd_mixed(const float *oi, const float *of, int64_t M, const void *rho, int rho_f32,
+                           const GridArgs &ga, int nq, const QuadRule *qr, int B, double G, double *g, double *gz,
+                           int *status, cudaStream_t st) {
+    const RowSplit rs = row_split(ga.nx);
+    const int64_t tiles = (M + 63) / 64;
+    const int c = pair_cluster(tiles * B, (int64_t)rs.nch * nq * ga.ny * ga.nz);
+    return pair_launch(direct_fwd_mixed, tiles, B, c, st, oi, of, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
 }
 
 // Transpose: one thread per voxel, observers (with their weights) staged in
@@ -308,18 +505,12 @@ gf_status direct_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B,
     const int64_t M = plan->M;
     if (M == 0) return GF_OK;
     const GridArgs ga = grid_args(plan);
-    const dim3 grid(ceil_div(M, kTile), B);
     const int f32 = rho_dtype == GF_DTYPE_F32;
-    if (plan->opt.precision == GF_PREC_FP64) {
-        direct_fwd_f64<<<grid, kTile, 0, st>>>(plan->d_obs, M, rho, f32, ga, quad_device(plan),
-                                               plan->G, g, gz, plan->d_status);
-    } else {
-        direct_fwd_mixed<<<grid, kTile, 0, st>>>(reinterpret_cast<const float *>(plan->d_obs_ivox),
-                                                 plan->d_obs_fvox, M, rho, f32, ga,
-                                                 quad_device(plan), plan->G, g, gz, plan->d_status);
-    }
-    GF_KERNEL_DONE();
-    return GF_OK;
+    if (plan->opt.precision == GF_PREC_FP64)
+        return launch_fwd_f64(plan->d_obs, M, rho, f32, ga, plan->quad.nq, quad_device(plan), B, plan->G, g, gz,
+                              plan->d_status, st);
+    return launch_fwd_mixed(reinterpret_cast<const float *>(plan->d_obs_ivox), plan->d_obs_fvox, M, rho, f32, ga,
+                            plan->quad.nq, quad_device(plan), B, plan->G, g, gz, plan->d_status, st);
 }
 
 gf_status direct_adjoint(gf_plan_s *plan, const double *r, int ncomp, int B, double *grad,
@@ -505,10 +696,6 @@ extern "C" gf_status gf_direct_forward_static(const gf_grid *grid, const gf_quad
     GF_KERNEL_DONE();
     split_voxel_coords<<<ceil_div(M, 256), 256, 0, st>>>(obs_dev, M, ga, oi, of);
     GF_KERNEL_DONE();
-    direct_fwd_mixed<<<dim3(ceil_div(M, kTile), B), kTile, 0, st>>>(oi, of, M, rho_dev,
-                                                                     rho_dtype == GF_DTYPE_F32, ga, d_qr,
-                                                                     G > 0.0 ? G : 6.67428e-11, g_dev, gz_dev,
-                                                                     nullptr);
-    GF_KERNEL_DONE();
-    return GF_OK;
+    return launch_fwd_mixed(oi, of, M, rho_dev, rho_dtype == GF_DTYPE_F32, ga, qr.nq, d_qr, B,
+                            G > 0.0 ? G : 6.67428e-11, g_dev, gz_dev, nullptr, st);
 }

@@ -31,13 +31,13 @@
 
 #include "fmm_math.cuh"
 #include "gf_fmm.cuh"
+#include "gf_pair.cuh"
 #include "gf_prim.cuh"
 #include "gf_simd.cuh"
 
 namespace gf {
 namespace {
 
-constexpr int kPtTile = 256;
 constexpr double kPointsPerLeaf = 48.0;
 
 // ---------------------------------------------------------------- hexahedra
@@ -149,69 +149,80 @@ __global__ void hex_sources_fix(const double *__restrict__ verts, int64_t ncell,
 }
 
 // ---------------------------------------------------------------- direct
-__device__ __forceinline__ void neumaier_p(double &s, double &c, double x) {
-    const double t = s + x;
-    c += (fabs(s) >= fabs(x)) ? ((s - t) + x) : ((x - t) + s);
-    s = t;
-}
-
 __device__ __forceinline__ double load_rho_p(const void *rho, int f32, int64_t i) {
     return f32 ? (double)__ldg(reinterpret_cast<const float *>(rho) + i) : __ldg(reinterpret_cast<const double *>(rho) + i);
 }
 
-// One thread per observer; sources staged kPtTile at a time per block with
-// their masses rho_{c(s)} a_s of batch member blockIdx.y.
-__global__ void __launch_bounds__(kPtTile)
+// Tiles of 64 observers (two per lane); the warps of a cluster take the
+// sources 32 at a time (gf_pair.cuh), each lane staging one with its mass
+// rho_{c(s)} a_s of batch member blockIdx.y.  16 FP64 instructions a pair,
+// bound by the FP64 pipe.
+__global__ void __launch_bounds__(kPairThreads)
 direct_points_f64(const double *__restrict__ obs, int64_t M, const double *__restrict__ src,
                   const double *__restrict__ wt, int64_t S, int per_cell, int64_t ncell, const void *__restrict__ rho,
                   int rho_f32, double G, double *__restrict__ g, double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ double sx[kPtTile], sy[kPtTile], sz[kPtTile], sm[kPtTile];
+    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
+    __shared__ __align__(16) double2 stage[kPairWarps][32][2];   // (x, y), (z, mass)
+    const int C = (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
-    const int64_t j = (int64_t)blockIdx.x * kPtTile + threadIdx.x;
-    const bool active = j < M;
-    const double rx = active ? obs[3 * j] : 0.0, ry = active ? obs[3 * j + 1] : 0.0, rz = active ? obs[3 * j + 2] : 0.0;
-    double s0 = 0, c0 = 0, s1 = 0, c1 = 0, s2 = 0, c2 = 0;
-    bool bad = false;
-    for (int64_t t0 = 0; t0 < S; t0 += kPtTile) {
-        const int64_t s = t0 + threadIdx.x;
-        __syncthreads();
-        if (s < S) {
-            sx[threadIdx.x] = src[3 * s];
-            sy[threadIdx.x] = src[3 * s + 1];
-            sz[threadIdx.x] = src[3 * s + 2];
-            const double r = load_rho_p(rho, rho_f32, (int64_t)b * ncell + s / per_cell);
-            bad |= !isfinite(r);
-            sm[threadIdx.x] = r * wt[s];
-        } else {
-            sx[threadIdx.x] = sy[threadIdx.x] = sz[threadIdx.x] = sm[threadIdx.x] = 0.0;
-        }
-        __syncthreads();
-        const int cnt = (S - t0) < kPtTile ? (int)(S - t0) : kPtTile;
-        double px = 0, py = 0, pz = 0;
-#pragma unroll 4
-        for (int u = 0; u < cnt; ++u) {
-            const double dx = rx - sx[u], dy = ry - sy[u], dz = rz - sz[u];
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double ri = rsqrt(r2);
-            const double k3 = (r2 > 0.0) ? sm[u] * (ri * ri * ri) : 0.0;
-            px = fma(k3, dx, px);
-            py = fma(k3, dy, py);
-            pz = fma(k3, dz, pz);
-        }
-        neumaier_p(s0, c0, px);
-        neumaier_p(s1, c1, py);
-        neumaier_p(s2, c2, pz);
+    const int64_t tile = blockIdx.x / C;
+    double r[6], s[6], c[6], a[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+        const int64_t j = tile * 64 + (v / 3) * 32 + lane;
+        r[v] = j < M ? obs[3 * j + v % 3] : 0.0;
+        s[v] = c[v] = a[v] = 0.0;
     }
-    if (bad && status && blockIdx.x == 0) atomicOr(status, 1);
-    if (active) {
-        const double vx = G * (s0 + c0), vy = G * (s1 + c1), vz = G * (s2 + c2);
-        if (g) {
-            double *o = g + ((int64_t)b * M + j) * 3;
-            o[0] = vx;
-            o[1] = vy;
-            o[2] = vz;
+    bool bad = false;
+    double2(*st)[2] = stage[warp];
+    int since = 0;
+    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += (int64_t)C * kPairThreads) {
+        const int64_t i = t0 + lane;
+        __syncwarp();
+        if (i < S) {
+            const double rv = load_rho_p(rho, rho_f32, (int64_t)b * ncell + i / per_cell);
+            bad |= !isfinite(rv);
+            st[lane][0] = make_double2(src[3 * i], src[3 * i + 1]);
+            st[lane][1] = make_double2(src[3 * i + 2], rv * wt[i]);
         }
-        if (gz) gz[(int64_t)b * M + j] = vz;
+        __syncwarp();
+        const int cnt = (int)min((int64_t)32, S - t0);
+#pragma unroll 2
+        for (int e = 0; e < cnt; ++e) {
+            const double2 p = st[e][0], q = st[e][1];
+#pragma unroll
+            for (int u = 0; u < 6; u += 3) {
+                const double dx = r[u] - p.x, dy = r[u + 1] - p.y, dz = r[u + 2] - q.x;
+                const double k3 = inv_r3(fma(dx, dx, fma(dy, dy, dz * dz)), q.y);
+                a[u] = fma(k3, dx, a[u]);
+                a[u + 1] = fma(k3, dy, a[u + 1]);
+                a[u + 2] = fma(k3, dz, a[u + 2]);
+            }
+        }
+        since += cnt;
+        if (since >= 256) {
+            since = 0;
+#pragma unroll
+            for (int v = 0; v < 6; ++v) {
+                two_sum_d(s[v], c[v], a[v]);
+                a[v] = 0.0;
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 6; ++v) two_sum_d(s[v], c[v], a[v]);
+    if (bad && status && tile == 0) atomicOr(status, 1);
+    const double tot = cluster_total<6>(s, c, red);
+    const int t = threadIdx.x;
+    if (rank == 0 && t < 6 * 32) {
+        const int v = t >> 5;
+        const int64_t j = tile * 64 + (v / 3) * 32 + (t & 31);
+        if (j < M) {
+            if (g) g[((int64_t)b * M + j) * 3 + v % 3] = G * tot;
+            if (gz && v % 3 == 2) gz[(int64_t)b * M + j] = G * tot;
+        }
     }
 }
 
@@ -231,69 +242,114 @@ __global__ void split_points(const double *__restrict__ x, int64_t n, double lo0
 }
 
 // Mixed precision: the separation (ri - si) + (rf - sf) in quanta is an exact
-// integer difference plus one rounding; FP32 kernel, FP64 sum of the tiles.
-__global__ void __launch_bounds__(kPtTile)
+// integer difference plus one rounding; FP32 pair terms, compensated FP32
+// sums of about 256 sources, FP64 beyond.  Sources are staged as packed pairs
+// (f32x2), so one instruction does two pairs of an observer.
+__global__ void __launch_bounds__(kPairThreads)
 direct_points_mixed(const float *__restrict__ oi, const float *__restrict__ of, int64_t M,
                     const float *__restrict__ si, const float *__restrict__ sf, const double *__restrict__ wt,
                     int64_t S, int per_cell, int64_t ncell, const void *__restrict__ rho, int rho_f32, float q,
                     double Gq, double *__restrict__ g, double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ float ti[kPtTile][3], tf[kPtTile][3], tm[kPtTile];
+    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
+    // per pair of sources: integer parts {x0,x1, y0,y1}, {z0,z1, m0,m1}, fractions {x, y}, {z, -}
+    __shared__ __align__(16) float stage[kPairWarps][16 * 16];
+    const int C = (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
-    const int64_t j = (int64_t)blockIdx.x * kPtTile + threadIdx.x;
-    const bool active = j < M;
-    float ri[3] = {0.f, 0.f, 0.f}, rf[3] = {0.f, 0.f, 0.f};
-    if (active)
-        for (int a = 0; a < 3; ++a) {
-            ri[a] = oi[3 * j + a];
-            rf[a] = of[3 * j + a];
-        }
-    double ax = 0, ay = 0, az = 0;
+    const int64_t tile = blockIdx.x / C;
+    uint64_t RI[6], RF[6], A[6];
+    float h[6], l[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+        const int64_t j = tile * 64 + (v / 3) * 32 + lane;
+        const float x = j < M ? oi[3 * j + v % 3] : 0.f, f = j < M ? of[3 * j + v % 3] : 0.f;
+        RI[v] = pk2(x, x);
+        RF[v] = pk2(f, f);
+        A[v] = 0;
+        h[v] = l[v] = 0.f;
+    }
     bool bad = false;
     const double inv_q3 = 1.0 / ((double)q * (double)q * (double)q);
-    for (int64_t t0 = 0; t0 < S; t0 += kPtTile) {
-        const int64_t s = t0 + threadIdx.x;
-        __syncthreads();
-        if (s < S) {
-            for (int a = 0; a < 3; ++a) {
-                ti[threadIdx.x][a] = si[3 * s + a];
-                tf[threadIdx.x][a] = sf[3 * s + a];
+    float *st = stage[warp];
+    auto merge = [&]() {
+#pragma unroll
+        for (int v = 0; v < 6; ++v) {
+            float x0, x1;
+            up2(A[v], x0, x1);
+            two_sum(h[v], l[v], x0 + x1);
+            A[v] = 0;
+        }
+    };
+    int since = 0;
+    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += (int64_t)C * kPairThreads) {
+        const int64_t i = t0 + lane;
+        __syncwarp();
+        {
+            float *rec = st + (lane >> 1) * 16 + (lane & 1);
+            float v[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // past the end: massless
+            if (i < S) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    v[d] = si[3 * i + d];
+                    v[4 + d] = sf[3 * i + d];
+                }
+                const double r = load_rho_p(rho, rho_f32, (int64_t)b * ncell + i / per_cell);
+                bad |= !isfinite(r);
+                v[3] = (float)(r * wt[i] * inv_q3);   // mass in quantum units
             }
-            const double r = load_rho_p(rho, rho_f32, (int64_t)b * ncell + s / per_cell);
-            bad |= !isfinite(r);
-            tm[threadIdx.x] = (float)(r * wt[s] * inv_q3);   // mass in quantum units
-        } else {
-            for (int a = 0; a < 3; ++a) ti[threadIdx.x][a] = tf[threadIdx.x][a] = 0.f;
-            tm[threadIdx.x] = 0.f;
+#pragma unroll
+            for (int d = 0; d < 7; ++d) rec[2 * d] = v[d];
         }
-        __syncthreads();
-        const int cnt = (S - t0) < kPtTile ? (int)(S - t0) : kPtTile;
-        float px = 0.f, py = 0.f, pz = 0.f;
-#pragma unroll 4
-        for (int u = 0; u < cnt; ++u) {
-            const float dx = (ri[0] - ti[u][0]) + (rf[0] - tf[u][0]);
-            const float dy = (ri[1] - ti[u][1]) + (rf[1] - tf[u][1]);
-            const float dz = (ri[2] - ti[u][2]) + (rf[2] - tf[u][2]);
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            const float rinv = rsqrtf(r2);
-            const float k3 = (r2 > 0.f) ? tm[u] * (rinv * rinv * rinv) : 0.f;
-            px = fmaf(k3, dx, px);
-            py = fmaf(k3, dy, py);
-            pz = fmaf(k3, dz, pz);
+        __syncwarp();
+        const int cnt = (int)min((int64_t)32, S - t0);
+#pragma unroll 2
+        for (int e = 0; e < (cnt + 1) / 2; ++e) {
+            const ulonglong2 p0 = *reinterpret_cast<const ulonglong2 *>(st + 16 * e),
+                             p1 = *reinterpret_cast<const ulonglong2 *>(st + 16 * e + 4),
+                             p2 = *reinterpret_cast<const ulonglong2 *>(st + 16 * e + 8);
+            const uint64_t p3 = *reinterpret_cast<const uint64_t *>(st + 16 * e + 12);
+#pragma unroll
+            for (int u = 0; u < 6; u += 3) {
+                const uint64_t dx = add2(sub2(RI[u], p0.x), sub2(RF[u], p2.x));
+                const uint64_t dy = add2(sub2(RI[u + 1], p0.y), sub2(RF[u + 1], p2.y));
+                const uint64_t dz = add2(sub2(RI[u + 2], p1.x), sub2(RF[u + 2], p3));
+                const uint64_t R2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                float r0, r1;
+                up2(R2, r0, r1);
+                const uint64_t Q = pk2(rsqrt_ftz(r0), rsqrt_ftz(r1));
+                float k0, k1;
+                up2(mul2(mul2(Q, Q), mul2(Q, p1.y)), k0, k1);
+                // a source on the observer contributes nothing
+                const uint64_t K = pk2(r0 > 1e-37f ? k0 : 0.f, r1 > 1e-37f ? k1 : 0.f);
+                A[u] = fma2(K, dx, A[u]);
+                A[u + 1] = fma2(K, dy, A[u + 1]);
+                A[u + 2] = fma2(K, dz, A[u + 2]);
+            }
         }
-        ax += (double)px;
-        ay += (double)py;
-        az += (double)pz;
+        since += cnt;
+        if (since >= 256) {
+            since = 0;
+            merge();
+        }
     }
-    if (bad && status && blockIdx.x == 0) atomicOr(status, 1);
-    if (active) {
-        const double vx = Gq * ax, vy = Gq * ay, vz = Gq * az;
-        if (g) {
-            double *o = g + ((int64_t)b * M + j) * 3;
-            o[0] = vx;
-            o[1] = vy;
-            o[2] = vz;
+    merge();
+    if (bad && status && tile == 0) atomicOr(status, 1);
+    double s[6], c[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+        s[v] = (double)h[v];
+        c[v] = (double)l[v];
+    }
+    const double tot = cluster_total<6>(s, c, red);
+    const int t = threadIdx.x;
+    if (rank == 0 && t < 6 * 32) {
+        const int v = t >> 5;
+        const int64_t j = tile * 64 + (v / 3) * 32 + (t & 31);
+        if (j < M) {
+            if (g) g[((int64_t)b * M + j) * 3 + v % 3] = Gq * tot;
+            if (gz && v % 3 == 2) gz[(int64_t)b * M + j] = Gq * tot;
         }
-        if (gz) gz[(int64_t)b * M + j] = vz;
     }
 }
 
@@ -1122,19 +1178,15 @@ gf_status points_direct_forward(gf_plan_s *plan, const void *rho, int rho_dtype,
     const PointSet &P = plan->pts;
     const int64_t M = plan->M;
     if (M == 0) return GF_OK;
-    const dim3 grid(ceil_div(M, kPtTile), B);
     const int f32 = rho_dtype == GF_DTYPE_F32;
-    if (plan->opt.precision == GF_PREC_FP64 || P.S == 0) {
-        direct_points_f64<<<grid, kPtTile, 0, st>>>(plan->d_obs, M, P.x, P.a, P.S, P.per_cell, P.ncell, rho, f32,
-                                                   plan->G, g, gz, plan->d_status);
-    } else {
-        // mass and separations in quanta: g = G / q^2 * (quantum-unit sum)
-        direct_points_mixed<<<grid, kPtTile, 0, st>>>(P.oi, P.of, M, P.xi, P.xf, P.a, P.S, P.per_cell,
-                                                     P.ncell, rho, f32, (float)P.q, plan->G * P.q, g, gz,
-                                                     plan->d_status);
-    }
-    GF_KERNEL_DONE();
-    return GF_OK;
+    const int64_t tiles = (M + 63) / 64;
+    const int cl = pair_cluster(tiles * B, (P.S + 31) / 32);
+    if (plan->opt.precision == GF_PREC_FP64 || P.S == 0)
+        return pair_launch(direct_points_f64, tiles, B, cl, st, plan->d_obs, M, P.x, P.a, P.S, P.per_cell, P.ncell, rho,
+                           f32, plan->G, g, gz, plan->d_status);
+    // mass and separations in quanta: g = G / q^2 * (quantum-unit sum)
+    return pair_launch(direct_points_mixed, tiles, B, cl, st, P.oi, P.of, M, P.xi, P.xf, P.a, P.S, P.per_cell, P.ncell,
+                       rho, f32, (float)P.q, plan->G * P.q, g, gz, plan->d_status);
 }
 
 gf_status points_fmm_create(gf_plan_s *plan, const double *src, const double *wt, const double *obs,
