@@ -120,19 +120,18 @@ __global__ void build_p2m(int p, int K, int b, const QuadRule *__restrict__ qr, 
     }
 }
 
-// P2M into the parent level: Q[o][v][k] = sum_i P[v][i] T_o[i][k] for the
-// 8 child positions o (T_o the M2M operator, input component major), i.e.
-// the parent expansion contributed by unit mass at voxel v of child o.
-// Grid (8, b3), one thread per output component.
-__global__ void compose_p2m_up(const double *__restrict__ P, const double *__restrict__ m2m, int K, int b3,
-                               double *__restrict__ Q) {
-    const int o = blockIdx.x, v = blockIdx.y;
-    const double *pv = P + (size_t)v * K;
-    const double *T = m2m + (size_t)o * K * K;
+// P2M into the parent level of the child at the all-positive position 7:
+// Q[v][k] = sum_i P[v][i] T_7[i][k] (T_7 its M2M operator, input component
+// major), the parent expansion of unit mass at voxel v of that child.  The
+// other children's are its mirror images (gf_xlate.cu).  One block per voxel.
+__global__ void compose_p2m_up(const double *__restrict__ P, const double *__restrict__ T7, int K,
+                               double *__restrict__ Q, float *__restrict__ Qf) {
+    const double *pv = P + (size_t)blockIdx.x * K;
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         double s = 0.0;
-        for (int i = 0; i < K; ++i) s += pv[i] * T[(size_t)i * K + k];
-        Q[((size_t)o * b3 + v) * K + k] = s;
+        for (int i = 0; i < K; ++i) s += pv[i] * T7[(size_t)i * K + k];
+        Q[(size_t)blockIdx.x * K + k] = s;
+        Qf[(size_t)blockIdx.x * K + k] = (float)s;
     }
 }
 
@@ -516,135 +515,6 @@ template <class T>
 bool p2m_fused_ok(const FmmPlan *F) {
     const int b3 = F->b * F->b * F->b;
     return F->b <= 4 && p2m_fused_pitch(F->K) <= 320 && p2m_fused_smem<T>(b3, F->K, F->KS) <= 200 * 1024;
-}
-
-// Top-level translations in FP64 (mixed precision keeps the M2M into
-// level 2 and the L2L out of it in double).  The work is small but FP64 is
-// slow, so each block computes 32 output coefficients of one box and its 8
-// warps split the input coefficients; the partial sums meet in shared
-// memory.  Grid: (boxes, ceil(K / 32)), 256 threads.
-constexpr int kTopWarps = 8;
-
-// Batch members [b0, b0 + nb) of B are handled by one launch (nb bounded by
-// shared memory).
-// sum_{i0 <= i < i1} t[i K] x[i] with four partial sums, so that four
-// table loads are in flight at once (the FP64 top-level translations are
-// bound by the latency of these loads, not by arithmetic)
-template <class Tc>
-__device__ __forceinline__ Tc dot_strided(const Tc *__restrict__ t, const Tc *x, int i0, int i1, int K) {
-    Tc a0 = Tc(0), a1 = Tc(0), a2 = Tc(0), a3 = Tc(0);
-    int i = i0;
-    for (; i + 3 < i1; i += 4) {
-        const Tc t0 = t[(size_t)i * K], t1 = t[(size_t)(i + 1) * K], t2 = t[(size_t)(i + 2) * K],
-                 t3 = t[(size_t)(i + 3) * K];
-        a0 += t0 * x[i];
-        a1 += t1 * x[i + 1];
-        a2 += t2 * x[i + 2];
-        a3 += t3 * x[i + 3];
-    }
-    for (; i < i1; ++i) a0 += t[(size_t)i * K] * x[i];
-    return (a0 + a1) + (a2 + a3);
-}
-
-__host__ __device__ inline size_t top_smem(int nexp, int nb, int K) {
-    return sizeof(double) * ((size_t)nexp * nb * K + (size_t)kTopWarps * nb * 32);
-}
-
-// M2M: parent ME[k] = sum over existing children c, inputs i of
-// T_oct(c)[i][k] * child ME[i].  amax (may be null): the largest |ME[k]|
-// written into parents [alo, ahi), as float bits with atomicMax.
-template <class Ts, class Tc>
-__global__ void __launch_bounds__(kTopWarps * 32)
-m2m_kernel(const Ts *__restrict__ me_c, Block3 bc, Ts *__restrict__ me_p, Block3 bp, int B, int b0, int nb, int K,
-           int ldk, const Tc *__restrict__ tab, uint32_t *amax = nullptr, int64_t alo = 0, int64_t ahi = 0) {
-    extern __shared__ unsigned char shraw[];
-    Tc *xs = reinterpret_cast<Tc *>(shraw);   // [8][nb][K] child expansions
-    Tc *red = xs + 8 * nb * K;                // [kTopWarps][nb][32] partial sums
-    __shared__ int present[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t pi = blockIdx.x;
-    const int k = blockIdx.y * 32 + lane;
-    const int64_t px = bp.lo[0] + pi % bp.n[0], py = bp.lo[1] + (pi / bp.n[0]) % bp.n[1],
-                  pz = bp.lo[2] + pi / (bp.n[0] * bp.n[1]);
-    for (int e = threadIdx.x; e < 8 * nb * K; e += blockDim.x) {
-        const int oct = e / (nb * K), r = e - oct * nb * K;
-        const int64_t cx = 2 * px + (oct & 1) - bc.lo[0], cy = 2 * py + ((oct >> 1) & 1) - bc.lo[1],
-                      cz = 2 * pz + ((oct >> 2) & 1) - bc.lo[2];
-        const bool in = cx >= 0 && cx < bc.n[0] && cy >= 0 && cy < bc.n[1] && cz >= 0 && cz < bc.n[2];
-        const int rb = r / K, rk = r - rb * K;
-        xs[e] = in ? (Tc)me_c[(((cz * bc.n[1] + cy) * bc.n[0] + cx) * B + b0 + rb) * ldk + rk] : Tc(0);
-        if (r == 0) present[oct] = in;
-    }
-    __syncthreads();
-    const int per = (K + kTopWarps - 1) / kTopWarps;
-    const int i0 = warp * per, i1 = min(K, i0 + per);
-    for (int bb = 0; bb < nb; ++bb) {
-        Tc acc = Tc(0);
-        if (k < K)
-            for (int oct = 0; oct < 8; ++oct) {
-                if (!present[oct]) continue;
-                const Tc *t = tab + (size_t)oct * K * K + k;
-                const Tc *x = xs + (oct * nb + bb) * K;
-                acc += dot_strided(t, x, i0, i1, K);
-            }
-        red[(warp * nb + bb) * 32 + lane] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nb * 32; e += blockDim.x) {
-        const int bb = e / 32, kk = blockIdx.y * 32 + (e & 31);
-        if (kk >= K) continue;
-        Tc acc = Tc(0);
-        for (int w = 0; w < kTopWarps; ++w) acc += red[(w * nb + bb) * 32 + (e & 31)];
-        const Ts v = (Ts)acc;
-        me_p[(pi * B + b0 + bb) * ldk + kk] = v;
-        if (amax && pi >= alo && pi < ahi && v != Ts(0) && v == v)   // NaN is skipped, as fmaxf does
-            atomicMax(amax, __float_as_uint(fabsf((float)v)));
-    }
-}
-
-// L2L: child LE[k] += sum_i T_oct[i][k] * parent LE[i], one block per
-// (observer box of level l, 32 outputs).
-template <class Ts, class Tc>
-__global__ void __launch_bounds__(kTopWarps * 32)
-l2l_kernel(const Ts *__restrict__ le_p, const uint64_t *__restrict__ tkey, const int32_t *__restrict__ tparent,
-           Ts *__restrict__ le_c, int B, int b0, int nb, int K, int ldk, const Tc *__restrict__ tab) {
-    extern __shared__ unsigned char shraw[];
-    Tc *xs = reinterpret_cast<Tc *>(shraw);   // [nb][K]
-    Tc *red = xs + nb * K;                    // [kTopWarps][nb][32]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t = blockIdx.x;
-    const int k = blockIdx.y * 32 + lane;
-    const int oct = (int)(tkey[t] & 7);
-    const int64_t par = tparent[t];
-    for (int e = threadIdx.x; e < nb * K; e += blockDim.x) {
-        const int rb = e / K, rk = e - rb * K;
-        xs[e] = (Tc)le_p[(par * B + b0 + rb) * ldk + rk];
-    }
-    __syncthreads();
-    const int per = (K + kTopWarps - 1) / kTopWarps;
-    const int i0 = warp * per, i1 = min(K, i0 + per);
-    const Tc *tb = tab + (size_t)oct * K * K + k;
-    for (int bb = 0; bb < nb; ++bb) {
-        Tc acc = Tc(0);
-        if (k < K) acc = dot_strided(tb, xs + bb * K, i0, i1, K);
-        red[(warp * nb + bb) * 32 + lane] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nb * 32; e += blockDim.x) {
-        const int bb = e / 32, kk = blockIdx.y * 32 + (e & 31);
-        if (kk >= K) continue;
-        Tc acc = Tc(0);
-        for (int w = 0; w < kTopWarps; ++w) acc += red[(w * nb + bb) * 32 + (e & 31)];
-        Ts *o = le_c + (t * B + b0 + bb) * ldk + kk;
-        *o = (Ts)((Tc)*o + acc);
-    }
-}
-
-// Largest batch chunk whose shared memory fits one block.
-inline int top_batch_chunk(int nexp, int B, int K) {
-    int nb = B;
-    while (nb > 1 && top_smem(nexp, nb, K) > 200 * 1024) nb = (nb + 1) / 2;
-    return nb;
 }
 
 // ---------------------------------------------------------------- evaluation
@@ -1458,6 +1328,7 @@ gf_status get_tables(int device, int p, cudaStream_t st, const Tables **out) {
     transpose_ops<<<8, 256, 0, st>>>(T->l2l_d, T->al2l_d, T->al2l_f, T->K, 8, 0);
     GF_KERNEL_DONE();
     GF_TRY(m2l_prepare_tables(T, st));
+    GF_TRY(xlate_prepare_tables(T, st));
     GF_TRY(upload_l2p_coefs());
     GF_CUDA(cudaStreamSynchronize(st));
     g_tabs.push_back(T);
@@ -1472,10 +1343,10 @@ struct P2MEntry {
     int device, p, b, nq;
     int exact;             // closed-form voxels: moments integrated exactly
     double xi[kMaxQuad][3], wn[kMaxQuad];
-    double *pd;
-    float *pf;
-    float *tc = nullptr;   // tensor-core image (built on first use)
-    float *up_tc = nullptr;   // tensor-core image of the P2M into the parent level
+    double *pd = nullptr;
+    float *pf = nullptr;
+    double *ud = nullptr;  // 4^3-voxel leaves: P2M into the parent level from position 7 [64][K]
+    float *uf = nullptr, *uq = nullptr;   // FP32 copy, and in quad order
 };
 std::mutex g_p2m_mu;
 std::vector<P2MEntry *> g_p2m;
@@ -1490,6 +1361,9 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
             !memcmp(e->xi, q.xi, sizeof(double) * 3 * q.nq) && !memcmp(e->wn, q.wn, sizeof(double) * q.nq)) {
             F->p2m_d = e->pd;
             F->p2m_f = e->pf;
+            F->p2m_up_d = e->ud;
+            F->p2m_up_f = e->uf;
+            F->p2m_up_q = e->uq;
             return GF_OK;
         }
     P2MEntry *e = new P2MEntry();
@@ -1502,8 +1376,14 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
     memcpy(e->wn, q.wn, sizeof(double) * q.nq);
     const int b3 = F->b * F->b * F->b, K = F->K;
     if (cudaMalloc(&e->pd, sizeof(double) * b3 * K) != cudaSuccess ||
-        cudaMalloc(&e->pf, sizeof(float) * b3 * K) != cudaSuccess) {
+        cudaMalloc(&e->pf, sizeof(float) * b3 * K) != cudaSuccess ||
+        (F->b == 4 && (cudaMalloc(&e->ud, sizeof(double) * b3 * K) != cudaSuccess ||
+                       cudaMalloc(&e->uf, sizeof(float) * b3 * K) != cudaSuccess))) {
         cudaGetLastError();
+        cudaFree(e->pd);
+        cudaFree(e->pf);
+        cudaFree(e->ud);
+        cudaFree(e->uf);
         delete e;
         set_error("cannot allocate the P2M matrix");
         return GF_ERR_OOM;
@@ -1516,51 +1396,19 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
         build_p2m<<<b3, 128, shm, st>>>(F->p, K, F->b, quad_device(plan), e->pd, e->pf);
     }
     GF_KERNEL_DONE();
+    if (e->ud) {
+        compose_p2m_up<<<b3, 128, 0, st>>>(e->pd, F->tab->m2m_d + (size_t)7 * K * K, K, e->ud, e->uf);
+        GF_KERNEL_DONE();
+        GF_TRY(xlate_quad_table(F->tab, e->uf, b3, &e->uq, st));
+    }
     GF_CUDA(cudaStreamSynchronize(st));   // other streams may use the cached matrix next
     g_p2m.push_back(e);
     F->p2m_d = e->pd;
     F->p2m_f = e->pf;
+    F->p2m_up_d = e->ud;
+    F->p2m_up_f = e->uf;
+    F->p2m_up_q = e->uq;
     return GF_OK;
-}
-
-gf_status get_p2m_tc(gf_plan_s *plan, cudaStream_t st) {
-    FmmPlan *F = plan->fmm;
-    std::lock_guard<std::mutex> lk(g_p2m_mu);
-    for (P2MEntry *e : g_p2m) {
-        if (e->pd != F->p2m_d) continue;
-        if (!e->tc) {
-            const int b3 = F->b * F->b * F->b, npad = F->tab->tc_npad;
-            if (cudaMalloc(&e->tc, sizeof(float) * (size_t)(b3 / 16) * 2 * npad * 16) != cudaSuccess) {
-                cudaGetLastError();
-                e->tc = nullptr;
-                set_error("cannot allocate the P2M tensor-core image");
-                return GF_ERR_OOM;
-            }
-            GF_TRY(build_p2m_tc_image(e->pd, F->K, npad, b3, e->tc, st));
-            GF_CUDA(cudaStreamSynchronize(st));
-        }
-        if (!e->up_tc) {
-            const int b3 = F->b * F->b * F->b, npad = F->tab->tc_npad;
-            double *q = nullptr;
-            if (cudaMalloc(&q, sizeof(double) * 8 * (size_t)b3 * F->K) != cudaSuccess ||
-                cudaMalloc(&e->up_tc, sizeof(float) * 8 * (size_t)(b3 / 16) * 2 * npad * 16) != cudaSuccess) {
-                cudaGetLastError();
-                if (q) cudaFree(q);
-                e->up_tc = nullptr;
-                set_error("cannot allocate the tensor-core image of the P2M into the parent level");
-                return GF_ERR_OOM;
-            }
-            compose_p2m_up<<<dim3(8, b3), 128, 0, st>>>(e->pd, F->tab->m2m_d, F->K, b3, q);
-            GF_KERNEL_DONE();
-            GF_TRY(build_p2m_up_tc_image(q, F->K, npad, b3, e->up_tc, st));
-            GF_CUDA(cudaStreamSynchronize(st));
-            cudaFree(q);
-        }
-        F->p2m_tc = e->tc;
-        F->p2m_up_tc = e->up_tc;
-        return GF_OK;
-    }
-    return GF_OK;   // no cached matrix: the P2M stays on the SIMT path
 }
 
 gf_status fmm_alloc_workspaces(gf_plan_s *plan, cudaStream_t st) {
@@ -1708,48 +1556,42 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     FmmPlan *F = plan->fmm;
     const int K = F->K, L = F->L;
     const int b3 = F->b * F->b * F->b;
-    const Tables *tab = F->tab;
     const bool pts = F->points;
     const bool fused = !pts && p2m_fused_ok<T>(F);
-    bool up = false;   // level L-1 expansions made straight from the leaf masses
-    F->amax_fused = false;
+    const Block3 lb = block_of(F->lev[L]);
+    // 4^3-voxel leaves under a mirror-symmetric rule: the folded P2M kernels
+    const bool fold = !pts && p2m_fold_ok(plan) && lb.n[1] * 4 <= 65535 && lb.n[2] * 4 * B <= 65535;
+    bool up = false;   // level L-1 expansions made straight from the density grid
+    // the folded kernels that write each level's expansions also take the
+    // largest |input| of the slabs its M2L reads, in place of a pass over
+    // those rows before the M2L
+    F->amax_fused = fold && F->tc_amax != nullptr;
+    if (F->amax_fused) GF_CUDA(cudaMemsetAsync(F->tc_amax, 0, (kMaxLevels + 1) * sizeof(uint32_t), st));
     if (pts) {
         // a0 + a3 for point sources: masses in leaf order, P2M over each leaf's points
         GF_TRY(points_masses<T>(plan, rho, rho_dtype, B, st));
         stage_mark(plan, 1, st);
         GF_TRY(points_p2m<T>(plan, B, st));
-    }
-    if (fused) {
-        // a0 + a3: leaf-blocked densities and P2M (timed as P2M): on the
-        // tensor cores for 4^3-voxel leaves in mixed precision, else fused
+    } else if (fold) {
+        // a0 + a3 (timed as P2M): leaf-blocked masses and leaf expansions, of
+        // every leaf or -- when the expansions of level L-1 come straight from
+        // the grid -- of the z-slabs that the leaf level's M2L (and so the near
+        // field) reaches
         stage_mark(plan, 1, st);
-        const Block3 lb = block_of(F->lev[F->L]);
-        if (sizeof(T) == 4 && F->b == 4 && p2m_tc_ok(plan, B) && lb.n[1] * 4 <= 65535 &&
-            lb.n[2] * 4 * B <= 65535) {
-            // Leaf-blocked masses (read by the near field and the leaf P2M)
-            // of every leaf, or -- when the expansions of level L-1 come
-            // straight from the density grid -- of the z-slabs that the leaf
-            // level's M2L (and so the near field) reaches.
-            up = p2m_up_ok(plan, B);
-            const bool from_grid = up && p2m_up_grid_ok(plan, rho, rho_dtype);
-            // the kernels that write each level's expansions (the tensor-core
-            // P2M and M2M kinds, the FP64 M2M into level 2) also take the
-            // largest |input| of the slabs the M2L reads, in place of a pass
-            // over those rows before the M2L
-            F->amax_fused = F->tc_amax != nullptr;
-            if (F->amax_fused) GF_CUDA(cudaMemsetAsync(F->tc_amax, 0, (kMaxLevels + 1) * sizeof(uint32_t), st));
-            const FmmLevel &lf = F->lev[L];
-            const int64_t z0 = from_grid ? lf.m2l_z0 : 0;
-            const int64_t nz = from_grid ? std::max<int64_t>(0, lf.m2l_z1 - lf.m2l_z0 + 1) : lb.n[2];
-            GF_TRY((launch_blocking<T, 4>(plan, rho, rho_dtype == GF_DTYPE_F32, B, z0, nz, st)));
-            GF_TRY(p2m_run_tc(plan, B, st));   // every leaf, or only the slabs the M2L reads
-            if (up) GF_TRY(p2m_up_run_tc(plan, B, from_grid ? (const float *)rho : nullptr, st));
-        } else {
-            GF_TRY(launch_p2m_fused<T>(plan, rho, rho_dtype == GF_DTYPE_F32, B, st));
-        }
+        up = L - 1 > 2;   // level 2 keeps its FP64 M2M
+        const FmmLevel &lf = F->lev[L];
+        const int64_t z0 = up ? lf.m2l_z0 : 0;
+        const int64_t nz = up ? std::max<int64_t>(0, lf.m2l_z1 - lf.m2l_z0 + 1) : lb.n[2];
+        const int64_t slab = lb.n[0] * lb.n[1];
+        GF_TRY((launch_blocking<T, 4>(plan, rho, rho_dtype == GF_DTYPE_F32, B, z0, nz, st)));
+        GF_TRY(p2m_leaf_run<T>(plan, B, z0 * slab, nz * slab, st));
+        if (up) GF_TRY(p2m_up_run<T>(plan, rho, rho_dtype == GF_DTYPE_F32, B, st));
+    } else if (fused) {
+        stage_mark(plan, 1, st);
+        GF_TRY(launch_p2m_fused<T>(plan, rho, rho_dtype == GF_DTYPE_F32, B, st));
     }
     // a0: leaf-blocked densities
-    if (!fused && !pts) {
+    if (!fused && !fold && !pts) {
         const FmmLevel &lv = F->lev[L];
         const int64_t total = lv.ns * B * b3;
         const unsigned grid = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 16);
@@ -1758,9 +1600,9 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
                                                  block_of(lv), F->b, B, (T *)F->mass, plan->d_status);
         GF_KERNEL_DONE();
     }
-    if (!fused && !pts) stage_mark(plan, 1, st);
+    if (!fused && !fold && !pts) stage_mark(plan, 1, st);
     // a3: P2M at the leaves
-    if (!fused && !pts) {
+    if (!fused && !fold && !pts) {
         const FmmLevel &lv = F->lev[L];
         const unsigned grid = ceil_div(lv.ns, kP2MLeaves);
         const size_t shm = sizeof(T) * kP2MLeaves * B * b3;
@@ -1771,28 +1613,12 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     }
     stage_mark(plan, 2, st);
     // a4: M2M up to level 2.  In mixed precision the translation into the
-    // top level (2) is done in FP64 on the per-box kernel; the deeper levels
-    // run in the batched kernel in the plan's precision.
+    // top level (2) is done in FP64, the deeper ones in FP32.
     for (int l = up ? L - 2 : L - 1; l >= 2; --l) {
-        const FmmLevel &ch = F->lev[l + 1], &pa = F->lev[l];
-        if (sizeof(T) == 4 && l <= 2) {
-            const int nbc = top_batch_chunk(8, B, K);
-            GF_TRY((ensure_smem(m2m_kernel<T, double>, top_smem(8, nbc, K))));
-            for (int b0 = 0; b0 < B; b0 += nbc) {
-                const int nb = std::min(nbc, B - b0);
-                const int64_t slab = pa.sn[0] * pa.sn[1];
-                const bool am = F->amax_fused && pa.m2l_z1 >= pa.m2l_z0;
-                m2m_kernel<T, double><<<dim3((unsigned)pa.ns, ceil_div(K, 32)), kTopWarps * 32,
-                                        top_smem(8, nb, K), st>>>((const T *)ch.me, block_of(ch), (T *)pa.me,
-                                                                  block_of(pa), B, b0, nb, K, F->KS, tab->m2m_d,
-                                                                  am ? F->tc_amax + l : nullptr,
-                                                                  am ? pa.m2l_z0 * slab : 0,
-                                                                  am ? (pa.m2l_z1 + 1) * slab : 0);
-                GF_KERNEL_DONE();
-            }
-        } else {
+        if (sizeof(T) == 4 && l <= 2)
+            GF_TRY((translate_run<T, double>(plan, l, 0, B, st)));
+        else
             GF_TRY((translate_run<T, T>(plan, l, 0, B, st)));
-        }
     }
     stage_mark(plan, 3, st);
     // a7-a9 set up before the M2L: the near field of the evaluation only
@@ -1818,20 +1644,10 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     for (int l = 3; l <= L; ++l) {
         const FmmLevel &lv = F->lev[l];
         if (lv.nt == 0) continue;
-        const FmmLevel &pa = F->lev[l - 1];
-        if (sizeof(T) == 4 && l - 1 <= 2) {
-            const int nbc = top_batch_chunk(1, B, K);
-            GF_TRY((ensure_smem(l2l_kernel<T, double>, top_smem(1, nbc, K))));
-            for (int b0 = 0; b0 < B; b0 += nbc) {
-                const int nb = std::min(nbc, B - b0);
-                l2l_kernel<T, double><<<dim3((unsigned)lv.nt, ceil_div(K, 32)), kTopWarps * 32,
-                                        top_smem(1, nb, K), st>>>((const T *)pa.le, lv.tkey, lv.tparent,
-                                                                  (T *)lv.le, B, b0, nb, K, F->KS, tab->l2l_d);
-                GF_KERNEL_DONE();
-            }
-        } else {
+        if (sizeof(T) == 4 && l - 1 <= 2)
+            GF_TRY((translate_run<T, double>(plan, l, 1, B, st)));
+        else
             GF_TRY((translate_run<T, T>(plan, l, 1, B, st)));
-        }
     }
     stage_mark(plan, 6, st);
     // a7-a9: near field + L2P + combine + scatter

@@ -44,15 +44,13 @@ struct Tables {
     // (rows of 64 bytes):
     //   m2l_tc, am2l_tc  [343 slots][tc_nck_h chunks of 32 inputs][hi|lo][Npad][32]
     //                    FP16 parts of T_o[k_out][k_in] * colscale[k_out]
-    //   m2m_tc, l2l_tc   [8][tc_nck chunks of 16 inputs][hi|lo][Npad][16]
-    //                    TF32 parts of the operator
     // colscale (m2l_cs / am2l_cs: [Npad] scale, then [Npad] its inverse) is
     // the power of two that brings each output column's largest entry over
     // all offsets into (2^13, 2^14], so that both FP16 parts of every entry
     // that matters are normal numbers.
     void *m2l_tc = nullptr, *am2l_tc = nullptr;
     float *m2l_cs = nullptr, *am2l_cs = nullptr;
-    int tc_npad = 0, tc_nck = 0, tc_nck_h = 0;
+    int tc_npad = 0, tc_nck_h = 0;
     double *m2l_d = nullptr;
     float *m2l_f = nullptr;
     double *m2m_d = nullptr, *l2l_d = nullptr;
@@ -62,7 +60,12 @@ struct Tables {
     //   am2m[oct] = (T_M2M,oct)^T,  al2l[oct] = (T_L2L,oct)^T
     double *am2l_d = nullptr, *am2m_d = nullptr, *al2l_d = nullptr;
     float *am2l_f = nullptr, *am2m_f = nullptr, *al2l_f = nullptr;
-    float *m2m_tc = nullptr, *l2l_tc = nullptr;   // [8] operator images (tensor-core translations)
+    // Quads: four components of one parity class, ordered by degree
+    // (gf_xlate.cu); the FP32 operators of position 7 (M2M, L2L, M2M^T, L2L^T)
+    // as [K rounded up to 4][quad][4].
+    int nquad = 0;
+    int *quad_k = nullptr, *quad_info = nullptr;
+    float *quad_f[4] = {};
 };
 
 gf_status get_tables(int device, int p, cudaStream_t st, const Tables **out);
@@ -92,6 +95,11 @@ struct FmmPlan {
     void *nsum = nullptr;         // [B][M][6] near-field sums (hi, lo per component) in observer-key order
     double *p2m_d = nullptr;      // [b^3][K] quadrature-folded P2M matrix
     float *p2m_f = nullptr;
+    // 4^3-voxel leaves: [64][K], the leaf P2M followed by the M2M to the parent
+    // for the child at position 7 (gf_xlate.cu: the other positions mirror it)
+    double *p2m_up_d = nullptr;
+    float *p2m_up_f = nullptr;
+    float *p2m_up_q = nullptr;    // the FP32 matrix in quad order [64][quad][4]
     const Tables *tab = nullptr;
     void *tc_levels = nullptr;                  // tensor-core M2L level table
     // largest |input| of each level's M2L (bits of a non-negative float;
@@ -118,14 +126,6 @@ struct FmmPlan {
     bool adj_ready = false;                      // adjoint structures built (on first adjoint)
     void *tc_levels_adj = nullptr;
     std::vector<unsigned char> tc_levels_adj_host;
-    float *p2m_tc = nullptr;                     // tensor-core P2M operator image
-    // tensor-core image of the P2M into level L-1: for each child position
-    // o of a parent, Q_o[v][k] = sum_i P[v][i] M2M_o[i][k] (the leaf P2M
-    // followed by the M2M to the parent), so a parent's expansion comes
-    // straight from the masses of its 8 child leaves
-    float *p2m_up_tc = nullptr;
-    void *tc_xlate = nullptr;                    // tensor-core M2M / L2L / P2M level tables
-    std::vector<unsigned char> tc_xlate_host;
 };
 
 // adjoint set-up and driver (gf_adjoint.cu)

@@ -169,8 +169,6 @@ void fmm_destroy(gf_plan_s *plan);
 void plan_release(gf_plan_s *plan);
 gf_status fmm_info(const gf_plan_s *plan, gf_plan_info *info);
 gf_status fmm_work_counts(gf_plan_s *plan, cudaStream_t st);
-// The plan's P2M matrix as a tensor-core image, cached with the matrix.
-gf_status get_p2m_tc(gf_plan_s *plan, cudaStream_t st);
 gf_status fmm_export_tree(gf_plan_s *plan, int level, int32_t *perm, uint64_t *keys,
                           uint64_t *box_keys, int64_t *ilist, int64_t *near_);
 size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_options *opt);
@@ -206,10 +204,10 @@ __host__ __device__ __forceinline__ bool in_source_part(int64_t X, int64_t Y, in
     return c >= lo && c < hi;
 }
 
-// Opt a kernel in to more than 48 KB of dynamic shared memory.
+// Opt a kernel in to more than 48 KB of shared memory (up to 1 KB of it static).
 template <class Kern>
 inline gf_status ensure_smem(Kern kernel, size_t bytes) {
-    if (bytes > 48 * 1024) {
+    if (bytes > 47 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) {
             set_error("cannot reserve %zu bytes of shared memory: %s", bytes, cudaGetErrorString(e));

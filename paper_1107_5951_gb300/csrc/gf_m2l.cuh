@@ -8,14 +8,9 @@ namespace gf {
 
 gf_status m2l_upload_offsets(const signed char h_il[8][189][3]);
 gf_status m2l_prepare_tables(Tables *T, cudaStream_t st);
-// Tensor-core image of a P2M matrix [b3][K] (b3 a multiple of 16).
-gf_status build_p2m_tc_image(const double *pd, int K, int npad, int b3, float *img, cudaStream_t st);
-// Tensor-core image of the P2M into the parent level (8 operators [b3][K]).
-gf_status build_p2m_up_tc_image(const double *q, int K, int npad, int b3, float *img, cudaStream_t st);
-
 // LE_l[t] = sum over the interaction list of box t of T_o * ME_l[t + o],
 // for every observer box t of every level (overwrites each LE_l).  Mixed
-// precision runs on the tensor cores (tcgen05, 3xTF32) unless the plan asks
+// precision runs on the tensor cores (tcgen05, FP16 parts) unless the plan asks
 // for the SIMT kernel; FP64 runs on the SIMT kernel.
 // adj: the transpose, MEdual_l[s] = sum_{o in IL(class of s)} T_{-o}^T LEdual_l[s + o]
 // over every source box s (observer boxes found through the level's map).
@@ -26,9 +21,7 @@ gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t
 template <class T>
 gf_status m2l_level(gf_plan_s *plan, int level, int B, bool adj, cudaStream_t st);
 
-// Batched translations (Ts = storage, Tc = arithmetic); in mixed precision
-// the forward M2M / L2L run on the tensor cores (3xTF32), otherwise on the
-// SIMT cores:
+// Translations between levels (gf_xlate.cu; Ts = storage, Tc = arithmetic):
 //   kind 0  M2M into `level` from level + 1 (store)
 //   kind 1  L2L into `level` from level - 1 (update)
 //   kind 2  M2M^T into `level` from level - 1 (update), over source boxes
@@ -36,27 +29,23 @@ gf_status m2l_level(gf_plan_s *plan, int level, int B, bool adj, cudaStream_t st
 template <class Ts, class Tc>
 gf_status translate_run(gf_plan_s *plan, int level, int kind, int B, cudaStream_t st);
 
+// The tables that the translations read beside the operators themselves, and
+// any FP32 matrix [rows][K] in their component order (allocated here).
+gf_status xlate_prepare_tables(Tables *T, cudaStream_t st);
+gf_status xlate_quad_table(const Tables *T, const float *src, int rows, float **dst, cudaStream_t st);
+
+// P2M of 4^3-voxel leaves under a mirror-symmetric rule (p2m_fold_ok): the
+// leaves [first, first + count) from their leaf-blocked masses, and every box
+// of level L - 1 straight from the density grid.
+bool p2m_fold_ok(const gf_plan_s *plan);
+template <class T>
+gf_status p2m_leaf_run(gf_plan_s *plan, int B, int64_t first, int64_t count, cudaStream_t st);
+template <class T>
+gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaStream_t st);
+
 // Plan-time set-up of the tensor-core path (level descriptors on the device).
 gf_status m2l_tc_prepare(gf_plan_s *plan);
 // The adjoint's level tables (built on the plan's first adjoint call).
 gf_status m2l_tc_prepare_adj(gf_plan_s *plan);
-
-// P2M on the tensor cores (mixed precision, leaves of 16k voxels): ME of
-// every leaf = P^T x its leaf-blocked masses.  p2m_tc_ok says whether the
-// plan and batch size allow it.
-bool p2m_tc_ok(const gf_plan_s *plan, int B);
-gf_status p2m_run_tc(gf_plan_s *plan, int B, cudaStream_t st);
-// Whether the parent level's expansions can come straight from the leaf
-// masses (p2m_up_run_tc) instead of P2M at every leaf and the M2M out of the
-// leaf level: mixed precision on the tensor cores, L - 1 > 2 (level 2 keeps
-// its FP64 M2M).  The leaf expansions are then computed only for the z-slabs
-// that the leaf level's M2L reads.
-bool p2m_up_ok(const gf_plan_s *plan, int B);
-// Whether the P2M into level L-1 can read the densities straight from the
-// caller's grid (FP32, 16-byte aligned, every axis and the grid's place in
-// the tree multiples of the 4-voxel leaf edge); grid NULL: the leaf-blocked
-// masses of every leaf.
-bool p2m_up_grid_ok(const gf_plan_s *plan, const void *rho, int rho_dtype);
-gf_status p2m_up_run_tc(gf_plan_s *plan, int B, const float *grid, cudaStream_t st);
 
 }  // namespace gf
