@@ -1,18 +1,15 @@
-// gf_m2l.cu -- M2L over the interaction list, as a batched dense contraction.
-//
-// Observer boxes of a level are grouped by parity class (their position in
-// the parent), because the 189 interaction-list offsets depend only on that
-// class.  A block takes up to 32 columns -- (box, batch member) pairs of one
-// class -- and, offset by offset, multiplies the K x K operator T_o by the
-// K x 32 matrix of gathered source expansions ME[t + o], accumulating the
-// K x 32 result in registers.  Sources outside the source block contribute
-// zero columns.  Each output is written once, so the result is deterministic.
+// gf_m2l.cu -- M2L over the interaction list, as a batched dense contraction:
+// on the tensor cores in mixed precision (tiles of 128 columns of one parity
+// class, offset by offset), on the SIMT cores otherwise (columns folded by
+// mirror symmetry).  Sources outside the source block contribute zeros.  Each
+// output is written once, so the result is deterministic.
 #include <cuda_fp16.h>
 #include <string.h>
 
 #include <algorithm>
 #include <vector>
 
+#include "gf_fold.cuh"
 #include "gf_m2l.cuh"
 
 namespace gf {
@@ -114,33 +111,6 @@ gf_status m2l_prepare_tables(Tables *T, cudaStream_t st) {
 
 namespace {
 
-struct M2LArgs {
-    const void *me;    // input rows (forward: ME_l; adjoint: LE_l duals)
-    void *le;          // output rows (forward: LE_l; adjoint: ME_l duals)
-    int K, ldk, B, nbox;
-    const int32_t *order;
-    int64_t cls_off[9];
-    const uint64_t *tkey;
-    int64_t blo[3], bn[3];   // source block of the level
-    const void *tab;   // [343][K][K], input component major
-    int adj;           // adjoint: columns are source boxes, inputs via imap
-    const int32_t *imap;
-    int64_t mlo[3], mn[3];
-    int shift;                   // level - 2
-    uint32_t part_lo, part_hi;   // source partition (forward)
-};
-
-constexpr int kCK = 32;  // input components per shared-memory chunk
-
-template <class T>
-struct XStride {
-    static constexpr int v = 36;
-};
-template <>
-struct XStride<double> {
-    static constexpr int v = 34;
-};
-
 __device__ __forceinline__ int64_t dm(uint64_t k, int s) {
     int64_t c = 0;
     for (int bit = 0; bit < 21; ++bit) c |= (int64_t)((k >> (3 * bit + s)) & 1) << bit;
@@ -168,128 +138,176 @@ __device__ __forceinline__ void class_box(int cls, const int64_t *lo, const int6
     z = i0[2] + 2 * (j / (c[0] * c[1]));
 }
 
-template <class T, int RPT>
-__global__ void __launch_bounds__(256)
-m2l_simt(M2LArgs a) {
-    constexpr int S = XStride<T>::v;
-    constexpr int KP = 32 * RPT;
-    extern __shared__ unsigned char shraw[];
-    T *Xs = reinterpret_cast<T *>(shraw);  // [kCK][S]
-    T *Ts = Xs + kCK * S;                  // [kCK][KP]
-    __shared__ int64_t tbox[32];
-    __shared__ int tc[32][3];
-    __shared__ int64_t srow[32];
-    const int cls = blockIdx.y;
-    const int64_t cbeg = a.cls_off[cls], ccnt = a.cls_off[cls + 1] - cbeg;
-    const int64_t tile0 = (int64_t)blockIdx.x * a.nbox;
-    if (tile0 >= ccnt) return;
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    const int K = a.K, B = a.B;
-    const T *me = reinterpret_cast<const T *>(a.me);
-    const T *tab = reinterpret_cast<const T *>(a.tab);
-    if (tid < 32) {
-        const int64_t s = tile0 + tid;
-        if (tid < a.nbox && s < ccnt) {
-            if (!a.adj) {
-                const int64_t t = a.order[cbeg + s];
-                tbox[tid] = t;
-                const uint64_t key = a.tkey[t];
-                tc[tid][0] = (int)(dm(key, 0) - a.blo[0]);
-                tc[tid][1] = (int)(dm(key, 1) - a.blo[1]);
-                tc[tid][2] = (int)(dm(key, 2) - a.blo[2]);
-            } else {
-                int64_t x, y, z;
-                class_box(cls, a.blo, a.bn, s, x, y, z);
-                tbox[tid] = (z * a.bn[1] + y) * a.bn[0] + x;
-                tc[tid][0] = (int)x;
-                tc[tid][1] = (int)y;
-                tc[tid][2] = (int)z;
-            }
+// ---------------------------------------------------------------- SIMT
+// The M2L on the SIMT cores (FP64 plans; GF_FLAG_M2L_SIMT; degrees beyond one
+// MMA's width), folded by mirror symmetry: the up to eight offsets
+// (+-a, +-b, +-c) of a box's list have operators that are signed copies of
+// T_(a, b, c), so their sources are folded (an 8-point Walsh-Hadamard transform)
+// and take one K x K product: 56 products for the 189 offsets of an interior
+// box, 28 for the 63 of a box above its sources.  The FP64 pipe (two
+// instructions a clock and SM) bounds it, so everything else -- gathering,
+// table reads, index work -- only has to stay out of its way.  One launch
+// takes every level (the longest lists, the upper levels, first); a block owns
+// P columns (box, batch member), any parity classes mixed, and runs the 56
+// magnitudes in turn; thread (i, group) sums component i of a 16-byte group of
+// columns.  128^3 voxels, p = 14, 256^2 stations, FP64: the M2L 275 -> 10.8 ms
+// (each level a launch of 8..64 blocks before, one after another; the FP64 pipe
+// is now 95% busy on an active SM).
+struct FoldLevel {
+    const void *in;          // forward: ME_l; adjoint: LE_l duals
+    void *out;               // forward: LE_l; adjoint: ME_l duals
+    const uint64_t *tkey;    // forward: observer boxes
+    const int32_t *imap;     // adjoint: observer box of a place, or -1
+    int32_t blo[3], bn[3];   // source block
+    int32_t mlo[3], mn[3];   // adjoint: extent of the map
+    uint32_t ncol, blk0;     // columns; first block of the level
+};
+
+struct FoldM2LArgs {
+    FoldLevel lv[kMaxLevels + 1];
+    int lmin, lmax;
+    int K, ldk, B, adj;
+    const void *tab;             // [343][K][K], input component major
+    uint32_t part_lo, part_hi;   // source partition (forward)
+};
+
+template <class T, int P>
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 640, sizeof(T) == 8 ? 2 : 1)
+m2l_fold(const __grid_constant__ FoldM2LArgs a) {
+    constexpr int G = Lay<T, P>::G, NG = Lay<T, P>::NG;
+    constexpr int Q = sizeof(T) == 8 ? 2 : 4;   // staged inputs per thread (FP64: two blocks' registers fit an SM)
+    extern __shared__ __align__(16) unsigned char shraw[];
+    T *xs = reinterpret_cast<T *>(shraw);   // folded inputs (Lay)
+    __shared__ int64_t crow[P * 8];
+    __shared__ int ccoord[P][3], cmember[P];
+    const int K = a.K, tid = threadIdx.x, nthr = blockDim.x;
+    int l = a.lmin;
+    while (l < a.lmax && blockIdx.x >= a.lv[l + 1].blk0) ++l;
+    const FoldLevel &L = a.lv[l];
+    const uint32_t col0 = (blockIdx.x - L.blk0) * P;
+    if (tid < P) {   // the columns' boxes, relative to the source block
+        const uint32_t col = min(col0 + tid, L.ncol - 1), box = col / (uint32_t)a.B;
+        cmember[tid] = (int)(col - box * a.B);
+        if (!a.adj) {
+            const uint64_t key = L.tkey[box];
+            for (int d = 0; d < 3; ++d) ccoord[tid][d] = (int)dm(key, d) - L.blo[d];
         } else {
-            tbox[tid] = -1;
+            const uint32_t yz = box / (uint32_t)L.bn[0], z = yz / (uint32_t)L.bn[1];
+            ccoord[tid][0] = (int)(box - yz * L.bn[0]);
+            ccoord[tid][1] = (int)(yz - z * L.bn[1]);
+            ccoord[tid][2] = (int)z;
         }
     }
-    __syncthreads();
-    T acc[RPT][4];
-#pragma unroll
-    for (int r = 0; r < RPT; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
-    for (int oi = 0; oi < 189; ++oi) {
-        const int dx = c_il[cls][oi][0], dy = c_il[cls][oi][1], dz = c_il[cls][oi][2];
+    const bool on = tid < K * NG;
+    const int grp = on ? tid / K : 0, i = on ? tid - grp * K : 0, cls = parity_of(i);
+    const T *in = reinterpret_cast<const T *>(L.in);
+    Acc<T, G> acc;
+    acc.zero();
+    for (int mag = 0; mag < 64; ++mag) {
+        const int ma[3] = {mag & 3, (mag >> 2) & 3, mag >> 4};
+        if (max(ma[0], max(ma[1], ma[2])) < 2) continue;
+        __syncthreads();   // the previous magnitude's inputs have been used
         int any = 0;
-        if (tid < 32) {
-            const int slot = tid / B, bb = tid - slot * B;
+        if (tid < 8 * P) {
+            // source at (s_x a, s_y b, s_z c), s = - where the bit of o is clear
+            const int c = tid >> 3, o = tid & 7;
             int64_t row = -1;
-            if (slot < a.nbox && tbox[slot] >= 0) {
-                const int64_t sx = tc[slot][0] + dx, sy = tc[slot][1] + dy, sz = tc[slot][2] + dz;
-                if (!a.adj) {
-                    if (sx >= 0 && sy >= 0 && sz >= 0 && sx < a.bn[0] && sy < a.bn[1] && sz < a.bn[2] &&
-                        in_source_part(sx + a.blo[0], sy + a.blo[1], sz + a.blo[2], a.shift, a.part_lo, a.part_hi))
-                        row = (((sz * a.bn[1] + sy) * a.bn[0] + sx) * B + bb) * a.ldk;
-                } else {
-                    const int64_t wx = sx + a.blo[0] - a.mlo[0], wy = sy + a.blo[1] - a.mlo[1],
-                                  wz = sz + a.blo[2] - a.mlo[2];
-                    if (wx >= 0 && wy >= 0 && wz >= 0 && wx < a.mn[0] && wy < a.mn[1] && wz < a.mn[2]) {
-                        const int32_t m = a.imap[(wz * a.mn[1] + wy) * a.mn[0] + wx];
-                        if (m >= 0) row = ((int64_t)m * B + bb) * a.ldk;
-                    }
+            int s[3];
+            bool ok = col0 + c < L.ncol;
+            for (int d = 0; d < 3; ++d) {
+                const int off = ((o >> d) & 1) ? ma[d] : -ma[d];
+                const int t = ccoord[c][d], par = (t + L.blo[d]) & 1;
+                // the list reaches [-2, 3] from an even place, [-3, 2] from an odd
+                // one; a zero component is counted once
+                ok = ok && off >= -2 - par && off <= 3 - par && (ma[d] != 0 || ((o >> d) & 1));
+                s[d] = t + off;
+            }
+            if (ok && !a.adj) {
+                ok = s[0] >= 0 && s[1] >= 0 && s[2] >= 0 && s[0] < L.bn[0] && s[1] < L.bn[1] && s[2] < L.bn[2] &&
+                     in_source_part(s[0] + L.blo[0], s[1] + L.blo[1], s[2] + L.blo[2], l - 2, a.part_lo, a.part_hi);
+                if (ok) row = ((((int64_t)s[2] * L.bn[1] + s[1]) * L.bn[0] + s[0]) * a.B + cmember[c]) * a.ldk;
+            } else if (ok) {
+                const int w[3] = {s[0] + L.blo[0] - L.mlo[0], s[1] + L.blo[1] - L.mlo[1], s[2] + L.blo[2] - L.mlo[2]};
+                if (w[0] >= 0 && w[1] >= 0 && w[2] >= 0 && w[0] < L.mn[0] && w[1] < L.mn[1] && w[2] < L.mn[2]) {
+                    const int32_t m = L.imap[((int64_t)w[2] * L.mn[1] + w[1]) * L.mn[0] + w[0]];
+                    if (m >= 0) row = ((int64_t)m * a.B + cmember[c]) * a.ldk;
                 }
             }
-            srow[tid] = row;
-            any = row >= 0;
+            crow[tid] = row;
+            any = row >= 0 ? 1 << o : 0;
         }
-        if (!__syncthreads_or(any)) continue;
-        const T *tabo = tab + (size_t)((dz + 3) * 49 + (dy + 3) * 7 + (dx + 3)) * K * K;
-        for (int c0 = 0; c0 < K; c0 += kCK) {
-            for (int e = tid; e < kCK * 32; e += 256) {
-                const int cc = e % kCK, j = e / kCK;
-                const int64_t row = srow[j];
-                const int c = c0 + cc;
-                Xs[cc * S + j] = (row >= 0 && c < K) ? me[row + c] : T(0);
+        const int sides = tid < 32 * ((8 * P + 31) / 32) ? __reduce_or_sync(0xffffffffu, any) : 0;
+        const int has = __syncthreads_or(sides) ? 1 : 0;
+        if (!has) continue;
+        // Q inputs of one column per thread; a mirror pair with one side
+        // missing throughout the column needs no additions
+        for (int e = tid; e < (((K + 3) & ~3) / Q) * P; e += nthr) {
+            const int c = e % P, j0 = Q * (e / P);
+            T v[Q][8];
+            int have = 0;
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                const int64_t row = crow[c * 8 + o];
+                have |= (row >= 0) << o;
+                if constexpr (Q == 4) {
+                    T w[4];
+                    load4<T, T>(in, row, j0, K, w);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q][o] = w[q];
+                } else {
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) v[q][o] = row >= 0 && j0 + q < K ? __ldg(in + row + j0 + q) : T(0);
+                }
             }
-            for (int e = tid; e < kCK * KP; e += 256) {
-                const int cc = e / KP, k = e - cc * KP;
-                const int c = c0 + cc;
-                Ts[e] = (c < K && k < K) ? tabo[(size_t)c * K + k] : T(0);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int hi_set = d == 0 ? 0xaa : d == 1 ? 0xcc : 0xf0;
+                const bool lo_any = have & ~hi_set & 0xff, hi_any = have & hi_set;
+#pragma unroll
+                for (int o = 0; o < 8; ++o)
+                    if (!((o >> d) & 1)) {
+                        const int h = o | (1 << d);
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) {
+                            const T lo = v[q][o], hi = v[q][h];
+                            if (lo_any && hi_any) {
+                                v[q][o] = hi + lo;
+                                v[q][h] = hi - lo;
+                            } else if (hi_any) {
+                                v[q][o] = hi;
+                            } else {
+                                v[q][h] = -lo;
+                            }
+                        }
+                    }
+                have |= (have & hi_set) >> (1 << d) | (have & ~hi_set & 0xff) << (1 << d);
             }
-            __syncthreads();
-#pragma unroll 4
-            for (int cc = 0; cc < kCK; ++cc) {
-                T xv[4], tv[RPT];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) xv[c] = Xs[cc * S + tx * 4 + c];
+            for (int q = 0; q < Q; ++q) {
+                const int sw = parity_of(j0 + q) ^ (((j0 + q) >> 2) & 7);
 #pragma unroll
-                for (int r = 0; r < RPT; ++r) tv[r] = Ts[cc * KP + ty * RPT + r];
-#pragma unroll
-                for (int r = 0; r < RPT; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] += tv[r] * xv[c];
+                for (int d = 0; d < 8; ++d) xs[Lay<T, P>::at(j0 + q, d ^ sw, c)] = v[q][d];
             }
-            __syncthreads();
+        }
+        __syncthreads();
+        const T *t = reinterpret_cast<const T *>(a.tab) + (size_t)((ma[2] + 3) * 49 + (ma[1] + 3) * 7 + ma[0] + 3) * K * K + i;
+#pragma unroll 2
+        for (int g = 0; 4 * g < K; ++g) {
+            T tv[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) tv[q] = 4 * g + q < K ? __ldg(t + (size_t)(4 * g + q) * K) : T(0);
+            const T *x = xs + ((size_t)(4 * g * NG + grp) * 8 + (cls ^ (g & 7) ^ (grp & 7))) * G;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc.add(0, tv[q], x + q * 8 * P);
         }
     }
-    T *le = reinterpret_cast<T *>(a.le);
+    if (!on) return;
+    T *out = reinterpret_cast<T *>(L.out);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int j = tx * 4 + c;
-        const int slot = j / B, bb = j - slot * B;
-        if (slot >= a.nbox || tbox[slot] < 0) continue;
-#pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-            const int k = ty * RPT + r;
-            if (k < K) le[(tbox[slot] * B + bb) * a.ldk + k] = acc[r][c];
-        }
+    for (int c = 0; c < G; ++c) {
+        const uint32_t col = col0 + grp * G + c;
+        if (col < L.ncol) out[(int64_t)col * a.ldk + i] = acc.get(c);
     }
-}
-
-template <class T, int RPT>
-gf_status launch_simt(const M2LArgs &a, int64_t max_tiles, cudaStream_t st) {
-    const size_t shm = sizeof(T) * (kCK * XStride<T>::v + kCK * 32 * RPT);
-    GF_TRY(ensure_smem(m2l_simt<T, RPT>, shm));
-    m2l_simt<T, RPT><<<dim3((unsigned)max_tiles, 8), 256, shm, st>>>(a);
-    GF_KERNEL_DONE();
-    return GF_OK;
 }
 
 // ---------------------------------------------------------------- tcgen05
@@ -1244,58 +1262,73 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
 
 }  // namespace
 
-template <class T>
-gf_status m2l_level(gf_plan_s *plan, int level, int B, bool adj, cudaStream_t st) {
-    FmmPlan *F = plan->fmm;
-    const FmmLevel &lv = F->lev[level];
-    M2LArgs a;
-    a.me = adj ? lv.le : lv.me;
-    a.le = adj ? lv.me : lv.le;
-    a.K = F->K;
-    a.ldk = F->KS;
-    a.B = B;
-    a.nbox = std::max(1, 32 / B);
-    a.order = lv.m2l_order;
-    a.adj = adj ? 1 : 0;
-    a.imap = F->imap[level];
-    a.shift = level - 2;
-    a.part_lo = adj ? 0u : plan->part_lo;
-    a.part_hi = adj ? 64u : plan->part_hi;
-    int64_t maxc = 0;
-    for (int c = 0; c <= 8; ++c) a.cls_off[c] = adj ? F->scls_off[level][c] : lv.cls_off[c];
-    for (int c = 0; c < 8; ++c) maxc = std::max<int64_t>(maxc, a.cls_off[c + 1] - a.cls_off[c]);
-    a.tkey = lv.tkey;
-    for (int d = 0; d < 3; ++d) {
-        a.blo[d] = lv.slo[d];
-        a.bn[d] = lv.sn[d];
-        a.mlo[d] = F->mlo[level][d];
-        a.mn[d] = F->mn[level][d];
+template <class T, int P>
+gf_status launch_m2l_fold(FoldM2LArgs &a, cudaStream_t st) {
+    uint64_t blocks = 0;
+    for (int l = a.lmin; l <= a.lmax; ++l) {
+        a.lv[l].blk0 = (uint32_t)blocks;
+        blocks += (a.lv[l].ncol + (uint64_t)P - 1) / P;
     }
-    if (adj)
-        a.tab = sizeof(T) == 8 ? (const void *)F->tab->am2l_d : (const void *)F->tab->am2l_f;
-    else
-        a.tab = sizeof(T) == 8 ? (const void *)F->tab->m2l_d : (const void *)F->tab->m2l_f;
+    if (blocks == 0) return GF_OK;
+    const size_t shm = sizeof(T) * (size_t)((a.K + 3) & ~3) * 8 * P;
+    GF_TRY((ensure_smem(m2l_fold<T, P>, shm)));
+    const int threads = (a.K * Lay<T, P>::NG + 31) & ~31;
+    m2l_fold<T, P><<<(unsigned)blocks, threads, shm, st>>>(a);
+    GF_KERNEL_DONE();
+    return GF_OK;
+}
+
+// Every level of the M2L (adj: of its transpose) on the SIMT cores.
+template <class T>
+gf_status m2l_run_fold(gf_plan_s *plan, int B, bool adj, cudaStream_t st) {
+    FmmPlan *F = plan->fmm;
     if (B > 32) {
         set_error("M2L supports at most 32 batch members");
         return GF_ERR_UNSUPPORTED;
     }
-    const int64_t tiles = (maxc + a.nbox - 1) / a.nbox;
-    if (tiles == 0) return GF_OK;
-    const int rpt = (F->K + 31) / 32;
-    switch (rpt) {
-        case 1: return launch_simt<T, 1>(a, tiles, st);
-        case 2: return launch_simt<T, 2>(a, tiles, st);
-        case 3: return launch_simt<T, 3>(a, tiles, st);
-        case 4: return launch_simt<T, 4>(a, tiles, st);
-        case 5: return launch_simt<T, 5>(a, tiles, st);
-        case 6: return launch_simt<T, 6>(a, tiles, st);
-        case 7: return launch_simt<T, 7>(a, tiles, st);
-        case 8: return launch_simt<T, 8>(a, tiles, st);
-        case 9: return launch_simt<T, 9>(a, tiles, st);
-        case 10: return launch_simt<T, 10>(a, tiles, st);
-        default:
-            set_error("expansion degree too large for the M2L kernel");
-            return GF_ERR_UNSUPPORTED;
+    FoldM2LArgs a;
+    memset(&a, 0, sizeof(a));
+    int64_t total = 0;
+    for (int l = 2; l <= F->L; ++l) {
+        const FmmLevel &lv = F->lev[l];
+        FoldLevel &t = a.lv[l];
+        t.in = adj ? lv.le : lv.me;
+        t.out = adj ? lv.me : lv.le;
+        t.tkey = lv.tkey;
+        t.imap = F->imap[l];
+        for (int d = 0; d < 3; ++d) {
+            t.blo[d] = (int32_t)lv.slo[d];
+            t.bn[d] = (int32_t)lv.sn[d];
+            t.mlo[d] = (int32_t)F->mlo[l][d];
+            t.mn[d] = (int32_t)F->mn[l][d];
+        }
+        const int64_t ncol = (adj ? lv.ns : lv.nt) * B;
+        t.ncol = (uint32_t)ncol;
+        total += ncol;
+    }
+    if (total > (int64_t)0x7fffffff) {
+        set_error("too many expansions for one launch (%lld)", (long long)total);
+        return GF_ERR_UNSUPPORTED;
+    }
+    a.lmin = 2;
+    a.lmax = F->L;
+    a.K = F->K;
+    a.ldk = F->KS;
+    a.B = B;
+    a.adj = adj ? 1 : 0;
+    a.part_lo = adj ? 0u : plan->part_lo;
+    a.part_hi = adj ? 64u : plan->part_hi;
+    const Tables *Tb = F->tab;
+    a.tab = sizeof(T) == 8 ? (const void *)(adj ? Tb->am2l_d : Tb->m2l_d) : (const void *)(adj ? Tb->am2l_f : Tb->m2l_f);
+    // columns per block: more share a table element, fewer fill the SMs evenly
+    const int64_t sms = sm_count();
+    if constexpr (sizeof(T) == 8) {
+        if (total >= 8 * sms && F->K <= 256) return launch_m2l_fold<T, 4>(a, st);   // at most 512 threads
+        if (total >= sms) return launch_m2l_fold<T, 2>(a, st);
+        return launch_m2l_fold<T, 1>(a, st);
+    } else {
+        if (total >= 16 * sms) return launch_m2l_fold<T, 8>(a, st);
+        return launch_m2l_fold<T, 2>(a, st);
     }
 }
 
@@ -1308,11 +1341,7 @@ gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t
     if (tc) return m2l_run_tc(plan, B, adj, st, fork);
     if (!adj) stage_mark(plan, 4, st);   // no input split on this path
     if (fork) GF_CUDA(cudaEventRecord(fork, st));
-    for (int l = 2; l <= F->L; ++l) {
-        if (F->lev[l].nt == 0 && !adj) continue;   // the adjoint writes every source box
-        GF_TRY(m2l_level<T>(plan, l, B, adj, st));
-    }
-    return GF_OK;
+    return m2l_run_fold<T>(plan, B, adj, st);
 }
 
 template gf_status m2l_run<float>(gf_plan_s *, int, bool, cudaStream_t, cudaEvent_t);

@@ -18,8 +18,6 @@ gf_status m2l_prepare_tables(Tables *T, cudaStream_t st);
 // launched (after the input split).
 template <class T>
 gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t fork = nullptr);
-template <class T>
-gf_status m2l_level(gf_plan_s *plan, int level, int B, bool adj, cudaStream_t st);
 
 // Translations between levels (gf_xlate.cu; Ts = storage, Tc = arithmetic):
 //   kind 0  M2M into `level` from level + 1 (store)
