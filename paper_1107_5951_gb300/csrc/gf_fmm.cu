@@ -135,6 +135,24 @@ __global__ void compose_p2m_up(const double *__restrict__ P, const double *__res
     }
 }
 
+// The P2M matrices of position 7 transposed for the adjoint, rows in class
+// order: ut[c][v] = Q[v][perm_c], lt[c][v] = P[octant voxel v][perm_c] (zeros for
+// perm_c = -1).  One block per row.
+__global__ void transpose_p2m(const double *__restrict__ P, const double *__restrict__ Q, const int *__restrict__ perm,
+                              int K, double *__restrict__ utd, float *__restrict__ utf, double *__restrict__ ltd,
+                              float *__restrict__ ltf) {
+    const int c = blockIdx.x, v = threadIdx.x, k = perm[c];
+    const double q = k >= 0 ? Q[(size_t)v * K + k] : 0.0;
+    utd[c * 64 + v] = q;
+    utf[c * 64 + v] = (float)q;
+    if (v < 8) {
+        const double x =
+            k >= 0 ? P[(size_t)(((2 + (v >> 2)) * 4 + 2 + ((v >> 1) & 1)) * 4 + 2 + (v & 1)) * K + k] : 0.0;
+        ltd[c * 8 + v] = x;
+        ltf[c * 8 + v] = (float)x;
+    }
+}
+
 // P2M matrix of closed-form voxels (SUM-AN): P[v][k] = the k-th real component
 // of conj R((x - c)/b) integrated over voxel v (unit volume in voxel units),
 // by a Gauss-Legendre rule of m nodes per axis, exact for every regular solid
@@ -1347,9 +1365,23 @@ struct P2MEntry {
     float *pf = nullptr;
     double *ud = nullptr;  // 4^3-voxel leaves: P2M into the parent level from position 7 [64][K]
     float *uf = nullptr, *uq = nullptr;   // FP32 copy, and in quad order
+    double *utd = nullptr, *ltd = nullptr;   // transposes in class order [K][64], [K][8]
+    float *utf = nullptr, *ltf = nullptr;
 };
 std::mutex g_p2m_mu;
 std::vector<P2MEntry *> g_p2m;
+
+static void use_p2m(FmmPlan *F, const P2MEntry *e) {
+    F->p2m_d = e->pd;
+    F->p2m_f = e->pf;
+    F->p2m_up_d = e->ud;
+    F->p2m_up_f = e->uf;
+    F->p2m_up_q = e->uq;
+    F->p2m_upt_d = e->utd;
+    F->p2m_upt_f = e->utf;
+    F->p2m_leaft_d = e->ltd;
+    F->p2m_leaft_f = e->ltf;
+}
 
 gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
     FmmPlan *F = plan->fmm;
@@ -1359,11 +1391,7 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
     for (P2MEntry *e : g_p2m)
         if (e->device == plan->device && e->p == F->p && e->b == F->b && e->nq == q.nq && e->exact == exact &&
             !memcmp(e->xi, q.xi, sizeof(double) * 3 * q.nq) && !memcmp(e->wn, q.wn, sizeof(double) * q.nq)) {
-            F->p2m_d = e->pd;
-            F->p2m_f = e->pf;
-            F->p2m_up_d = e->ud;
-            F->p2m_up_f = e->uf;
-            F->p2m_up_q = e->uq;
+            use_p2m(F, e);
             return GF_OK;
         }
     P2MEntry *e = new P2MEntry();
@@ -1374,16 +1402,19 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
     e->exact = exact;
     memcpy(e->xi, q.xi, sizeof(double) * 3 * q.nq);
     memcpy(e->wn, q.wn, sizeof(double) * q.nq);
-    const int b3 = F->b * F->b * F->b, K = F->K;
+    const int b3 = F->b * F->b * F->b, K = F->K, KP = F->tab->cls_off[8];
     if (cudaMalloc(&e->pd, sizeof(double) * b3 * K) != cudaSuccess ||
         cudaMalloc(&e->pf, sizeof(float) * b3 * K) != cudaSuccess ||
         (F->b == 4 && (cudaMalloc(&e->ud, sizeof(double) * b3 * K) != cudaSuccess ||
-                       cudaMalloc(&e->uf, sizeof(float) * b3 * K) != cudaSuccess))) {
+                       cudaMalloc(&e->uf, sizeof(float) * b3 * K) != cudaSuccess ||
+                       cudaMalloc(&e->utd, sizeof(double) * b3 * KP) != cudaSuccess ||
+                       cudaMalloc(&e->utf, sizeof(float) * b3 * KP) != cudaSuccess ||
+                       cudaMalloc(&e->ltd, sizeof(double) * 8 * KP) != cudaSuccess ||
+                       cudaMalloc(&e->ltf, sizeof(float) * 8 * KP) != cudaSuccess))) {
         cudaGetLastError();
-        cudaFree(e->pd);
-        cudaFree(e->pf);
-        cudaFree(e->ud);
-        cudaFree(e->uf);
+        for (void *m : {(void *)e->pd, (void *)e->pf, (void *)e->ud, (void *)e->uf, (void *)e->utd, (void *)e->utf,
+                        (void *)e->ltd, (void *)e->ltf})
+            cudaFree(m);
         delete e;
         set_error("cannot allocate the P2M matrix");
         return GF_ERR_OOM;
@@ -1400,14 +1431,12 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
         compose_p2m_up<<<b3, 128, 0, st>>>(e->pd, F->tab->m2m_d + (size_t)7 * K * K, K, e->ud, e->uf);
         GF_KERNEL_DONE();
         GF_TRY(xlate_quad_table(F->tab, e->uf, b3, &e->uq, st));
+        transpose_p2m<<<KP, 64, 0, st>>>(e->pd, e->ud, F->tab->cls_perm, K, e->utd, e->utf, e->ltd, e->ltf);
+        GF_KERNEL_DONE();
     }
     GF_CUDA(cudaStreamSynchronize(st));   // other streams may use the cached matrix next
     g_p2m.push_back(e);
-    F->p2m_d = e->pd;
-    F->p2m_f = e->pf;
-    F->p2m_up_d = e->ud;
-    F->p2m_up_f = e->uf;
-    F->p2m_up_q = e->uq;
+    use_p2m(F, e);
     return GF_OK;
 }
 

@@ -66,6 +66,9 @@ struct Tables {
     int nquad = 0;
     int *quad_k = nullptr, *quad_info = nullptr;
     float *quad_f[4] = {};
+    int *cls_perm = nullptr;   // components grouped by parity class, ascending within one, each class
+                               // filled up to a multiple of four with -1
+    int cls_off[9] = {};       // class c: cls_perm[cls_off[c] .. cls_off[c + 1]); [8]: the length
 };
 
 gf_status get_tables(int device, int p, cudaStream_t st, const Tables **out);
@@ -100,6 +103,10 @@ struct FmmPlan {
     double *p2m_up_d = nullptr;
     float *p2m_up_f = nullptr;
     float *p2m_up_q = nullptr;    // the FP32 matrix in quad order [64][quad][4]
+    // the transposes for the adjoint, rows in class order (zeros where it has
+    // none): [cls_off[8]][64] (up) and [..][8] (the leaf's octant at position 7)
+    double *p2m_upt_d = nullptr, *p2m_leaft_d = nullptr;
+    float *p2m_upt_f = nullptr, *p2m_leaft_f = nullptr;
     const Tables *tab = nullptr;
     void *tc_levels = nullptr;                  // tensor-core M2L level table
     // largest |input| of each level's M2L (bits of a non-negative float;

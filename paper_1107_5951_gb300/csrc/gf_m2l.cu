@@ -348,6 +348,7 @@ struct TcLevel {
     int64_t blo[3], bn[3];
     int64_t cls_off[9];
     int adj;
+    int64_t slab0;        // adjoint: boxes of the source block before [blo, bn)
     const int32_t *imap;
     int64_t mlo[3], mn[3];
     const uint32_t *amax;        // largest |input| of the level (float bits)
@@ -912,7 +913,7 @@ m2l_tc(TcArgs a) {
                 } else {
                     int64_t ox, oy, oz;
                     class_box(pc.cls, L.blo, L.bn, os, ox, oy, oz);
-                    obox = (oz * L.bn[1] + oy) * L.bn[0] + ox;
+                    obox = L.slab0 + (oz * L.bn[1] + oy) * L.bn[0] + ox;
                 }
                 // 16-byte stores of the whole half row: columns from K up to
                 // Npad hold zeros (the operator images are zero there) and stay
@@ -975,6 +976,11 @@ gf_status m2l_tc_prepare_adj(gf_plan_s *plan) {
                 t.mlo[d] = F->mlo[l][d];
                 t.mn[d] = F->mn[l][d];
             }
+            if (adj) {   // output: the z-slabs an interaction list reaches
+                t.blo[2] += lv.m2l_z0;
+                t.bn[2] = std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
+                t.slab0 = lv.m2l_z0 * lv.sn[0] * lv.sn[1];
+            }
             for (int c = 0; c <= 8; ++c) t.cls_off[c] = adj ? F->scls_off[l][c] : lv.cls_off[c];
             t.amax = F->tc_amax + (adj ? kMaxLevels + 1 : 0) + l;
             t.split = (adj ? F->tc_split_adj : F->tc_split) + split_offset(F, adj, l);
@@ -1026,6 +1032,11 @@ gf_status m2l_tc_prepare(gf_plan_s *plan) {
                 t.bn[d] = lv.sn[d];
                 t.mlo[d] = F->mlo[l][d];
                 t.mn[d] = F->mn[l][d];
+            }
+            if (adj) {   // output: the z-slabs an interaction list reaches
+                t.blo[2] += lv.m2l_z0;
+                t.bn[2] = std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
+                t.slab0 = lv.m2l_z0 * lv.sn[0] * lv.sn[1];
             }
             for (int c = 0; c <= 8; ++c) t.cls_off[c] = adj ? F->scls_off[l][c] : lv.cls_off[c];
             t.amax = F->tc_amax + (adj ? kMaxLevels + 1 : 0) + l;
@@ -1302,7 +1313,14 @@ gf_status m2l_run_fold(gf_plan_s *plan, int B, bool adj, cudaStream_t st) {
             t.mlo[d] = (int32_t)F->mlo[l][d];
             t.mn[d] = (int32_t)F->mn[l][d];
         }
-        const int64_t ncol = (adj ? lv.ns : lv.nt) * B;
+        int64_t ncol = lv.nt * B;
+        if (adj) {   // the z-slabs an interaction list reaches
+            const int64_t slab = lv.sn[0] * lv.sn[1];
+            t.blo[2] += (int32_t)lv.m2l_z0;
+            t.bn[2] = (int32_t)std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
+            t.out = (T *)lv.me + lv.m2l_z0 * slab * B * F->KS;
+            ncol = t.bn[2] * slab * B;
+        }
         t.ncol = (uint32_t)ncol;
         total += ncol;
     }

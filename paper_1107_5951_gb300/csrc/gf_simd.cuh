@@ -301,5 +301,48 @@ __device__ __forceinline__ double f32_to_f64(float f) {
                                             ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 
+// h + l as a double, |l| <= |h| (a compensated FP32 pair), with integer
+// operations: the low part is added to the high part's bit pattern in units of
+// its last place (exact but for bits below the double's last place, which are
+// cut).  An FP64 addition takes as long as 64 of these instructions here.
+__device__ __forceinline__ double pair_to_f64(float h, float l) {
+    const float s = h + l, e = l - (s - h);
+    const unsigned sb = __float_as_uint(s), eb = __float_as_uint(e);
+    const int es = (int)((sb >> 23) & 0xff), ee = (int)((eb >> 23) & 0xff);
+    if (es == 0 || es == 0xff) return f32_to_f64(s);
+    unsigned long long v = ((unsigned long long)(es - 127 + 1023) << 52) | ((unsigned long long)(sb & 0x7fffffu) << 29);
+    if (ee != 0) {
+        const int sh = ee - es + 29;   // e = m 2^sh last places of s
+        const unsigned m = (eb & 0x7fffffu) | 0x800000u;
+        unsigned long long d = sh >= 0 ? (unsigned long long)m << min(sh, 30) : (sh > -32 ? (unsigned long long)(m >> -sh) : 0ull);
+        const bool opp = ((sb ^ eb) >> 31) != 0;
+        if (opp && (sb & 0x7fffffu) == 0) d <<= 1;   // below a power of two the places are half as wide
+        v = opp ? v - d : v + d;
+    }
+    return __longlong_as_double((long long)(v | ((unsigned long long)(sb >> 31) << 63)));
+}
+
+// A scale factor x = (h + l) 2^e, h + l in [1, 2) to 2^-47, for compensated FP32
+// results; |e| <= 800 (scale_pair: false beyond, or x not positive).
+struct ScalePair {
+    float h, l;
+    int e;
+};
+// (h + l) x as a double
+__device__ __forceinline__ double scaled_pair(float h, float l, ScalePair k) {
+    const float p = h * k.h;
+    const long long r = __double_as_longlong(pair_to_f64(p, fmaf(h, k.h, -p) + fmaf(h, k.l, l * k.h)));
+    const int ex = (int)((r >> 52) & 0x7ff);
+    return __longlong_as_double(ex == 0 || ex == 0x7ff ? r : r + ((long long)k.e << 52));
+}
+inline bool scale_pair(double x, ScalePair &k) {
+    int e = 0;
+    const double f = 2.0 * std::frexp(x, &e);   // x = f 2^(e - 1)
+    k.h = (float)f;
+    k.l = (float)(f - (double)k.h);
+    k.e = e - 1;
+    return f >= 1.0 && f < 2.0 && e > -800 && e < 800;
+}
+
 }  // namespace
 }  // namespace gf

@@ -762,6 +762,15 @@ gf_status xlate_prepare_tables(Tables *T, cudaStream_t st) {
             ++n;
         }
     }
+    std::vector<int> perm;
+    for (int c = 0; c < 8; ++c) {
+        T->cls_off[c] = (int)perm.size();
+        for (const Quad &q : quads)   // before the sort by degree: classes in turn, each a whole number of quads
+            if (q.cls == c) perm.insert(perm.end(), q.k, q.k + 4);
+    }
+    T->cls_off[8] = (int)perm.size();
+    GF_CUDA(cudaMalloc(&T->cls_perm, perm.size() * sizeof(int)));
+    GF_TRY(upload_small(T->cls_perm, perm.data(), perm.size() * sizeof(int), st));
     std::stable_sort(quads.begin(), quads.end(), [](const Quad &x, const Quad &y) { return x.hi < y.hi; });
     T->nquad = (int)quads.size();
     std::vector<int> qk, info;

@@ -35,3 +35,8 @@ def test_many_columns_match_few(p, n):
         for b in (0, 15):
             ref = few.adjoint(r[b])
             assert float((grad[b] - ref).norm() / ref.norm()) <= 2e-6
+        r = torch.randn((16, wk.n_obs, 3), generator=gen, device=DEV, dtype=torch.float64)
+        grad = many.adjoint(r, ncomp=3)
+        for b in (0, 15):
+            ref = few.adjoint(r[b], ncomp=3)
+            assert float((grad[b] - ref).norm() / ref.norm()) <= 2e-6
