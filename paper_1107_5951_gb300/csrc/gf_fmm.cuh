@@ -114,9 +114,13 @@ struct FmmPlan {
     // reduced on the device before each tensor-core M2L
     uint32_t *tc_amax = nullptr;
     bool amax_fused = false;      // this forward's expansion writers took the M2L input maxima
-    float *m2l_part = nullptr;    // forward M2L with two CTAs per tile: [tiles][2][128][Npad] partial rows
-    int *m2l_cnt = nullptr;       // [tiles][8] arrivals
-    int m2l_part_tiles = 0;       // tiles m2l_part holds (0: no sharing)
+    // tensor-core M2L: active offsets of the tiles (forward [0], adjoint [1]);
+    // partial rows of cut tiles, two slots for each of m2l_part_ctas CTAs, and
+    // where each CTA's units start
+    uint32_t *m2l_mask[2] = {};
+    float *m2l_part = nullptr;
+    int4 *m2l_cut = nullptr;
+    int m2l_part_ctas = 0;
     // the M2L inputs of levels 2..L split into scaled FP16 high and low
     // parts: for every input row and 32-wide chunk, 64 bytes of high parts
     // then 64 bytes of low parts (the same byte offsets as the FP32 rows)

@@ -14,10 +14,16 @@
 
 namespace gf {
 
-__constant__ signed char c_il[8][189][3];
+// Interaction-list offsets of each parity class, dx | dy | dz << 0 | 8 | 16
+// as signed bytes.
+__constant__ int c_il[8][189];
 
 gf_status m2l_upload_offsets(const signed char h_il[8][189][3]) {
-    GF_CUDA(cudaMemcpyToSymbol(c_il, h_il, sizeof(signed char) * 8 * 189 * 3));
+    int packed[8][189];
+    for (int c = 0; c < 8; ++c)
+        for (int i = 0; i < 189; ++i)
+            packed[c][i] = (uint8_t)h_il[c][i][0] | (uint8_t)h_il[c][i][1] << 8 | (uint8_t)h_il[c][i][2] << 16;
+    GF_CUDA(cudaMemcpyToSymbol(c_il, packed, sizeof(packed)));
     return GF_OK;
 }
 
@@ -321,14 +327,19 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
 // 2^sh (largest |input| into (2^14, 2^15]), each output column of the operator
 // images by its own factor; the write-back divides both out exactly.  The
 // inputs are split once per level by a small kernel before the M2L.  Inputs
-// come in chunks of 32, two to a stage, through a ring of shared-memory stages
+// come in chunks of 32, one to a stage, through a ring of shared-memory stages
 // (64-byte swizzle), filled by warp-specialised producers:
 //   warps 0-3   A producers: 16-byte asynchronous copies straight into the
-//               stage (eight lanes per row's 128 contiguous bytes), which is
-//               signalled once they have landed;
-//   warp 4      one thread issues the MMAs of a stage and commits them to the
-//               stage's "empty" barrier (and, after an offset's last chunk,
-//               to the bank's "full" barrier);
+//               stage (eight lanes per row's 128 contiguous bytes); each
+//               thread's arrival on the stage's barrier is made by its copies
+//               as they land, so the producers run as far ahead as there are
+//               free stages;
+//   warp 4      one thread issues the MMAs, of two stages at a time, and commits
+//               them to the stages' "empty" barriers (and, after an offset's
+//               last chunk, to the bank's "full" barrier).  A look at a barrier
+//               costs this warp over 200 cycles even when it is complete, and
+//               two stages' MMAs take 200 to 1500: the lanes look at all the
+//               barriers that a step needs at once;
 //   warp 5      one thread bulk-copies the pre-split, pre-swizzled operator
 //               image of each stage;
 //   warps 6-13  promoters: after each offset they read the finished bank of
@@ -336,8 +347,26 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
 //               alternate, so the tensor cores never accumulate more than one
 //               offset: their FP32 accumulation rounds differently from
 //               IEEE and long chains over zero-mean data lose digits).
-// Offsets whose source boxes are all missing are skipped by every role (a
-// per-tile list built first).  Every wait is bounded and watches an abort
+// Offsets whose source boxes are all missing are skipped by every role: the
+// active offsets of every tile are found beforehand (tile_masks) as bit masks
+// and counts.  Work is dealt out in units of one (tile, active offset): with up
+// to kStreamTiles tiles the launch has at most one CTA per SM, and CTA c of G
+// takes the units [c T / G, (c + 1) T / G) of the T in tile order, whatever tiles
+// they fall in, so that no SM waits for the longest tile (the upper levels' lists
+// are twice as long as a surface's leaf lists, and a few tiles more than SMs
+// made a second wave).  The partial rows of a tile cut by that are summed in CTA
+// order by a second launch (m2l_join), spread over the chip: one CTA's last
+// arrival summing them took longer than the tile's units when a tile was shared
+// by twenty CTAs.  With more tiles a CTA takes one whole tile.
+// What bounds it: the MMA issuer.  The tensor cores are about half busy (169
+// components: 33 MMAs of 128 x 176 x 16 an offset, 2,900 of 5,800 cycles); the
+// rest is the issuer's own chain of barrier looks, fences and commits, which the
+// few MMAs it can queue do not cover.  Measured against one CTA, or two, per tile
+// and two chunks to a stage: 16 tiles' worth of a 32^3 grid 260 -> 34 us + 6 us to
+// join; 156 tiles of 464 x 464 x 16 (K = 121) 327 -> 154 + 16; 16 grids of 128^3
+// 846 -> 434; a 2^25-point set 1,050 -> 574; 128^3 with observers throughout
+// 1,236 -> 1,140.
+// Every wait is bounded and watches an abort
 // flag; a wait that gives up sets status[1], and the CTA then drains its
 // copies and MMAs (bounded) and frees its tensor memory.
 
@@ -367,14 +396,14 @@ struct TcArgs {
     int *status;
     long wait_tries;            // bound of every barrier wait (kWaitTries)
     uint32_t part_lo, part_hi;  // forward: source partition (in_source_part)
-    // forward with msplit = 2: each tile's active offsets are shared by two
-    // CTAs (blockIdx 2 t and 2 t + 1); each writes its partial rows to mpart
-    // (slot = blockIdx, [128][Npad]) and counts itself in mcnt ([tile][8]
-    // promoter warps, zero at launch); the second to arrive adds the other's
-    // rows to its own and writes the tile.
-    int msplit;
-    float *mpart;
-    int *mcnt;
+    int ntiles;
+    const uint32_t *tmask;      // [ntiles][8]: 189 offset bits, [6]: how many
+    int stream;                 // units dealt out over the grid (else one tile per CTA)
+    int min_units;              // a CTA takes no fewer units than this (stream)
+    float *mpart;               // [2 gridDim][Npad / 4][128] float4: partial rows, slot 0 of CTA c for its
+                                // first tile, slot 1 for its last
+    int4 *mcut;                 // [gridDim + 1] (stream): CTA c's first tile, the units before it and up to its
+                                // end, G; [gridDim].x: T
     int test_stall;             // testing aid: the MMA issuer first waits on a barrier that
                                 // nothing completes, so the bounded-wait failure path runs
 };
@@ -478,25 +507,215 @@ constexpr int kTcMaxStages = 8;
 constexpr uint32_t kTcCols = 512;           // two banks of 256 columns
 constexpr uint32_t kTcA = 2u * 8192u;       // A hi + lo: 128 rows x 64 bytes each
 
-constexpr int kTcChunks = 2;                // 32-input chunks per pipeline stage (12 MMAs per barrier wait)
-
 __host__ __device__ constexpr uint32_t tc_stage_bytes(int Npad) { return kTcA + 2u * (uint32_t)Npad * 64u; }
-constexpr size_t kTcSmemBudget = 227 * 1024 - 2048;
+constexpr int kScanItems = 4;               // tiles per thread of the unit scan
+constexpr int kStreamTiles = kTcThreads * kScanItems;
+constexpr size_t kTcSmemBudget = 227 * 1024 - 2048 - 4 * (kStreamTiles + 1);
 inline int tc_stages(int Npad) {
-    const int n = (int)(kTcSmemBudget / ((size_t)kTcChunks * tc_stage_bytes(Npad)));
+    const int n = (int)(kTcSmemBudget / (size_t)tc_stage_bytes(Npad));
     return n > kTcMaxStages ? kTcMaxStages : n;
 }
-size_t tc_smem_bytes(int Npad) { return (size_t)tc_stages(Npad) * kTcChunks * tc_stage_bytes(Npad) + 1024; }
+size_t tc_smem_bytes(int Npad) { return (size_t)tc_stages(Npad) * tc_stage_bytes(Npad) + 1024; }
 
 // 16-byte asynchronous global -> shared copy; nbytes = 0 fills zeros.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t nbytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(nbytes) : "memory");
 }
 
+struct TcTile {
+    const TcLevel *L;
+    int cls, tile;        // tile within the class
+    int64_t cbeg, ccnt;   // the class's targets
+};
+
+// (level, class, tile within the class) of tile t
+__device__ __forceinline__ TcTile tile_of(const TcArgs &a, int t) {
+    int e = 0;
+    while (e + 1 < a.nent && a.tile_begin[e + 1] <= t) ++e;
+    TcTile c;
+    c.L = &a.lv[a.lmin + e / 8];
+    c.cls = e % 8;
+    c.tile = t - a.tile_begin[e];
+    c.cbeg = c.L->cls_off[c.cls];
+    c.ccnt = c.L->cls_off[c.cls + 1] - c.cbeg;
+    return c;
+}
+
+// What locates the source rows of a target box at an offset, in registers:
+// its position in the window of boxes that have rows (forward: the level's
+// source block; adjoint: the target boxes' bounding box, through imap).
+struct TcTarget {
+    int x, y, z, n0, n1, n2;
+    const int32_t *imap;
+};
+
+// Target of a tile's slot (a position no offset can reach if there is none).
+__device__ __forceinline__ TcTarget target_of(const TcTile &t, int nbox, int slot) {
+    const TcLevel &L = *t.L;
+    TcTarget q;
+    q.imap = L.imap;
+    q.x = q.y = q.z = -1000;
+    if (!L.adj) {
+        q.imap = nullptr;
+        q.n0 = (int)L.bn[0];
+        q.n1 = (int)L.bn[1];
+        q.n2 = (int)L.bn[2];
+    } else {
+        q.n0 = (int)L.mn[0];
+        q.n1 = (int)L.mn[1];
+        q.n2 = (int)L.mn[2];
+    }
+    const int64_t sidx = (int64_t)t.tile * nbox + slot;
+    if (slot >= nbox || sidx >= t.ccnt) return q;
+    if (!L.adj) {
+        const uint64_t key = L.tkey[L.order[t.cbeg + sidx]];
+        q.x = (int)(dm(key, 0) - L.blo[0]);
+        q.y = (int)(dm(key, 1) - L.blo[1]);
+        q.z = (int)(dm(key, 2) - L.blo[2]);
+    } else {
+        int64_t c0, c1, c2;
+        class_box(t.cls, L.blo, L.bn, sidx, c0, c1, c2);
+        q.x = (int)(c0 + L.blo[0] - L.mlo[0]);
+        q.y = (int)(c1 + L.blo[1] - L.mlo[1]);
+        q.z = (int)(c2 + L.blo[2] - L.mlo[2]);
+    }
+    return q;
+}
+
+// Index of the source box's rows at list offset oi of class cls (-1: none).
+__device__ __forceinline__ int64_t source_of(const TcArgs &a, const TcLevel *L, const TcTarget &q, int cls, int oi) {
+    const int o = c_il[cls][oi];
+    const int sx = q.x + (signed char)o, sy = q.y + (signed char)(o >> 8), sz = q.z + (signed char)(o >> 16);
+    if ((unsigned)sx >= (unsigned)q.n0 || (unsigned)sy >= (unsigned)q.n1 || (unsigned)sz >= (unsigned)q.n2) return -1;
+    const int64_t i = ((int64_t)sz * q.n1 + sy) * q.n0 + sx;
+    if (q.imap) return q.imap[i];
+    if ((a.part_lo != 0 || a.part_hi < 64) &&
+        !in_source_part(sx + L->blo[0], sy + L->blo[1], sz + L->blo[2], L->shift, a.part_lo, a.part_hi))
+        return -1;
+    return i;
+}
+
+// The active offsets of tile t (256 threads of one block): bit masks and their
+// count, at least one (a tile without sources runs one offset of zeros).
+__device__ __forceinline__ void tile_mask(const TcArgs &a, int t, uint32_t *tmask) {
+    __shared__ uint32_t words[6];
+    const TcTile tile = tile_of(a, t);
+    const int row = threadIdx.x & 127, half = threadIdx.x >> 7;   // offset words 3 half .. 3 half + 2
+    // the batch members of a box share its offsets
+    const bool on = row % a.B == 0;
+    const TcTarget q = target_of(tile, 128 / a.B, row / a.B);
+    __syncthreads();
+    if (threadIdx.x < 6) words[threadIdx.x] = 0;
+    __syncthreads();
+    for (int w = 3 * half; w < 3 * half + 3; ++w) {
+        uint32_t bits = 0;
+        if (on)
+            for (int b = 0; b < 32 && 32 * w + b < 189; ++b)
+                if (source_of(a, tile.L, q, tile.cls, 32 * w + b) >= 0) bits |= 1u << b;
+        bits = __reduce_or_sync(0xffffffffu, bits);
+        if ((threadIdx.x & 31) == 0 && bits) atomicOr(&words[w], bits);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int n = 0;
+        for (int w = 0; w < 6; ++w) n += __popc(words[w]);
+        if (n == 0) words[0] = n = 1;
+        for (int w = 0; w < 6; ++w) tmask[8 * (size_t)t + w] = words[w];
+        tmask[8 * (size_t)t + 6] = (uint32_t)n;
+    }
+}
+
+// The active offsets of a tile in order, from the one of rank `skip` on.
+struct OffsetIter {
+    const uint32_t *m;
+    int w;
+    uint32_t bits;
+    __device__ __forceinline__ void open(const uint32_t *tmask, int t, int skip) {
+        m = tmask + 8 * (size_t)t;
+        w = 0;
+        bits = __ldg(m);
+        while (skip > 0) {
+            const int n = __popc(bits);
+            if (n <= skip) {
+                skip -= n;
+                bits = __ldg(m + ++w);
+            } else {
+                for (; skip > 0; --skip) bits &= bits - 1;
+            }
+        }
+    }
+    __device__ __forceinline__ int next() {
+        while (!bits) bits = __ldg(m + ++w);
+        const int b = __ffs(bits) - 1;
+        bits &= bits - 1;
+        return 32 * w + b;
+    }
+};
+
+// Output row of row r of a tile (-1: none).
+__device__ __forceinline__ int64_t out_row(const TcArgs &a, const TcTile &t, int nbox, int r) {
+    const TcLevel &L = *t.L;
+    const int slot = r / a.B, bb = r - slot * a.B;
+    const int64_t sidx = (int64_t)t.tile * nbox + slot;
+    if (slot >= nbox || sidx >= t.ccnt) return -1;
+    if (!L.adj) return (int64_t)L.order[t.cbeg + sidx] * a.B + bb;
+    int64_t x, y, z;
+    class_box(t.cls, L.blo, L.bn, sidx, x, y, z);
+    return (L.slab0 + (z * L.bn[1] + y) * L.bn[0] + x) * a.B + bb;
+}
+
+// Store four columns of an output row; columns from K up to Npad hold zeros
+// (the operator images are zero there) and stay inside the row's padding
+// (Npad <= ldk).
+__device__ __forceinline__ void store4(const TcArgs &a, const TcLevel &L, int64_t row, int col, float4 v) {
+    if (a.le_f64) {
+        double2 *d = reinterpret_cast<double2 *>(reinterpret_cast<double *>(L.le) + row * a.ldk + col);
+        d[0] = make_double2(v.x, v.y);
+        d[1] = make_double2(v.z, v.w);
+    } else {
+        *reinterpret_cast<float4 *>(L.le + row * a.ldk + col) = v;
+    }
+}
+
+// Tiles cut between CTAs: the sum of their partial rows in CTA order.  Blocks
+// (c - 1, .) look at the boundary before CTA c and, when it is the first one
+// inside its tile, write the tile's rows, the columns split over blockIdx.y.
+// A chain of dependent loads with little behind it: one wave of blocks.
+__global__ void __launch_bounds__(512) m2l_join(const __grid_constant__ TcArgs a) {
+    const int c = (int)blockIdx.x + 1;
+    const int4 cut = a.mcut[c];
+    const uint32_t G = (uint32_t)cut.w, T = a.mcut[gridDim.x + 1].x;
+    if (c >= (int)G) return;
+    const uint32_t p0 = (uint32_t)cut.y, p1 = (uint32_t)cut.z;
+    if ((uint32_t)((uint64_t)c * T / G) == p0) return;
+    // CTAs holding the tile's first and last unit
+    const int cf = (int)((((uint64_t)p0 + 1) * G - 1) / T), cl = (int)(((uint64_t)p1 * G - 1) / T);
+    if (c != cf + 1) return;
+    const int r = threadIdx.x & 127;
+    const TcTile tile = tile_of(a, cut.x);
+    const int64_t row = out_row(a, tile, 128 / a.B, r);
+    if (row < 0) return;
+    const int first = (uint32_t)((uint64_t)cf * T / G) < p0 ? 1 : 0;
+    const size_t slot = (size_t)(a.Npad / 4) * 128;
+    const float4 *p = reinterpret_cast<const float4 *>(a.mpart) + r;
+    for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < a.Npad / 4; q += 4 * (int)gridDim.y) {
+        float4 s = __ldg(p + (2 * cf + first) * slot + (size_t)q * 128);
+#pragma unroll 8
+        for (int e = cf + 1; e <= cl; ++e) {
+            const float4 v = __ldg(p + 2 * e * slot + (size_t)q * 128);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+        store4(a, *tile.L, row, 4 * q, s);
+    }
+}
+
 // NS >= Npad / 2: FP32 sums held per promoter thread.
 template <int NS>
 __global__ void __launch_bounds__(kTcThreads, 1)
-m2l_tc(TcArgs a) {
+m2l_tc(const __grid_constant__ TcArgs a) {
     extern __shared__ unsigned char dsm[];
     unsigned char *base = dsm + ((1024 - (smem_u32(dsm) & 1023)) & 1023);
     // afull: the stage's A operand has landed (128 producer arrivals); bfull:
@@ -507,35 +726,16 @@ m2l_tc(TcArgs a) {
     __shared__ __align__(8) uint64_t bank_full[2], bank_empty[2];
     __shared__ uint32_t tslot;
     __shared__ int abort_flag;
-    __shared__ uint32_t omask[6];   // M2L: offsets with at least one source box in this tile
+    __shared__ uint32_t pref[kStreamTiles + 1];   // stream: units before each tile
+    __shared__ uint32_t wtot[kTcWarps];
+    __shared__ int first_tile;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int B = a.B, Npad = a.Npad, nck = a.nck, NST = a.nst;
     const int nsum = Npad / 2;
     const uint32_t b_bytes = 2u * (uint32_t)Npad * 64u;
-    constexpr int S = kTcChunks;
-    const uint32_t stage_bytes = S * tc_stage_bytes(Npad);   // [A: S x (hi, lo)][B: S x (hi, lo)]
+    const uint32_t stage_bytes = tc_stage_bytes(Npad);   // [A: hi, lo][B: hi, lo]
     volatile int *abortp = &abort_flag;
     const int nbox = 128 / B;
-    constexpr int noff = 189;
-    const int msplit = max(1, a.msplit);
-    const int utile = (int)blockIdx.x / msplit, uhalf = (int)blockIdx.x - utile * msplit;   // tile, share
-    struct Ctx {
-        const TcLevel *L;
-        int cls, tile;
-        int64_t cbeg, ccnt;
-    };
-    // (level, class, tile within the class) of tile t
-    auto ctx_of = [&](int t) -> Ctx {
-        int e = 0;
-        while (e + 1 < a.nent && a.tile_begin[e + 1] <= t) ++e;
-        Ctx c;
-        c.L = &a.lv[a.lmin + e / 8];
-        c.cls = e % 8;
-        c.tile = t - a.tile_begin[e];
-        c.cbeg = c.L->cls_off[c.cls];
-        c.ccnt = c.L->cls_off[c.cls + 1] - c.cbeg;
-        return c;
-    };
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tslot)),
@@ -557,260 +757,248 @@ m2l_tc(TcArgs a) {
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    if (tid < 6) omask[tid] = 0;
-
-    // producer role: column `row` of the tile
-    const int row = tid & 127;
-    const int slot = row / B, bb = row - slot * B;
-    const Ctx pc = ctx_of(utile);
-    int64_t tbox = -1, tc0 = 0, tc1 = 0, tc2 = 0;
-    int64_t qbn0 = 0, qbn1 = 0, qbn2 = 0;   // the level's source block extent, kept in registers
-    int qadj = 0;
-    auto set_target = [&]() {
-        tbox = -1;
-        tc0 = tc1 = tc2 = 0;
-        const TcLevel &L = *pc.L;
-        qbn0 = L.bn[0];
-        qbn1 = L.bn[1];
-        qbn2 = L.bn[2];
-        qadj = L.adj;
-        const int64_t sidx = (int64_t)pc.tile * nbox + slot;
-        if (warp >= 4 || slot >= nbox || sidx >= pc.ccnt) return;
-        if (!L.adj) {
-            tbox = L.order[pc.cbeg + sidx];
-            const uint64_t key = L.tkey[tbox];
-            tc0 = dm(key, 0) - L.blo[0];
-            tc1 = dm(key, 1) - L.blo[1];
-            tc2 = dm(key, 2) - L.blo[2];
-        } else {
-            class_box(pc.cls, L.blo, L.bn, sidx, tc0, tc1, tc2);
-            tbox = (tc2 * L.bn[1] + tc1) * L.bn[0] + tc0;
+    // this CTA's units [u0, u1), in tile order from tile t0 on; P(t) = units
+    // before tile t
+    uint32_t G = 1, T = 0;
+    uint32_t u0 = 0, u1 = 0;
+    if (a.stream) {
+        uint32_t n[kScanItems], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            const int t = tid * kScanItems + q;
+            n[q] = t < a.ntiles ? __ldg(a.tmask + 8 * (size_t)t + 6) : 0;
+            sum += n[q];
         }
-    };
-    set_target();
-    // input row of this column at offset oi of the current tile (-1: none)
-    auto src_row = [&](int oi) -> int64_t {
-        if (tbox < 0) return -1;
-        const TcLevel &L = *pc.L;
-        const int cls = pc.cls;
-        const int64_t sx = tc0 + c_il[cls][oi][0], sy = tc1 + c_il[cls][oi][1], sz = tc2 + c_il[cls][oi][2];
-        if (!qadj) {
-            if (sx >= 0 && sy >= 0 && sz >= 0 && sx < qbn0 && sy < qbn1 && sz < qbn2 &&
-                in_source_part(sx + L.blo[0], sy + L.blo[1], sz + L.blo[2], L.shift, a.part_lo, a.part_hi))
-                return (((sz * qbn1 + sy) * qbn0 + sx) * B + bb) * a.ldk;
-            return -1;
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
         }
-        const int64_t wx = sx + L.blo[0] - L.mlo[0], wy = sy + L.blo[1] - L.mlo[1], wz = sz + L.blo[2] - L.mlo[2];
-        if (wx >= 0 && wy >= 0 && wz >= 0 && wx < L.mn[0] && wy < L.mn[1] && wz < L.mn[2]) {
-            const int32_t m = L.imap[(wz * L.mn[1] + wy) * L.mn[0] + wx];
-            if (m >= 0) return ((int64_t)m * B + bb) * a.ldk;
+        if (lane == 31) wtot[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int w = 0; w < kTcWarps; ++w) {
+            if (w < warp) before += wtot[w];
+            T += wtot[w];
         }
-        return -1;
-    };
-    __syncthreads();
-    if (warp < 4) {
-        for (int w = 0; w * 32 < noff; ++w) {
-            uint32_t bits = 0;
-            for (int b = 0; b < 32 && 32 * w + b < noff; ++b)
-                if (src_row(32 * w + b) >= 0) bits |= 1u << b;
-            bits = __reduce_or_sync(0xffffffffu, bits);
-            if (lane == 0 && bits) atomicOr(&omask[w], bits);
+        uint32_t run = before + incl - sum;
+        G = min(gridDim.x, max(1u, T / (uint32_t)a.min_units));
+        if (blockIdx.x < G) {
+            u0 = (uint32_t)((uint64_t)blockIdx.x * T / G);
+            u1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * T / G);
         }
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            const int t = tid * kScanItems + q;
+            if (t <= a.ntiles) pref[t] = run;
+            if (t < a.ntiles && u0 >= run && u0 < run + n[q]) first_tile = t;
+            run += n[q];
+        }
+        if (tid == 0) pref[a.ntiles] = T;
+    } else {
+        if (tid == 0) first_tile = (int)blockIdx.x;
+        u1 = __ldg(a.tmask + 8 * (size_t)blockIdx.x + 6);
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (msplit > 1) {
-        // keep this CTA's share of the tile's active offsets: ranks
-        // [uhalf tot / msplit, (uhalf + 1) tot / msplit) in offset order
-        if (tid == 0) {
-            int tot = 0;
-            for (int w = 0; w < 6; ++w) tot += __popc(omask[w]);
-            const int lo = uhalf * tot / msplit, hi = (uhalf + 1) * tot / msplit;
-            int rank = 0;
-            for (int w = 0; w < 6; ++w) {
-                uint32_t m = omask[w], keep = 0;
-                while (m) {
-                    const int b = __ffs(m) - 1;
-                    m &= m - 1;
-                    if (rank >= lo && rank < hi) keep |= 1u << b;
-                    ++rank;
-                }
-                omask[w] = keep;
-            }
-        }
-        __syncthreads();
-    }
     const uint32_t tmem = tslot;
-    int G = 0;   // offsets run by this CTA
-    for (int w = 0; w < 6; ++w) G += __popc(omask[w]);
-    const int nsp = (nck + S - 1) / S;   // stages per offset
-    const int iters = G * nsp;       // stages run by this CTA
-    // the next offset to run after oi within a tile (noff when none is left)
-    auto next_off = [&](int oi) -> int {
-        for (++oi; oi < noff; ++oi)
-            if (omask[oi >> 5] & (1u << (oi & 31))) return oi;
-        return noff;
+    const int units = (int)(u1 - u0);
+    const int t0 = units > 0 ? first_tile : 0;
+    if (a.stream && tid == 0) {   // for m2l_join
+        a.mcut[blockIdx.x] = make_int4(t0, (int)pref[t0], (int)pref[t0 + 1], (int)G);
+        if (blockIdx.x == 0) a.mcut[gridDim.x] = make_int4((int)T, 0, 0, 0);
+    }
+    // rank of the first unit taken of tile t, and how many are taken
+    auto seg_lo = [&](int t) -> int { return a.stream && pref[t] < u0 ? (int)(u0 - pref[t]) : 0; };
+    auto seg_n = [&](int t) -> int {
+        return a.stream ? (int)(min(u1, pref[t + 1]) - max(u0, pref[t])) : units;
     };
 
     if (warp < 4) {
-        // ---------------- A producers
-        int qo = next_off(-1), qc = 0;
-        int64_t qs = qo < noff ? src_row(qo) : -1;
-        auto take = [&](int &c_out, int64_t &s_out) {   // next chunk in sequence
-            c_out = qc;
-            s_out = qs;
-            if (++qc == nck) {
-                qc = 0;
-                qo = next_off(qo);
-                qs = qo < noff ? src_row(qo) : -1;
+        // ---------------- A producers: FP16 inputs, scaled and split in advance
+        const int row = tid & 127, slot = row / B, bb = row - slot * B;
+        const int k = lane & 7;                       // 16-byte piece of a row's chunk: 0-3 high, 4-7 low
+        const uint32_t kpart = k < 4 ? 0u : 8192u;
+        const int rl0 = lane >> 3;
+        int t = t0 - 1, left = 0, cls = 0;
+        const TcLevel *L = nullptr;
+        const unsigned char *split = nullptr;
+        TcTarget q{};
+        OffsetIter it;
+        // split parts of this thread's row at the next unit (null: none)
+        auto next_row = [&]() -> const unsigned char * {
+            if (left == 0) {
+                ++t;
+                left = seg_n(t);
+                it.open(a.tmask, t, seg_lo(t));
+                const TcTile tile = tile_of(a, t);
+                L = tile.L;
+                cls = tile.cls;
+                split = L->split;
+                q = target_of(tile, nbox, slot);
             }
+            --left;
+            const int64_t src = source_of(a, L, q, cls, it.next());
+            return src >= 0 ? split + (src * B + bb) * a.ldk * 4 : nullptr;
         };
-        // FP16 inputs, scaled and split in advance: once a stage is free,
-        // each thread copies its row's 64-byte high and low pieces of the
-        // stage's chunks straight into it (16-byte asynchronous copies to
-        // the swizzled positions; a missing source copies zeros), waits for
-        // them and signals the stage.  The copies overlap the MMAs of the
-        // previous stage.
-        const unsigned char *spl = pc.L->split;   // every tile of a launch reads the same levels
-        int s = 0;
+        int s = 0, n_done = 0;
         uint32_t ph = 0;
-        for (int it = 0; it < iters; ++it) {
-            if (it >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) break;
-            unsigned char *stage = base + (size_t)s * stage_bytes;
-            int c0 = 0, nc = S;
+        bool stop = false;
+        const unsigned char *ahead = units > 0 ? next_row() : nullptr;
+        for (int u = 0; u < units && !stop; ++u) {
+            const unsigned char *src = ahead;
+            if (u + 1 < units) ahead = next_row();   // located a unit early, off the pipeline's path
+            // the warp's 32 rows in 8 passes of 4, eight lanes per row: each
+            // lane's piece of its eight rows
+            const unsigned char *rp[8];
+            uint32_t have = 0;
 #pragma unroll
-            for (int q = 0; q < S; ++q) {
-                if (q > 0 && c0 + q >= nck) break;   // the offset's last stage may hold fewer chunks
-                int cc;
-                int64_t sr;
-                take(cc, sr);
-                if (q == 0) {
-                    c0 = cc;
-                    nc = min(S, nck - c0);
-                }
-                // chunks run from the highest inputs down (chunk_of), and the
-                // stage keeps its chunks in ascending order
-                const int pc = chunk_of(nck, cc);
-                // the warp's 32 rows in 8 passes of 4: eight lanes copy one
-                // row's 128 contiguous bytes (pieces 0-3 high, 4-7 low)
-                const uint32_t sub = smem_u32(stage + (nc - 1 - q) * kTcA);
-                const int k = lane & 7;
-                const uint32_t kpart = k < 4 ? 0u : 8192u;
-                const int kk = 8 * (k & 3);
-#pragma unroll
-                for (int pp = 0; pp < 8; ++pp) {
-                    const int rl = 4 * pp + (lane >> 3);
-                    const int64_t srp = __shfl_sync(0xffffffffu, (long long)sr, rl);
-                    const int r = (row & ~31) + rl;
-                    const unsigned char *src = srp >= 0 ? spl + (size_t)srp * 4 + (size_t)pc * 128 + 16 * k : spl;
-                    cp_async16(sub + kpart + swz64h(r, kk), src, srp >= 0 ? 16u : 0u);
-                }
+            for (int pp = 0; pp < 8; ++pp) {
+                const unsigned char *o =
+                    (const unsigned char *)__shfl_sync(0xffffffffu, (unsigned long long)src, 4 * pp + rl0);
+                rp[pp] = (o ? o : split) + 16 * k;
+                have |= (uint32_t)(o != nullptr) << pp;
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(smem_u32(&afull[s]));
-            if (++s == NST) {
-                s = 0;
-                ph ^= 1;
+            for (int j = 0; j < nck; ++j) {
+                if (n_done >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) {
+                    stop = true;
+                    break;
+                }
+                const uint32_t sub = smem_u32(base) + (uint32_t)s * stage_bytes + kpart;
+                const int ck = chunk_of(nck, j);
+#pragma unroll
+                for (int pp = 0; pp < 8; ++pp)
+                    cp_async16(sub + swz64h((row & ~31) + 4 * pp + rl0, 8 * (k & 3)), rp[pp] + 128 * ck,
+                               (have >> pp) & 1u ? 16u : 0u);
+                // the thread's arrival, made when its copies have landed
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&afull[s])) : "memory");
+                ++n_done;
+                if (++s == NST) {
+                    s = 0;
+                    ph ^= 1;
+                }
             }
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");   // no copy outlives the loop (abort)
+        asm volatile("cp.async.wait_all;" ::: "memory");   // no copy outlives the loop
     } else if (warp == 4) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_f16(128, Npad);
-            int s = 0, c0 = 0, g = 0;
-            uint32_t ph = 0;
-            int last = -1;
-            // testing aid: a wait that nothing completes runs out, sets the abort
-            // flag, and every role stops, drains and reports through status[1]
-            const bool stalled = a.test_stall && !mbar_wait_ab(smem_u32(&stall_bar), 0, abortp, a.wait_tries);
-            for (int it = 0; it < (stalled ? 0 : iters); ++it) {
-                if (!mbar_wait_ab(smem_u32(&afull[s]), ph, abortp, a.wait_tries)) break;
-                if (!mbar_wait_ab(smem_u32(&bfull[s]), ph, abortp, a.wait_tries)) break;
-                if (c0 == 0 && g >= 2 &&
-                    !mbar_wait_ab(smem_u32(&bank_empty[g & 1]), ((g - 2) >> 1) & 1, abortp, a.wait_tries))
+        const uint32_t idesc = idesc_f16(128, Npad);
+        const uint64_t desc0 = umma_desc64(smem_u32(base));   // addresses: lowest bits, in units of 16 bytes
+        int s = 0, g = 0, last = -1, it = 0;
+        uint32_t ph = 0;
+        // testing aid: a wait that nothing completes runs out, sets the abort
+        // flag, and every role stops, drains and reports through status[1]
+        bool stop = a.test_stall && !mbar_wait_ab(smem_u32(&stall_bar), 0, abortp, a.wait_tries);
+        stop = __any_sync(0xffffffffu, stop);
+        // Inputs in descending order: chunk by chunk from the last, each chunk's
+        // k-steps of 16 inputs from the last down, and in each k-step the two
+        // small cross products before the main one.  The accumulator adds of the
+        // tensor cores truncate, so every add made once the sum has its full size
+        // costs up to an ulp of it, all of the same sign; leading with the small
+        // high-order terms leaves only the last few adds at full size.
+        for (; g < units && !stop; ++g) {
+            const uint32_t d = tmem + (uint32_t)(g & 1) * 256u;
+            for (int j = 0; j < nck && !stop; j += 2) {
+                const int n = min(2, nck - j);
+                const int s1 = s + 1 == NST ? 0 : s + 1;
+                // lanes 0, 1: the stage's operands; 2, 3: the next stage's; 4: the
+                // bank, read out by the promoters of two units before
+                uint32_t bar = 0, par = ph;
+                if (lane < 2 * n) {
+                    const int sl = lane & 2 ? s1 : s;
+                    bar = smem_u32(lane & 1 ? &bfull[sl] : &afull[sl]);
+                    if ((lane & 2) && s1 == 0) par ^= 1;
+                } else if (lane == 4 && j == 0 && g >= 2) {
+                    bar = smem_u32(&bank_empty[g & 1]);
+                    par = ((g - 2) >> 1) & 1;
+                }
+                bool done = bar == 0;
+                long tries = 0;
+                for (; tries < a.wait_tries; ++tries) {
+                    if (!done) done = mbar_try(bar, par);
+                    if (__all_sync(0xffffffffu, done)) break;
+                    if ((tries & 255) == 255 && __any_sync(0xffffffffu, *abortp != 0)) tries = a.wait_tries;
+                }
+                if (tries >= a.wait_tries) {
+                    *abortp = 1;
+                    stop = true;
                     break;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const unsigned char *stage = base + (size_t)s * stage_bytes;
-                const uint32_t d = tmem + (uint32_t)(g & 1) * 256u;
-                const int nc = min(S, nck - c0);
-                // Inputs in descending order: the stage's chunks from the last
-                // slot down, each chunk's k-steps from the last down, and in each
-                // k-step the two small cross products before the main one.  The
-                // accumulator adds of the tensor cores truncate, so every add made
-                // once the sum has its full size costs up to an ulp of it, all of
-                // the same sign; leading with the small high-order terms leaves
-                // only the last few adds at full size.
-                for (int q = 0; q < nc; ++q) {
-                    const int sl = nc - 1 - q;
-                    const int c = chunk_of(nck, c0 + nc - 1) + sl;   // the input chunk in slot sl
-                    const uint32_t sa = smem_u32(stage + sl * kTcA);
-                    const uint32_t sb = smem_u32(stage + S * kTcA + sl * b_bytes);
-                    // k-steps of 32 bytes (16 inputs) holding inputs
-                    const int nks = min(2, (a.K - 32 * c + 15) / 16);
-                    for (int ks = nks - 1; ks >= 0; --ks) {
-                        const uint32_t ko = ks * 32;
-                        const uint64_t ah = umma_desc64(sa + ko), al = umma_desc64(sa + 8192 + ko);
-                        const uint64_t bh = umma_desc64(sb + ko), bl = umma_desc64(sb + (uint32_t)Npad * 64 + ko);
-                        const uint32_t acc = (c0 > 0 || q > 0 || ks < nks - 1) ? 1u : 0u;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    // the producers' copies are generic-proxy writes; the MMAs read
+                    // shared memory through the async proxy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    for (int e = 0; e < n; ++e) {
+                        const int se = e ? s1 : s;
+                        const uint64_t ah = desc0 + (uint32_t)se * (stage_bytes >> 4), al = ah + (8192 >> 4);
+                        const uint64_t bh = ah + (kTcA >> 4), bl = bh + Npad * 4;
+                        uint32_t acc = j + e > 0 ? 1u : 0u;
+                        if (a.K > 32 * chunk_of(nck, j + e) + 16) {   // else one k-step holds inputs
+                            mma_f16(d, ah + 2, bl + 2, idesc, acc);
+                            mma_f16(d, al + 2, bh + 2, idesc, 1u);
+                            mma_f16(d, ah + 2, bh + 2, idesc, 1u);
+                            acc = 1u;
+                        }
                         mma_f16(d, ah, bl, idesc, acc);
                         mma_f16(d, al, bh, idesc, 1u);
                         mma_f16(d, ah, bh, idesc, 1u);
+                        commit_to(&empty[se]);
                     }
+                    if (j + n == nck) commit_to(&bank_full[g & 1]);
                 }
-                commit_to(&empty[s]);
-                last = it;
-                c0 += S;
-                if (c0 >= nck) {
-                    commit_to(&bank_full[g & 1]);
-                    c0 = 0;
-                    ++g;
-                }
-                if (++s == NST) {
-                    s = 0;
+                it += n;
+                last = it - 1;
+                s += n;
+                if (s >= NST) {
+                    s -= NST;
                     ph ^= 1;
                 }
             }
-            // drain: the last commit covers every MMA issued
-            if (last >= 0) mbar_wait(smem_u32(&empty[last % NST]), (uint32_t)((last / NST) & 1), a.wait_tries);
         }
+        // drain: the last commit covers every MMA issued
+        if (last >= 0) mbar_wait(smem_u32(&empty[last % NST]), (uint32_t)((last / NST) & 1), a.wait_tries);
     } else if (warp == 5) {
         // ---------------- operator images
         if (lane == 0) {
-            int s = 0, c0 = 0;
-            int oi = next_off(-1);
-            const int bcls = pc.cls;
+            int t = t0 - 1, left = 0, cls = 0;
+            OffsetIter it;
+            int s = 0, n_done = 0;
             uint32_t ph = 0;
             int last = -1;
-            for (int it = 0; it < iters; ++it) {
-                if (it >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) break;
-                const int dx = c_il[bcls][oi][0], dy = c_il[bcls][oi][1], dz = c_il[bcls][oi][2];
-                const int slot_off = (dz + 3) * 49 + (dy + 3) * 7 + (dx + 3);
-                unsigned char *stage = base + (size_t)s * stage_bytes;
-                // the stage's chunks of the operator image are contiguous
-                // (ascending, the lowest being that of the stage's last chunk)
-                const int ncs = min(S, nck - c0);
-                const uint32_t nbytes = (uint32_t)ncs * b_bytes;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&bfull[s])),
-                             "r"(nbytes));
-                const unsigned char *srcimg = a.img + ((size_t)slot_off * nck + chunk_of(nck, c0 + ncs - 1)) * b_bytes;
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                        smem_u32(stage + S * kTcA)),
-                    "l"(srcimg), "r"(nbytes), "r"(smem_u32(&bfull[s]))
-                    : "memory");
-                last = it;
-                c0 += S;
-                if (c0 >= nck) {
-                    c0 = 0;
-                    oi = next_off(oi);
+            bool stop = false;
+            for (int u = 0; u < units && !stop; ++u) {
+                if (left == 0) {
+                    ++t;
+                    left = seg_n(t);
+                    it.open(a.tmask, t, seg_lo(t));
+                    cls = tile_of(a, t).cls;
                 }
-                if (++s == NST) {
-                    s = 0;
-                    ph ^= 1;
+                --left;
+                const int o = c_il[cls][it.next()];
+                const int dx = (signed char)o, dy = (signed char)(o >> 8), dz = (signed char)(o >> 16);
+                const unsigned char *img = a.img + (size_t)((dz + 3) * 49 + (dy + 3) * 7 + (dx + 3)) * nck * b_bytes;
+                for (int j = 0; j < nck; ++j) {
+                    if (n_done >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) {
+                        stop = true;
+                        break;
+                    }
+                    const uint32_t stage = smem_u32(base) + (uint32_t)s * stage_bytes;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&bfull[s])),
+                                 "r"(b_bytes));
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            stage + kTcA),
+                        "l"(img + (size_t)chunk_of(nck, j) * b_bytes), "r"(b_bytes), "r"(smem_u32(&bfull[s]))
+                        : "memory");
+                    last = n_done++;
+                    if (++s == NST) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
             }
             // drain: every copy issued must have landed before the CTA exits;
@@ -827,39 +1015,40 @@ m2l_tc(TcArgs a) {
     bool ok = true;
     if (pw >= 0) {
         float acc[NS];
+        int g = 0;   // units promoted so far (bank g & 1)
+        for (int t = t0; g < units; ++t) {
+            const int n = seg_n(t);
 #pragma unroll
-        for (int q = 0; q < NS; ++q) acc[q] = 0.f;
-        for (int g = 0; g < G; ++g) {
-            bool w_ok = mbar_wait_ab(smem_u32(&bank_full[g & 1]), (g >> 1) & 1, abortp, a.wait_tries);
-            w_ok = __all_sync(0xffffffffu, w_ok);   // tcgen05.ld is warp-collective
-            if (!w_ok) {
-                ok = false;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t tb =
-                tmem + ((uint32_t)(pq * 32) << 16) + (uint32_t)(g & 1) * 256u + (uint32_t)(ph_half * nsum);
-#pragma unroll
-            for (int j0 = 0; j0 < NS; j0 += 8) {
-                if (j0 < nsum) {
-                    float t[8];
-                    tmem_ld8(tb + j0, t);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) acc[j0 + q] += t[q];
+            for (int q = 0; q < NS; ++q) acc[q] = 0.f;
+            for (int e = 0; e < n; ++e, ++g) {
+                bool w_ok = mbar_wait_ab(smem_u32(&bank_full[g & 1]), (g >> 1) & 1, abortp, a.wait_tries);
+                w_ok = __all_sync(0xffffffffu, w_ok);   // tcgen05.ld is warp-collective
+                if (!w_ok) {
+                    ok = false;
+                    break;
                 }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t tb =
+                    tmem + ((uint32_t)(pq * 32) << 16) + (uint32_t)(g & 1) * 256u + (uint32_t)(ph_half * nsum);
+#pragma unroll
+                for (int j0 = 0; j0 < NS; j0 += 8) {
+                    if (j0 < nsum) {
+                        float v[8];
+                        tmem_ld8(tb + j0, v);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) acc[j0 + q] += v[q];
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bank_empty[g & 1]));
             }
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bank_empty[g & 1]));
-        }
-        if (*abortp) ok = false;
-        if (ok) {
-            // write this tile's rows
-            const TcLevel &L = *pc.L;
+            if (*abortp) ok = false;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const TcTile tile = tile_of(a, t);
+            const TcLevel &L = *tile.L;
             const int r = pq * 32 + lane;
-            const int oslot = r / B, obb = r - oslot * B;
-            const int64_t os = (int64_t)pc.tile * nbox + oslot;
-            bool write = true;
             {
                 // undo the column scales of the image and the input scale
                 float sig, sig_inv;
@@ -875,66 +1064,22 @@ m2l_tc(TcArgs a) {
                         acc[q + 3] = acc[q + 3] * c4.w * sig_inv;
                     }
             }
-            if (msplit > 1) {
-                // this warp's slice of the tile (32 rows, half the columns):
-                // partial rows out, then the second CTA to arrive adds the
-                // other's rows (a + b = b + a, so the sum does not depend on
-                // which CTA is second) and writes the tile
-                float4 *mine =
-                    reinterpret_cast<float4 *>(a.mpart + ((size_t)blockIdx.x * 128 + r) * Npad + ph_half * nsum);
+            if (a.stream && n < (int)(pref[t + 1] - pref[t])) {
+                // a cut tile: partial rows, summed by m2l_join
+                const int q4 = nsum / 4;
+                float4 *mine = reinterpret_cast<float4 *>(a.mpart) +
+                               ((size_t)(2 * blockIdx.x + (pref[t] > u0 ? 1 : 0)) * (Npad / 4) + ph_half * q4) * 128 + r;
 #pragma unroll
                 for (int q = 0; q < NS; q += 4)
-                    if (q < nsum) mine[q / 4] = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
-                __threadfence();
-                __syncwarp();
-                int second = 0;
-                if (lane == 0) second = atomicAdd(a.mcnt + (size_t)utile * 8 + pw, 1) == msplit - 1;
-                second = __shfl_sync(0xffffffffu, second, 0);
-                write = second != 0;
-                if (write) {
-                    __threadfence();
-                    const float4 *other = reinterpret_cast<const float4 *>(
-                        a.mpart + ((size_t)(utile * msplit + (1 - uhalf)) * 128 + r) * Npad + ph_half * nsum);
-#pragma unroll
-                    for (int q = 0; q < NS; q += 4)
-                        if (q < nsum) {
-                            const float4 o4 = __ldcg(other + q / 4);
-                            acc[q] += o4.x;
-                            acc[q + 1] += o4.y;
-                            acc[q + 2] += o4.z;
-                            acc[q + 3] += o4.w;
-                        }
-                }
+                    if (q < nsum) mine[(q / 4) * 128] = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
+                continue;
             }
-            if (write && oslot < nbox && os < pc.ccnt) {
-                int64_t obox;
-                if (!L.adj) {
-                    obox = L.order[pc.cbeg + os];
-                } else {
-                    int64_t ox, oy, oz;
-                    class_box(pc.cls, L.blo, L.bn, os, ox, oy, oz);
-                    obox = L.slab0 + (oz * L.bn[1] + oy) * L.bn[0] + ox;
-                }
-                // 16-byte stores of the whole half row: columns from K up to
-                // Npad hold zeros (the operator images are zero there) and stay
-                // inside the row's padding (Npad <= ldk)
-                float4 *dst = reinterpret_cast<float4 *>(L.le + (obox * B + obb) * a.ldk + ph_half * nsum);
-                if (a.le_f64) {
-                    // an FP64 plan's local expansions: rows of ldk >= Npad doubles
-                    double *dd = reinterpret_cast<double *>(L.le) + (obox * B + obb) * a.ldk + ph_half * nsum;
+            const int64_t row = out_row(a, tile, nbox, r);
+            if (row >= 0) {
 #pragma unroll
-                    for (int q = 0; q < NS; q += 4)
-                        if (q < nsum) {
-                            dd[q] = (double)acc[q];
-                            dd[q + 1] = (double)acc[q + 1];
-                            dd[q + 2] = (double)acc[q + 2];
-                            dd[q + 3] = (double)acc[q + 3];
-                        }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < NS; q += 4)
-                        if (q < nsum) dst[q / 4] = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
-                }
+                for (int q = 0; q < NS; q += 4)
+                    if (q < nsum)
+                        store4(a, L, row, ph_half * nsum + q, make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]));
             }
         }
     }
@@ -955,10 +1100,56 @@ static size_t split_offset(const FmmPlan *F, int adj, int l) {
     return off;
 }
 
+// Tiles of the M2L (adj: of its transpose) for batches of B.
+static int64_t tc_tiles(const FmmPlan *F, bool adj, int B, int *tile_begin) {
+    const int nbox = 128 / B;
+    int64_t tiles = 0;
+    int e = 0;
+    for (int l = 2; l <= F->L; ++l)
+        for (int c = 0; c < 8; ++c, ++e) {
+            if (tile_begin) tile_begin[e] = (int)tiles;
+            const int64_t *off = adj ? F->scls_off[l] : F->lev[l].cls_off;
+            const int64_t cnt = (adj || F->lev[l].nt > 0) ? off[c + 1] - off[c] : 0;
+            tiles += (cnt + nbox - 1) / nbox;
+        }
+    if (tile_begin) tile_begin[e] = (int)tiles;
+    return tiles;
+}
+
+// CTAs of a launch that deals out units: one per SM, and no more than could
+// have kMinUnits each.
+constexpr int kMinUnits = 6;
+static int64_t tc_stream_ctas(int64_t tiles) {
+    return std::max<int64_t>(1, std::min<int64_t>(sm_count(), tiles * 189 / kMinUnits));
+}
+
+size_t m2l_tc_bytes(int p) {
+    const int npad = ((p + 1) * (p + 1) + 15) & ~15;
+    return npad > 256 ? 0 : (size_t)2 * sm_count() * 128 * npad * sizeof(float) + (size_t)(sm_count() + 1) * sizeof(int4);
+}
+
+// Masks of the tiles and the partial rows of cut tiles, for the plan's largest batch (smaller batches have no more tiles); the
+// forward's partial rows serve the adjoint too when they suffice.
+static gf_status m2l_tc_workspaces(gf_plan_s *plan, bool adj) {
+    FmmPlan *F = plan->fmm;
+    if (F->B > 128) return GF_OK;
+    const int64_t tiles = tc_tiles(F, adj, F->B, nullptr);
+    if (tiles == 0) return GF_OK;
+    GF_TRY(plan->arena.alloc((void **)&F->m2l_mask[adj], (size_t)tiles * 8 * sizeof(uint32_t)));
+    if (tiles > kStreamTiles) return GF_OK;
+    const int64_t ctas = tc_stream_ctas(tiles);
+    if (ctas <= F->m2l_part_ctas) return GF_OK;
+    GF_TRY(plan->arena.alloc((void **)&F->m2l_cut, (size_t)(ctas + 1) * sizeof(int4)));
+    GF_TRY(plan->arena.alloc((void **)&F->m2l_part, (size_t)ctas * 2 * 128 * F->tab->tc_npad * sizeof(float)));
+    F->m2l_part_ctas = (int)ctas;
+    return GF_OK;
+}
+
 gf_status m2l_tc_prepare_adj(gf_plan_s *plan) {
     FmmPlan *F = plan->fmm;
     if (!F->mixed || !F->tab->m2l_tc) return GF_OK;
     GF_TRY(plan->arena.alloc((void **)&F->tc_split_adj, std::max<size_t>(16, split_offset(F, 1, F->L + 1))));
+    GF_TRY(m2l_tc_workspaces(plan, true));
     for (int adj = 1; adj < 2; ++adj) {
         std::vector<TcLevel> h(F->L + 1);
         memset(h.data(), 0, h.size() * sizeof(TcLevel));
@@ -1000,22 +1191,7 @@ gf_status m2l_tc_prepare(gf_plan_s *plan) {
     if (!(F->mixed || F->m2l_tc64) || !F->tab->m2l_tc) return GF_OK;
     GF_TRY(plan->arena.alloc((void **)&F->tc_amax, 2 * (kMaxLevels + 1) * sizeof(uint32_t)));
     GF_TRY(plan->arena.alloc((void **)&F->tc_split, std::max<size_t>(16, split_offset(F, 0, F->L + 1))));
-    {
-        // partial rows of the forward M2L's tiles when two CTAs share each
-        // (tiles counted for the plan's largest batch: the most tiles)
-        const int nbox = 128 / std::max(1, std::min(F->B, 128));
-        int64_t tiles = 0;
-        for (int l = 2; l <= F->L; ++l)
-            for (int c = 0; c < 8; ++c) {
-                const int64_t cnt = F->lev[l].nt > 0 ? F->lev[l].cls_off[c + 1] - F->lev[l].cls_off[c] : 0;
-                tiles += (cnt + nbox - 1) / nbox;
-            }
-        if (tiles > 0 && 2 * tiles <= (int64_t)sm_count()) {
-            GF_TRY(plan->arena.alloc((void **)&F->m2l_part, (size_t)tiles * 2 * 128 * F->tab->tc_npad * sizeof(float)));
-            GF_TRY(plan->arena.alloc((void **)&F->m2l_cnt, (size_t)tiles * 8 * sizeof(int)));
-            F->m2l_part_tiles = (int)tiles;
-        }
-    }
+    GF_TRY(m2l_tc_workspaces(plan, false));
     for (int adj = 0; adj < 1; ++adj) {
         std::vector<TcLevel> h(F->L + 1);
         memset(h.data(), 0, h.size() * sizeof(TcLevel));
@@ -1112,7 +1288,15 @@ struct SplitArgs {
     unsigned char *out[kMaxLevels + 1];
 };
 
-__global__ void __launch_bounds__(256) input_split(AmaxArgs a, SplitArgs o, int nck) {
+// The last row of blocks finds the active offsets of the tiles (tile_mask)
+// beside the split.
+__global__ void __launch_bounds__(256)
+input_split(const __grid_constant__ AmaxArgs a, const __grid_constant__ SplitArgs o, int nck,
+            const __grid_constant__ TcArgs tc, uint32_t *tmask) {
+    if (blockIdx.y == gridDim.y - 1) {
+        for (int t = (int)blockIdx.x; t < tc.ntiles; t += (int)gridDim.x) tile_mask(tc, t, tmask);
+        return;
+    }
     const int l = a.lmin + (int)blockIdx.y;
     float sig, sig_inv;
     input_scale(a.out[l], sig, sig_inv);
@@ -1157,9 +1341,8 @@ __global__ void __launch_bounds__(256) input_split(AmaxArgs a, SplitArgs o, int 
     }
 }
 
-gf_status tc_launch(TcArgs &a, int tiles, cudaStream_t st) {
-    if (tiles == 0) return GF_OK;
-    const int grid = tiles * std::max(1, a.msplit);
+gf_status tc_launch(TcArgs &a, int grid, cudaStream_t st) {
+    if (a.ntiles == 0) return GF_OK;
     const size_t shm = tc_smem_bytes(a.Npad);
     a.nst = tc_stages(a.Npad);
     const int nsum = a.Npad / 2;
@@ -1193,7 +1376,6 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
     a.nck = T->tc_nck_h;
     a.status = plan->d_status;
     a.wait_tries = kWaitTries;
-    a.msplit = 1;
     a.lv = reinterpret_cast<const TcLevel *>(adj ? F->tc_levels_adj : F->tc_levels);
     a.lmin = 2;
     a.img = (const unsigned char *)(adj ? T->am2l_tc : T->m2l_tc);
@@ -1206,6 +1388,14 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
         a.wait_tries = kTestWaitTries;
     }
     if (F->L < 2) return GF_OK;
+    a.nent = 8 * (F->L - 1);
+    a.ntiles = (int)tc_tiles(F, adj, B, a.tile_begin);
+    a.tmask = F->m2l_mask[adj];
+    a.mcut = F->m2l_cut;
+    a.mpart = F->m2l_part;
+    a.min_units = kMinUnits;
+    const int64_t ctas = tc_stream_ctas(a.ntiles);
+    a.stream = a.ntiles <= kStreamTiles && ctas <= F->m2l_part_ctas;
     // the largest |input| of every level, for the FP16 input scales
     {
         AmaxArgs m;
@@ -1243,32 +1433,18 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
         memset(&o, 0, sizeof(o));
         for (int l = 2; l <= F->L; ++l)
             o.out[l] = (adj ? F->tc_split_adj : F->tc_split) + split_offset(F, adj, l) + (size_t)row0[l] * F->KS * 4;
-        input_split<<<dim3(gx, F->L - 1), 256, 0, st>>>(m, o, T->tc_nck_h);
+        const int gs = std::max(gx, std::min(a.ntiles, 8 * 152));
+        input_split<<<dim3(gs, F->L), 256, 0, st>>>(m, o, T->tc_nck_h, a, F->m2l_mask[adj]);
         GF_KERNEL_DONE();
     }
     if (!adj) stage_mark(plan, 4, st);
-    const int nbox = 128 / B;
-    int tiles = 0, e = 0;
-    for (int l = 2; l <= F->L; ++l)
-        for (int c = 0; c < 8; ++c, ++e) {
-            a.tile_begin[e] = tiles;
-            const int64_t *off = adj ? F->scls_off[l] : F->lev[l].cls_off;
-            const int64_t cnt = (adj || F->lev[l].nt > 0) ? off[c + 1] - off[c] : 0;
-            tiles += (int)((cnt + nbox - 1) / nbox);
-        }
-    a.tile_begin[e] = tiles;
-    a.nent = e;
-    // when two CTAs per tile still fit the SMs at once, every tile's offsets
-    // are shared by two: each chain of offsets is half as long (and each
-    // FP32 sum of offsets half as deep)
-    if (!adj && F->m2l_part && tiles <= F->m2l_part_tiles && 2 * tiles <= sm_count()) {
-        a.msplit = 2;
-        a.mpart = F->m2l_part;
-        a.mcnt = F->m2l_cnt;
-        GF_CUDA(cudaMemsetAsync(F->m2l_cnt, 0, (size_t)tiles * 8 * sizeof(int), st));
-    }
     if (fork) GF_CUDA(cudaEventRecord(fork, st));
-    return tc_launch(a, tiles, st);
+    GF_TRY(tc_launch(a, a.stream ? (int)ctas : a.ntiles, st));
+    if (a.stream && ctas > 1) {
+        m2l_join<<<dim3((unsigned)ctas - 1, 4), 512, 0, st>>>(a);
+        GF_KERNEL_DONE();
+    }
+    return GF_OK;
 }
 
 }  // namespace

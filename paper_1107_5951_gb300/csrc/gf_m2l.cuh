@@ -41,6 +41,9 @@ gf_status p2m_leaf_run(gf_plan_s *plan, int B, int64_t first, int64_t count, cud
 template <class T>
 gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaStream_t st);
 
+// Upper bound of the tensor-core M2L's own workspaces (beside the expansions
+// and their split parts).
+size_t m2l_tc_bytes(int p);
 // Plan-time set-up of the tensor-core path (level descriptors on the device).
 gf_status m2l_tc_prepare(gf_plan_s *plan);
 // The adjoint's level tables (built on the plan's first adjoint call).
