@@ -1591,10 +1591,10 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     // 4^3-voxel leaves under a mirror-symmetric rule: the folded P2M kernels
     const bool fold = !pts && p2m_fold_ok(plan) && lb.n[1] * 4 <= 65535 && lb.n[2] * 4 * B <= 65535;
     bool up = false;   // level L-1 expansions made straight from the density grid
-    // the folded kernels that write each level's expansions also take the
-    // largest |input| of the slabs its M2L reads, in place of a pass over
+    // the kernels that write each level's expansions (folded, or the points'
+    // P2M) also take the largest |input| of the slabs its M2L reads, in place of a pass over
     // those rows before the M2L
-    F->amax_fused = fold && F->tc_amax != nullptr;
+    F->amax_fused = (fold || pts) && F->tc_amax != nullptr;
     if (F->amax_fused) GF_CUDA(cudaMemsetAsync(F->tc_amax, 0, (kMaxLevels + 1) * sizeof(uint32_t), st));
     if (pts) {
         // a0 + a3 for point sources: masses in leaf order, P2M over each leaf's points

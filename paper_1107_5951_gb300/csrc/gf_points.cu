@@ -483,264 +483,251 @@ __global__ void point_masses(const void *__restrict__ rho, int rho_f32, const in
     if (e >= S * B) return;
     const int b = (int)(e / S);
     const int64_t i = e - (int64_t)b * S;
-    const double r = load_rho_p(rho, rho_f32, (int64_t)b * ncell + perm[i] / per_cell);
+    const int64_t src = (int64_t)b * ncell + perm[i] / per_cell;
+    if constexpr (sizeof(T) == 4) {
+        if (rho_f32) {   // one rounding of the product, without the FP64 pipe
+            const float r = ((const float *)rho)[src];
+            if (!isfinite(r)) atomicOr(status, 1);
+            m[e] = r * loc[4 * i + 3];
+            return;
+        }
+    }
+    const double r = load_rho_p(rho, rho_f32, src);
     if (!isfinite(r)) atomicOr(status, 1);
     m[e] = (T)(r * (double)loc[4 * i + 3]);
 }
 
-// Recursion coefficients of the regular harmonics (the recursion of
-// fmm_math.cuh) for the point P2M, n <= kMaxP: for m < n, t = n (n + 1) / 2 + m,
-//   c_pa[t] = (2n - 1) / sqrt((n + m)(n - m)),
-//   c_pb[t] = sqrt((n - 1 + m)(n - 1 - m)) / sqrt((n + m)(n - m))  (0 for n = m + 1),
-// and c_pf[n] = -sqrt((2n - 1) / (2n)), the sectoral step into R_n^n; in
-// FP64 and rounded to FP32.
-constexpr int kPT = (kMaxP + 1) * (kMaxP + 2) / 2;
-__constant__ double c_pa[kPT], c_pb[kPT], c_pf[kMaxP + 1];
-__constant__ float c_paf[kPT], c_pbf[kPT], c_pff[kMaxP + 1];
-
-template <class T>
-__device__ __forceinline__ T coef(const double *d, const float *f, int i) {
-    if constexpr (sizeof(T) == 4)
-        return f[i];
-    else
-        return d[i];
-}
-
 // P2M over the points of each leaf: ME_n^m = sum_i m_i conj(R_n^m(x_i - c)),
-// x_i - c the point's offset from the leaf centre (leaf units).  One warp
-// per leaf, 64 points per round: each lane runs the recursion for two
-// points at once (the sectoral steps R_m^m, then the upward steps in n for
-// each order m, the coefficients uniform across the warp) and writes the
-// two points' mass-weighted harmonics, summed, into its own row of the
-// warp's shared-memory block ([32][K], odd row stride); the lanes then sum
-// the 32 rows column by column into the expansion.
-constexpr int kP2MRound = 64;
+// x_i - c the point's offset from the leaf centre (leaf units).
+//
+// R_n^m = s_nm (x + iy)^m Q_n^m(z, r^2) with a real Q that starts at Q_m^m = 1
+// and follows Q_n = z Q_{n-1} - c_nm r^2 Q_{n-2}, c_nm = ((n-1)^2 - m^2) /
+// ((2n-1)(2n-3)) (the regular harmonics' recursion divided by its leading
+// coefficients, whose product is s_nm), so a term costs three operations for
+// Q and one for each real component, and s_nm is applied to the sums.
+//
+// What bounds it is the FP32 (FP64) issue rate, so nothing is spent on a sum
+// across lanes: a lane owns two orders of one leaf, m <= p/2 and p + 1 - m (p
+// even; none beside m = 0) or p - m (p odd) -- p + 1 or p + 2 terms whatever m,
+// held in registers -- and walks over the leaf's points.  A warp
+// takes 32 / GL leaves at once, GL >= p/2 + 1 lanes each; a leaf of more than
+// kP2MBig points is taken by the whole warp, its lane groups' sums added at the
+// end.  The points come through shared memory, one entry (FP32: a pair of
+// points) made by each lane at a time: z and r^2, and the mass-weighted powers
+// of x + iy, 16 bytes each, read back by the lanes of a leaf without bank
+// conflicts (their orders are neighbours, entries an odd number of 16 bytes
+// apart).  FP32 sums run over two points at once as packed pairs.
+// A lane per point, with the harmonics summed over the warp through shared
+// memory, took 3,254 us for 2^25 points in leaves of 48 at p = 12.
+constexpr int kP2MWarps = 4;
+constexpr int kP2MBig = 256;    // points from which a leaf takes the whole warp
+constexpr int kP2MSeg = 1024;   // points of such a leaf summed before its row is updated
+__constant__ double c_ps[(kMaxP + 1) * (kMaxP + 1)];   // s_nm by real component
 
-template <class T>
-constexpr int p2m_warps() {
-    return sizeof(T) == 4 ? 4 : 2;
+__device__ __forceinline__ uint64_t v_mul(uint64_t a, uint64_t b) { return mul2(a, b); }
+__device__ __forceinline__ uint64_t v_fma(uint64_t a, uint64_t b, uint64_t c) { return fma2(a, b, c); }
+__device__ __forceinline__ double v_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ double v_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float v_sum(uint64_t v) {
+    float l, h;
+    up2(v, l, h);
+    return l + h;
 }
+__device__ __forceinline__ double v_sum(double v) { return v; }
+__device__ __forceinline__ void v_dup(float c, uint64_t &v) { v = pk2(c, c); }
+__device__ __forceinline__ void v_dup(double c, double &v) { v = c; }
 
-inline int p2m_stride(int K) { return K | 1; }
+// 16-byte shared-memory entries an odd number apart from point to point
+inline __host__ __device__ int p2m_stride(int p) { return (p + 2) | 1; }
 
-template <class T>
-__global__ void __launch_bounds__(p2m_warps<T>() * 32)
-point_p2m(const T *__restrict__ loc, const T *__restrict__ mass, const int64_t *__restrict__ leaf_beg,
-          int64_t nleaf, int64_t S, int p, int B, int ldk, int stride, T *__restrict__ me) {
-    extern __shared__ unsigned char shraw[];
-    constexpr int W = p2m_warps<T>();
-    constexpr int kMaxCols = (kMaxP + 1) * (kMaxP + 1) / 32 + 2;   // ceil(ldk / 32) for ldk <= 320
+// NS >= terms of a lane; SW <= p - p/2 + 1, the first term at which a
+// lane can turn to its second order (selects are what the ALU does here).
+template <class T, int GL, int NS, int SW>
+__global__ void __launch_bounds__(kP2MWarps * 32, NS <= (sizeof(T) == 4 ? 13 : 11) ? 4 : 3)
+point_p2m(const T *__restrict__ loc, const T *__restrict__ mass, const int64_t *__restrict__ leaf_beg, int64_t nleaf,
+          int64_t S, int p, int B, int ldk, T *__restrict__ me, uint32_t *__restrict__ amax, int64_t amax_lo,
+          int64_t amax_hi) {
+    extern __shared__ __align__(16) unsigned char shraw[];
+    constexpr int NG = 32 / GL, PT = sizeof(T) == 4 ? 2 : 1;
+    constexpr int PTS = PT * GL;   // points a lane group stages at a time
+    using V = std::conditional_t<sizeof(T) == 4, uint64_t, double>;
+    struct __align__(16) V2 {
+        V a, b;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T *rows = reinterpret_cast<T *>(shraw) + (size_t)warp * 32 * stride;
-    T *row = rows + lane * stride;
-    const int K = (p + 1) * (p + 1);
-    for (int64_t leaf = (int64_t)blockIdx.x * W + warp; leaf < nleaf; leaf += (int64_t)gridDim.x * W) {
-        const int64_t i0 = leaf_beg[leaf], i1 = leaf_beg[leaf + 1];
-        for (int bb = 0; bb < B; ++bb) {
-            T acc[kMaxCols];
+    const int grp = lane / GL, tk = lane % GL;
+    const int K = (p + 1) * (p + 1), steps = p % 2 ? p + 2 : p + 1, stride = p2m_stride(p);
+    V2 *sh = reinterpret_cast<V2 *>(shraw) + (size_t)warp * 32 * stride;
+    V2 *own = sh + lane * stride;               // the entry this lane stages
+    const V2 *grp_sh = sh + grp * GL * stride;
+    // orders of this lane; lanes beyond p / 2 repeat the last one's, unwritten
+    const int m1 = min(tk, p / 2), m2 = p % 2 ? p - m1 : min(p, p + 1 - m1);
+    const int sw = p - m1 + 1;   // term sw is the first of order m2 (p even, m1 = 0: beyond the last)
+    V nc[NS];   // -c_nm of each term
 #pragma unroll
-            for (int j = 0; j < kMaxCols; ++j) acc[j] = T(0);
-            for (int64_t r0 = i0; r0 < i1; r0 += kP2MRound) {
-                const int64_t ia = r0 + lane, ib = r0 + 32 + lane;
-                T xa = T(0), ya = T(0), za = T(0), qa = T(0), xb = T(0), yb = T(0), zb = T(0), qb = T(0), w;
-                if (ia < i1) {
-                    ld_loc(loc, ia, xa, ya, za, w);
-                    qa = mass[(int64_t)bb * S + ia];
-                }
-                if (ib < i1) {
-                    ld_loc(loc, ib, xb, yb, zb, w);
-                    qb = mass[(int64_t)bb * S + ib];
-                }
-                const T r2a = xa * xa + ya * ya + za * za, r2b = xb * xb + yb * yb + zb * zb;
-                T sra = T(1), sia = T(0), srb = T(1), sib = T(0);   // R_m^m of both points
-                for (int m = 0; m <= p; ++m) {
-                    if (m > 0) {
-                        const T f = coef<T>(c_pf, c_pff, m);
-                        const T fxa = f * xa, fya = f * ya, fxb = f * xb, fyb = f * yb;
-                        const T nra = fxa * sra - fya * sia, nia = fxa * sia + fya * sra;
-                        const T nrb = fxb * srb - fyb * sib, nib = fxb * sib + fyb * srb;
-                        sra = nra;
-                        sia = nia;
-                        srb = nrb;
-                        sib = nib;
-                    }
-                    T cra = sra, cia = sia, crb = srb, cib = sib;
-                    T pra = T(0), pia = T(0), prb = T(0), pib = T(0);
-                    int k = m * m + (m == 0 ? 0 : 2 * m - 1);   // R_m^m's real index
-                    for (int n = m;; ++n) {
-                        // the two points' mass-weighted conj(R_n^m), summed
-                        const T vr = qa * cra + qb * crb, vi = qa * cia + qb * cib;
-                        if (m == 0) {
-                            row[k] = vr;
-                        } else {
-                            row[k] = vr;
-                            row[k + 1] = -vi;
-                        }
-                        if (n == p) break;
-                        k += 2 * n + 1;   // the same order one degree up: (n + 1)^2 - n^2
-                        const int t = (n + 1) * (n + 2) / 2 + m;
-                        const T av = coef<T>(c_pa, c_paf, t), bv = coef<T>(c_pb, c_pbf, t);
-                        const T aza = av * za, brea = bv * r2a, azb = av * zb, breb = bv * r2b;
-                        const T nra = aza * cra - brea * pra, nia = aza * cia - brea * pia;
-                        const T nrb = azb * crb - breb * prb, nib = azb * cib - breb * pib;
-                        pra = cra;
-                        pia = cia;
-                        prb = crb;
-                        pib = cib;
-                        cra = nra;
-                        cia = nia;
-                        crb = nrb;
-                        cib = nib;
-                    }
-                }
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < kMaxCols; ++j) {
-                    const int kk = lane + 32 * j;
-                    if (kk < K) {
-                        T sum = T(0);
-#pragma unroll 8
-                        for (int r = 0; r < 32; ++r) sum += rows[r * stride + kk];
-                        acc[j] += sum;
-                    }
-                }
-                __syncwarp();
-            }
-            T *dst = me + (leaf * B + bb) * ldk;
-#pragma unroll
-            for (int j = 0; j < kMaxCols; ++j) {
-                const int kk = lane + 32 * j;
-                if (kk < ldk) dst[kk] = kk < K ? acc[j] : T(0);
-            }
-        }
+    for (int i = 0; i < NS; ++i) {
+        const int m = i < sw ? m1 : m2, n = i < sw ? m1 + i : m2 + i - sw;
+        const T c = n >= m + 2 ? T((n - 1) * (n - 1) - m * m) / T((2 * n - 1) * (2 * n - 3)) : T(0);
+        v_dup(-c, nc[i]);
     }
-}
-
-// The FP32 P2M, the same sums in packed pairs: a lane's two points form
-// one f32x2 value and one packed instruction advances both recursions (the
-// coefficients are stored as duplicated pairs).  The harmonics are made in
-// groups of consecutive orders m holding at most kGrpEnt real entries; a
-// group's entries go to the warp's [32][kGrpEnt + 1] block and are summed
-// over the rows before the next group starts (the sectoral steps below the
-// group's first order are redone, a few complex products), so a warp needs
-// 8 KB of shared memory and many warps fit an SM.  In each order the upward
-// recursion overwrites the older of its two values (no register moves).
-constexpr int kGrpEnt = 64;
-constexpr int kMaxGroups = 12;
-constexpr int kGrpStride = kGrpEnt + 1;
-constexpr int kP2MWarpsF = 4;
-
-struct P2MGroups {
-    int ng;
-    int m_lo[kMaxGroups + 1];   // group g: orders [m_lo[g], m_lo[g + 1])
-    int ent0[kMaxGroups + 1];   // its entries [ent0[g], ent0[g + 1]) in generation order
-};
-__constant__ float2 c_a2[kPT], c_nb2[kPT], c_f2[kMaxP + 1], c_nf2[kMaxP + 1];
-__constant__ P2MGroups c_grp[kMaxP + 1];
-__constant__ short c_ktab[kMaxP + 1][(kMaxP + 1) * (kMaxP + 1)];   // real index of each generated entry
-
-__device__ __forceinline__ uint64_t ldc2(const float2 &v) { return pk2(v.x, v.y); }
-
-__global__ void __launch_bounds__(kP2MWarpsF * 32)
-point_p2m_f32(const float *__restrict__ loc, const float *__restrict__ mass, const int64_t *__restrict__ leaf_beg,
-              int64_t nleaf, int64_t S, int p, int B, int ldk, float *__restrict__ me) {
-    __shared__ float rows_all[kP2MWarpsF][32 * kGrpStride];
-    __shared__ short kt[(kMaxP + 1) * (kMaxP + 1)];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int K = (p + 1) * (p + 1);
-    for (int i = threadIdx.x; i < K; i += blockDim.x) kt[i] = c_ktab[p][i];
+    V one;
+    v_dup(T(1), one);
+    __shared__ T sc[(kMaxP + 1) * (kMaxP + 1)];
+    for (int k = threadIdx.x; k < K; k += blockDim.x) sc[k] = (T)c_ps[k];
     __syncthreads();
-    float *rows = rows_all[warp];
-    float *row = rows + lane * kGrpStride;
-    const int ng = c_grp[p].ng;
-    for (int64_t leaf = (int64_t)blockIdx.x * kP2MWarpsF + warp; leaf < nleaf;
-         leaf += (int64_t)gridDim.x * kP2MWarpsF) {
-        const int64_t i0 = leaf_beg[leaf], i1 = leaf_beg[leaf + 1];
-        for (int bb = 0; bb < B; ++bb) {
-            float *dst = me + (leaf * B + bb) * ldk;
-            for (int k = K + lane; k < ldk; k += 32) dst[k] = 0.f;
-            for (int g = 0; g < ng; ++g) {
-                const int mlo = c_grp[p].m_lo[g], mhi = c_grp[p].m_lo[g + 1];
-                const int ne = c_grp[p].ent0[g + 1] - c_grp[p].ent0[g];
-                float acc0 = 0.f, acc1 = 0.f;
-                for (int64_t r0 = i0; r0 < i1; r0 += kP2MRound) {
-                    const int64_t ia = r0 + lane, ib = r0 + 32 + lane;
-                    float xa = 0.f, ya = 0.f, za = 0.f, qa = 0.f, xb = 0.f, yb = 0.f, zb = 0.f, qb = 0.f, w;
-                    if (ia < i1) {
-                        ld_loc(loc, ia, xa, ya, za, w);
-                        qa = mass[(int64_t)bb * S + ia];
-                    }
-                    if (ib < i1) {
-                        ld_loc(loc, ib, xb, yb, zb, w);
-                        qb = mass[(int64_t)bb * S + ib];
-                    }
-                    const uint64_t X = pk2(xa, xb), Y = pk2(ya, yb), Z = pk2(za, zb), Q = pk2(qa, qb);
-                    const uint64_t R2 = fma2(Z, Z, fma2(Y, Y, mul2(X, X)));
-                    uint64_t SR = pk2(1.f, 1.f), SI = 0;   // R_m^m of both points
-                    auto sectoral = [&](int m) {
-                        const uint64_t FX = mul2(ldc2(c_f2[m]), X), FY = mul2(ldc2(c_f2[m]), Y),
-                                       NFY = mul2(ldc2(c_nf2[m]), Y);
-                        const uint64_t nr = fma2(FX, SR, mul2(NFY, SI)), ni = fma2(FX, SI, mul2(FY, SR));
-                        SR = nr;
-                        SI = ni;
-                    };
-                    for (int m = 1; m < mlo; ++m) sectoral(m);
-                    int j = 0;
-                    auto put = [&](uint64_t vr, uint64_t vi, bool re_only) {
-                        float l, h;
-                        up2(mul2(Q, vr), l, h);
-                        row[j] = l + h;
-                        if (!re_only) {
-                            up2(mul2(Q, vi), l, h);
-                            row[j + 1] = -(l + h);   // conj
-                        }
-                        j += re_only ? 1 : 2;
-                    };
-                    for (int m = mlo; m < mhi; ++m) {
-                        if (m > 0) sectoral(m);
-                        const bool m0 = m == 0;
-                        uint64_t Cr = SR, Ci = SI, Pr = 0, Pi = 0;   // R_n^m, R_{n-1}^m
-                        put(Cr, Ci, m0);
-                        int t = (m + 1) * (m + 2) / 2 + m;      // coefficient index of (n + 1, m), n = m
-                        for (int n = m; n < p; n += 2) {
-                            {   // P <- R_{n+1}^m
-                                const uint64_t AZ = mul2(ldc2(c_a2[t]), Z), NB = mul2(ldc2(c_nb2[t]), R2);
-                                Pr = fma2(AZ, Cr, mul2(NB, Pr));
-                                Pi = fma2(AZ, Ci, mul2(NB, Pi));
-                                put(Pr, Pi, m0);
-                                t += n + 2;
-                            }
-                            if (n + 1 == p) break;
-                            {   // C <- R_{n+2}^m
-                                const uint64_t AZ = mul2(ldc2(c_a2[t]), Z), NB = mul2(ldc2(c_nb2[t]), R2);
-                                Cr = fma2(AZ, Pr, mul2(NB, Cr));
-                                Ci = fma2(AZ, Pi, mul2(NB, Ci));
-                                put(Cr, Ci, m0);
-                                t += n + 3;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    if (lane < ne) {
-                        float sum = 0.f;
-#pragma unroll 8
-                        for (int r = 0; r < 32; ++r) sum += rows[r * kGrpStride + lane];
-                        acc0 += sum;
-                    }
-                    if (lane + 32 < ne) {
-                        float sum = 0.f;
-#pragma unroll 8
-                        for (int r = 0; r < 32; ++r) sum += rows[r * kGrpStride + lane + 32];
-                        acc1 += sum;
-                    }
-                    __syncwarp();
+    float big_in = 0.f;   // largest |component| written in [amax_lo, amax_hi)
+
+    V ar[NS], ai[NS];
+    // add the points base + ((c step + off) PTS + PT tk + e), c < nchunk, below end
+    auto add_points = [&](int64_t base, int64_t end, int nchunk, int step, int off, const T *mb) {
+        for (int c = 0; c < nchunk; ++c) {
+            const int64_t first = base + (int64_t)(c * step + off) * PTS, i0 = first + PT * tk;
+            T x[PT], y[PT], z[PT], q[PT], w;
+#pragma unroll
+            for (int e = 0; e < PT; ++e) {
+                x[e] = y[e] = z[e] = q[e] = T(0);
+                if (i0 + e < end) {
+                    ld_loc(loc, i0 + e, x[e], y[e], z[e], w);
+                    q[e] = mb[i0 + e];
                 }
-                const int e0 = c_grp[p].ent0[g];
-                if (lane < ne) dst[kt[e0 + lane]] = acc0;
-                if (lane + 32 < ne) dst[kt[e0 + lane + 32]] = acc1;
+            }
+            V X, Y, NY, Z, WR, WI;
+            if constexpr (PT == 2) {
+                X = pk2(x[0], x[1]);
+                Y = pk2(y[0], y[1]);
+                NY = pk2(-y[0], -y[1]);
+                Z = pk2(z[0], z[1]);
+                WR = pk2(q[0], q[1]);
+                WI = 0;
+            } else {
+                X = x[0];
+                Y = y[0];
+                NY = -y[0];
+                Z = z[0];
+                WR = q[0];
+                WI = 0.0;
+            }
+            __syncwarp();   // the entries of the chunk before have been read
+            own[0] = V2{Z, v_fma(Z, Z, v_fma(Y, Y, v_mul(X, X)))};
+            own[1] = V2{WR, WI};
+            for (int m = 1; m <= p; ++m) {
+                const V nr = v_fma(X, WR, v_mul(NY, WI)), ni = v_fma(X, WI, v_mul(Y, WR));
+                WR = nr;
+                WI = ni;
+                own[1 + m] = V2{WR, WI};
+            }
+            __syncwarp();
+            // entries that hold points, over the warp's leaves
+            const int64_t rest = end - first;
+            const int mine = rest <= 0 ? 0 : (int)((min(rest, (int64_t)PTS) + PT - 1) / PT);
+            const int cnt = __reduce_max_sync(0xffffffffu, mine);
+            for (int e = 0; e < cnt; ++e) {
+                const V2 *pe = grp_sh + e * stride;
+                const V2 zr = pe[0], w1 = pe[1 + m1], w2 = pe[1 + m2];
+                V wr = w1.a, wi = w1.b, Q = one, P = zr.b;   // P is multiplied by 0 first
+#pragma unroll
+                for (int i = 0; i < NS; ++i) {
+                    if (i > 0) {
+                        if (i >= steps) break;
+                        const V n = v_fma(zr.a, Q, v_mul(v_mul(nc[i], zr.b), P));
+                        P = Q;
+                        Q = n;
+                        if (i >= SW && i == sw) {
+                            Q = one;
+                            wr = w2.a;
+                            wi = w2.b;
+                        }
+                    }
+                    ar[i] = v_fma(wr, Q, ar[i]);
+                    ai[i] = v_fma(wi, Q, ai[i]);
+                }
+            }
+        }
+    };
+    auto clear = [&]() {
+#pragma unroll
+        for (int i = 0; i < NS; ++i) v_dup(T(0), ar[i]), v_dup(T(0), ai[i]);
+    };
+    // the sums into row `leaf` (whole: all lane groups' sums into it; add: on top of it)
+    auto write = [&](int64_t leaf, int bb, bool whole, bool add, bool last) {
+        T *dst = me + (leaf * B + bb) * ldk;
+        const bool on = leaf < nleaf && tk <= p / 2 && (!whole || grp == 0);
+        const bool in = amax && leaf >= amax_lo && leaf < amax_hi && last;
+        auto put = [&](int k, T v) {
+            const T r = add ? dst[k] + v : v;
+            dst[k] = r;
+            if (in) big_in = fmaxf(big_in, fabsf((float)r));
+        };
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            if (i >= steps) break;
+            T re = v_sum(ar[i]), im = v_sum(ai[i]);
+            if (whole) {
+#pragma unroll
+                for (int o = GL; o < 32; o *= 2) {
+                    re += __shfl_xor_sync(0xffffffffu, re, o);
+                    im += __shfl_xor_sync(0xffffffffu, im, o);
+                }
+            }
+            const int m = i < sw ? m1 : m2, n = i < sw ? m1 + i : m2 + i - sw;
+            if (on) {
+                const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+                put(k, sc[k] * re);
+                if (m > 0) put(k + 1, -sc[k] * im);   // conj
+            }
+        }
+        if (leaf < nleaf && (!whole || grp == 0))
+            for (int k = K + tk; k < ldk; k += GL) dst[k] = T(0);
+    };
+
+    const int64_t nwarp = (int64_t)gridDim.x * kP2MWarps;
+    for (int64_t leaf0 = ((int64_t)blockIdx.x * kP2MWarps + warp) * NG; leaf0 < nleaf; leaf0 += nwarp * NG) {
+        const int64_t leaf = leaf0 + grp;
+        const int64_t i0 = leaf < nleaf ? leaf_beg[leaf] : 0, i1 = leaf < nleaf ? leaf_beg[leaf + 1] : 0;
+        const bool any_big = __any_sync(0xffffffffu, i1 - i0 > kP2MBig);
+        for (int bb = 0; bb < B; ++bb) {
+            const T *mb = mass + (int64_t)bb * S;
+            if (!any_big) {
+                clear();
+                const int n = __reduce_max_sync(0xffffffffu, (int)((i1 - i0 + PTS - 1) / PTS));
+                add_points(i0, i1, n, 1, 0, mb);
+                write(leaf, bb, false, false, true);
+                continue;
+            }
+            for (int q = 0; q < NG; ++q) {
+                const int64_t b0 = __shfl_sync(0xffffffffu, (long long)i0, q * GL);
+                const int64_t b1 = __shfl_sync(0xffffffffu, (long long)i1, q * GL);
+                if (leaf0 + q >= nleaf) break;
+                for (int64_t s0 = b0;; s0 += kP2MSeg) {
+                    const int64_t s1 = min(b1, s0 + kP2MSeg);
+                    clear();
+                    add_points(s0, s1, (int)((s1 - s0 + NG * PTS - 1) / (NG * PTS)), NG, grp, mb);
+                    write(leaf0 + q, bb, true, s0 > b0, s1 == b1);
+                    if (s1 == b1) break;
+                }
             }
         }
     }
+    if (amax) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) big_in = fmaxf(big_in, __shfl_xor_sync(0xffffffffu, big_in, o));
+        if (lane == 0 && big_in > 0.f) atomicMax(amax, __float_as_uint(big_in));
+    }
+}
+
+template <class T, int GL, int NS, int SW>
+gf_status launch_point_p2m(const gf_plan_s *plan, int B, uint32_t *amax, int64_t lo, int64_t hi, cudaStream_t st) {
+    const FmmPlan *F = plan->fmm;
+    const PointSet &P = plan->pts;
+    const FmmLevel &lv = F->lev[F->L];
+    const size_t shm = (size_t)kP2MWarps * 32 * p2m_stride(F->p) * 16;
+    GF_TRY((ensure_smem(point_p2m<T, GL, NS, SW>, shm)));
+    const int64_t per_block = kP2MWarps * (32 / GL);
+    const unsigned grid = (unsigned)std::min<int64_t>((lv.ns + per_block - 1) / per_block, 152 * 64);
+    point_p2m<T, GL, NS, SW><<<grid, kP2MWarps * 32, shm, st>>>((const T *)P.loc, (const T *)F->mass, P.leaf_beg, lv.ns,
+                                                            P.S, F->p, B, F->KS, (T *)lv.me, amax, lo, hi);
+    GF_KERNEL_DONE();
+    return GF_OK;
 }
 
 // Near field over the points of the 27 neighbour leaves + the L2P gradient
@@ -1020,82 +1007,19 @@ gf_status upload_point_tables(int device) {
     static unsigned long long done = 0;
     std::lock_guard<std::mutex> lk(mu);
     if (device >= 0 && device < 64 && ((done >> device) & 1ull)) return GF_OK;
-    double pa[kPT] = {}, pb[kPT] = {}, pf[kMaxP + 1] = {};
-    for (int n = 1; n <= kMaxP; ++n) {
-        for (int m = 0; m < n; ++m) {
-            const int t = n * (n + 1) / 2 + m;
-            const double inv = 1.0 / std::sqrt((double)((n + m) * (n - m)));
-            pa[t] = (2 * n - 1) * inv;
-            pb[t] = n - 1 > m ? std::sqrt((double)((n - 1 + m) * (n - 1 - m))) * inv : 0.0;
+    // s_nm: prod_{j <= m} -sqrt((2j-1) / (2j)) for the sectoral steps, then
+    // prod_{j = m+1..n} (2j-1) / sqrt((j+m)(j-m))
+    double ps[(kMaxP + 1) * (kMaxP + 1)] = {};
+    double sect = 1.0;
+    for (int m = 0; m <= kMaxP; ++m) {
+        if (m > 0) sect *= -std::sqrt((2.0 * m - 1.0) / (2.0 * m));
+        double v = sect;
+        for (int n = m; n <= kMaxP; ++n) {
+            if (n > m) v *= (2 * n - 1) / std::sqrt((double)((n + m) * (n - m)));
+            ps[n * n + (m == 0 ? 0 : 2 * m - 1)] = v;
         }
-        pf[n] = -std::sqrt((2.0 * n - 1.0) / (2.0 * n));
     }
-    float paf[kPT], pbf[kPT], pff[kMaxP + 1];
-    for (int t = 0; t < kPT; ++t) {
-        paf[t] = (float)pa[t];
-        pbf[t] = (float)pb[t];
-    }
-    for (int n = 0; n <= kMaxP; ++n) pff[n] = (float)pf[n];
-    GF_CUDA(cudaMemcpyToSymbol(c_pa, pa, sizeof(pa)));
-    GF_CUDA(cudaMemcpyToSymbol(c_pb, pb, sizeof(pb)));
-    GF_CUDA(cudaMemcpyToSymbol(c_pf, pf, sizeof(pf)));
-    {
-        // packed pairs, and the order groups and entry order of the FP32 P2M
-        float2 a2[kPT], nb2[kPT], f2[kMaxP + 1], nf2[kMaxP + 1];
-        for (int t = 0; t < kPT; ++t) {
-            a2[t] = make_float2(paf[t], paf[t]);
-            nb2[t] = make_float2(-pbf[t], -pbf[t]);
-        }
-        for (int n = 0; n <= kMaxP; ++n) {
-            f2[n] = make_float2(pff[n], pff[n]);
-            nf2[n] = make_float2(-pff[n], -pff[n]);
-        }
-        static P2MGroups grp[kMaxP + 1];
-        static short ktab[kMaxP + 1][(kMaxP + 1) * (kMaxP + 1)];
-        memset(grp, 0, sizeof(grp));
-        memset(ktab, 0, sizeof(ktab));
-        for (int pp = 1; pp <= kMaxP; ++pp) {
-            P2MGroups &G = grp[pp];
-            int e = 0, cur = 0;
-            G.ng = 0;
-            G.m_lo[0] = 0;
-            G.ent0[0] = 0;
-            for (int m = 0; m <= pp; ++m) {
-                const int em = m == 0 ? pp + 1 : 2 * (pp + 1 - m);
-                if (cur + em > kGrpEnt) {   // close the group before order m
-                    ++G.ng;
-                    G.m_lo[G.ng] = m;
-                    G.ent0[G.ng] = e;
-                    cur = 0;
-                }
-                for (int n = m; n <= pp; ++n) {
-                    if (m == 0) {
-                        ktab[pp][e++] = (short)(n * n);
-                    } else {
-                        ktab[pp][e++] = (short)(n * n + 2 * m - 1);
-                        ktab[pp][e++] = (short)(n * n + 2 * m);
-                    }
-                }
-                cur += em;
-            }
-            ++G.ng;
-            G.m_lo[G.ng] = pp + 1;
-            G.ent0[G.ng] = e;
-            if (G.ng > kMaxGroups || e != (pp + 1) * (pp + 1)) {
-                set_error("internal: P2M order groups for p = %d", pp);
-                return GF_ERR_CUDA;
-            }
-        }
-        GF_CUDA(cudaMemcpyToSymbol(c_a2, a2, sizeof(a2)));
-        GF_CUDA(cudaMemcpyToSymbol(c_nb2, nb2, sizeof(nb2)));
-        GF_CUDA(cudaMemcpyToSymbol(c_f2, f2, sizeof(f2)));
-        GF_CUDA(cudaMemcpyToSymbol(c_nf2, nf2, sizeof(nf2)));
-        GF_CUDA(cudaMemcpyToSymbol(c_grp, grp, sizeof(grp)));
-        GF_CUDA(cudaMemcpyToSymbol(c_ktab, ktab, sizeof(ktab)));
-    }
-    GF_CUDA(cudaMemcpyToSymbol(c_paf, paf, sizeof(paf)));
-    GF_CUDA(cudaMemcpyToSymbol(c_pbf, pbf, sizeof(pbf)));
-    GF_CUDA(cudaMemcpyToSymbol(c_pff, pff, sizeof(pff)));
+    GF_CUDA(cudaMemcpyToSymbol(c_ps, ps, sizeof(ps)));
     GF_TRY(upload_l2p_coefs());
     if (device >= 0 && device < 64) done |= 1ull << device;
     return GF_OK;
@@ -1343,24 +1267,20 @@ gf_status points_masses(gf_plan_s *plan, const void *rho, int rho_dtype, int B, 
 template <class T>
 gf_status points_p2m(gf_plan_s *plan, int B, cudaStream_t st) {
     FmmPlan *F = plan->fmm;
-    const PointSet &P = plan->pts;
     const FmmLevel &lv = F->lev[F->L];
-    if constexpr (sizeof(T) == 4) {
-        const unsigned grid = (unsigned)std::min<int64_t>((lv.ns + kP2MWarpsF - 1) / kP2MWarpsF, 152 * 64);
-        point_p2m_f32<<<grid, kP2MWarpsF * 32, 0, st>>>((const float *)P.loc, (const float *)F->mass, P.leaf_beg,
-                                                        lv.ns, P.S, F->p, B, F->KS, (float *)lv.me);
-        GF_KERNEL_DONE();
-        return GF_OK;
-    }
-    constexpr int W = p2m_warps<T>();
-    const int stride = p2m_stride(F->K);
-    const size_t shm = sizeof(T) * W * 32 * (size_t)stride;
-    GF_TRY(ensure_smem(point_p2m<T>, shm));
-    const unsigned grid = (unsigned)std::min<int64_t>((lv.ns + W - 1) / W, 152 * 64);
-    point_p2m<T><<<grid, W * 32, shm, st>>>((const T *)P.loc, (const T *)F->mass, P.leaf_beg, lv.ns, P.S, F->p, B,
-                                            F->KS, stride, (T *)lv.me);
-    GF_KERNEL_DONE();
-    return GF_OK;
+    // the rows whose largest component scales the leaf level's M2L inputs
+    const int64_t slab = lv.sn[0] * lv.sn[1];
+    const bool in = F->amax_fused && lv.m2l_z1 >= lv.m2l_z0;
+    uint32_t *amax = in ? F->tc_amax + F->L : nullptr;
+    const int64_t lo = in ? lv.m2l_z0 * slab : 0, hi = in ? (lv.m2l_z1 + 1) * slab : 0;
+    // lanes per leaf: the power of two that holds the p/2 + 1 lanes' orders;
+    // terms per lane in a few sizes (what a size has beyond them is skipped)
+    const int p = F->p;
+    if (p <= 7) return launch_point_p2m<T, 4, 9, 2>(plan, B, amax, lo, hi, st);
+    if (p <= 10) return launch_point_p2m<T, 8, 11, 5>(plan, B, amax, lo, hi, st);
+    if (p <= 12) return launch_point_p2m<T, 8, 13, 7>(plan, B, amax, lo, hi, st);
+    if (p <= 15) return launch_point_p2m<T, 8, 17, 8>(plan, B, amax, lo, hi, st);
+    return launch_point_p2m<T, 16, 17, 9>(plan, B, amax, lo, hi, st);
 }
 
 template <class T>
