@@ -1,5 +1,5 @@
 // gf_prim.cuh -- device-wide primitives used by the tree build:
-// exclusive scan and a stable LSD radix sort of (uint64 key, int32 value).
+// exclusive scan and a stable LSD radix sort of keys with their indices.
 #pragma once
 
 #include "gf_internal.cuh"
@@ -15,10 +15,15 @@ size_t sort_scratch_bytes(int64_t n);
 gf_status exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, void *scratch,
                              cudaStream_t st);
 
-// Stable sort of keys (the low `bits` bits matter) carrying vals.  Results
-// end in keys/vals; keys_alt/vals_alt are ping-pong buffers of size n.
-gf_status radix_sort_u64(uint64_t *keys, int32_t *vals, uint64_t *keys_alt, int32_t *vals_alt,
-                         int64_t n, int bits, void *scratch, cudaStream_t st);
+// Stable sort of n keys (the low `bits` bits matter; K = uint32_t or uint64_t)
+// with their indices: sorted keys in keys, where each came from in vals.  The
+// unsorted keys are in radix_sort_input(...), one of the two ping-pong buffers
+// of size n (so that the last pass ends in keys without a copy).
+template <class K>
+K *radix_sort_input(K *keys, K *keys_alt, int bits);
+template <class K>
+gf_status radix_sort(K *keys, int32_t *vals, K *keys_alt, int32_t *vals_alt, int64_t n, int bits, void *scratch,
+                     cudaStream_t st);
 
 // min/max of the three coordinates of n points [n][3] (FP64) into out[6]
 // (min x,y,z, max x,y,z); out must hold 12 doubles (6 of scratch).

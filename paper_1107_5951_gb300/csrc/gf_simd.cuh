@@ -266,26 +266,14 @@ __device__ __forceinline__ float fix_to_f32(long long v) {
                            (unsigned)((n >> 40) & 0x7fffffull));
 }
 
-// v 2^-k as a double (|v| < 2^63; exact for |v| < 2^53, else truncated).
-__device__ __forceinline__ double fix_to_f64(long long v, int k) {
-    if (v == 0) return 0.0;
-    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    const int lz = __clzll((long long)a);
-    const unsigned long long n = a << lz;   // leading one at bit 63
-    const long long e = 63 - lz - k + 1023;
-    return __longlong_as_double((long long)((v < 0 ? 0x8000000000000000ull : 0ull) |
-                                            ((unsigned long long)e << 52) | ((n >> 11) & 0xfffffffffffffull)));
-}
-
-// trunc(f 2^k) for a float f with |f 2^k| < 2^62.
-__device__ __forceinline__ long long f32_to_fix(float f, int k) {
-    const unsigned b = __float_as_uint(f);
-    const int e = (int)((b >> 23) & 0xff);
-    if (e == 0) return 0;
-    const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
-    const int sh = e - 150 + k;
-    const long long v = sh >= 0 ? (m << sh) : (sh > -32 ? (m >> -sh) : 0);
-    return (b >> 31) ? -v : v;
+// A double as a float by truncation, integer operations only: below the normal
+// FP32 range zero, above it (and for NaN) infinity.
+__device__ __forceinline__ float f32_trunc(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi = (unsigned)(b >> 32), sign = hi & 0x80000000u;
+    const int e = (int)((hi >> 20) & 0x7ff) - 1023;
+    const unsigned mag = ((unsigned)(e + 127) << 23) | ((unsigned)(b >> 29) & 0x7fffffu);
+    return __uint_as_float(sign | (e < -126 ? 0u : e > 127 ? 0x7f800000u : mag));
 }
 
 // A float as a double (subnormals read as zero; infinities and NaNs kept).

@@ -64,7 +64,7 @@ struct Geo {
 // Leaf key of every observer: floor((x - lo) * inv_s) with one rounded
 // subtraction and one rounded multiplication, clamped to the root.
 __global__ void obs_keys(const double *__restrict__ obs, int64_t M, Geo g, uint64_t *__restrict__ keys,
-                         int32_t *__restrict__ vals, int *__restrict__ status) {
+                         int *__restrict__ status) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
     const float top = (float)((1ll << g.L) - 1);
@@ -88,7 +88,6 @@ __global__ void obs_keys(const double *__restrict__ obs, int64_t M, Geo g, uint6
         c[a] = (int64_t)fl;
     }
     keys[j] = morton(c[0], c[1], c[2]);
-    vals[j] = (int32_t)j;
 }
 
 // The tree is built without host round trips: counts stay on the device
@@ -568,9 +567,9 @@ gf_status fmm_observer_tree(gf_plan_s *plan, const double *obs, const double oz[
     GF_TRY(A.alloc(&scratch, scr));
     F->okey = keys;
     if (M > 0) {
-        obs_keys<<<ceil_div(M, 256), 256, 0, st>>>(obs, M, g, keys, F->perm, plan->d_status);
+        obs_keys<<<ceil_div(M, 256), 256, 0, st>>>(obs, M, g, radix_sort_input(keys, keys2, 3 * L), plan->d_status);
         GF_KERNEL_DONE();
-        GF_TRY(radix_sort_u64(keys, F->perm, keys2, vals2, M, 3 * L, scratch, st));
+        GF_TRY(radix_sort(keys, F->perm, keys2, vals2, M, 3 * L, scratch, st));
     }
 
     // ---- leaves and their ancestors.  Counts stay on the device (d_cnt:
