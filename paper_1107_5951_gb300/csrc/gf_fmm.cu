@@ -1190,7 +1190,240 @@ __global__ void __launch_bounds__(kFarWarps * 32, 6) eval_far_kernel(EvalArgs a,
     }
 }
 
-// Near field + far field of closed-form voxels (SUM-AN in the FMM): one warp
+constexpr int kAnNb = 12;                          // voxels per axis of the 27-leaf block of closed-form voxels
+constexpr int kAnBlock = kAnNb * kAnNb * kAnNb;
+
+// Near field of closed-form voxels (SUM-AN in the FMM) in FP32: the sums of
+// eval_kernel's mode 1, the far field following as for quadrature voxels.  One
+// warp per half work item, an observer per lane; the densities of the item's 27
+// neighbour leaves (a 12^3 voxel block, 4^3-voxel leaves) are staged in the
+// warp's shared-memory slice.  The sums are those of an_near_block with radius 2:
+// - Voxels beyond Chebyshev distance 2 of the observer's own: two voxels of a row
+//   at a time as packed pairs.  With r^2 = x^2 + Y, Y, y and z constant on a row,
+//   the midpoint rule and the cube's l = 4 term are x (A + B x^2) and, summed over
+//   the row, y (sum A + y^2 sum B): 22 packed operations for two voxels.  The
+//   voxels of the closed form get r^2 = 1e36, so that they add zero; rows of
+//   leaves without sources are passed over.
+// - The others in closed form on their 6^3 corner lattice, by offset from the
+//   observer's voxel, so that the sign of every coordinate, and with it the form
+//   of every logarithm, is the same across the warp; the corner weights of a row
+//   are differences of column sums.
+// Bound by the instruction issue, logarithms and arctangents above all.  One
+// observer's voxels one by one, both forms and the L2P's square roots and
+// divisions in one kernel, took 1,690 us for 512 x 512 stations over 128^3 voxels;
+// now 600 us and 40 us of far field.
+//
+// Quotients and roots from the approximate reciprocals, refined by their
+// residual (in the last place); operands are normal numbers here.
+__device__ __forceinline__ float an_quot(float n, float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    const float q = n * r;
+    return fmaf(fmaf(-q, d, n), r, q);
+}
+__device__ __forceinline__ float an_root(float x) {
+    const float y = rsqrt_ftz(x), r = x * y;
+    return x > 0.f ? fmaf(fmaf(-r, r, x), 0.5f * y, r) : 0.f;
+}
+
+// atan(n / d), d != 0, as the angle of the smaller to the larger of |n| and |d|:
+// one division for both ranges.  On [0, 1] t + t s q(s), s = t^2, q of degree 8
+// fitted to the smallest largest relative error (2.4e-9; evaluated, 1.2 units in
+// the last place).
+__device__ __forceinline__ float an_angle(float n, float d) {
+    const float an = fabsf(n), ad = fabsf(d);
+    const float t = an_quot(fminf(an, ad), fmaxf(an, ad)), s = t * t;
+    float q = -0.0017539296532049775f;
+    q = fmaf(q, s, 0.010726941749453545f);
+    q = fmaf(q, s, -0.030804593116044998f);
+    q = fmaf(q, s, 0.05755209922790527f);
+    q = fmaf(q, s, -0.08377315104007721f);
+    q = fmaf(q, s, 0.1094203069806099f);
+    q = fmaf(q, s, -0.142619326710701f);
+    q = fmaf(q, s, 0.1999826580286026f);
+    q = fmaf(q, s, -0.3333328366279602f);
+    float r = fmaf(q * s, t, t);
+    if (an > ad) r = (1.57079637f - r) - 4.37113883e-8f;   // pi / 2 in two parts
+    return __uint_as_float(__float_as_uint(r) ^ ((__float_as_uint(n) ^ __float_as_uint(d)) & 0x80000000u));
+}
+
+// ln(a + R), R = sqrt(a^2 + q); 0 when q is zero
+__device__ __forceinline__ float an_ln_of(float a, float q, float R) {
+    float x = a + R;
+    if (a < 0.f) x = an_quot(q, R - a);
+    return q > 0.f ? logf(x) : 0.f;
+}
+
+constexpr int kAnWarps = 4;
+inline __host__ __device__ int near_an_slice() { return kAnBlock + 32; }   // floats: densities, 27 leaf numbers
+
+__global__ void __launch_bounds__(kAnWarps * 32, 7) near_an_kernel(EvalArgs a) {
+    extern __shared__ __align__(16) unsigned char shraw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *blk = reinterpret_cast<float *>(shraw) + (size_t)warp * near_an_slice();
+    int *slots = reinterpret_cast<int *>(blk + kAnBlock);
+    const float *tloc = reinterpret_cast<const float *>(a.tloc);
+    const float *mass = reinterpret_cast<const float *>(a.mass);
+    float *ns = reinterpret_cast<float *>(a.nsum);
+    constexpr float c = 7.f / 192.f;
+    const uint64_t c3 = pk2(3.f * c, 3.f * c), nc9 = pk2(-9.f * c, -9.f * c), one = pk2(1.f, 1.f), half = pk2(0.5f, 0.5f);
+    const int64_t units = 2 * a.n_items;
+    for (int64_t un = (int64_t)blockIdx.x * kAnWarps + warp; un < units; un += (int64_t)gridDim.x * kAnWarps) {
+        const int4 item = a.items[un >> 1];
+        const int r0 = 32 * (int)(un & 1);
+        if (r0 >= item.z) continue;
+        const int leaf = item.x;
+        const uint64_t key = a.tkey[leaf];
+        const bool on = r0 + lane < item.z;
+        const int64_t i0 = item.y + (on ? r0 + lane : r0);
+        // position in the block (own leaf at [4, 8)) and the voxel it is in
+        const float tx = tloc[3 * i0] + 6.f, ty = tloc[3 * i0 + 1] + 6.f, tz = tloc[3 * i0 + 2] + 6.f;
+        const int vi = min(max((int)floorf(tx), 2), kAnNb - 3), vj = min(max((int)floorf(ty), 2), kAnNb - 3),
+                  vk = min(max((int)floorf(tz), 2), kAnNb - 3);
+        uint32_t have;   // the neighbour leaves that hold sources
+        int slot = -1;
+        {
+            int64_t lc[3] = {0, 0, 0};
+            for (int bit = 0; bit < a.L; ++bit)
+                for (int d = 0; d < 3; ++d) lc[d] |= (int64_t)((key >> (3 * bit + d)) & 1) << bit;
+            if (lane < 27) {
+                const int64_t X = lc[0] + lane % 3 - 1, Y = lc[1] + (lane / 3) % 3 - 1, Z = lc[2] + lane / 9 - 1;
+                const int64_t sx = X - a.blk.lo[0], sy = Y - a.blk.lo[1], sz = Z - a.blk.lo[2];
+                if (sx >= 0 && sy >= 0 && sz >= 0 && sx < a.blk.n[0] && sy < a.blk.n[1] && sz < a.blk.n[2] &&
+                    in_source_part(X, Y, Z, a.L - 2, a.part_lo, a.part_hi))
+                    slot = (int)((sz * a.blk.n[1] + sy) * a.blk.n[0] + sx);
+            }
+            have = __ballot_sync(0xffffffffu, slot >= 0);
+            __syncwarp();   // the unit before has read its slots
+            slots[lane] = slot;
+        }
+        uint64_t X2[6], XP[6];   // offsets along x of the row's pairs of voxels, and their squares
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            XP[q] = pk2(tx - (2 * q + 0.5f), tx - (2 * q + 1.5f));
+            X2[q] = mul2(XP[q], XP[q]);
+        }
+        const uint32_t nearx = 0x1fu << (vi - 2);
+        for (int bb = 0; bb < a.B; ++bb) {
+            __syncwarp();
+            // one 4-voxel row of a leaf per lane and step: rows (z, y) of 3 leaves
+            for (int e = lane; e < 3 * kAnNb * kAnNb; e += 32) {
+                const int xl = e % 3, yz = e / 3, y = yz % kAnNb, z = yz / kAnNb;
+                const int l = (z >> 2) * 9 + (y >> 2) * 3 + xl;
+                const int sl = slots[l];
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (sl >= 0)
+                    v = __ldg(reinterpret_cast<const float4 *>(mass + ((int64_t)sl * a.B + bb) * 64) + (z & 3) * 4 + (y & 3));
+                *reinterpret_cast<float4 *>(blk + yz * kAnNb + 4 * xl) = v;
+            }
+            __syncwarp();
+            float sx = 0.f, ex = 0.f, sy = 0.f, ey = 0.f, sz = 0.f, ez = 0.f;
+            for (int k = 0; k < kAnNb; ++k) {
+                const float z = tz - (k + 0.5f), z2 = z * z;
+                for (int j = 0; j < kAnNb; ++j) {
+                    if (!(have >> ((k >> 2) * 9 + (j >> 2) * 3) & 7u)) continue;
+                    const float y = ty - (j + 0.5f), y2 = y * y;
+                    const float q2 = y2 + z2, q4 = y2 * y2 + z2 * z2;
+                    const uint64_t Q2 = pk2(q2, q2), Q4 = pk2(q4, q4);
+                    const uint32_t skip = max(abs(j - vj), abs(k - vk)) <= 2 ? nearx : 0u;
+                    const bool any = __any_sync(0xffffffffu, skip != 0u);
+                    const float4 *row = reinterpret_cast<const float4 *>(blk + (k * kAnNb + j) * kAnNb);
+                    uint64_t SA = 0, SB = 0, GX = 0;
+#pragma unroll
+                    for (int q = 0; q < 6; q += 2) {
+                        const float4 m4 = row[q / 2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const uint64_t M = h ? pk2(m4.z, m4.w) : pk2(m4.x, m4.y);
+                            uint64_t R2 = add2(X2[q + h], Q2);
+                            if (any) {
+                                float ra, rb;
+                                up2(R2, ra, rb);
+                                R2 = pk2((skip >> (2 * (q + h))) & 1u ? 1e36f : ra,
+                                         (skip >> (2 * (q + h))) & 2u ? 1e36f : rb);
+                            }
+                            float ra, rb;
+                            up2(R2, ra, rb);
+                            uint64_t I = pk2(rsqrt_ftz(ra), rsqrt_ftz(rb));
+                            // one Newton step: I += I/2 (1 - R2 I^2)
+                            const uint64_t E = fma2(mul2(R2 ^ 0x8000000080000000ull, I), I, one);
+                            I = fma2(mul2(half, I), E, I);
+                            const uint64_t I2 = mul2(I, I), I3 = mul2(I, I2), I9 = mul2(I3, mul2(I3, I3));
+                            const uint64_t S4 = fma2(X2[q + h], X2[q + h], Q4);
+                            // A = r^-3 + c r^-9 (3 r^2 - 9 S4 / r^2), B = 4 c r^-9 (its 4 c at the row's end)
+                            const uint64_t A = fma2(I9, fma2(nc9, mul2(S4, I2), mul2(c3, R2)), I3);
+                            const uint64_t MA = mul2(M, A), MB = mul2(M, I9);
+                            SA = add2(SA, MA);
+                            SB = add2(SB, MB);
+                            GX = fma2(fma2(mul2(MB, pk2(4.f * c, 4.f * c)), X2[q + h], MA), XP[q + h], GX);
+                        }
+                    }
+                    float lo, hi;
+                    up2(SA, lo, hi);
+                    const float sa = lo + hi;
+                    up2(SB, lo, hi);
+                    const float sb = 4.f * c * (lo + hi);
+                    up2(GX, lo, hi);
+                    two_sum(sx, ex, lo + hi);
+                    two_sum(sy, ey, y * (sa + sb * y2));
+                    two_sum(sz, ez, z * (sa + sb * z2));
+                }
+            }
+            // closed form: corners v - 2 .. v + 3 of the 5^3 voxels around the observer's
+            const float *own = blk + ((vk - 2) * kAnNb + vj - 2) * kAnNb + vi - 2;
+            for (int K = 0; K < 6; ++K) {
+                const float w = (float)(vk - 2 + K) - tz, w2 = w * w;
+                float qp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // column sums of the row before
+                for (int J = 0; J < 6; ++J) {
+                    float t[5];   // signed density sums of the corner row's 5 voxel columns
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) {
+                        const float up = K < 5 && J < 5 ? own[(K * kAnNb + J) * kAnNb + i] : 0.f;
+                        const float dn = K > 0 && J < 5 ? own[((K - 1) * kAnNb + J) * kAnNb + i] : 0.f;
+                        const float q = dn - up;
+                        t[i] = q - qp[i];
+                        qp[i] = q;
+                    }
+                    float gx = 0.f, gy = 0.f, gz = 0.f;
+                    const float v = (float)(vj - 2 + J) - ty, v2 = v * v, qu = v2 + w2;
+                    float tp = 0.f;
+#pragma unroll 1   // the body is some 250 instructions: six copies overflow the instruction cache
+                    for (int I = 0; I < 6; ++I) {
+                        const float D = t[0] - tp;
+                        tp = t[0];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) t[i] = t[i + 1];
+                        t[4] = 0.f;
+                        if (!__any_sync(0xffffffffu, D != 0.f)) continue;
+                        const float u = (float)(vi - 2 + I) - tx, u2 = u * u;
+                        const float R = an_root(u2 + qu);
+                        const float Lu = an_ln_of(u, qu, R), Lv = an_ln_of(v, u2 + w2, R), Lw = an_ln_of(w, u2 + v2, R);
+                        const float au = u != 0.f ? u * an_angle(v * w, u * R) : 0.f;
+                        const float av = v != 0.f ? v * an_angle(w * u, v * R) : 0.f;
+                        const float aw = w != 0.f ? w * an_angle(u * v, w * R) : 0.f;
+                        gx += D * (v * Lw + w * Lv - au);
+                        gy += D * (w * Lu + u * Lw - av);
+                        gz += D * (u * Lv + v * Lu - aw);
+                    }
+                    two_sum(sx, ex, gx);
+                    two_sum(sy, ey, gy);
+                    two_sum(sz, ez, gz);
+                }
+            }
+            if (on) {
+                float *q = ns + ((int64_t)bb * a.M + i0) * 6;
+                q[0] = sx;
+                q[1] = ex;
+                q[2] = sy;
+                q[3] = ey;
+                q[4] = sz;
+                q[5] = ez;
+            }
+        }
+    }
+}
+
+// Near field + far field of closed-form voxels in FP64: one warp
 // per work item, two observers per lane.  The densities of the item's 27
 // neighbour leaves (a 12^3 voxel block, 4^3-voxel leaves) are staged in the
 // warp's shared-memory slice; each observer takes the voxels within
@@ -1198,9 +1431,6 @@ __global__ void __launch_bounds__(kFarWarps * 32, 6) eval_far_kernel(EvalArgs a,
 // lattice and the others by the midpoint rule with a uniform cube's l = 4
 // term (an_near_block); the far field is the L2P gradient of the leaf's
 // local expansion (made from exact voxel moments).
-constexpr int kAnNb = 12;                          // voxels per axis of the 27-leaf block
-constexpr int kAnBlock = kAnNb * kAnNb * kAnNb;
-
 inline __host__ __device__ int eval_an_slice(int P2) { return (kAnBlock + 3 * P2 + 27 * 2 + 7) & ~7; }
 
 template <class T, int RAD>
@@ -1566,6 +1796,12 @@ gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_
         const unsigned fg = (unsigned)std::min<int64_t>((F->n_items + kFarWarps - 1) / kFarWarps, 152 * 64);
         const unsigned rg = std::min<unsigned>(fg, resident_blocks(eval_far_kernel, kFarWarps * 32, fshm));
         eval_far_kernel<<<rg, kFarWarps * 32, fshm, st>>>(a, F->leaf_beg);
+    } else if (sizeof(T) == 4 && (plan->opt.reserved0 & GF_FLAG_SUM_AN)) {
+        const size_t ashm = sizeof(float) * kAnWarps * near_an_slice();
+        GF_TRY((ensure_smem(near_an_kernel, ashm)));
+        const unsigned ag = (unsigned)std::min<int64_t>((2 * F->n_items + kAnWarps - 1) / kAnWarps, 152 * 64);
+        near_an_kernel<<<std::min<unsigned>(ag, resident_blocks(near_an_kernel, kAnWarps * 32, ashm)), kAnWarps * 32, ashm,
+                         st>>>(a);
     } else if (sizeof(T) == 4 && n1 == 4) {
         GF_TRY((ensure_smem(eval_kernel<float, 4>, shm)));
         const unsigned rg = std::min<unsigned>(grid, resident_blocks(eval_kernel<float, 4>, kEvalWarps * 32, shm));
@@ -1660,7 +1896,7 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     EvalArgs ea;
     int n1 = 0;
     if (eval_on) n1 = eval_setup<T>(plan, B, g, gz, ea);
-    const bool beside = eval_on && !an && plan->side && !plan->timing;
+    const bool beside = eval_on && !(an && sizeof(T) == 8) && plan->side && !plan->timing;
     // a5/a6: M2L at every level (each overwrites its level's LE), then the
     // L2L chain from level 3 down, which adds each finished parent LE.
     GF_TRY(m2l_run<T>(plan, B, false, st, beside ? plan->ev_fork : nullptr));   // marks the input split's end (4)
@@ -1682,19 +1918,14 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     // a7-a9: near field + L2P + combine + scatter
     if (pts) {
         GF_TRY(points_eval<T>(plan, B, g, gz, st));
-    } else if (eval_on && an) {
-        // closed-form voxels: radius 2 in FP32, 4 in FP64 (the closed form
-        // cancels like (d/h)^3, so the precision sets how far it is used;
-        // beyond it the corrected midpoint rule errs like (h/d)^6)
+    } else if (eval_on && an && sizeof(T) == 8) {
+        // closed-form voxels: radius 2 in FP32 (near_an_kernel), 4 in FP64 (the
+        // closed form cancels like (d/h)^3, so the precision sets how far it is
+        // used; beyond it the corrected midpoint rule errs like (h/d)^6)
         const unsigned grid = (unsigned)std::min<int64_t>((F->n_items + kEvalWarps - 1) / kEvalWarps, 152 * 64);
         const size_t shan = sizeof(T) * kEvalWarps * eval_an_slice(F->p * F->p) + 64;
-        if (sizeof(T) == 4) {
-            GF_TRY((ensure_smem(eval_an_kernel<T, 2>, shan)));
-            eval_an_kernel<T, 2><<<grid, kEvalWarps * 32, shan, st>>>(ea);
-        } else {
-            GF_TRY((ensure_smem(eval_an_kernel<T, 4>, shan)));
-            eval_an_kernel<T, 4><<<grid, kEvalWarps * 32, shan, st>>>(ea);
-        }
+        GF_TRY((ensure_smem(eval_an_kernel<double, 4>, shan)));
+        eval_an_kernel<double, 4><<<grid, kEvalWarps * 32, shan, st>>>(ea);
         GF_KERNEL_DONE();
     } else if (eval_on) {
         if (beside)
