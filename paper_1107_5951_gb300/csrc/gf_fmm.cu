@@ -1698,7 +1698,8 @@ gf_status fmm_alloc_workspaces(gf_plan_s *plan, cudaStream_t st) {
     }
     GF_TRY(get_tables(plan->device, F->p, st, &F->tab));
     if (!F->points) GF_TRY(get_p2m(plan, st));
-    return m2l_tc_prepare(plan);
+    GF_TRY(m2l_tc_prepare(plan));
+    return m2l_oz_prepare(plan);
 }
 
 // ---------------------------------------------------------------- forward

@@ -37,7 +37,15 @@ struct FmmLevel {
 //   m2l_*[off][c][k]  off = (dz+3)*49 + (dy+3)*7 + (dx+3)
 //   m2m_*[oct][c][k], l2l_*[oct][c][k]  oct = (x&1) | (y&1)<<1 | (z&1)<<2
 //                                          of the child box
+// Digit images of the FP64 M2L on the tensor cores (gf_m2l.cu).
+struct OzTables {
+    unsigned char *img = nullptr;
+    double *cinv = nullptr;
+    int *se = nullptr;
+};
+
 struct Tables {
+    OzTables *oz = new OzTables();   // filled by the first plan that uses it
     int device = -1, p = 0, K = 0, Kp = 0;   // Kp = K rounded up to 8
     // Tensor-core operand images (mixed precision), one bulk copy per
     // pipeline stage, in the 64-byte-swizzled K-major shared-memory layout
@@ -120,6 +128,13 @@ struct FmmPlan {
     uint32_t *m2l_mask[2] = {};
     float *m2l_part = nullptr;
     int4 *m2l_cut = nullptr;
+    // FP64 M2L on the tensor cores (oz != nullptr): split inputs of levels 2..L
+    // (the z-slabs the M2L reads), their rows' scales, partial rows
+    const OzTables *oz = nullptr;
+    unsigned char *oz_split = nullptr;
+    double *oz_rscale = nullptr, *oz_part = nullptr;
+    void *oz_levels = nullptr;
+    int64_t oz_row0[kMaxLevels + 1] = {};
     int m2l_part_ctas = 0;
     // the M2L inputs of levels 2..L split into scaled FP16 high and low
     // parts: for every input row and 32-wide chunk, 64 bytes of high parts

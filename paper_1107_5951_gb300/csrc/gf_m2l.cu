@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "gf_fold.cuh"
@@ -381,7 +382,9 @@ struct TcLevel {
     const int32_t *imap;
     int64_t mlo[3], mn[3];
     const uint32_t *amax;        // largest |input| of the level (float bits)
-    const unsigned char *split;  // the level's inputs split into scaled FP16 parts
+    const unsigned char *split;  // the level's inputs split into scaled FP16 parts (FP64 slices: BF16 digits)
+    const double *rscale;        // FP64 slices: the rows' scales
+    int64_t src0;                // FP64 slices: first box of the source block that has split rows
     int shift;                   // level - 2 (source partition test)
 };
 
@@ -1090,6 +1093,588 @@ m2l_tc(const __grid_constant__ TcArgs a) {
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols));
 }
 
+// ------------------------------------------------ FP64 from BF16 digits
+// The FP64 M2L on the tensor cores (GB300's FP64 pipe runs at 1/64 of its FP32
+// rate; its tensor cores add 8-bit integers' products exactly).  Every input row
+// is scaled by a power of two of its own and every operator column by one of its
+// own, and both are written as kSl = 7 digits in base 256, -128..128, exact in
+// BF16 (56 bits); powers of two per input component, taken from the operators,
+// balance the orders first.  Digit products of equal weight, i + j = d <= 6, add
+// up in one FP32 accumulator, d of them for up to 304 inputs of at most 2^14:
+// below 2^24 for d <= 3, so exact, and beyond it only where the weight is 2^-32 and
+// less of the first digits'.  (The splitting into exactly multipliable slices is
+// Ozaki, Ogita, Oishi and Rump's, 2012.)  What is left out, d >= 7, and the last
+// place of the digits are some 2^-54 of a row's largest term, as much as FP64
+// rounds away in one of its additions.
+//
+// The pipeline is m2l_tc's: tiles of 128 targets, units of one (tile, column
+// group, offset) dealt out over the grid, chunks of 16 inputs in a ring of stages
+// (32-byte rows, 32-byte swizzle), seven accumulators of up to 64 columns in
+// tensor memory.  After an offset the promoters turn the seven sums into one
+// 64-bit integer, exactly, and add it to FP64 sums with the source row's scale.
+// The batch members go one after the other, tiles of 128 boxes of one member:
+// where a tile is cut decides how its sum associates, and a member's result is
+// the same alone and in a batch.
+// Bound by shared-memory and L2 operand traffic and by the promoters, which the
+// tensor cores wait for (no second bank fits).  128^3 with 1,360 targets at p = 14:
+// 1,710 us, where the SIMT M2L takes 10.8 ms; the fields differ by 2e-16.
+constexpr int kSl = 7;
+constexpr int kOzCols = 64;                              // columns of a group, at most
+constexpr uint32_t kOzA = kSl * 128u * 32u;              // A slices of a stage
+__host__ __device__ constexpr uint32_t oz_stage_bytes(int ng) { return kOzA + (uint32_t)kSl * ng * 32u; }
+inline int oz_stages(int ng) {
+    const int n = (int)(kTcSmemBudget / oz_stage_bytes(ng));
+    return n > kTcMaxStages ? kTcMaxStages : n;
+}
+inline int oz_groups(int K) { return (K + kOzCols - 1) / kOzCols; }
+inline int oz_group_cols(int K) { return ((K + oz_groups(K) - 1) / oz_groups(K) + 15) & ~15; }
+inline int oz_chunks(int K) { return (K + 15) / 16; }
+constexpr int kOzRowChunk = 256;                         // bytes of a row's chunk: 7 slices of 16 digits, padded
+
+struct OzArgs {
+    TcArgs t;                   // ntiles: of 128 targets; the launch's are (tile, group) pairs
+    int ngrp, ng, nck;          // column groups, columns of a group, chunks of 16 inputs
+    int nb, bb;                 // batch members of the rows, and the one this launch does (t.B = 1)
+    const unsigned char *img;   // [343][ngrp][nck][kSl][ng rows of 32 bytes, swizzled]
+    const double *cinv;         // [ngrp ng] inverse column scales
+    double *part;               // [2 gridDim][ng][128] partial rows
+};
+
+// Byte offset of 16-byte half h of row r in a slice (8-row atoms of 256 bytes).
+__host__ __device__ __forceinline__ uint32_t swz32(int r, int h) {
+    return (uint32_t)r * 32u + (uint32_t)((h ^ ((r >> 2) & 1)) << 4);
+}
+
+__device__ __forceinline__ uint64_t umma_desc32(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;             // leading byte offset (unused, swizzled K-major)
+    d |= (uint64_t)(256 >> 4) << 32;    // stride byte offset: one 8-row atom
+    d |= (uint64_t)1 << 46;             // descriptor version
+    d |= (uint64_t)6 << 61;             // 32-byte swizzle
+    return d;
+}
+
+// D = FP32, A = B = BF16 (format 1), both K-major
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// Digits of v, |v| <= 2^55, as BF16: v = sum_i d_i 256^(6 - i).
+__device__ __forceinline__ void bf16_digits(long long v, uint16_t d[kSl]) {
+#pragma unroll
+    for (int i = kSl - 1; i >= 0; --i) {
+        const int q = i > 0 ? (int)(signed char)(v & 255) : (int)v;
+        v = (v - q) >> 8;
+        d[i] = (uint16_t)(__float_as_uint((float)q) >> 16);   // |q| <= 128: 8 bits
+    }
+}
+
+// The integer v as FP64, truncated to 53 bits, without the FP64 pipe
+__device__ __forceinline__ double i64_to_f64(long long v) {
+    const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)m);
+    const unsigned long long n = m << (lz & 63);   // leading one at bit 63
+    const unsigned hi = (v < 0 ? 0x80000000u : 0u) + ((unsigned)(63 - lz + 1022) << 20) + (unsigned)(n >> 43);
+    return m ? __hiloint2double((int)hi, (int)(unsigned)(n >> 11)) : 0.0;
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ OzArgs o) {
+    extern __shared__ unsigned char dsm[];
+    unsigned char *base = dsm + ((1024 - (smem_u32(dsm) & 1023)) & 1023);
+    __shared__ __align__(8) uint64_t afull[kTcMaxStages], bfull[kTcMaxStages], empty[kTcMaxStages];
+    __shared__ __align__(8) uint64_t bank_full, bank_empty;
+    __shared__ uint32_t tslot;
+    __shared__ int abort_flag;
+    __shared__ uint32_t pref[kStreamTiles + 1];   // stream: units before each (tile, group)
+    __shared__ uint32_t wtot[kTcWarps];
+    __shared__ int first_tile;
+    const TcArgs &a = o.t;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nck = o.nck, NST = a.nst, NG = o.ng, ngrp = o.ngrp;
+    const int ntg = a.ntiles * ngrp;
+    const uint32_t stage_bytes = oz_stage_bytes(NG), b_bytes = (uint32_t)kSl * NG * 32u;
+    volatile int *abortp = &abort_flag;
+    constexpr int nbox = 128;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tslot)),
+                     "r"(kTcCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < NST; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&afull[i])), "r"(128));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bfull[i])), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty[i])), "r"(1));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bank_full)), "r"(1));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bank_empty)), "r"(8));
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    // this CTA's units [u0, u1), as in m2l_tc with (tile, group) pairs for tiles
+    uint32_t G = 1, T = 0, u0 = 0, u1 = 0;
+    if (a.stream) {
+        uint32_t n[kScanItems], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            const int t = tid * kScanItems + q;
+            n[q] = t < ntg ? __ldg(a.tmask + 8 * (size_t)(t / ngrp) + 6) : 0;
+            sum += n[q];
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int q = 1; q < 32; q <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, q);
+            if (lane >= q) incl += v;
+        }
+        if (lane == 31) wtot[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int w = 0; w < kTcWarps; ++w) {
+            if (w < warp) before += wtot[w];
+            T += wtot[w];
+        }
+        uint32_t run = before + incl - sum;
+        G = min(gridDim.x, max(1u, T / (uint32_t)a.min_units));
+        if (blockIdx.x < G) {
+            u0 = (uint32_t)((uint64_t)blockIdx.x * T / G);
+            u1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * T / G);
+        }
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            const int t = tid * kScanItems + q;
+            if (t <= ntg) pref[t] = run;
+            if (t < ntg && u0 >= run && u0 < run + n[q]) first_tile = t;
+            run += n[q];
+        }
+        if (tid == 0) pref[ntg] = T;
+    } else {
+        if (tid == 0) first_tile = (int)blockIdx.x;
+        u1 = __ldg(a.tmask + 8 * (size_t)((int)blockIdx.x / ngrp) + 6);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tslot;
+    const int units = (int)(u1 - u0);
+    const int t0 = units > 0 ? first_tile : 0;
+    if (a.stream && tid == 0) {   // for m2l_oz_join
+        a.mcut[blockIdx.x] = make_int4(t0, (int)pref[t0], (int)pref[t0 + 1], (int)G);
+        if (blockIdx.x == 0) a.mcut[gridDim.x] = make_int4((int)T, 0, 0, 0);
+    }
+    auto seg_lo = [&](int t) -> int { return a.stream && pref[t] < u0 ? (int)(u0 - pref[t]) : 0; };
+    auto seg_n = [&](int t) -> int {
+        return a.stream ? (int)(min(u1, pref[t + 1]) - max(u0, pref[t])) : units;
+    };
+    // the source box's row index of row `row` of the tile, unit by unit (-1: none)
+    struct Rows {
+        int t, left, cls, slot;
+        const TcLevel *L;
+        TcTarget q;
+        OffsetIter it;
+    };
+    auto next_row = [&](Rows &w) -> int64_t {
+        if (w.left == 0) {
+            ++w.t;
+            w.left = seg_n(w.t);
+            w.it.open(a.tmask, w.t / ngrp, seg_lo(w.t));
+            const TcTile tile = tile_of(a, w.t / ngrp);
+            w.L = tile.L;
+            w.cls = tile.cls;
+            w.q = target_of(tile, nbox, w.slot);
+        }
+        --w.left;
+        const int64_t src = source_of(a, w.L, w.q, w.cls, w.it.next());
+        return src >= 0 ? (src - w.L->src0) * o.nb + o.bb : -1;
+    };
+
+    bool ok = true;
+    if (warp < 4) {
+        // ---------------- A producers: 16 lanes per row's 14 pieces of 16 bytes
+        Rows w{};
+        w.t = t0 - 1;
+        w.slot = tid;
+        const int piece = lane & 15;
+        const int64_t ldb = (int64_t)nck * kOzRowChunk;
+        int s = 0, n_done = 0;
+        uint32_t ph = 0;
+        bool stop = false;
+        const unsigned char *ahead = nullptr;
+        auto locate = [&]() {
+            const int64_t r = next_row(w);
+            ahead = r >= 0 ? w.L->split + r * ldb : nullptr;
+        };
+        if (units > 0) locate();
+        const unsigned char *any = units > 0 ? w.L->split : nullptr;   // a valid address for rows without a source
+        for (int u = 0; u < units && !stop; ++u) {
+            const unsigned char *src = ahead;
+            if (u + 1 < units) locate();
+            const unsigned char *rp[16];
+            uint32_t have = 0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const unsigned char *q =
+                    (const unsigned char *)__shfl_sync(0xffffffffu, (unsigned long long)src, 2 * i + (lane >> 4));
+                rp[i] = (q ? q : any) + 16 * piece;
+                have |= (uint32_t)(q != nullptr) << i;
+            }
+            for (int j = 0; j < nck; ++j) {
+                if (n_done >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) {
+                    stop = true;
+                    break;
+                }
+                if (piece < 2 * kSl) {
+                    const uint32_t sub = smem_u32(base) + (uint32_t)s * stage_bytes + (uint32_t)(piece >> 1) * 4096u;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        cp_async16(sub + swz32(warp * 32 + 2 * i + (lane >> 4), piece & 1), rp[i] + j * kOzRowChunk,
+                                   (have >> i) & 1u ? 16u : 0u);
+                }
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&afull[s])) : "memory");
+                ++n_done;
+                if (++s == NST) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");   // no copy outlives the loop
+    } else if (warp == 4) {
+        // ---------------- MMA issuer
+        const uint32_t idesc = idesc_bf16(128, NG);
+        const uint64_t desc0 = umma_desc32(smem_u32(base));
+        int s = 0, last = -1, it = 0;
+        uint32_t ph = 0;
+        bool stop = false;
+        for (int g = 0; g < units && !stop; ++g) {
+            for (int j = 0; j < nck && !stop; ++j) {
+                // lanes 0, 1: the stage's operands; 2: the bank, read out after the unit before
+                uint32_t bar = 0, par = ph;
+                if (lane < 2) {
+                    bar = smem_u32(lane ? &bfull[s] : &afull[s]);
+                } else if (lane == 2 && j == 0 && g >= 1) {
+                    bar = smem_u32(&bank_empty);
+                    par = (g - 1) & 1;
+                }
+                bool done = bar == 0;
+                long tries = 0;
+                for (; tries < a.wait_tries; ++tries) {
+                    if (!done) done = mbar_try(bar, par);
+                    if (__all_sync(0xffffffffu, done)) break;
+                    if ((tries & 255) == 255 && __any_sync(0xffffffffu, *abortp != 0)) tries = a.wait_tries;
+                }
+                if (tries >= a.wait_tries) {
+                    *abortp = 1;
+                    stop = true;
+                    break;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint64_t ad = desc0 + (uint32_t)s * (stage_bytes >> 4), bd = ad + (kOzA >> 4);
+#pragma unroll
+                    for (int i = 0; i < kSl; ++i)
+#pragma unroll
+                        for (int e = 0; e < kSl - i; ++e)
+                            mma_f16(tmem + (uint32_t)((i + e) * NG), ad + i * (4096 >> 4), bd + (uint32_t)(e * NG * 2), idesc,
+                                    j > 0 || i > 0 ? 1u : 0u);
+                    commit_to(&empty[s]);
+                    if (j + 1 == nck) commit_to(&bank_full);
+                }
+                last = it++;
+                if (++s == NST) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+        }
+        if (last >= 0) mbar_wait(smem_u32(&empty[last % NST]), (uint32_t)((last / NST) & 1), a.wait_tries);
+    } else if (warp == 5) {
+        // ---------------- operator images
+        if (lane == 0) {
+            int t = t0 - 1, left = 0, cls = 0;
+            OffsetIter it;
+            int s = 0, n_done = 0, last = -1;
+            uint32_t ph = 0;
+            bool stop = false;
+            for (int u = 0; u < units && !stop; ++u) {
+                if (left == 0) {
+                    ++t;
+                    left = seg_n(t);
+                    it.open(a.tmask, t / ngrp, seg_lo(t));
+                    cls = tile_of(a, t / ngrp).cls;
+                }
+                --left;
+                const int q = c_il[cls][it.next()];
+                const int dx = (signed char)q, dy = (signed char)(q >> 8), dz = (signed char)(q >> 16);
+                const unsigned char *img =
+                    o.img + ((size_t)((dz + 3) * 49 + (dy + 3) * 7 + (dx + 3)) * ngrp + t % ngrp) * nck * b_bytes;
+                for (int j = 0; j < nck; ++j) {
+                    if (n_done >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) {
+                        stop = true;
+                        break;
+                    }
+                    const uint32_t stage = smem_u32(base) + (uint32_t)s * stage_bytes;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&bfull[s])),
+                                 "r"(b_bytes));
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            stage + kOzA),
+                        "l"(img + (size_t)j * b_bytes), "r"(b_bytes), "r"(smem_u32(&bfull[s]))
+                        : "memory");
+                    last = n_done++;
+                    if (++s == NST) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            // drain, as in m2l_tc
+            for (int j = last - NST + 1 > 0 ? last - NST + 1 : 0; j <= last; ++j)
+                mbar_wait(smem_u32(&bfull[j % NST]), (uint32_t)((j / NST) & 1), a.wait_tries);
+        }
+    } else {
+        // ---------------- promoters: a row and half the columns per thread
+        constexpr int NH = kOzCols / 2;
+        const int pw = warp - 6, pq = warp & 3, half = pw >> 2, nh = NG / 2;
+        const int r = pq * 32 + lane;
+        Rows w{};
+        w.t = t0 - 1;
+        w.slot = r;
+        double acc[NH];
+        int64_t ahead = units > 0 ? next_row(w) : -1;
+        double scale = ahead >= 0 ? __ldg(w.L->rscale + ahead) : 0.0;
+        int g = 0;
+        for (int t = t0; g < units; ++t) {
+            const int n = seg_n(t);
+#pragma unroll
+            for (int q = 0; q < NH; ++q) acc[q] = 0.0;
+            for (int e = 0; e < n; ++e, ++g) {
+                const double sc = scale;
+                if (g + 1 < units) {   // the next unit's scale, on its way meanwhile
+                    ahead = next_row(w);
+                    scale = ahead >= 0 ? __ldg(w.L->rscale + ahead) : 0.0;
+                }
+                bool w_ok = mbar_wait_ab(smem_u32(&bank_full), g & 1, abortp, a.wait_tries);
+                w_ok = __all_sync(0xffffffffu, w_ok);   // tcgen05.ld is warp-collective
+                if (!w_ok) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t tb = tmem + ((uint32_t)(pq * 32) << 16) + (uint32_t)(half * nh);
+#pragma unroll
+                for (int c0 = 0; c0 < NH; c0 += 4) {
+                    if (c0 < nh) {
+                        uint32_t d[kSl][4];
+#pragma unroll
+                        for (int i = 0; i < kSl; ++i)
+                            asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                         : "=r"(d[i][0]), "=r"(d[i][1]), "=r"(d[i][2]), "=r"(d[i][3])
+                                         : "r"(tb + (uint32_t)(i * NG + c0)));
+                        // (the registers pass through the wait: nothing reads them before it)
+                        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                                     : "+r"(d[0][0]), "+r"(d[0][1]), "+r"(d[0][2]), "+r"(d[0][3]), "+r"(d[1][0]),
+                                       "+r"(d[1][1]), "+r"(d[1][2]), "+r"(d[1][3]), "+r"(d[2][0]), "+r"(d[2][1]),
+                                       "+r"(d[2][2]), "+r"(d[2][3]), "+r"(d[3][0]), "+r"(d[3][1]));
+                        asm volatile("" : "+r"(d[3][2]), "+r"(d[3][3]), "+r"(d[4][0]), "+r"(d[4][1]), "+r"(d[4][2]),
+                                          "+r"(d[4][3]), "+r"(d[5][0]), "+r"(d[5][1]), "+r"(d[5][2]), "+r"(d[5][3]),
+                                          "+r"(d[6][0]), "+r"(d[6][1]), "+r"(d[6][2]), "+r"(d[6][3]));
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            int v[kSl];
+#pragma unroll
+                            for (int i = 0; i < kSl; ++i) v[i] = __float2int_rn(__uint_as_float(d[i][c]));
+                            // in units of 256^-5 of the first digits' products; |d_0| <= 304 2^14 and so on:
+                            // below 2^62
+                            long long x = (long long)(v[0] * 256 + v[1]) * 65536 + (long long)v[2] * 256 + v[3];
+                            x = x * 65536 + (long long)v[4] * 256 + v[5] + ((v[6] + 128) >> 8);
+                            acc[c0 + c] = fma(i64_to_f64(x), sc, acc[c0 + c]);
+                        }
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bank_empty));
+            }
+            if (*abortp) ok = false;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const int col0 = (t % ngrp) * NG + half * nh;
+            if (a.stream && n < (int)(pref[t + 1] - pref[t])) {
+                // a cut tile: partial rows, summed by m2l_oz_join
+                double *mine = o.part + ((size_t)(2 * blockIdx.x + (pref[t] > u0 ? 1 : 0)) * NG + half * nh) * 128 + r;
+#pragma unroll
+                for (int q = 0; q < NH; ++q)
+                    if (q < nh) mine[q * 128] = acc[q];
+                continue;
+            }
+            const TcTile tile = tile_of(a, t / ngrp);
+            const int64_t row = out_row(a, tile, nbox, r);
+            if (row >= 0) {
+                double *dst = reinterpret_cast<double *>(tile.L->le) + (row * o.nb + o.bb) * a.ldk + col0;
+#pragma unroll
+                for (int q = 0; q < NH; ++q)
+                    if (q < nh && col0 + q < a.K) dst[q] = acc[q] * __ldg(o.cinv + col0 + q);
+            }
+        }
+    }
+    const bool failed = __syncthreads_or(!ok || abort_flag);
+    if (failed && tid == 0) atomicOr(a.status + 1, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols));
+}
+
+// The cut (tile, group)s' partial rows, summed in CTA order (see m2l_join).
+__global__ void __launch_bounds__(512) m2l_oz_join(const __grid_constant__ OzArgs o) {
+    const TcArgs &a = o.t;
+    const int c = (int)blockIdx.x + 1;
+    const int4 cut = a.mcut[c];
+    const uint32_t G = (uint32_t)cut.w, T = a.mcut[gridDim.x + 1].x;
+    if (c >= (int)G) return;
+    const uint32_t p0 = (uint32_t)cut.y, p1 = (uint32_t)cut.z;
+    if ((uint32_t)((uint64_t)c * T / G) == p0) return;
+    const int cf = (int)((((uint64_t)p0 + 1) * G - 1) / T), cl = (int)(((uint64_t)p1 * G - 1) / T);
+    if (c != cf + 1) return;
+    const int r = threadIdx.x & 127;
+    const TcTile tile = tile_of(a, cut.x / o.ngrp);
+    const int64_t row = out_row(a, tile, 128, r);
+    if (row < 0) return;
+    const int first = (uint32_t)((uint64_t)cf * T / G) < p0 ? 1 : 0;
+    const int col0 = (cut.x % o.ngrp) * o.ng;
+    double *dst = reinterpret_cast<double *>(tile.L->le) + (row * o.nb + o.bb) * a.ldk + col0;
+    const double *p = o.part + r;
+    const size_t slot = (size_t)o.ng * 128;
+    for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < o.ng && col0 + q < a.K; q += 4 * (int)gridDim.y) {
+        double s = __ldg(p + (2 * cf + first) * slot + (size_t)q * 128);
+#pragma unroll 8
+        for (int e = cf + 1; e <= cl; ++e) s += __ldg(p + 2 * e * slot + (size_t)q * 128);
+        dst[q] = s * __ldg(o.cinv + col0 + q);
+    }
+}
+
+// Power-of-two exponents of the operator set: se[k] per input component, ce[n]
+// per output column, |T_o[n][k]| 2^(-se[k] - ce[n]) <= 1 over all offsets, each
+// reached within a factor of two or so.  One block; two sweeps.
+__global__ void __launch_bounds__(1024) oz_exponents(const double *__restrict__ cmax, int K, int *__restrict__ se,
+                                                     int *__restrict__ ce) {
+    __shared__ int c1[(kMaxP + 1) * (kMaxP + 1)], s1[(kMaxP + 1) * (kMaxP + 1)];
+    auto expo = [](double v) { return v > 0.0 ? ilogb(v) + 1 : -2000; };   // v < 2^expo
+    for (int n = threadIdx.x; n < K; n += blockDim.x) {
+        int e = -2000;
+        for (int k = 0; k < K; ++k) e = max(e, expo(cmax[(size_t)k * K + n]));
+        c1[n] = e;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        int e = -2000;
+        for (int n = 0; n < K; ++n)
+            if (c1[n] > -2000) e = max(e, expo(cmax[(size_t)k * K + n]) - c1[n]);
+        s1[k] = e > -1000 ? e : 0;
+        se[k] = s1[k];
+    }
+    __syncthreads();
+    for (int n = threadIdx.x; n < K; n += blockDim.x) {
+        int e = -2000;
+        for (int k = 0; k < K; ++k) e = max(e, expo(cmax[(size_t)k * K + n]) - s1[k]);
+        ce[n] = e > -1000 ? e : 0;
+    }
+}
+
+// Largest |T_o[n][k]| over the offsets, per (k, n).
+__global__ void oz_absmax(const double *__restrict__ tab, int KK, double *__restrict__ cmax) {
+    const int e = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (e >= KK) return;
+    double m = 0.0;
+    for (int off = 0; off < 343; ++off) {
+        const int dx = off % 7 - 3, dy = (off / 7) % 7 - 3, dz = off / 49 - 3;
+        if (max(abs(dx), max(abs(dy), abs(dz))) >= 2) m = fmax(m, fabs(tab[(size_t)off * KK + e]));
+    }
+    cmax[e] = m;
+}
+
+__global__ void oz_images(const double *__restrict__ tab, int K, int ngrp, int ng, int nck, const int *__restrict__ se,
+                          const int *__restrict__ ce, double *__restrict__ cinv, unsigned char *__restrict__ img) {
+    const int off = blockIdx.x, grp = blockIdx.y;
+    const int dx = off % 7 - 3, dy = (off / 7) % 7 - 3, dz = off / 49 - 3;
+    const bool used = max(abs(dx), max(abs(dy), abs(dz))) >= 2;
+    const size_t tile = (size_t)kSl * ng * 32;
+    unsigned char *dst = img + ((size_t)off * ngrp + grp) * nck * tile;
+    for (int e = threadIdx.x; e < nck * ng * 16; e += blockDim.x) {
+        const int kk = e % 16, n = e / 16 % ng, ck = e / (16 * ng), k = 16 * ck + kk, col = grp * ng + n;
+        long long v = 0;
+        if (used && k < K && col < K)
+            v = llrint(ldexp(tab[(size_t)off * K * K + (size_t)k * K + col], 55 - se[k] - ce[col]));
+        uint16_t d[kSl];
+        bf16_digits(v, d);
+#pragma unroll
+        for (int i = 0; i < kSl; ++i)
+            *reinterpret_cast<uint16_t *>(dst + ck * tile + (size_t)i * ng * 32 + swz32(n, kk >> 3) + (kk & 7) * 2) = d[i];
+    }
+    if (off == 0)
+        for (int n = threadIdx.x; n < ng; n += blockDim.x)
+            cinv[grp * ng + n] = grp * ng + n < K ? ldexp(1.0, ce[grp * ng + n]) : 0.0;
+}
+
+// The inputs' rows as digits, and the rows' scales: one warp per row; the last
+// row of blocks finds the tiles' active offsets.
+struct OzSplitArgs {
+    const double *in[kMaxLevels + 1];
+    unsigned char *out[kMaxLevels + 1];
+    double *rscale[kMaxLevels + 1];
+    int64_t rows[kMaxLevels + 1];
+    const int *se;
+    int lmin, ldk, K, nck;
+};
+
+__global__ void __launch_bounds__(256)
+oz_split(const __grid_constant__ OzSplitArgs o, const __grid_constant__ TcArgs tc, uint32_t *tmask) {
+    if (blockIdx.y == gridDim.y - 1) {
+        for (int t = (int)blockIdx.x; t < tc.ntiles; t += (int)gridDim.x) tile_mask(tc, t, tmask);
+        return;
+    }
+    const int l = o.lmin + (int)blockIdx.y, lane = threadIdx.x & 31;
+    constexpr int NV = ((kMaxP + 1) * (kMaxP + 1) + 31) / 32;
+    int sk[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) sk[q] = lane + 32 * q < o.K ? __ldg(o.se + lane + 32 * q) : 0;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < o.rows[l]; r += (int64_t)gridDim.x * 8) {
+        const double *src = o.in[l] + r * o.ldk;
+        double x[NV];
+        int em = 0;   // largest biased exponent of x 2^se, 0x7ff + ... for infinities and NaN
+        bool bad = false;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int k = lane + 32 * q;
+            x[q] = k < o.K ? __ldg(src + k) : 0.0;
+            const int e = (int)((__double_as_longlong(x[q]) >> 52) & 0x7ff);
+            bad |= e == 0x7ff;
+            if (e > 0) em = max(em, e + sk[q]);
+        }
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, q));
+        bad = __any_sync(0xffffffffu, bad);
+        const int E = em - 1022;   // |x 2^se| < 2^E
+        if (lane == 0) o.rscale[l][r] = bad ? __longlong_as_double(0x7ff8000000000000ll) : em > 0 ? ldexp(1.0, E - 54) : 0.0;
+        unsigned char *dst = o.out[l] + r * (int64_t)o.nck * kOzRowChunk;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int k = lane + 32 * q;
+            if (k >= 16 * o.nck) continue;
+            // one bit more, rounded off
+            const long long v = bad || em <= 0 ? 0 : (to_fix(x[q], 56 - E + sk[q]) + 1) >> 1;
+            uint16_t d[kSl];
+            bf16_digits(v, d);
+#pragma unroll
+            for (int i = 0; i < kSl; ++i)
+                *reinterpret_cast<uint16_t *>(dst + (k >> 4) * kOzRowChunk + i * 32 + (k & 15) * 2) = d[i];
+        }
+    }
+}
+
 }  // namespace
 
 // Bytes of the split FP16 inputs of levels 2..l-1 (the start of level l in
@@ -1123,9 +1708,11 @@ static int64_t tc_stream_ctas(int64_t tiles) {
     return std::max<int64_t>(1, std::min<int64_t>(sm_count(), tiles * 189 / kMinUnits));
 }
 
-size_t m2l_tc_bytes(int p) {
+size_t m2l_tc_bytes(int p, bool fp64) {
     const int npad = ((p + 1) * (p + 1) + 15) & ~15;
-    return npad > 256 ? 0 : (size_t)2 * sm_count() * 128 * npad * sizeof(float) + (size_t)(sm_count() + 1) * sizeof(int4);
+    const size_t cuts = (size_t)(sm_count() + 1) * sizeof(int4) + 65536;
+    if (fp64) return (size_t)2 * sm_count() * 128 * kOzCols * sizeof(double) + cuts;
+    return npad > 256 ? 0 : (size_t)2 * sm_count() * 128 * npad * sizeof(float) + cuts;
 }
 
 // Masks of the tiles and the partial rows of cut tiles, for the plan's largest batch (smaller batches have no more tiles); the
@@ -1526,6 +2113,203 @@ gf_status m2l_run_fold(gf_plan_s *plan, int B, bool adj, cudaStream_t st) {
     }
 }
 
+// ---------------------------------------------------------------- FP64 on the tensor cores
+namespace {
+
+std::mutex g_oz_mu;
+
+// The digit images of an operator set, built with the first plan that uses
+// them and kept as long as the tables they come from.
+gf_status oz_tables(const Tables *T, cudaStream_t st, const OzTables **out) {
+    std::lock_guard<std::mutex> lk(g_oz_mu);
+    OzTables &z = *T->oz;
+    if (!z.img) {
+        const int K = T->K, ngrp = oz_groups(K), ng = oz_group_cols(K), nck = oz_chunks(K);
+        double *cmax = nullptr;
+        int *e = nullptr;
+        unsigned char *img = nullptr;
+        const size_t nimg = (size_t)343 * ngrp * nck * kSl * ng * 32;
+        cudaError_t err = cudaMalloc(&cmax, ((size_t)K * K + (size_t)ngrp * ng) * sizeof(double));
+        if (err == cudaSuccess) err = cudaMalloc(&e, 2 * (size_t)K * sizeof(int));
+        if (err == cudaSuccess) err = cudaMalloc(&img, nimg);
+        if (err == cudaSuccess) {
+            double *cinv = cmax + (size_t)K * K;
+            oz_absmax<<<ceil_div(K * K, 256), 256, 0, st>>>(T->m2l_d, K * K, cmax);
+            oz_exponents<<<1, 1024, 0, st>>>(cmax, K, e, e + K);
+            oz_images<<<dim3(343, ngrp), 256, 0, st>>>(T->m2l_d, K, ngrp, ng, nck, e, e + K, cinv, img);
+            err = cudaGetLastError();
+            if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+            if (err == cudaSuccess) {
+                z.cinv = cinv;
+                z.se = e;
+                z.img = img;
+            }
+        }
+        if (!z.img) {
+            cudaFree(cmax);
+            cudaFree(e);
+            cudaFree(img);
+            cudaGetLastError();
+            *out = nullptr;   // no room: the SIMT M2L serves the plan
+            return err == cudaErrorMemoryAllocation ? GF_OK : GF_ERR_CUDA;
+        }
+    }
+    *out = &z;
+    return GF_OK;
+}
+
+// Rows of a level's split inputs: the z-slabs its M2L reads.
+int64_t oz_rows(const FmmLevel &lv) {
+    return lv.m2l_z1 >= lv.m2l_z0 ? (lv.m2l_z1 - lv.m2l_z0 + 1) * lv.sn[0] * lv.sn[1] : 0;
+}
+
+}  // namespace
+
+// FP64 plans: the digit M2L's workspaces, when it is the faster one and they
+// fit what the plan's size was announced as (gf_plan_bytes; point plans have no
+// announced size).
+gf_status m2l_oz_prepare(gf_plan_s *plan) {
+    FmmPlan *F = plan->fmm;
+    F->oz = nullptr;
+    if (F->mixed || F->m2l_tc64 || F->L < 2 || F->B > 32 || (plan->opt.reserved0 & GF_FLAG_M2L_SIMT)) return GF_OK;
+    const int K = F->K, ngrp = oz_groups(K), ng = oz_group_cols(K), nck = oz_chunks(K);
+    const int64_t tiles = tc_tiles(F, false, 1, nullptr);
+    if (tiles == 0 || tiles * ngrp > 0x7fffffff) return GF_OK;
+    int64_t cols = 0, rows = 0;
+    for (int l = 2; l <= F->L; ++l) {
+        cols += F->lev[l].nt * F->B;
+        rows += oz_rows(F->lev[l]) * F->B;
+    }
+    // Microseconds, from measurements at p = 4 to 16: a (tile, group, offset) unit
+    // here, some 130 offsets to a tile padded to 128 targets, against a wave of the
+    // SIMT M2L, which takes as many targets to a block as it would.  16^3 to 48^3
+    // grids under a plane of observers (20 to 189 targets) stay there: 48^3 at
+    // p = 12 1,109 us against 1,173 for the whole forward; from 64^3 on (340 targets)
+    // the digits win: 2,256 against 1,271 us, 128^3 12.6 against 6.9 ms at p = 14.
+    const double oz_us = F->B * (tiles * 130.0 * ngrp / sm_count() + 2.0) * (1.2 * nck + 8.0);
+    const int64_t sms = sm_count(), P = cols >= 8 * sms && K <= 256 ? 4 : cols >= sms ? 2 : 1;
+    const double fold_us = 0.8e-4 * K * K * (double)((cols + sms * P - 1) / (sms * P) * (sms * P));
+    if (oz_us > 0.85 * fold_us) return GF_OK;
+    const int64_t ctas = std::min<int64_t>(sm_count(), tiles * ngrp * 189);
+    const bool stream = tiles * ngrp <= kStreamTiles;
+    const size_t row_bytes = (size_t)nck * kOzRowChunk;
+    const size_t need = (size_t)rows * (row_bytes + sizeof(double)) + (size_t)tiles * 8 * sizeof(uint32_t) +
+                        (F->L + 1) * sizeof(TcLevel) +
+                        (stream ? (size_t)ctas * 2 * ng * 128 * sizeof(double) + (size_t)(ctas + 1) * sizeof(int4) : 0) + 4096;
+    const size_t grows = need + 4096 > plan->arena.left ? std::max(need + 4096, plan->arena.next) : 0;
+    if (!F->points && plan->arena.bytes + grows > fmm_bytes_estimate(&plan->grid, plan->quad.nq, plan->M, &plan->opt))
+        return GF_OK;
+    const OzTables *z = nullptr;
+    GF_TRY(oz_tables(F->tab, plan->arena.stream, &z));
+    if (!z) return GF_OK;
+    unsigned char *mem = nullptr;
+    if (plan->arena.alloc((void **)&mem, need) != GF_OK) {   // no room: the SIMT M2L serves the plan
+        cudaGetLastError();
+        return GF_OK;
+    }
+    auto take = [&](size_t n) {
+        unsigned char *p = mem;
+        mem += (n + 255) & ~(size_t)255;
+        return p;
+    };
+    F->oz_split = take((size_t)rows * row_bytes);
+    F->oz_rscale = (double *)take((size_t)rows * sizeof(double));
+    F->m2l_mask[0] = (uint32_t *)take((size_t)tiles * 8 * sizeof(uint32_t));
+    F->oz_part = stream ? (double *)take((size_t)ctas * 2 * ng * 128 * sizeof(double)) : nullptr;
+    F->m2l_cut = stream ? (int4 *)take((size_t)(ctas + 1) * sizeof(int4)) : nullptr;
+    std::vector<TcLevel> h(F->L + 1);
+    memset(h.data(), 0, h.size() * sizeof(TcLevel));
+    int64_t r0 = 0;
+    for (int l = 2; l <= F->L; ++l) {
+        const FmmLevel &lv = F->lev[l];
+        TcLevel &t = h[l];
+        t.le = (float *)lv.le;
+        t.order = lv.m2l_order;
+        t.tkey = lv.tkey;
+        for (int d = 0; d < 3; ++d) {
+            t.blo[d] = lv.slo[d];
+            t.bn[d] = lv.sn[d];
+        }
+        for (int c = 0; c <= 8; ++c) t.cls_off[c] = lv.cls_off[c];
+        t.shift = l - 2;
+        t.split = F->oz_split + r0 * row_bytes;
+        t.rscale = F->oz_rscale + r0;
+        t.src0 = oz_rows(lv) > 0 ? lv.m2l_z0 * lv.sn[0] * lv.sn[1] : 0;
+        F->oz_row0[l] = r0;
+        r0 += oz_rows(lv) * F->B;
+    }
+    F->oz_levels = take(h.size() * sizeof(TcLevel));
+    GF_TRY(upload_small(F->oz_levels, h.data(), h.size() * sizeof(TcLevel), plan->arena.stream));
+    F->oz = z;
+    return GF_OK;
+}
+
+static gf_status m2l_run_oz(gf_plan_s *plan, int B, cudaStream_t st, cudaEvent_t fork) {
+    FmmPlan *F = plan->fmm;
+    const OzTables *z = F->oz;
+    OzArgs o;
+    memset(&o, 0, sizeof(o));
+    TcArgs &a = o.t;
+    a.K = F->K;
+    a.ldk = F->KS;
+    a.B = 1;
+    a.status = plan->d_status;
+    a.wait_tries = kWaitTries;
+    a.lv = reinterpret_cast<const TcLevel *>(F->oz_levels);
+    a.lmin = 2;
+    a.part_lo = plan->part_lo;
+    a.part_hi = plan->part_hi;
+    a.nent = 8 * (F->L - 1);
+    a.ntiles = (int)tc_tiles(F, false, 1, a.tile_begin);
+    a.tmask = F->m2l_mask[0];
+    a.mcut = F->m2l_cut;
+    a.min_units = 1;
+    o.nb = B;
+    o.ngrp = oz_groups(F->K);
+    o.ng = oz_group_cols(F->K);
+    o.nck = oz_chunks(F->K);
+    o.img = z->img;
+    o.cinv = z->cinv;
+    o.part = F->oz_part;
+    a.nst = oz_stages(o.ng);
+    const int64_t ntg = (int64_t)a.ntiles * o.ngrp;
+    a.stream = ntg <= kStreamTiles && o.part;
+    OzSplitArgs p;
+    memset(&p, 0, sizeof(p));
+    p.se = z->se;
+    p.lmin = 2;
+    p.ldk = F->KS;
+    p.K = F->K;
+    p.nck = o.nck;
+    int64_t most = 1;
+    for (int l = 2; l <= F->L; ++l) {
+        const FmmLevel &lv = F->lev[l];
+        p.rows[l] = oz_rows(lv) * B;
+        p.in[l] = (const double *)lv.me + (p.rows[l] > 0 ? lv.m2l_z0 * lv.sn[0] * lv.sn[1] : 0) * B * F->KS;
+        p.out[l] = F->oz_split + F->oz_row0[l] * o.nck * kOzRowChunk;
+        p.rscale[l] = F->oz_rscale + F->oz_row0[l];
+        most = std::max(most, p.rows[l]);
+    }
+    const int gx = (int)std::min<int64_t>(8 * 152, std::max<int64_t>((most + 7) / 8, std::min(a.ntiles, 8 * 152)));
+    oz_split<<<dim3(gx, F->L), 256, 0, st>>>(p, a, F->m2l_mask[0]);
+    GF_KERNEL_DONE();
+    stage_mark(plan, 4, st);
+    if (fork) GF_CUDA(cudaEventRecord(fork, st));
+    if (a.ntiles == 0) return GF_OK;
+    const size_t shm = (size_t)a.nst * oz_stage_bytes(o.ng) + 1024;
+    GF_TRY(ensure_smem(m2l_oz, shm));
+    const int64_t grid = a.stream ? std::min<int64_t>(sm_count(), ntg * 189) : ntg;
+    for (o.bb = 0; o.bb < B; ++o.bb) {
+        m2l_oz<<<(unsigned)grid, kTcThreads, shm, st>>>(o);
+        GF_KERNEL_DONE();
+        if (a.stream && grid > 1) {
+            m2l_oz_join<<<dim3((unsigned)grid - 1, 2), 512, 0, st>>>(o);
+            GF_KERNEL_DONE();
+        }
+    }
+    return GF_OK;
+}
+
 template <class T>
 gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t fork) {
     FmmPlan *F = plan->fmm;
@@ -1533,6 +2317,7 @@ gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t
                     !(plan->opt.reserved0 & GF_FLAG_M2L_SIMT) && B <= 128 &&
                     tc_stages(F->tab->tc_npad) >= 2;
     if (tc) return m2l_run_tc(plan, B, adj, st, fork);
+    if (sizeof(T) == 8 && !adj && F->oz) return m2l_run_oz(plan, B, st, fork);
     if (!adj) stage_mark(plan, 4, st);   // no input split on this path
     if (fork) GF_CUDA(cudaEventRecord(fork, st));
     return m2l_run_fold<T>(plan, B, adj, st);

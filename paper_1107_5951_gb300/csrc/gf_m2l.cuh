@@ -42,10 +42,13 @@ template <class T>
 gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaStream_t st);
 
 // Upper bound of the tensor-core M2L's own workspaces (beside the expansions
-// and their split parts).
-size_t m2l_tc_bytes(int p);
+// and their split parts; fp64: of the digit M2L).
+size_t m2l_tc_bytes(int p, bool fp64);
 // Plan-time set-up of the tensor-core path (level descriptors on the device).
 gf_status m2l_tc_prepare(gf_plan_s *plan);
+// FP64 plans: workspaces of the M2L on the tensor cores by BF16 digits, where
+// that is the faster one.
+gf_status m2l_oz_prepare(gf_plan_s *plan);
 // The adjoint's level tables (built on the plan's first adjoint call).
 gf_status m2l_tc_prepare_adj(gf_plan_s *plan);
 

@@ -403,7 +403,7 @@ size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_optio
     bytes += nleaf * b * b * b * rs * opt->max_batch;          // blocked densities
     if (opt->precision == GF_PREC_MIXED)                         // M2L inputs split into FP16 parts
         bytes += nsrc * ((K + 31) / 32 * 32) * 4.0 * opt->max_batch;
-    if (opt->precision == GF_PREC_MIXED || (opt->reserved0 & GF_FLAG_M2L_TENSOR)) bytes += (double)m2l_tc_bytes(opt->p);
+    bytes += (double)m2l_tc_bytes(opt->p, opt->precision != GF_PREC_MIXED && !(opt->reserved0 & GF_FLAG_M2L_TENSOR));
     bytes += (double)M * (8 + 4 + 4 + 12 + 24) + ntgt * 24;       // keys, perm, locals, box tables
     bytes += (double)M * 32 + 8e6;                                // sort buffers and scratch
     return (size_t)bytes;
