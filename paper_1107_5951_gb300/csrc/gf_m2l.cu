@@ -1159,13 +1159,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// Digits of v, |v| <= 2^55, as BF16: v = sum_i d_i 256^(6 - i).
+// Digits of v, |v| <= 2^55, as BF16: v = sum_i d_i 256^(6 - i), those of -v the
+// negatives of v's.
 __device__ __forceinline__ void bf16_digits(long long v, uint16_t d[kSl]) {
+    const uint16_t sign = v < 0 ? 0x8000u : 0u;
+    v = v < 0 ? -v : v;
 #pragma unroll
     for (int i = kSl - 1; i >= 0; --i) {
         const int q = i > 0 ? (int)(signed char)(v & 255) : (int)v;
         v = (v - q) >> 8;
-        d[i] = (uint16_t)(__float_as_uint((float)q) >> 16);   // |q| <= 128: 8 bits
+        d[i] = (uint16_t)(__float_as_uint((float)q) >> 16) ^ (q ? sign : 0u);   // |q| <= 128: 8 bits
     }
 }
 
@@ -1490,7 +1493,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ 
                             // in units of 256^-5 of the first digits' products; |d_0| <= 304 2^14 and so on:
                             // below 2^62
                             long long x = (long long)(v[0] * 256 + v[1]) * 65536 + (long long)v[2] * 256 + v[3];
-                            x = x * 65536 + (long long)v[4] * 256 + v[5] + ((v[6] + 128) >> 8);
+                            x = x * 65536 + (long long)v[4] * 256 + v[5] + v[6] / 256;
                             acc[c0 + c] = fma(i64_to_f64(x), sc, acc[c0 + c]);
                         }
                     }
@@ -1665,7 +1668,8 @@ oz_split(const __grid_constant__ OzSplitArgs o, const __grid_constant__ TcArgs t
             const int k = lane + 32 * q;
             if (k >= 16 * o.nck) continue;
             // one bit more, rounded off
-            const long long v = bad || em <= 0 ? 0 : (to_fix(x[q], 56 - E + sk[q]) + 1) >> 1;
+            long long v = bad || em <= 0 ? 0 : to_fix(x[q], 56 - E + sk[q]);
+            v = (v + (v >= 0 ? 1 : -1)) / 2;
             uint16_t d[kSl];
             bf16_digits(v, d);
 #pragma unroll
