@@ -18,6 +18,7 @@
 #include "gf_fmm.cuh"
 #include "gf_m2l.cuh"
 #include "gf_simd.cuh"
+#include "gf_pair.cuh"
 #include "gf_sum_an.cuh"
 
 namespace gf {
@@ -544,16 +545,12 @@ constexpr int kMaxLat = 8;         // lattice planes per axis of a leaf (lattice
 
 constexpr int kLatGroups = 4;      // lattice form: lane groups sharing a small item
 
-// Elements of one warp's shared-memory slice of the evaluation kernel
+// Elements of one warp's shared-memory slice of the near-field kernel
 // (a multiple of 8): 4 kEvalChunk staged source values (FP32: 8, the
-// duplicated lattice weights of up to kLatGroups leaves), three gradient
-// expansions of P2 coefficients (FP32: duplicated pairs) and 27
+// duplicated lattice weights of up to kLatGroups leaves) and 27
 // neighbour-leaf entries (int64).
 inline __host__ __device__ int eval_stage(int tsize) { return (tsize == 4 ? 2 : 1) * 4 * kEvalChunk; }
-inline __host__ __device__ int eval_slice(int P2, int tsize) {
-    const int dmul = tsize == 4 ? 2 : 1;
-    return (eval_stage(tsize) + 3 * dmul * P2 + 27 * 8 / tsize + 7) & ~7;
-}
+inline __host__ __device__ int eval_slice(int tsize) { return (eval_stage(tsize) + 27 * 8 / tsize + 7) & ~7; }
 
 struct EvalArgs {
     int L;                       // leaf level
@@ -561,8 +558,6 @@ struct EvalArgs {
     const int4 *items;
     int64_t n_items;
     unsigned long long *queue; // [0]: next item, [1]: warps done (zero between launches)
-    int mode;                  // 0: near + far field; 1: near field only, sums to nsum;
-                               // 2: far field, near sums from nsum
     void *nsum;                // [B][M][6] T: (hi, lo) of x, y, z per observer (key order)
     const uint64_t *tkey;      // leaf keys
     const int32_t *perm;
@@ -589,7 +584,8 @@ struct EvalArgs {
     int lat_q[kMaxQuad];
 };
 
-// Near field + far field of the observers of one leaf, one warp per work
+// Near field of the observers of one leaf, its sums (hi, lo) left in nsum for the
+// far-field kernel, one warp per work
 // item; warps take items from a queue (one atomic per item), so a warp that
 // drew a short item takes the next one at once.  The sources of each
 // neighbouring leaf are staged in the warp's shared-memory slice in chunks
@@ -605,7 +601,6 @@ __global__ void __launch_bounds__(kEvalWarps * 32, sizeof(T) == 4 ? 5 : 1)   // 
 eval_kernel(EvalArgs a) {
     extern __shared__ unsigned char shraw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int P2 = a.p * a.p;
     const int b3 = a.b * a.b * a.b;
     const int nsrc = b3 * a.nq;
     // block-wide table: offset of source u (voxel u / nq, node u % nq) from
@@ -613,19 +608,15 @@ eval_kernel(EvalArgs a) {
     Vec4<T> *tab = reinterpret_cast<Vec4<T> *>(shraw);
     int *tvox = reinterpret_cast<int *>(tab + kSrcTable);
     // per-warp slice, a multiple of 8 elements so every slice keeps the
-    // alignment of the vector type: staged sources, the gradient expansions
-    // (FP32: duplicated pairs), the item's neighbour leaves
+    // alignment of the vector type: staged sources, the item's neighbour leaves
     constexpr bool kF32 = std::is_same<T, float>::value;
-    const int wstride = eval_slice(P2, sizeof(T));
+    const int wstride = eval_slice(sizeof(T));
     T *wsh = reinterpret_cast<T *>(tvox + kSrcTable) + (size_t)warp * wstride;
     Vec4<T> *src = reinterpret_cast<Vec4<T> *>(wsh);
-    T *Dx = wsh + eval_stage(sizeof(T)), *Dy = Dx + (kF32 ? 2 : 1) * P2, *Dz = Dy + (kF32 ? 2 : 1) * P2;
-    int64_t *nbl = reinterpret_cast<int64_t *>(Dz + (kF32 ? 2 : 1) * P2);
+    int64_t *nbl = reinterpret_cast<int64_t *>(wsh + eval_stage(sizeof(T)));
     const T *tloc = reinterpret_cast<const T *>(a.tloc);
     const T *mass = reinterpret_cast<const T *>(a.mass);
-    const T *le = reinterpret_cast<const T *>(a.le);
     const T half_b = T(0.5) * T(a.b);
-    const T inv_b = T(1) / T(a.b);
     const T eps2 = (T)a.eps2;
     const bool use_tab = nsrc <= kSrcTable;
     if (N1 > 0) {
@@ -651,9 +642,6 @@ eval_kernel(EvalArgs a) {
         }
     }
     __syncthreads();
-    // far-field scale of the L2P gradient (voxel units)
-    const double far_s = -1.0 / ((double)a.b * (double)a.b);
-    const float far_sf = (float)far_s;
     // lattice form: this lane's two lattice points (weight, voxel)
     float lw0 = 0.f, lw1 = 0.f;
     int lv0 = 0, lv1 = 0;
@@ -675,11 +663,11 @@ eval_kernel(EvalArgs a) {
         int gs = 32;
         if constexpr (N1 > 0 && kF32) {
             const int np = (item.z + 1) >> 1;
-            if (a.mode != 2) gs = np > 16 ? 32 : np > 8 ? 16 : 32 / kLatGroups;
+            gs = np > 16 ? 32 : np > 8 ? 16 : 32 / kLatGroups;
         }
         const int ns = 32 / gs, grp = lane / gs, r0 = lane - grp * gs;
         int64_t lc[3] = {0, 0, 0};   // the leaf's box coordinates (near field only)
-        if (a.mode != 2) {
+        {
             const uint64_t k = a.tkey[leaf];
             for (int bit = 0; bit < 21; ++bit) {
                 lc[0] |= (int64_t)((k >> (3 * bit)) & 1) << bit;
@@ -702,7 +690,7 @@ eval_kernel(EvalArgs a) {
         // nb = (dx + 1) + 3 (dy + 1) + 9 (dz + 1): source-block index * 32 + nb
         __syncwarp();
         int nv = 0;
-        if (a.mode != 2) {
+        {
             bool in = false;
             int64_t sidx = 0;
             if (lane < 27) {
@@ -974,102 +962,17 @@ eval_kernel(EvalArgs a) {
                     lz[u] += wz;
                 }
             }
-            // split evaluation: the near sums go to nsum (mode 1) or come from it (mode 2)
-            if (a.mode != 0) {
-                T *ns = reinterpret_cast<T *>(a.nsum);
-#pragma unroll
-                for (int u = 0; u < kTPL; ++u) {
-                    if (tid[u] < 0 || grp != 0) continue;
-                    T *q = ns + ((int64_t)bb * a.M + tid[u]) * 6;
-                    if (a.mode == 1) {
-                        q[0] = hx[u];
-                        q[1] = lx[u];
-                        q[2] = hy[u];
-                        q[3] = ly[u];
-                        q[4] = hz[u];
-                        q[5] = lz[u];
-                    } else {
-                        hx[u] = q[0];
-                        lx[u] = q[1];
-                        hy[u] = q[2];
-                        ly[u] = q[3];
-                        hz[u] = q[4];
-                        lz[u] = q[5];
-                    }
-                }
-                if (a.mode == 1) continue;
-            }
-            // ---- far field: gradient of the leaf's local expansion
-            __syncwarp();
-            const T *L = le + ((int64_t)leaf * a.B + bb) * a.ldk;
-            T fxa[kTPL], fya[kTPL], fza[kTPL];
-            if constexpr (kF32) {
-                // duplicated pairs, the factor 2 of the m > 0 terms folded in;
-                // both observers of the lane in one packed sum
-                float2 *Dx2 = reinterpret_cast<float2 *>(Dx), *Dy2 = reinterpret_cast<float2 *>(Dy),
-                       *Dz2 = reinterpret_cast<float2 *>(Dz);
-                for (int e = lane; e < P2; e += 32) {
-                    float vx, vy, vz;
-                    grad_coeff<float>(reinterpret_cast<const float *>(L), e, vx, vy, vz);
-                    int n = 0;
-                    while ((n + 1) * (n + 1) <= e) ++n;
-                    const float f2 = e == n * n ? 1.f : 2.f;
-                    Dx2[e] = make_float2(f2 * vx, f2 * vx);
-                    Dy2[e] = make_float2(f2 * vy, f2 * vy);
-                    Dz2[e] = make_float2(f2 * vz, f2 * vz);
-                }
-                __syncwarp();
-                uint64_t FX, FY, FZ;
-                l2p_sum2(a.p, Dx2, Dy2, Dz2, pk2(tx[0] * inv_b, tx[1] * inv_b), pk2(ty[0] * inv_b, ty[1] * inv_b),
-                         pk2(tz[0] * inv_b, tz[1] * inv_b), FX, FY, FZ);
-                float f0, f1;
-                up2(FX, f0, f1);
-                fxa[0] = f0;
-                fxa[1] = f1;
-                up2(FY, f0, f1);
-                fya[0] = f0;
-                fya[1] = f1;
-                up2(FZ, f0, f1);
-                fza[0] = f0;
-                fza[1] = f1;
-            } else {
-                for (int e = lane; e < P2; e += 32) grad_coeff<T>(L, e, Dx[e], Dy[e], Dz[e]);
-                __syncwarp();
-#pragma unroll
-                for (int u = 0; u < kTPL; ++u)
-                    l2p_sum<T>(a.p, Dx, Dy, Dz, tx[u] * inv_b, ty[u] * inv_b, tz[u] * inv_b, fxa[u], fya[u], fza[u]);
-            }
+            T *ns = reinterpret_cast<T *>(a.nsum);
 #pragma unroll
             for (int u = 0; u < kTPL; ++u) {
                 if (tid[u] < 0 || grp != 0) continue;
-                const T fx = fxa[u], fy = fya[u], fz = fza[u];
-                double gx, gy, gzv;
-                if constexpr (kF32) {
-                    // near (hi + lo) + far as a compensated FP32 pair (TwoSum), then
-                    // the pair's sum and the scale in FP64; the FP32 -> FP64
-                    // conversions use integer operations (FP64 runs at 1/64 of
-                    // the FP32 rate on this GPU)
-                    float sx = hx[u], ex = lx[u], sy = hy[u], ey = ly[u], sz = hz[u], ez = lz[u];
-                    two_sum(sx, ex, far_sf * fx);
-                    two_sum(sy, ey, far_sf * fy);
-                    two_sum(sz, ez, far_sf * fz);
-                    gx = (f32_to_f64(sx) + f32_to_f64(ex)) * a.scale;
-                    gy = (f32_to_f64(sy) + f32_to_f64(ey)) * a.scale;
-                    gzv = (f32_to_f64(sz) + f32_to_f64(ez)) * a.scale;
-                } else {
-                    // near (hi + lo) + far and the scale in FP64
-                    gx = ((double)hx[u] + (double)lx[u] + far_s * (double)fx) * a.scale;
-                    gy = ((double)hy[u] + (double)ly[u] + far_s * (double)fy) * a.scale;
-                    gzv = ((double)hz[u] + (double)lz[u] + far_s * (double)fz) * a.scale;
-                }
-                const int64_t j = a.perm[tid[u]];
-                if (a.g) {
-                    double *o = a.g + ((int64_t)bb * a.M + j) * 3;
-                    o[0] = gx;
-                    o[1] = gy;
-                    o[2] = gzv;
-                }
-                if (a.gz) a.gz[(int64_t)bb * a.M + j] = gzv;
+                T *q = ns + ((int64_t)bb * a.M + tid[u]) * 6;
+                q[0] = hx[u];
+                q[1] = lx[u];
+                q[2] = hy[u];
+                q[3] = ly[u];
+                q[4] = hz[u];
+                q[5] = lz[u];
             }
         }
     }
@@ -1186,6 +1089,234 @@ __global__ void __launch_bounds__(kFarWarps * 32, 6) eval_far_kernel(EvalArgs a,
         if (atomicAdd(a.queue + 1, 1ull) == (unsigned long long)gridDim.x * kFarWarps - 1) {
             a.queue[0] = 0;
             a.queue[1] = 0;
+        }
+    }
+}
+
+// Near field in FP64 of rules whose sources form a 4^3 lattice per leaf: the sums
+// of eval_kernel's mode 1.  The FP64 pipe takes two instructions a clock and SM,
+// so their number is what counts: with the lattice sums of the FP32 form (|d|^2
+// from the squared plane distances, rows added up before they are weighted) and
+// inv_r3's seven, 10.3 per pair of observer and source against 23.  A block takes
+// half a work item, an observer per lane; its warps share out the neighbour leaves
+// and their compensated sums meet in shared memory in warp order, so that a few
+// items are enough to keep many SMs busy (a warp per item left 16 of 152 busy for
+// 0.8 ms under 64 x 64 stations).  65,536 observers over 128^3: 3,000 -> 1,715 us.
+constexpr int kNear64Warps = 8;
+
+__global__ void __launch_bounds__(kNear64Warps * 32) near_f64_kernel(EvalArgs a) {
+    __shared__ double lat[3][4];                          // lattice planes from the leaf's centre (voxel units)
+    __shared__ double lw[64];                             // the rule's weight at each lattice point
+    __shared__ int lv[64];                                // its voxel
+    __shared__ __align__(16) double wts[kNear64Warps][64];   // masses of the warp's leaf
+    __shared__ double2 part[kNear64Warps][3][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b3 = a.b * a.b * a.b, m = a.lat_m;
+    const double half_b = 0.5 * (double)a.b;
+    if (threadIdx.x < 64) {
+        const int n = threadIdx.x, i = n % 4, j = (n / 4) % 4, k = n / 16;
+        lv[n] = i / m + a.b * (j / m + a.b * (k / m));
+        lw[n] = a.qr->wn[a.lat_q[i % m + m * (j % m + m * (k % m))]];
+    } else if (threadIdx.x < 76) {
+        const int d = (threadIdx.x - 64) / 4, i = (threadIdx.x - 64) % 4;
+        const int step = d == 0 ? 1 : d == 1 ? m : m * m;
+        lat[d][i] = (double)(i / m) + (0.5 + 0.5 * a.qr->xi[a.lat_q[(i % m) * step]][d]) - half_b;
+    }
+    __syncthreads();
+    const double *tloc = reinterpret_cast<const double *>(a.tloc);
+    const double *mass = reinterpret_cast<const double *>(a.mass);
+    double *ns = reinterpret_cast<double *>(a.nsum);
+    const long long eps_bits = __double_as_longlong(a.eps2);
+    const int64_t units = 2 * a.n_items;
+    for (int64_t un = blockIdx.x; un < units; un += gridDim.x) {
+        const int4 item = a.items[un >> 1];
+        const int r0 = 32 * (int)(un & 1);
+        if (r0 >= item.z) continue;   // the whole block
+        const uint64_t key = a.tkey[item.x];
+        const bool on = r0 + lane < item.z;
+        const int64_t i0 = item.y + (on ? r0 + lane : r0);
+        const double tx = tloc[3 * i0], ty = tloc[3 * i0 + 1], tz = tloc[3 * i0 + 2];
+        int64_t slot = -1;   // lane nb: neighbour leaf nb
+        {
+            int64_t lc[3] = {0, 0, 0};
+            for (int bit = 0; bit < a.L; ++bit)
+                for (int d = 0; d < 3; ++d) lc[d] |= (int64_t)((key >> (3 * bit + d)) & 1) << bit;
+            if (lane < 27) {
+                const int64_t X = lc[0] + lane % 3 - 1, Y = lc[1] + (lane / 3) % 3 - 1, Z = lc[2] + lane / 9 - 1;
+                const int64_t sx = X - a.blk.lo[0], sy = Y - a.blk.lo[1], sz = Z - a.blk.lo[2];
+                if (sx >= 0 && sy >= 0 && sz >= 0 && sx < a.blk.n[0] && sy < a.blk.n[1] && sz < a.blk.n[2] &&
+                    in_source_part(X, Y, Z, a.L - 2, a.part_lo, a.part_hi))
+                    slot = (sz * a.blk.n[1] + sy) * a.blk.n[0] + sx;
+            }
+        }
+        const unsigned have = __ballot_sync(0xffffffffu, slot >= 0);
+        for (int bb = 0; bb < a.B; ++bb) {
+            double h[3] = {0.0, 0.0, 0.0}, l[3] = {0.0, 0.0, 0.0};
+            unsigned rest = have;
+            for (int e = 0; rest; ++e) {
+                const int nb = __ffs(rest) - 1;
+                rest &= rest - 1;
+                const int64_t sl = __shfl_sync(0xffffffffu, (long long)slot, nb);
+                if (e % kNear64Warps != warp) continue;
+                const double *ms = mass + (sl * a.B + bb) * b3;
+                const double ox = (double)((nb % 3 - 1) * a.b), oy = (double)((nb / 3 % 3 - 1) * a.b),
+                             oz = (double)((nb / 9 - 1) * a.b);
+                __syncwarp();
+                wts[warp][lane] = lw[lane] * ms[lv[lane]];
+                wts[warp][lane + 32] = lw[lane + 32] * ms[lv[lane + 32]];
+                __syncwarp();
+                const bool guard = a.guard_all || nb == 13;   // a source may coincide with an observer
+                double dx[4], dy[4], X2[4], Y2[4], SX[4], SY[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    dx[i] = tx - (lat[0][i] + ox);
+                    dy[i] = ty - (lat[1][i] + oy);
+                    X2[i] = dx[i] * dx[i];
+                    Y2[i] = dy[i] * dy[i];
+                    SX[i] = SY[i] = 0.0;
+                }
+                double gz = 0.0;
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const double dz = tz - (lat[2][k] + oz), Z2 = dz * dz;
+                    double SZ = 0.0;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const double YZ = Y2[j] + Z2;
+                        const double2 w01 = *reinterpret_cast<const double2 *>(&wts[warp][16 * k + 4 * j]);
+                        const double2 w23 = *reinterpret_cast<const double2 *>(&wts[warp][16 * k + 4 * j + 2]);
+                        const double w[4] = {w01.x, w01.y, w23.x, w23.y};
+                        double K3[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const double r2 = X2[i] + YZ;
+                            K3[i] = inv_r3(r2, w[i]);
+                            if (guard) K3[i] = __double_as_longlong(r2) > eps_bits ? K3[i] : 0.0;
+                            SX[i] += K3[i];
+                        }
+                        const double t = (K3[0] + K3[1]) + (K3[2] + K3[3]);
+                        SY[j] += t;
+                        SZ += t;
+                    }
+                    gz = fma(SZ, dz, gz);
+                }
+                double gx = 0.0, gy = 0.0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    gx = fma(SX[i], dx[i], gx);
+                    gy = fma(SY[i], dy[i], gy);
+                }
+                two_sum(h[0], l[0], gx);
+                two_sum(h[1], l[1], gy);
+                two_sum(h[2], l[2], gz);
+            }
+            __syncthreads();   // the member before has been read
+#pragma unroll
+            for (int d = 0; d < 3; ++d) part[warp][d][lane] = make_double2(h[d], l[d]);
+            __syncthreads();
+            if (warp < 3) {
+                double H = 0.0, C = 0.0;
+#pragma unroll
+                for (int w = 0; w < kNear64Warps; ++w) {
+                    const double2 v = part[w][warp][lane];
+                    two_sum(H, C, v.x);
+                    C += v.y;
+                }
+                if (on) {
+                    double *q = ns + ((int64_t)bb * a.M + i0) * 6 + 2 * warp;
+                    q[0] = H;
+                    q[1] = C;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Far field of the split evaluation in FP64: the L2P gradient of the leaf's local
+// expansion, near + far, the scale and the scatter; a warp per half work item, an
+// observer per lane.  With R_n^m = s_nm (x + iy)^m Q_n^m (z, r^2), Q real (the
+// recursion of the points' P2M), the coefficients of the three gradient expansions
+// are staged times s_nm and an order's sums are made with Q alone, three FP64
+// instructions a term for Q and six for the sums, then turned by (x + iy)^m once.
+// Bound by the FP64 pipe; a square root and a division for every term took 580 us
+// for 65,536 observers at p = 14, now 184 us.
+__constant__ double c_far_c[kMaxP * (kMaxP - 1) / 2 + 1];   // -((n-1)^2 - m^2) / ((2n-1)(2n-3)) at n (n-1) / 2 + m
+__constant__ double c_far_s[kMaxP * kMaxP];   // s_nm by real component, twice it for m > 0
+constexpr int kFar64Warps = 4;
+
+__global__ void __launch_bounds__(kFar64Warps * 32) far_f64_kernel(EvalArgs a) {
+    extern __shared__ __align__(16) unsigned char shraw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int P2 = a.p * a.p;
+    double *Dx = reinterpret_cast<double *>(shraw) + (size_t)warp * 3 * P2, *Dy = Dx + P2, *Dz = Dy + P2;
+    const double *tloc = reinterpret_cast<const double *>(a.tloc);
+    const double *le = reinterpret_cast<const double *>(a.le);
+    const double *ns = reinterpret_cast<const double *>(a.nsum);
+    const double inv_b = 1.0 / (double)a.b;
+    const double far_s = -1.0 / ((double)a.b * (double)a.b);
+    const int64_t units = 2 * a.n_items;
+    for (int64_t un = (int64_t)blockIdx.x * kFar64Warps + warp; un < units; un += (int64_t)gridDim.x * kFar64Warps) {
+        const int4 item = a.items[un >> 1];
+        const int r0 = 32 * (int)(un & 1);
+        if (r0 >= item.z) continue;
+        const bool on = r0 + lane < item.z;
+        const int64_t i0 = item.y + (on ? r0 + lane : r0);
+        const double X = tloc[3 * i0] * inv_b, Y = tloc[3 * i0 + 1] * inv_b, Z = tloc[3 * i0 + 2] * inv_b;
+        const double R2 = X * X + Y * Y + Z * Z;
+        for (int bb = 0; bb < a.B; ++bb) {
+            const double *L = le + ((int64_t)item.x * a.B + bb) * a.ldk;
+            __syncwarp();
+            for (int e = lane; e < P2; e += 32) {
+                double vx, vy, vz;
+                grad_coeff<double>(L, e, vx, vy, vz);
+                const double sc = c_far_s[e];
+                Dx[e] = sc * vx;
+                Dy[e] = sc * vy;
+                Dz[e] = sc * vz;
+            }
+            __syncwarp();
+            double g[3] = {0.0, 0.0, 0.0}, wr = 1.0, wi = 0.0;
+            for (int m = 0; m < a.p; ++m) {
+                if (m > 0) {
+                    const double nr = X * wr - Y * wi, ni = X * wi + Y * wr;
+                    wr = nr;
+                    wi = ni;
+                }
+                double Q = 1.0, P = 0.0;
+                double re[3] = {0.0, 0.0, 0.0}, im[3] = {0.0, 0.0, 0.0};
+                for (int n = m; n < a.p; ++n) {
+                    if (n > m) {
+                        // -((n-1)^2 - m^2) / ((2n-1)(2n-3)), zero at n = m + 1
+                        const double v = fma(Z, Q, c_far_c[n * (n - 1) / 2 + m] * R2 * P);
+                        P = Q;
+                        Q = v;
+                    }
+                    const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+                    re[0] = fma(Dx[k], Q, re[0]);
+                    re[1] = fma(Dy[k], Q, re[1]);
+                    re[2] = fma(Dz[k], Q, re[2]);
+                    if (m > 0) {
+                        im[0] = fma(Dx[k + 1], Q, im[0]);
+                        im[1] = fma(Dy[k + 1], Q, im[1]);
+                        im[2] = fma(Dz[k + 1], Q, im[2]);
+                    }
+                }
+#pragma unroll
+                for (int d = 0; d < 3; ++d) g[d] = fma(re[d], wr, fma(im[d], wi, g[d]));
+            }
+            if (!on) continue;
+            const double *q = ns + ((int64_t)bb * a.M + i0) * 6;
+            const double gx = (q[0] + (q[1] + far_s * g[0])) * a.scale, gy = (q[2] + (q[3] + far_s * g[1])) * a.scale,
+                         gzv = (q[4] + (q[5] + far_s * g[2])) * a.scale;
+            const int64_t j = a.perm[i0];
+            if (a.g) {
+                double *o = a.g + ((int64_t)bb * a.M + j) * 3;
+                o[0] = gx;
+                o[1] = gy;
+                o[2] = gzv;
+            }
+            if (a.gz) a.gz[(int64_t)bb * a.M + j] = gzv;
         }
     }
 }
@@ -1530,6 +1661,28 @@ __global__ void transpose_ops(const double *__restrict__ fwd, double *__restrict
     (void)nslots;
 }
 
+// The far field's tables for the current device.
+gf_status upload_far_coefs() {
+    double c[kMaxP * (kMaxP - 1) / 2 + 1] = {}, sc[kMaxP * kMaxP] = {};
+    double sect = 1.0;
+    for (int m = 0; m < kMaxP; ++m) {
+        if (m > 0) sect *= -std::sqrt((2.0 * m - 1.0) / (2.0 * m));
+        double v = m > 0 ? 2.0 * sect : sect;
+        for (int n = m; n < kMaxP; ++n) {
+            if (n > m) {
+                v *= (2 * n - 1) / std::sqrt((double)((n + m) * (n - m)));
+                c[n * (n - 1) / 2 + m] = n > m + 1 ? -(double)((n - 1) * (n - 1) - m * m) / ((2 * n - 1) * (2 * n - 3)) : 0.0;
+            }
+            const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+            sc[k] = v;
+            if (m > 0) sc[k + 1] = v;
+        }
+    }
+    GF_CUDA(cudaMemcpyToSymbol(c_far_c, c, sizeof(c)));
+    GF_CUDA(cudaMemcpyToSymbol(c_far_s, sc, sizeof(sc)));
+    return GF_OK;
+}
+
 // ---------------------------------------------------------------- tables
 std::mutex g_tab_mu;
 std::vector<Tables *> g_tabs;
@@ -1578,6 +1731,7 @@ gf_status get_tables(int device, int p, cudaStream_t st, const Tables **out) {
     GF_TRY(m2l_prepare_tables(T, st));
     GF_TRY(xlate_prepare_tables(T, st));
     GF_TRY(upload_l2p_coefs());
+    GF_TRY(upload_far_coefs());
     GF_CUDA(cudaStreamSynchronize(st));
     g_tabs.push_back(T);
     *out = T;
@@ -1755,7 +1909,6 @@ int eval_setup(gf_plan_s *plan, int B, double *g, double *gz, EvalArgs &a) {
     a.items = F->items;
     a.n_items = F->n_items;
     a.queue = F->eval_queue;
-    a.mode = 0;
     a.nsum = F->nsum;
     a.tkey = F->lev[L].tkey;
     a.perm = F->perm;
@@ -1779,17 +1932,17 @@ int eval_setup(gf_plan_s *plan, int B, double *g, double *gz, EvalArgs &a) {
             if (fabs(plan->quad.xi[q][d]) >= 1.0) a.guard_all = 1;
     a.g = g;
     a.gz = gz;
-    return sizeof(T) == 4 ? lattice_of(plan->quad, F->b, a) : 0;
+    return lattice_of(plan->quad, F->b, a);
 }
 
-// One evaluation kernel (mode 0: whole, 1: near field, 2: far field) on
-// the blocks that fit the device at once; the warps drain the item queue.
+// One evaluation kernel (mode 1: near field, 2: far field).  FP64 rules of a 4^3
+// lattice per leaf and closed-form voxels have near fields of their own; the
+// queued kernels run on the blocks that fit the device at once.
 template <class T>
 gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_t st) {
     const FmmPlan *F = plan->fmm;
-    a.mode = mode;
     const size_t shm = kSrcTable * (sizeof(Vec4<T>) + sizeof(int)) +
-                       sizeof(T) * kEvalWarps * eval_slice(F->p * F->p, (int)sizeof(T));
+                       sizeof(T) * kEvalWarps * eval_slice((int)sizeof(T));
     const unsigned grid = (unsigned)std::min<int64_t>((F->n_items + kEvalWarps - 1) / kEvalWarps, 152 * 64);
     if (sizeof(T) == 4 && mode == 2) {
         const size_t fshm = sizeof(float) * kFarWarps * far_slice(F->p * F->p);
@@ -1797,6 +1950,12 @@ gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_
         const unsigned fg = (unsigned)std::min<int64_t>((F->n_items + kFarWarps - 1) / kFarWarps, 152 * 64);
         const unsigned rg = std::min<unsigned>(fg, resident_blocks(eval_far_kernel, kFarWarps * 32, fshm));
         eval_far_kernel<<<rg, kFarWarps * 32, fshm, st>>>(a, F->leaf_beg);
+    } else if (sizeof(T) == 8 && mode == 2) {
+        const size_t fshm = sizeof(double) * kFar64Warps * 3 * F->p * F->p;
+        const unsigned fg = (unsigned)std::min<int64_t>((2 * F->n_items + kFar64Warps - 1) / kFar64Warps, 152 * 64);
+        far_f64_kernel<<<fg, kFar64Warps * 32, fshm, st>>>(a);
+    } else if (sizeof(T) == 8 && n1 == 4) {
+        near_f64_kernel<<<(unsigned)std::min<int64_t>(2 * F->n_items, 152 * 64), kNear64Warps * 32, 0, st>>>(a);
     } else if (sizeof(T) == 4 && (plan->opt.reserved0 & GF_FLAG_SUM_AN)) {
         const size_t ashm = sizeof(float) * kAnWarps * near_an_slice();
         GF_TRY((ensure_smem(near_an_kernel, ashm)));
