@@ -533,8 +533,14 @@ struct TcTile {
 
 // (level, class, tile within the class) of tile t
 __device__ __forceinline__ TcTile tile_of(const TcArgs &a, int t) {
-    int e = 0;
-    while (e + 1 < a.nent && a.tile_begin[e + 1] <= t) ++e;
+    int e = 0, hi = a.nent;   // tile_begin[e] <= t < tile_begin[hi]
+    while (hi - e > 1) {
+        const int mid = (e + hi) >> 1;
+        if (a.tile_begin[mid] <= t)
+            e = mid;
+        else
+            hi = mid;
+    }
     TcTile c;
     c.L = &a.lv[a.lmin + e / 8];
     c.cls = e % 8;
