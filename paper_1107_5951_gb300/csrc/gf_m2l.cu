@@ -328,28 +328,26 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
 // 2^sh (largest |input| into (2^14, 2^15]), each output column of the operator
 // images by its own factor; the write-back divides both out exactly.  The
 // inputs are split once per level by a small kernel before the M2L.  Inputs
-// come in chunks of 32, one to a stage, through a ring of shared-memory stages
-// (64-byte swizzle), filled by warp-specialised producers:
-//   warps 0-3   A producers: 16-byte asynchronous copies straight into the
+// come in chunks of 32, one to a stage.  Two pipelines take the units of the CTA in
+// turn, each with a ring of shared-memory stages (64-byte swizzle), a tensor-memory
+// bank and warps of its own:
+//   warps 0-1, 2-3  A producers: 16-byte asynchronous copies straight into the
 //               stage (eight lanes per row's 128 contiguous bytes); each
 //               thread's arrival on the stage's barrier is made by its copies
 //               as they land, so the producers run as far ahead as there are
 //               free stages;
-//   warp 4      one thread issues the MMAs, of two stages at a time, and commits
-//               them to the stages' "empty" barriers (and, after an offset's
-//               last chunk, to the bank's "full" barrier).  A look at a barrier
-//               costs this warp over 200 cycles even when it is complete, and
-//               two stages' MMAs take 200 to 1500: the lanes look at all the
-//               barriers that a step needs at once;
-//   warp 5      one thread bulk-copies the pre-split, pre-swizzled operator
+//   warps 4, 14 one thread issues the MMAs of a stage and commits them to the
+//               stage's "empty" barrier (and, after an offset's last chunk,
+//               to the bank's "full" barrier);
+//   warps 5, 15 one thread bulk-copies the pre-split, pre-swizzled operator
 //               image of each stage;
-//   warps 6-13  promoters: after each offset they read the finished bank of
-//               tensor memory and add it into FP32 registers (two banks
-//               alternate, so the tensor cores never accumulate more than one
-//               offset: their FP32 accumulation rounds differently from
-//               IEEE and long chains over zero-mean data lose digits).
+//   warps 6-13  promoters, of both: after each offset they read the finished bank
+//               of tensor memory and add it into FP32 registers (the tensor
+//               cores never accumulate more than one offset: their FP32
+//               accumulation rounds differently from IEEE and long chains over
+//               zero-mean data lose digits).
 // Offsets whose source boxes are all missing are skipped by every role: the
-// active offsets of every tile are found beforehand (tile_masks) as bit masks
+// active offsets of every tile are found beforehand (tile_mask) as bit masks
 // and counts.  Work is dealt out in units of one (tile, active offset): with up
 // to kStreamTiles tiles the launch has at most one CTA per SM, and CTA c of G
 // takes the units [c T / G, (c + 1) T / G) of the T in tile order, whatever tiles
@@ -359,14 +357,16 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
 // order by a second launch (m2l_join), spread over the chip: one CTA's last
 // arrival summing them took longer than the tile's units when a tile was shared
 // by twenty CTAs.  With more tiles a CTA takes one whole tile.
-// What bounds it: the MMA issuer.  The tensor cores are about half busy (169
-// components: 33 MMAs of 128 x 176 x 16 an offset, 2,900 of 5,800 cycles); the
-// rest is the issuer's own chain of barrier looks, fences and commits, which the
-// few MMAs it can queue do not cover.  Measured against one CTA, or two, per tile
-// and two chunks to a stage: 16 tiles' worth of a 32^3 grid 260 -> 34 us + 6 us to
-// join; 156 tiles of 464 x 464 x 16 (K = 121) 327 -> 154 + 16; 16 grids of 128^3
-// 846 -> 434; a 2^25-point set 1,050 -> 574; 128^3 with observers throughout
-// 1,236 -> 1,140.
+// What bounds it: serial latencies.  169 components are 33 MMAs of 128 x 176 x 16
+// an offset, 2,900 cycles of the tensor cores; an issuing thread waits out most of
+// each MMA and spends as long again on barriers, fences and commits, and a stage's
+// refill (wake-up, 16 copies a thread, L2) takes longer than another stage's MMAs.
+// One pipeline took 5,800 cycles an offset; two, each hiding the other's, 5,000.
+// Measured against one CTA, or two, per tile and producers that waited for their
+// copies: 16 tiles' worth of a 32^3 grid 260 -> 33 us + 6 us to join; 156 tiles of
+// 464 x 464 x 16 (K = 121) 327 -> 127 + 14; 16 grids of 128^3 846 -> 397; a 2^25-point
+// set 1,050 -> 522; 128^3 with observers throughout 1,236 -> 1,011.  (A gather by TMA
+// of the rows took 20 cycles a row, three times as long in all.)
 // Every wait is bounded and watches an abort
 // flag; a wait that gives up sets status[1], and the CTA then drains its
 // copies and MMAs (bounded) and frees its tensor memory.
@@ -504,21 +504,21 @@ __device__ __forceinline__ void tmem_ld8(uint32_t ta, float *v) {
     for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-constexpr int kTcWarps = 14;
+constexpr int kTcWarps = 16;
 constexpr int kTcThreads = kTcWarps * 32;
-constexpr int kTcMaxStages = 8;
+constexpr int kTcMaxStages = 4;             // of each of the two pipelines
 constexpr uint32_t kTcCols = 512;           // two banks of 256 columns
 constexpr uint32_t kTcA = 2u * 8192u;       // A hi + lo: 128 rows x 64 bytes each
 
 __host__ __device__ constexpr uint32_t tc_stage_bytes(int Npad) { return kTcA + 2u * (uint32_t)Npad * 64u; }
-constexpr int kScanItems = 4;               // tiles per thread of the unit scan
+constexpr int kScanItems = 3;               // tiles per thread of the unit scan
 constexpr int kStreamTiles = kTcThreads * kScanItems;
 constexpr size_t kTcSmemBudget = 227 * 1024 - 2048 - 4 * (kStreamTiles + 1);
 inline int tc_stages(int Npad) {
-    const int n = (int)(kTcSmemBudget / (size_t)tc_stage_bytes(Npad));
+    const int n = (int)(kTcSmemBudget / (size_t)tc_stage_bytes(Npad)) / 2;   // per pipeline
     return n > kTcMaxStages ? kTcMaxStages : n;
 }
-size_t tc_smem_bytes(int Npad) { return (size_t)tc_stages(Npad) * tc_stage_bytes(Npad) + 1024; }
+size_t tc_smem_bytes(int Npad) { return 2 * (size_t)tc_stages(Npad) * tc_stage_bytes(Npad) + 1024; }
 
 // 16-byte asynchronous global -> shared copy; nbytes = 0 fills zeros.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t nbytes) {
@@ -727,10 +727,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 m2l_tc(const __grid_constant__ TcArgs a) {
     extern __shared__ unsigned char dsm[];
     unsigned char *base = dsm + ((1024 - (smem_u32(dsm) & 1023)) & 1023);
-    // afull: the stage's A operand has landed (128 producer arrivals); bfull:
-    // its operator image has landed (the copy's own transaction count, so the
-    // copying thread can always wait for its copies, whatever the producers do)
-    __shared__ __align__(8) uint64_t afull[kTcMaxStages], bfull[kTcMaxStages], empty[kTcMaxStages];
+    // Of each pipeline: afull: the stage's A operand has landed (64 producer
+    // arrivals); bfull: its operator image has landed (the copy's own transaction
+    // count, so the copying thread can always wait for its copies, whatever the
+    // producers do)
+    __shared__ __align__(8) uint64_t afull_[2][kTcMaxStages], bfull_[2][kTcMaxStages], empty_[2][kTcMaxStages];
     __shared__ __align__(8) uint64_t stall_bar;
     __shared__ __align__(8) uint64_t bank_full[2], bank_empty[2];
     __shared__ uint32_t tslot;
@@ -752,11 +753,11 @@ m2l_tc(const __grid_constant__ TcArgs a) {
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int i = 0; i < NST; ++i) {
-            // 128 producer threads; the operator copy's expect-tx arrival
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&afull[i])), "r"(128));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bfull[i])), "r"(1));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty[i])), "r"(1));
+        for (int i = 0; i < 2 * kTcMaxStages; ++i) {
+            // 64 producer threads; the operator copy's expect-tx arrival
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&afull_[0][0] + i)), "r"(64));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bfull_[0][0] + i)), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty_[0][0] + i)), "r"(1));
         }
         for (int i = 0; i < 2; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bank_full[i])), "r"(1));
@@ -825,61 +826,92 @@ m2l_tc(const __grid_constant__ TcArgs a) {
         return a.stream ? (int)(min(u1, pref[t + 1]) - max(u0, pref[t])) : units;
     };
 
+    // This role's pipeline: units pipe, pipe + 2, ... of the CTA's, in stages of its
+    // own ring.
+    const int pipe = warp < 4 ? warp >> 1 : warp >= 14 ? 1 : 0;
+    unsigned char *ring = base + (size_t)pipe * NST * stage_bytes;
+    uint64_t *afull = afull_[pipe], *bfull = bfull_[pipe], *empty = empty_[pipe];
+    // The units in order: tile, and offset within its class's list.
+    struct Walk {
+        int t, left, oi;
+        OffsetIter it;
+    };
+    auto step = [&](Walk &w) {
+        if (w.left == 0) {
+            ++w.t;
+            w.left = seg_n(w.t);
+            w.it.open(a.tmask, w.t, seg_lo(w.t));
+        }
+        --w.left;
+        w.oi = w.it.next();
+    };
+    Walk walk;
+    walk.t = t0 - 1;
+    walk.left = 0;
+
     if (warp < 4) {
-        // ---------------- A producers: FP16 inputs, scaled and split in advance
-        const int row = tid & 127, slot = row / B, bb = row - slot * B;
+        // ---------------- A producers: FP16 inputs, scaled and split in advance;
+        // a warp does rows [64 half, 64 half + 64) of its pipeline's stages
+        const int half = warp & 1;
         const int k = lane & 7;                       // 16-byte piece of a row's chunk: 0-3 high, 4-7 low
         const uint32_t kpart = k < 4 ? 0u : 8192u;
         const int rl0 = lane >> 3;
-        int t = t0 - 1, left = 0, cls = 0;
+        int opened = -1, cls = 0;
         const TcLevel *L = nullptr;
         const unsigned char *split = nullptr;
-        TcTarget q{};
-        OffsetIter it;
-        // split parts of this thread's row at the next unit (null: none)
-        auto next_row = [&]() -> const unsigned char * {
-            if (left == 0) {
-                ++t;
-                left = seg_n(t);
-                it.open(a.tmask, t, seg_lo(t));
-                const TcTile tile = tile_of(a, t);
+        TcTarget q[2];
+        const unsigned char *ahead[2] = {nullptr, nullptr};   // split parts of this lane's two rows at the next unit
+        auto locate = [&]() {
+            if (walk.t != opened) {
+                opened = walk.t;
+                const TcTile tile = tile_of(a, walk.t);
                 L = tile.L;
                 cls = tile.cls;
                 split = L->split;
-                q = target_of(tile, nbox, slot);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) q[e] = target_of(tile, nbox, (64 * half + 32 * e + lane) / B);
             }
-            --left;
-            const int64_t src = source_of(a, L, q, cls, it.next());
-            return src >= 0 ? split + (src * B + bb) * a.ldk * 4 : nullptr;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int64_t src = source_of(a, L, q[e], cls, walk.oi);
+                ahead[e] = src >= 0 ? split + (src * B + (64 * half + 32 * e + lane) % B) * a.ldk * 4 : nullptr;
+            }
         };
         int s = 0, n_done = 0;
         uint32_t ph = 0;
         bool stop = false;
-        const unsigned char *ahead = units > 0 ? next_row() : nullptr;
-        for (int u = 0; u < units && !stop; ++u) {
-            const unsigned char *src = ahead;
-            if (u + 1 < units) ahead = next_row();   // located a unit early, off the pipeline's path
-            // the warp's 32 rows in 8 passes of 4, eight lanes per row: each
-            // lane's piece of its eight rows
-            const unsigned char *rp[8];
+        if (pipe < units) {
+            if (pipe) step(walk);
+            step(walk);
+            locate();
+        }
+        for (int u = pipe; u < units && !stop; u += 2) {
+            // the warp's 64 rows in 16 passes of 4, eight lanes per row: each
+            // lane's piece of its sixteen rows
+            const unsigned char *rp[16];
             uint32_t have = 0;
 #pragma unroll
-            for (int pp = 0; pp < 8; ++pp) {
-                const unsigned char *o =
-                    (const unsigned char *)__shfl_sync(0xffffffffu, (unsigned long long)src, 4 * pp + rl0);
+            for (int pp = 0; pp < 16; ++pp) {
+                const unsigned char *o = (const unsigned char *)__shfl_sync(
+                    0xffffffffu, (unsigned long long)ahead[pp >> 3], 4 * (pp & 7) + rl0);
                 rp[pp] = (o ? o : split) + 16 * k;
                 have |= (uint32_t)(o != nullptr) << pp;
+            }
+            if (u + 2 < units) {   // located a unit early, off the pipeline's path
+                step(walk);
+                step(walk);
+                locate();
             }
             for (int j = 0; j < nck; ++j) {
                 if (n_done >= NST && !mbar_wait_ab(smem_u32(&empty[s]), ph ^ 1, abortp, a.wait_tries)) {
                     stop = true;
                     break;
                 }
-                const uint32_t sub = smem_u32(base) + (uint32_t)s * stage_bytes + kpart;
+                const uint32_t sub = smem_u32(ring) + (uint32_t)s * stage_bytes + kpart;
                 const int ck = chunk_of(nck, j);
 #pragma unroll
-                for (int pp = 0; pp < 8; ++pp)
-                    cp_async16(sub + swz64h((row & ~31) + 4 * pp + rl0, 8 * (k & 3)), rp[pp] + 128 * ck,
+                for (int pp = 0; pp < 16; ++pp)
+                    cp_async16(sub + swz64h(64 * half + 4 * pp + rl0, 8 * (k & 3)), rp[pp] + 128 * ck,
                                (have >> pp) & 1u ? 16u : 0u);
                 // the thread's arrival, made when its copies have landed
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&afull[s])) : "memory");
@@ -891,15 +923,16 @@ m2l_tc(const __grid_constant__ TcArgs a) {
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");   // no copy outlives the loop
-    } else if (warp == 4) {
-        // ---------------- MMA issuer
+    } else if (warp == 4 || warp == 14) {
+        // ---------------- MMA issuers
         const uint32_t idesc = idesc_f16(128, Npad);
-        const uint64_t desc0 = umma_desc64(smem_u32(base));   // addresses: lowest bits, in units of 16 bytes
-        int s = 0, g = 0, last = -1, it = 0;
+        const uint64_t desc0 = umma_desc64(smem_u32(ring));   // addresses: lowest bits, in units of 16 bytes
+        const uint32_t d = tmem + (uint32_t)pipe * 256u;
+        int s = 0, last = -1;
         uint32_t ph = 0;
         // testing aid: a wait that nothing completes runs out, sets the abort
         // flag, and every role stops, drains and reports through status[1]
-        bool stop = a.test_stall && !mbar_wait_ab(smem_u32(&stall_bar), 0, abortp, a.wait_tries);
+        bool stop = pipe == 0 && a.test_stall && !mbar_wait_ab(smem_u32(&stall_bar), 0, abortp, a.wait_tries);
         stop = __any_sync(0xffffffffu, stop);
         // Inputs in descending order: chunk by chunk from the last, each chunk's
         // k-steps of 16 inputs from the last down, and in each k-step the two
@@ -907,20 +940,15 @@ m2l_tc(const __grid_constant__ TcArgs a) {
         // tensor cores truncate, so every add made once the sum has its full size
         // costs up to an ulp of it, all of the same sign; leading with the small
         // high-order terms leaves only the last few adds at full size.
-        for (; g < units && !stop; ++g) {
-            const uint32_t d = tmem + (uint32_t)(g & 1) * 256u;
-            for (int j = 0; j < nck && !stop; j += 2) {
-                const int n = min(2, nck - j);
-                const int s1 = s + 1 == NST ? 0 : s + 1;
-                // lanes 0, 1: the stage's operands; 2, 3: the next stage's; 4: the
-                // bank, read out by the promoters of two units before
+        for (int g = pipe; g < units && !stop; g += 2)
+            for (int j = 0; j < nck; ++j) {
+                // lanes 0, 1: the stage's operands; 2: the bank, read out by the
+                // promoters of two units before
                 uint32_t bar = 0, par = ph;
-                if (lane < 2 * n) {
-                    const int sl = lane & 2 ? s1 : s;
-                    bar = smem_u32(lane & 1 ? &bfull[sl] : &afull[sl]);
-                    if ((lane & 2) && s1 == 0) par ^= 1;
-                } else if (lane == 4 && j == 0 && g >= 2) {
-                    bar = smem_u32(&bank_empty[g & 1]);
+                if (lane < 2) {
+                    bar = smem_u32(lane ? &bfull[s] : &afull[s]);
+                } else if (lane == 2 && j == 0 && g >= 2) {
+                    bar = smem_u32(&bank_empty[pipe]);
                     par = ((g - 2) >> 1) & 1;
                 }
                 bool done = bar == 0;
@@ -941,53 +969,43 @@ m2l_tc(const __grid_constant__ TcArgs a) {
                     // shared memory through the async proxy
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     asm volatile("tcgen05.fence::after_thread_sync;");
-                    for (int e = 0; e < n; ++e) {
-                        const int se = e ? s1 : s;
-                        const uint64_t ah = desc0 + (uint32_t)se * (stage_bytes >> 4), al = ah + (8192 >> 4);
-                        const uint64_t bh = ah + (kTcA >> 4), bl = bh + Npad * 4;
-                        uint32_t acc = j + e > 0 ? 1u : 0u;
-                        if (a.K > 32 * chunk_of(nck, j + e) + 16) {   // else one k-step holds inputs
-                            mma_f16(d, ah + 2, bl + 2, idesc, acc);
-                            mma_f16(d, al + 2, bh + 2, idesc, 1u);
-                            mma_f16(d, ah + 2, bh + 2, idesc, 1u);
-                            acc = 1u;
-                        }
-                        mma_f16(d, ah, bl, idesc, acc);
-                        mma_f16(d, al, bh, idesc, 1u);
-                        mma_f16(d, ah, bh, idesc, 1u);
-                        commit_to(&empty[se]);
+                    const uint64_t ah = desc0 + (uint32_t)s * (stage_bytes >> 4), al = ah + (8192 >> 4);
+                    const uint64_t bh = ah + (kTcA >> 4), bl = bh + Npad * 4;
+                    uint32_t acc = j > 0 ? 1u : 0u;
+                    if (a.K > 32 * chunk_of(nck, j) + 16) {   // else one k-step holds inputs
+                        mma_f16(d, ah + 2, bl + 2, idesc, acc);
+                        mma_f16(d, al + 2, bh + 2, idesc, 1u);
+                        mma_f16(d, ah + 2, bh + 2, idesc, 1u);
+                        acc = 1u;
                     }
-                    if (j + n == nck) commit_to(&bank_full[g & 1]);
+                    mma_f16(d, ah, bl, idesc, acc);
+                    mma_f16(d, al, bh, idesc, 1u);
+                    mma_f16(d, ah, bh, idesc, 1u);
+                    commit_to(&empty[s]);
+                    if (j + 1 == nck) commit_to(&bank_full[pipe]);
                 }
-                it += n;
-                last = it - 1;
-                s += n;
-                if (s >= NST) {
-                    s -= NST;
+                ++last;
+                if (++s == NST) {
+                    s = 0;
                     ph ^= 1;
                 }
             }
-        }
         // drain: the last commit covers every MMA issued
         if (last >= 0) mbar_wait(smem_u32(&empty[last % NST]), (uint32_t)((last / NST) & 1), a.wait_tries);
-    } else if (warp == 5) {
+    } else if (warp == 5 || warp == 15) {
         // ---------------- operator images
         if (lane == 0) {
-            int t = t0 - 1, left = 0, cls = 0;
-            OffsetIter it;
-            int s = 0, n_done = 0;
+            int s = 0, n_done = 0, opened = -1, cls = 0;
             uint32_t ph = 0;
-            int last = -1;
             bool stop = false;
-            for (int u = 0; u < units && !stop; ++u) {
-                if (left == 0) {
-                    ++t;
-                    left = seg_n(t);
-                    it.open(a.tmask, t, seg_lo(t));
-                    cls = tile_of(a, t).cls;
+            for (int u = pipe; u < units && !stop; u += 2) {
+                if (u > 0) step(walk);
+                step(walk);
+                if (walk.t != opened) {
+                    opened = walk.t;
+                    cls = tile_of(a, walk.t).cls;
                 }
-                --left;
-                const int o = c_il[cls][it.next()];
+                const int o = c_il[cls][walk.oi];
                 const int dx = (signed char)o, dy = (signed char)(o >> 8), dz = (signed char)(o >> 16);
                 const unsigned char *img = a.img + (size_t)((dz + 3) * 49 + (dy + 3) * 7 + (dx + 3)) * nck * b_bytes;
                 for (int j = 0; j < nck; ++j) {
@@ -995,7 +1013,7 @@ m2l_tc(const __grid_constant__ TcArgs a) {
                         stop = true;
                         break;
                     }
-                    const uint32_t stage = smem_u32(base) + (uint32_t)s * stage_bytes;
+                    const uint32_t stage = smem_u32(ring) + (uint32_t)s * stage_bytes;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&bfull[s])),
                                  "r"(b_bytes));
                     asm volatile(
@@ -1003,7 +1021,7 @@ m2l_tc(const __grid_constant__ TcArgs a) {
                             stage + kTcA),
                         "l"(img + (size_t)chunk_of(nck, j) * b_bytes), "r"(b_bytes), "r"(smem_u32(&bfull[s]))
                         : "memory");
-                    last = n_done++;
+                    ++n_done;
                     if (++s == NST) {
                         s = 0;
                         ph ^= 1;
@@ -1014,7 +1032,7 @@ m2l_tc(const __grid_constant__ TcArgs a) {
             // the last NST stages may still have copies in flight (earlier ones
             // were consumed by MMAs before their stage was reused), and each
             // stage's copy completes its own barrier
-            for (int j = last - NST + 1 > 0 ? last - NST + 1 : 0; j <= last; ++j)
+            for (int j = max(0, n_done - NST); j < n_done; ++j)
                 mbar_wait(smem_u32(&bfull[j % NST]), (uint32_t)((j / NST) & 1), a.wait_tries);
         }
     }
@@ -1022,7 +1040,7 @@ m2l_tc(const __grid_constant__ TcArgs a) {
     const int pw = warp - 6;
     const int pq = warp & 3, ph_half = pw >> 2;   // TMEM lane quarter, column half
     bool ok = true;
-    if (pw >= 0) {
+    if (pw >= 0 && pw < 8) {
         float acc[NS];
         int g = 0;   // units promoted so far (bank g & 1)
         for (int t = t0; g < units; ++t) {
@@ -1125,12 +1143,14 @@ m2l_tc(const __grid_constant__ TcArgs a) {
 // tensor cores wait for (no second bank fits).  128^3 with 1,360 targets at p = 14:
 // 1,710 us, where the SIMT M2L takes 10.8 ms; the fields differ by 2e-16.
 constexpr int kSl = 7;
+constexpr int kOzWarps = 14, kOzThreads = 32 * kOzWarps, kOzScanItems = 4, kOzMaxStages = 8;
+constexpr int kOzStreamTiles = kOzThreads * kOzScanItems;
 constexpr int kOzCols = 64;                              // columns of a group, at most
 constexpr uint32_t kOzA = kSl * 128u * 32u;              // A slices of a stage
 __host__ __device__ constexpr uint32_t oz_stage_bytes(int ng) { return kOzA + (uint32_t)kSl * ng * 32u; }
 inline int oz_stages(int ng) {
-    const int n = (int)(kTcSmemBudget / oz_stage_bytes(ng));
-    return n > kTcMaxStages ? kTcMaxStages : n;
+    const int n = (int)((227 * 1024 - 2048 - 4 * (kOzStreamTiles + 1)) / oz_stage_bytes(ng));
+    return n > kOzMaxStages ? kOzMaxStages : n;
 }
 inline int oz_groups(int K) { return (K + kOzCols - 1) / kOzCols; }
 inline int oz_group_cols(int K) { return ((K + oz_groups(K) - 1) / oz_groups(K) + 15) & ~15; }
@@ -1187,15 +1207,15 @@ __device__ __forceinline__ double i64_to_f64(long long v) {
     return m ? __hiloint2double((int)hi, (int)(unsigned)(n >> 11)) : 0.0;
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ OzArgs o) {
+__global__ void __launch_bounds__(kOzThreads, 1) m2l_oz(const __grid_constant__ OzArgs o) {
     extern __shared__ unsigned char dsm[];
     unsigned char *base = dsm + ((1024 - (smem_u32(dsm) & 1023)) & 1023);
-    __shared__ __align__(8) uint64_t afull[kTcMaxStages], bfull[kTcMaxStages], empty[kTcMaxStages];
+    __shared__ __align__(8) uint64_t afull[kOzMaxStages], bfull[kOzMaxStages], empty[kOzMaxStages];
     __shared__ __align__(8) uint64_t bank_full, bank_empty;
     __shared__ uint32_t tslot;
     __shared__ int abort_flag;
-    __shared__ uint32_t pref[kStreamTiles + 1];   // stream: units before each (tile, group)
-    __shared__ uint32_t wtot[kTcWarps];
+    __shared__ uint32_t pref[kOzStreamTiles + 1];   // stream: units before each (tile, group)
+    __shared__ uint32_t wtot[kOzWarps];
     __shared__ int first_tile;
     const TcArgs &a = o.t;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1224,10 +1244,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ 
     // this CTA's units [u0, u1), as in m2l_tc with (tile, group) pairs for tiles
     uint32_t G = 1, T = 0, u0 = 0, u1 = 0;
     if (a.stream) {
-        uint32_t n[kScanItems], sum = 0;
+        uint32_t n[kOzScanItems], sum = 0;
 #pragma unroll
-        for (int q = 0; q < kScanItems; ++q) {
-            const int t = tid * kScanItems + q;
+        for (int q = 0; q < kOzScanItems; ++q) {
+            const int t = tid * kOzScanItems + q;
             n[q] = t < ntg ? __ldg(a.tmask + 8 * (size_t)(t / ngrp) + 6) : 0;
             sum += n[q];
         }
@@ -1240,7 +1260,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ 
         if (lane == 31) wtot[warp] = incl;
         __syncthreads();
         uint32_t before = 0;
-        for (int w = 0; w < kTcWarps; ++w) {
+        for (int w = 0; w < kOzWarps; ++w) {
             if (w < warp) before += wtot[w];
             T += wtot[w];
         }
@@ -1251,8 +1271,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) m2l_oz(const __grid_constant__ 
             u1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * T / G);
         }
 #pragma unroll
-        for (int q = 0; q < kScanItems; ++q) {
-            const int t = tid * kScanItems + q;
+        for (int q = 0; q < kOzScanItems; ++q) {
+            const int t = tid * kOzScanItems + q;
             if (t <= ntg) pref[t] = run;
             if (t < ntg && u0 >= run && u0 < run + n[q]) first_tile = t;
             run += n[q];
@@ -2201,7 +2221,7 @@ gf_status m2l_oz_prepare(gf_plan_s *plan) {
     const double fold_us = 0.8e-4 * K * K * (double)((cols + sms * P - 1) / (sms * P) * (sms * P));
     if (oz_us > 0.85 * fold_us) return GF_OK;
     const int64_t ctas = std::min<int64_t>(sm_count(), tiles * ngrp * 189);
-    const bool stream = tiles * ngrp <= kStreamTiles;
+    const bool stream = tiles * ngrp <= kOzStreamTiles;
     const size_t row_bytes = (size_t)nck * kOzRowChunk;
     const size_t need = (size_t)rows * (row_bytes + sizeof(double)) + (size_t)tiles * 8 * sizeof(uint32_t) +
                         (F->L + 1) * sizeof(TcLevel) +
@@ -2283,7 +2303,7 @@ static gf_status m2l_run_oz(gf_plan_s *plan, int B, cudaStream_t st, cudaEvent_t
     o.part = F->oz_part;
     a.nst = oz_stages(o.ng);
     const int64_t ntg = (int64_t)a.ntiles * o.ngrp;
-    a.stream = ntg <= kStreamTiles && o.part;
+    a.stream = ntg <= kOzStreamTiles && o.part;
     OzSplitArgs p;
     memset(&p, 0, sizeof(p));
     p.se = z->se;
@@ -2310,7 +2330,7 @@ static gf_status m2l_run_oz(gf_plan_s *plan, int B, cudaStream_t st, cudaEvent_t
     GF_TRY(ensure_smem(m2l_oz, shm));
     const int64_t grid = a.stream ? std::min<int64_t>(sm_count(), ntg * 189) : ntg;
     for (o.bb = 0; o.bb < B; ++o.bb) {
-        m2l_oz<<<(unsigned)grid, kTcThreads, shm, st>>>(o);
+        m2l_oz<<<(unsigned)grid, kOzThreads, shm, st>>>(o);
         GF_KERNEL_DONE();
         if (a.stream && grid > 1) {
             m2l_oz_join<<<dim3((unsigned)grid - 1, 2), 512, 0, st>>>(o);
