@@ -993,12 +993,15 @@ eval_kernel(EvalArgs a) {
 // pairs that share every coefficient load; the warps take the evaluation
 // items (64 observers each) from the queue and skip every second item of a
 // leaf, which the warp holding the item before it covers.
+// Bound by the FP32 pipe.  With the real recursion of l2p_sum2 (nine operations a
+// term; the complex one took twelve) 2.1 M observers in 128^3 283 -> 227 us,
+// 464 x 464 x 16 with 512 x 512 stations 130 -> 101 us.
 constexpr int kFarWarps = 4;
 constexpr int kFarTargets = 128;
 static_assert(kFarTargets == 2 * kTPL * 32, "two evaluation items per far item");
 inline __host__ __device__ int far_slice(int P2) { return (6 * P2 + 7) & ~7; }   // floats per warp
 
-__global__ void __launch_bounds__(kFarWarps * 32, 6) eval_far_kernel(EvalArgs a, const int32_t *__restrict__ leaf_beg) {
+__global__ void __launch_bounds__(kFarWarps * 32, 5) eval_far_kernel(EvalArgs a, const int32_t *__restrict__ leaf_beg) {
     extern __shared__ float fsh[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int P2 = a.p * a.p;
@@ -1033,13 +1036,11 @@ __global__ void __launch_bounds__(kFarWarps * 32, 6) eval_far_kernel(EvalArgs a,
         for (int bb = 0; bb < a.B; ++bb) {
             const float *L = le + ((int64_t)leaf * a.B + bb) * a.ldk;
             __syncwarp();
-            // duplicated pairs, the factor 2 of the m > 0 terms folded in
+            // duplicated pairs, scaled
             for (int e = lane; e < P2; e += 32) {
                 float vx, vy, vz;
                 grad_coeff<float>(L, e, vx, vy, vz);
-                int n = 0;
-                while ((n + 1) * (n + 1) <= e) ++n;
-                const float f2 = e == n * n ? 1.f : 2.f;
+                const float f2 = __ldg(l2p_scale + e);
                 Dx2[e] = make_float2(f2 * vx, f2 * vx);
                 Dy2[e] = make_float2(f2 * vy, f2 * vy);
                 Dz2[e] = make_float2(f2 * vz, f2 * vz);
@@ -1664,20 +1665,7 @@ __global__ void transpose_ops(const double *__restrict__ fwd, double *__restrict
 // The far field's tables for the current device.
 gf_status upload_far_coefs() {
     double c[kMaxP * (kMaxP - 1) / 2 + 1] = {}, sc[kMaxP * kMaxP] = {};
-    double sect = 1.0;
-    for (int m = 0; m < kMaxP; ++m) {
-        if (m > 0) sect *= -std::sqrt((2.0 * m - 1.0) / (2.0 * m));
-        double v = m > 0 ? 2.0 * sect : sect;
-        for (int n = m; n < kMaxP; ++n) {
-            if (n > m) {
-                v *= (2 * n - 1) / std::sqrt((double)((n + m) * (n - m)));
-                c[n * (n - 1) / 2 + m] = n > m + 1 ? -(double)((n - 1) * (n - 1) - m * m) / ((2 * n - 1) * (2 * n - 3)) : 0.0;
-            }
-            const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
-            sc[k] = v;
-            if (m > 0) sc[k + 1] = v;
-        }
-    }
+    l2p_tables(c, sc);
     GF_CUDA(cudaMemcpyToSymbol(c_far_c, c, sizeof(c)));
     GF_CUDA(cudaMemcpyToSymbol(c_far_s, sc, sizeof(sc)));
     return GF_OK;

@@ -939,9 +939,7 @@ __global__ void __launch_bounds__(kPtWarps * 32) point_eval(PtEvalArgs a) {
                 for (int e = lane; e < P2; e += 32) {
                     float vx, vy, vz;
                     grad_coeff<float>(Lc, e, vx, vy, vz);
-                    int n = 0;
-                    while ((n + 1) * (n + 1) <= e) ++n;
-                    const float f2 = e == n * n ? 1.f : 2.f;
+                    const float f2 = __ldg(l2p_scale + e);
                     Dx2[e] = make_float2(f2 * vx, f2 * vx);
                     Dy2[e] = make_float2(f2 * vy, f2 * vy);
                     Dz2[e] = make_float2(f2 * vz, f2 * vz);

@@ -74,156 +74,139 @@ __device__ __forceinline__ void two_sum(T &hi, T &lo, T x) {
     hi = s;
 }
 
-// Coefficients of the regular-harmonic recursion of the L2P sums (the
-// recursion of fmm_math.cuh), for m < n < kMaxP at t = n (n + 1) / 2 + m:
-//   c_ra[t] = (2n - 1) / sqrt((n + m)(n - m)),
-//   c_rb[t] = sqrt((n - 1 + m)(n - 1 - m)) / sqrt((n + m)(n - m))  (0 for n = m + 1),
-// and c_rf[m] = -sqrt((2m - 1) / (2m)) for the sectoral step, so that the
-// FP32 evaluation needs no square roots or divisions.
-__constant__ float c_ra[kMaxP * (kMaxP + 1) / 2], c_rb[kMaxP * (kMaxP + 1) / 2], c_rf[kMaxP];
+// The L2P sums sum_{n<p, m} D_n^m conj(R_n^m(X)) of the gradient expansions
+// (l2p_sum of fmm_math.cuh) with R_n^m = s_nm (x + iy)^m Q_n^m(z, r^2), Q real:
+// Q_m^m = 1, Q_n = z Q_{n-1} - c_nm r^2 Q_{n-2}, c_nm = ((n-1)^2 - m^2) /
+// ((2n-1)(2n-3)).  s_nm (and the factor 2 of the m > 0 terms) is in the staged
+// coefficients, an order's sums are made with Q alone and turned by (x + iy)^m
+// once: nine operations a term instead of twelve, and no square roots or
+// divisions.  c_lq: -c_nm at n (n - 1) / 2 + m, m < n < kMaxP (zero at n = m + 1);
+// l2p_scale: s_nm, twice it for m > 0, by real component.
+__constant__ float c_lq[kMaxP * (kMaxP - 1) / 2 + 1];
+__device__ float l2p_scale[kMaxP * kMaxP];
 
-// sum_{n<p, m} D_n^m conj(R_n^m(X)) for the gradient expansions of
-// l2p_sum (fmm_math.cuh), for two points at once (packed pairs X, Y, Z).
-// D holds each coefficient as a duplicated pair {d, d}, with the factor 2
-// of the m > 0 terms folded in.
+// For two points at once (packed pairs X, Y, Z).  D holds each scaled
+// coefficient as a duplicated pair {d, d}.
 __device__ __forceinline__ void l2p_sum2(int p, const float2 *Dx, const float2 *Dy, const float2 *Dz, uint64_t X,
                                          uint64_t Y, uint64_t Z, uint64_t &gx, uint64_t &gy, uint64_t &gz) {
     const uint64_t r2 = fma2(Z, Z, fma2(Y, Y, mul2(X, X)));
-    uint64_t sr = pk2(1.f, 1.f), si = 0;
-    uint64_t ax = 0, ay = 0, az = 0;
+    const uint64_t NY = Y ^ 0x8000000080000000ull, one = pk2(1.f, 1.f);
+    uint64_t wr = one, wi = 0;
     auto ld = [](const float2 *d, int k) { return *reinterpret_cast<const uint64_t *>(d + k); };
+    gx = gy = gz = 0;
     for (int m = 0; m < p; ++m) {
-        if (m > 0) {
-            const float f = c_rf[m];
-            const uint64_t XF = mul2(X, pk2(f, f)), YF = mul2(Y, pk2(f, f)), YN = mul2(Y, pk2(-f, -f));
-            const uint64_t nr = fma2(XF, sr, mul2(YN, si));
-            const uint64_t ni = fma2(XF, si, mul2(YF, sr));
-            sr = nr;
-            si = ni;
-        }
-        uint64_t r1 = sr, i1 = si, r0 = 0, i0 = 0;
+        uint64_t Q = one, P = 0, xr = 0, xi = 0, yr = 0, yi = 0, zr = 0, zi = 0;
         for (int n = m; n < p; ++n) {
-            uint64_t cr = sr, ci = si;
             if (n > m) {
-                const int t = n * (n + 1) / 2 + m;
-                const float av = c_ra[t], bv = c_rb[t];
-                const uint64_t AZ = mul2(Z, pk2(av, av)), BN = mul2(r2, pk2(-bv, -bv));
-                cr = fma2(AZ, r1, mul2(BN, r0));
-                ci = fma2(AZ, i1, mul2(BN, i0));
-                r0 = r1;
-                i0 = i1;
-                r1 = cr;
-                i1 = ci;
+                const float c = c_lq[n * (n - 1) / 2 + m];
+                const uint64_t v = fma2(Z, Q, mul2(mul2(r2, pk2(c, c)), P));
+                P = Q;
+                Q = v;
             }
-            if (m == 0) {
-                const int k = n * n;
-                ax = fma2(ld(Dx, k), cr, ax);
-                ay = fma2(ld(Dy, k), cr, ay);
-                az = fma2(ld(Dz, k), cr, az);
-            } else {
-                const int k = n * n + 2 * m - 1;
-                ax = fma2(ld(Dx, k), cr, fma2(ld(Dx, k + 1), ci, ax));
-                ay = fma2(ld(Dy, k), cr, fma2(ld(Dy, k + 1), ci, ay));
-                az = fma2(ld(Dz, k), cr, fma2(ld(Dz, k + 1), ci, az));
+            const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+            xr = fma2(ld(Dx, k), Q, xr);
+            yr = fma2(ld(Dy, k), Q, yr);
+            zr = fma2(ld(Dz, k), Q, zr);
+            if (m > 0) {
+                xi = fma2(ld(Dx, k + 1), Q, xi);
+                yi = fma2(ld(Dy, k + 1), Q, yi);
+                zi = fma2(ld(Dz, k + 1), Q, zi);
             }
         }
+        gx = fma2(xr, wr, fma2(xi, wi, gx));
+        gy = fma2(yr, wr, fma2(yi, wi, gy));
+        gz = fma2(zr, wr, fma2(zi, wi, gz));
+        const uint64_t nr = fma2(X, wr, mul2(NY, wi)), ni = fma2(X, wi, mul2(Y, wr));
+        wr = nr;
+        wi = ni;
     }
-    gx = ax;
-    gy = ay;
-    gz = az;
 }
 
-
-// l2p_sum2 for two packed pairs of points at once (four points): the
-// recursion coefficients and every coefficient of D are loaded once for both.
+// l2p_sum2 for two packed pairs of points at once (four points): every
+// coefficient is loaded once for both.
 __device__ __forceinline__ void l2p_sum2x2(int p, const float2 *Dx, const float2 *Dy, const float2 *Dz,
                                            uint64_t X0, uint64_t Y0, uint64_t Z0, uint64_t X1, uint64_t Y1,
                                            uint64_t Z1, uint64_t g0[3], uint64_t g1[3]) {
     const uint64_t q0 = fma2(Z0, Z0, fma2(Y0, Y0, mul2(X0, X0)));
     const uint64_t q1 = fma2(Z1, Z1, fma2(Y1, Y1, mul2(X1, X1)));
-    uint64_t sr0 = pk2(1.f, 1.f), si0 = 0, sr1 = sr0, si1 = 0;
-    uint64_t ax0 = 0, ay0 = 0, az0 = 0, ax1 = 0, ay1 = 0, az1 = 0;
+    const uint64_t one = pk2(1.f, 1.f);
+    uint64_t wr0 = one, wi0 = 0, wr1 = one, wi1 = 0;
     auto ld = [](const float2 *d, int k) { return *reinterpret_cast<const uint64_t *>(d + k); };
+#pragma unroll
+    for (int d = 0; d < 3; ++d) g0[d] = g1[d] = 0;
     for (int m = 0; m < p; ++m) {
-        if (m > 0) {
-            const float f = c_rf[m];
-            const uint64_t F = pk2(f, f), FN = pk2(-f, -f);
-            uint64_t nr = fma2(mul2(X0, F), sr0, mul2(mul2(Y0, FN), si0));
-            uint64_t ni = fma2(mul2(X0, F), si0, mul2(mul2(Y0, F), sr0));
-            sr0 = nr;
-            si0 = ni;
-            nr = fma2(mul2(X1, F), sr1, mul2(mul2(Y1, FN), si1));
-            ni = fma2(mul2(X1, F), si1, mul2(mul2(Y1, F), sr1));
-            sr1 = nr;
-            si1 = ni;
-        }
-        uint64_t r10 = sr0, i10 = si0, r00 = 0, i00 = 0;
-        uint64_t r11 = sr1, i11 = si1, r01 = 0, i01 = 0;
+        uint64_t Q0 = one, P0 = 0, Q1 = one, P1 = 0;
+        uint64_t re0[3] = {0, 0, 0}, im0[3] = {0, 0, 0}, re1[3] = {0, 0, 0}, im1[3] = {0, 0, 0};
         for (int n = m; n < p; ++n) {
-            uint64_t cr0 = sr0, ci0 = si0, cr1 = sr1, ci1 = si1;
             if (n > m) {
-                const int t = n * (n + 1) / 2 + m;
-                const float av = c_ra[t], bv = c_rb[t];
-                const uint64_t A = pk2(av, av), BN = pk2(-bv, -bv);
-                const uint64_t AZ0 = mul2(Z0, A), BQ0 = mul2(q0, BN), AZ1 = mul2(Z1, A), BQ1 = mul2(q1, BN);
-                cr0 = fma2(AZ0, r10, mul2(BQ0, r00));
-                ci0 = fma2(AZ0, i10, mul2(BQ0, i00));
-                cr1 = fma2(AZ1, r11, mul2(BQ1, r01));
-                ci1 = fma2(AZ1, i11, mul2(BQ1, i01));
-                r00 = r10;
-                i00 = i10;
-                r10 = cr0;
-                i10 = ci0;
-                r01 = r11;
-                i01 = i11;
-                r11 = cr1;
-                i11 = ci1;
+                const float c = c_lq[n * (n - 1) / 2 + m];
+                const uint64_t C = pk2(c, c);
+                const uint64_t v0 = fma2(Z0, Q0, mul2(mul2(q0, C), P0)), v1 = fma2(Z1, Q1, mul2(mul2(q1, C), P1));
+                P0 = Q0;
+                Q0 = v0;
+                P1 = Q1;
+                Q1 = v1;
             }
-            if (m == 0) {
-                const int k = n * n;
-                const uint64_t dx = ld(Dx, k), dy = ld(Dy, k), dz = ld(Dz, k);
-                ax0 = fma2(dx, cr0, ax0);
-                ay0 = fma2(dy, cr0, ay0);
-                az0 = fma2(dz, cr0, az0);
-                ax1 = fma2(dx, cr1, ax1);
-                ay1 = fma2(dy, cr1, ay1);
-                az1 = fma2(dz, cr1, az1);
-            } else {
-                const int k = n * n + 2 * m - 1;
-                const uint64_t dxr = ld(Dx, k), dxi = ld(Dx, k + 1), dyr = ld(Dy, k), dyi = ld(Dy, k + 1),
-                               dzr = ld(Dz, k), dzi = ld(Dz, k + 1);
-                ax0 = fma2(dxr, cr0, fma2(dxi, ci0, ax0));
-                ay0 = fma2(dyr, cr0, fma2(dyi, ci0, ay0));
-                az0 = fma2(dzr, cr0, fma2(dzi, ci0, az0));
-                ax1 = fma2(dxr, cr1, fma2(dxi, ci1, ax1));
-                ay1 = fma2(dyr, cr1, fma2(dyi, ci1, ay1));
-                az1 = fma2(dzr, cr1, fma2(dzi, ci1, az1));
+            const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+            const uint64_t dr[3] = {ld(Dx, k), ld(Dy, k), ld(Dz, k)};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                re0[d] = fma2(dr[d], Q0, re0[d]);
+                re1[d] = fma2(dr[d], Q1, re1[d]);
+            }
+            if (m > 0) {
+                const uint64_t di[3] = {ld(Dx, k + 1), ld(Dy, k + 1), ld(Dz, k + 1)};
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    im0[d] = fma2(di[d], Q0, im0[d]);
+                    im1[d] = fma2(di[d], Q1, im1[d]);
+                }
             }
         }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            g0[d] = fma2(re0[d], wr0, fma2(im0[d], wi0, g0[d]));
+            g1[d] = fma2(re1[d], wr1, fma2(im1[d], wi1, g1[d]));
+        }
+        const uint64_t N0 = Y0 ^ 0x8000000080000000ull, N1 = Y1 ^ 0x8000000080000000ull;
+        uint64_t nr = fma2(X0, wr0, mul2(N0, wi0)), ni = fma2(X0, wi0, mul2(Y0, wr0));
+        wr0 = nr;
+        wi0 = ni;
+        nr = fma2(X1, wr1, mul2(N1, wi1));
+        ni = fma2(X1, wi1, mul2(Y1, wr1));
+        wr1 = nr;
+        wi1 = ni;
     }
-    g0[0] = ax0;
-    g0[1] = ay0;
-    g0[2] = az0;
-    g1[0] = ax1;
-    g1[1] = ay1;
-    g1[2] = az1;
 }
 
-// The recursion coefficients of l2p_sum2 for the current device.
-inline gf_status upload_l2p_coefs() {
-    constexpr int NT = kMaxP * (kMaxP + 1) / 2;
-    float ra[NT] = {}, rb[NT] = {}, rf[kMaxP] = {};
-    for (int n = 1; n < kMaxP; ++n)
-        for (int m = 0; m < n; ++m) {
-            const int t = n * (n + 1) / 2 + m;
-            const double inv = 1.0 / std::sqrt((double)((n + m) * (n - m)));
-            ra[t] = (float)((2 * n - 1) * inv);
-            rb[t] = n - 1 > m ? (float)(std::sqrt((double)((n - 1 + m) * (n - 1 - m))) * inv) : 0.f;
+// c[n (n - 1) / 2 + m] = -c_nm and sc[component] = the L2P scales, in FP64.
+inline void l2p_tables(double *c, double *sc) {
+    double sect = 1.0;
+    for (int m = 0; m < kMaxP; ++m) {
+        if (m > 0) sect *= -std::sqrt((2.0 * m - 1.0) / (2.0 * m));
+        double v = m > 0 ? 2.0 * sect : sect;
+        for (int n = m; n < kMaxP; ++n) {
+            if (n > m) {
+                v *= (2 * n - 1) / std::sqrt((double)((n + m) * (n - m)));
+                c[n * (n - 1) / 2 + m] =
+                    n > m + 1 ? -(double)((n - 1) * (n - 1) - m * m) / ((2 * n - 1) * (2 * n - 3)) : 0.0;
+            }
+            const int k = n * n + (m == 0 ? 0 : 2 * m - 1);
+            sc[k] = v;
+            if (m > 0) sc[k + 1] = v;
         }
-    for (int m = 1; m < kMaxP; ++m) rf[m] = (float)-std::sqrt((2.0 * m - 1.0) / (2.0 * m));
-    GF_CUDA(cudaMemcpyToSymbol(c_ra, ra, sizeof(ra)));
-    GF_CUDA(cudaMemcpyToSymbol(c_rb, rb, sizeof(rb)));
-    GF_CUDA(cudaMemcpyToSymbol(c_rf, rf, sizeof(rf)));
+    }
+}
+
+// The tables of l2p_sum2 for the current device.
+inline gf_status upload_l2p_coefs() {
+    double c[kMaxP * (kMaxP - 1) / 2 + 1] = {}, sc[kMaxP * kMaxP] = {};
+    l2p_tables(c, sc);
+    float cf[kMaxP * (kMaxP - 1) / 2 + 1], sf[kMaxP * kMaxP];
+    for (size_t i = 0; i < sizeof(cf) / sizeof(cf[0]); ++i) cf[i] = (float)c[i];
+    for (int i = 0; i < kMaxP * kMaxP; ++i) sf[i] = (float)sc[i];
+    GF_CUDA(cudaMemcpyToSymbol(c_lq, cf, sizeof(cf)));
+    GF_CUDA(cudaMemcpyToSymbol(l2p_scale, sf, sizeof(sf)));
     return GF_OK;
 }
 
