@@ -296,7 +296,7 @@ def level_boxes(info, l):
     return n
 
 
-SPLIT_PRODUCTS = 3              # tensor-core products per algorithmic one (FP16 or TF32 high/low parts)
+SPLIT_PRODUCTS = 3              # tensor-core products per algorithmic one (FP16 high/low parts)
 P2M_FLOPS_PER_HARMONIC = 10.0   # point P2M: one recursion step (6 flops) + the mass-weighted sum (4)
 
 
@@ -315,31 +315,30 @@ def fmm_roofline(stages, info, args, peaks, workload, nvox=None, rho_bytes=4, n_
                      "eval_kernel (near field) + eval_far_kernel (L2P, near + far, scatter)"),
             "m2l": ("tensor" if tensor else "alu", 2.0 * K * K * float(info.m2l_pairs),
                     "m2l_tc (tcgen05 FP16 parts, 3 products, all levels)" if tensor
-                    else "m2l_simt (all levels)")}
+                    else "m2l_oz (BF16 digits) or m2l_fold (all levels)")}
     if nvox is not None and L >= 2:
         ns = {l: level_boxes(info, l) for l in range(2, L + 1)}
-        # mixed precision on the tensor cores with L - 1 > 2: the P2M stage
-        # makes level L-1 straight from the densities (its essential traffic:
-        # the densities once, those expansions once) and the M2M stage starts
-        # from level L-1
-        up = tensor and L - 1 > 2
+        # 4^3-voxel leaves with L - 1 > 2: the P2M stage makes level L-1
+        # straight from the densities (its essential traffic: the densities
+        # once, those expansions once) and the M2M stage starts from level L-1
+        up = L - 1 > 2
         top = L - 1 if up else L
         work["p2m"] = ("hbm", float(nvox * rho_bytes + ns[top] * K * fbytes),
-                       "block_rows + m2l_tc P2M kinds (into level L-1 from the grid)" if up
-                       else ("block_rows + m2l_tc P2M kind" if tensor else "p2m_fused"))
+                       "block_rows + p2m_leaf_fold + p2m_up_quad (into level L-1 from the grid)" if up
+                       else "block_rows + p2m_leaf_fold")
         work["m2m"] = ("hbm", float(sum(ns[l] * K * fbytes for l in range(3, top + 1))
                                     + sum(ns[l] * K * fbytes for l in range(2, top))),
-                       "m2l_tc M2M kind + m2m_kernel (FP64 into level 2)" if tensor else "xlate_simt")
+                       "fold_quad + fold_kernel (FP64 into level 2)")
     if n_points is not None and L >= 2:
         # point sources: the P2M evaluates (p+1)(p+2)/2 complex harmonics per
         # point; the M2M reads each level's expansions once and writes the
         # parents' once
         ns = {l: level_boxes(info, l) for l in range(2, L + 1)}
         work["p2m"] = ("alu", P2M_FLOPS_PER_HARMONIC * (p + 1) * (p + 2) / 2 * float(n_points),
-                       "point_p2m_f32 (packed pair recursion)" if args.precision == "mixed" else "point_p2m")
+                       "point_p2m (two orders per lane)")
         work["m2m"] = ("hbm", float(sum(ns[l] * K * fbytes for l in range(3, L + 1))
                                     + sum(ns[l] * K * fbytes for l in range(2, L))),
-                       "m2l_tc M2M kind + m2m_kernel (FP64 into level 2)" if tensor else "xlate_simt")
+                       "fold_quad + fold_kernel (FP64 into level 2)")
     dom = max(work, key=lambda k: stages.get(k, 0.0))
     bound, amount, kern = work[dom]
     extra = {}

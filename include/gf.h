@@ -74,17 +74,20 @@ typedef struct {
 } gf_quad;
 
 enum { GF_MODE_DIRECT = 0, GF_MODE_FMM = 1 };
-/* GF_PREC_FP64: every stage in FP64.  GF_PREC_MIXED: FP32 near field with
+/* GF_PREC_FP64: every stage in FP64 (the forward M2L on the FP64 units or, where
+ * that is faster and the plan's announced size has room for its inputs, on the
+ * tensor cores from seven base-256 digits per value with exact sums: the error
+ * of FP64 additions).  GF_PREC_MIXED: FP32 near field with
  * compensated accumulation; tensor-core M2L on FP16 high/low parts of
  * power-of-two-scaled operands (three products, FP32 accumulation) and
- * split-TF32 P2M/M2M/L2L; FP64 for the top-level translations and the final
- * near+far sum.  Results stay within a relative L2 error of about 1e-5
+ * P2M/M2M/L2L in FP32 folded by mirror symmetry; FP64 for the top-level
+ * translations and the final near+far sum.  Results stay within a relative L2 error of about 1e-5
  * (p >= 10). */
 enum { GF_PREC_FP64 = 0, GF_PREC_MIXED = 1 };
 enum { GF_DTYPE_F64 = 0, GF_DTYPE_F32 = 1 };
 /* Option flags (gf_options.reserved0):
- *   GF_FLAG_M2L_SIMT  FMM, mixed precision: the M2L on the SIMT cores
- *                     instead of the tensor cores.
+ *   GF_FLAG_M2L_SIMT  FMM: the M2L on the SIMT cores instead of the tensor
+ *                     cores (either precision).
  *   GF_FLAG_SUM_AN    every voxel integrated in closed form (SUM-AN of
  *                     Sec. 2.1, the exact field of the piecewise-constant
  *                     density, finite on voxel faces, edges and corners)

@@ -3,9 +3,9 @@
 // evaluation (L2P plus the near-field direct sum, Eq. 10).
 //
 // Every kernel here works in voxel units (h = 1); see gf_fmm.cuh.  The
-// evaluation kernel fuses the near-field sum over the nearest-neighbour
-// leaves, the local-expansion gradient, the near+far sum in FP64 and the
-// scatter back to the caller's observer order.
+// evaluation is two kernels: the near-field sum over the nearest-neighbour
+// leaves, left per observer, and the local-expansion gradient with the
+// near+far sum in FP64 and the scatter back to the caller's observer order.
 #include <math.h>
 #include <string.h>
 
