@@ -14,11 +14,12 @@ constexpr int kScanThreads = 256;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;   // 1024
 
-// Sort tiles: 8 keys per thread, or 16 from kBigSort keys on (half the digit
-// counts to scan and longer runs to write; fewer keys would leave SMs idle).
-constexpr int kSortThreads = 256;
+// Sort tiles: 256 threads of 8 keys, or of 16 from kBigSort keys on (longer runs
+// to write; fewer keys would leave SMs idle).  512 threads of 16: the scatter of
+// 2^25 keys 164 us in place of 151.
 constexpr int64_t kBigSort = 4 << 20;
 constexpr int kRadix = 256;
+constexpr int kSmallTile = 256 * 8, kBigTile = 256 * 16;
 
 __device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
     const int lane = threadIdx.x & 31;
@@ -77,8 +78,7 @@ __global__ void write_total(int64_t *__restrict__ out, int64_t n, const int64_t 
 // loads), one block-wide scan of the run totals gives every run its offset,
 // and a second sweep scans the run row by row (the reads of four rows ahead of
 // the row in hand).  Latency is all there is to it: rows a warp reads at once
-// instead of a run per thread, 32,768 items (the digit counts of 262,144
-// observers) 59 -> 17 us.  Also the total into out[n] when asked.  (`in` may
+// instead of a run per thread, 32,768 items 59 -> 17 us.  Also the total into out[n] when asked.  (`in` may
 // alias `out`: the second sweep reads each item before writing it.)
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallRows = 32;   // per warp
@@ -150,44 +150,102 @@ gf_status scan_rec(const int64_t *in, int64_t *out, int64_t n, int64_t *scratch,
 }
 
 // -------------------------------------------------------------- radix sort
-template <class K, int R>
-__global__ void __launch_bounds__(kSortThreads)
-radix_hist(const K *__restrict__ keys, int64_t n, int shift, int64_t nblocks, int64_t *__restrict__ hist) {
-    __shared__ int cnt[kRadix];
-    cnt[threadIdx.x] = 0;
+// Counts of a pass: hist[digit][block] (rows of ld entries, a multiple of 4).
+template <class K, int T, int R>
+__global__ void __launch_bounds__(T)
+radix_hist(const K *__restrict__ keys, int64_t n, int shift, int64_t ld, uint32_t *__restrict__ hist) {
+    __shared__ uint32_t cnt[kRadix];
+    if (threadIdx.x < kRadix) cnt[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * (kSortThreads * R);
+    const int64_t base = (int64_t)blockIdx.x * (T * R);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int64_t i = base + r * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 0xff], 1);
+        const int64_t i = base + r * T + threadIdx.x;
+        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 0xff], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+    if (threadIdx.x < kRadix) hist[(int64_t)threadIdx.x * ld + blockIdx.x] = cnt[threadIdx.x];
+}
+
+// Exclusive scan of each digit's row in place, its total to tot[digit]: one block
+// a digit, 1,024 counts at a time; the scatter adds the digits' own scan.  All SMs
+// take part: for 262,144 keys 2.5 us where one block over all the digits' 32,768
+// counts took 24; for 2^25, 8 where tiles, their sums and a sweep to add them took 23.
+__global__ void __launch_bounds__(256)
+radix_rows(uint32_t *__restrict__ hist, int64_t nb, int64_t ld, uint32_t *__restrict__ tot) {
+    __shared__ uint32_t wsum[2][8];
+    uint32_t *row = hist + (int64_t)blockIdx.x * ld;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t run = 0;
+    int buf = 0;
+    for (int64_t b = 0; b < nb; b += 1024, buf ^= 1) {
+        const int64_t i = b + 4 * threadIdx.x;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < nb) {
+            v = *reinterpret_cast<const uint4 *>(row + i);
+            if (i + 1 >= nb) v.y = 0;
+            if (i + 2 >= nb) v.z = 0;
+            if (i + 3 >= nb) v.w = 0;
+        }
+        const uint32_t four = v.x + v.y + v.z + v.w;
+        uint32_t incl = four;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wsum[buf][warp] = incl;
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const uint32_t t = wsum[buf][w];
+            if (w < warp) before += t;
+            all += t;
+        }
+        if (i < nb) {
+            uint4 o;
+            o.x = run + before + incl - four;
+            o.y = o.x + v.x;
+            o.z = o.y + v.y;
+            o.w = o.z + v.z;
+            *reinterpret_cast<uint4 *>(row + i) = o;
+        }
+        run += all;
+    }
+    if (threadIdx.x == 0) tot[blockIdx.x] = run;
 }
 
 // Stable scatter.  Each warp ranks its own run of 32 R consecutive keys, row by
 // row, against its own digit counts (warp-level synchronisation only); one
 // block-wide step turns the warps' counts into offsets, and the keys go out
 // from registers.  Equal digits keep their relative order.  vals == nullptr:
-// the values are the indices.  Bound by the scattered writes (R keys
-// of a digit to a block, on average); ranking a block's row at a time, five block barriers to
-// 256 keys, it was bound by those: 200 us a pass over 2^25 (64-bit) keys, now 150.
-template <class K, int R>
-__global__ void __launch_bounds__(kSortThreads)
-radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int64_t n, int shift, int64_t nblocks,
-              const int64_t *__restrict__ offs, K *__restrict__ keys_out, int32_t *__restrict__ vals_out) {
-    constexpr int kWarps = kSortThreads / 32;
-    __shared__ int64_t first[kRadix];
-    __shared__ int wcnt[kWarps][kRadix];
+// the values are the indices.  Bound by the scattered writes (a tile's keys of a
+// digit are a run, 16 on average in the large tiles); ranking a block's row at a
+// time, five block barriers to 256 keys, it was bound by those: 200 us a pass over
+// 2^25 keys, now 150.
+template <class K, int T, int R>
+__global__ void __launch_bounds__(T)
+radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int64_t n, int shift, int64_t ld,
+              const uint32_t *__restrict__ offs, const uint32_t *__restrict__ tot, K *__restrict__ keys_out,
+              int32_t *__restrict__ vals_out) {
+    constexpr int kWarps = T / 32;
+    __shared__ uint32_t wcnt[kWarps][kRadix];
+    __shared__ uint32_t dsum[kRadix / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t base = (int64_t)blockIdx.x * (kSortThreads * R) + warp * (32 * R) + lane;
+    const int64_t base = (int64_t)blockIdx.x * (T * R) + warp * (32 * R) + lane;
     const unsigned lt_mask = (1u << lane) - 1u;
     K k[R];
     int32_t v[R];
-    int rank[R];
+    uint32_t rank[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) k[r] = base + 32 * r < n ? keys[base + 32 * r] : 0;
+    // thread d: where digit d's keys of this block begin
+    uint32_t mine = 0, start = 0;
+    if (threadIdx.x < kRadix) {
+        mine = tot[threadIdx.x];
+        start = offs[(int64_t)threadIdx.x * ld + blockIdx.x];
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = vals && base + 32 * r < n ? vals[base + 32 * r] : (int32_t)(base + 32 * r);
     for (int d = lane; d < kRadix; d += 32) wcnt[warp][d] = 0;
@@ -197,19 +255,28 @@ radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int6
         const bool valid = base + 32 * r < n;
         const int d = valid ? (int)((k[r] >> shift) & 0xff) : kRadix;   // invalid -> sentinel
         const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int old = valid ? wcnt[warp][d] : 0;
+        const uint32_t old = valid ? wcnt[warp][d] : 0;
         rank[r] = old + __popc(peers & lt_mask);
         __syncwarp();
         if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] = old + __popc(peers);
         __syncwarp();
     }
-    first[threadIdx.x] = offs[(int64_t)threadIdx.x * nblocks + blockIdx.x];
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (threadIdx.x < kRadix && lane == 31) dsum[warp] = incl;
     __syncthreads();
-    {   // exclusive prefix over warps for digit threadIdx.x
-        int acc = 0;
+    if (threadIdx.x < kRadix) {   // digit threadIdx.x: its keys of the warps before, from its own start
+        uint32_t acc = start + incl - mine;
+#pragma unroll
+        for (int w = 0; w < kRadix / 32; ++w)
+            if (w < warp) acc += dsum[w];
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
-            const int c = wcnt[w][threadIdx.x];
+            const uint32_t c = wcnt[w][threadIdx.x];
             wcnt[w][threadIdx.x] = acc;
             acc += c;
         }
@@ -218,22 +285,22 @@ radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int6
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (base + 32 * r < n) {
-            const int d = (int)((k[r] >> shift) & 0xff);
-            const int64_t pos = first[d] + wcnt[warp][d] + rank[r];
+            const uint32_t pos = wcnt[warp][(k[r] >> shift) & 0xff] + rank[r];
             keys_out[pos] = k[r];
             vals_out[pos] = v[r];
         }
 }
 
-template <class K, int R>
-gf_status radix_pass(const K *keys, const int32_t *vals, int64_t n, int shift, int64_t *hist, K *keys_out,
+template <class K, int T, int R>
+gf_status radix_pass(const K *keys, const int32_t *vals, int64_t n, int shift, uint32_t *hist, K *keys_out,
                      int32_t *vals_out, cudaStream_t st) {
-    const int64_t nb = (n + kSortThreads * R - 1) / (kSortThreads * R);
-    const int64_t h = nb * kRadix;
-    radix_hist<K, R><<<(unsigned)nb, kSortThreads, 0, st>>>(keys, n, shift, nb, hist);
+    const int64_t nb = (n + T * R - 1) / (T * R), ld = (nb + 3) / 4 * 4;
+    uint32_t *tot = hist + ld * kRadix;
+    radix_hist<K, T, R><<<(unsigned)nb, T, 0, st>>>(keys, n, shift, ld, hist);
     GF_KERNEL_DONE();
-    GF_TRY(scan_rec(hist, hist, h, hist + h + 1, st, false));
-    radix_scatter<K, R><<<(unsigned)nb, kSortThreads, 0, st>>>(keys, vals, n, shift, nb, hist, keys_out, vals_out);
+    radix_rows<<<kRadix, 256, 0, st>>>(hist, nb, ld, tot);
+    GF_KERNEL_DONE();
+    radix_scatter<K, T, R><<<(unsigned)nb, T, 0, st>>>(keys, vals, n, shift, ld, hist, tot, keys_out, vals_out);
     GF_KERNEL_DONE();
     return GF_OK;
 }
@@ -248,7 +315,8 @@ __device__ __forceinline__ unsigned long long order_key(double v) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-__global__ void bbox_keys(const double *__restrict__ p, int64_t n, unsigned long long *__restrict__ out) {
+__global__ void __launch_bounds__(256)
+bbox_keys(const double *__restrict__ p, int64_t n, unsigned long long *__restrict__ out) {
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0, 0, 0};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -259,6 +327,10 @@ __global__ void bbox_keys(const double *__restrict__ p, int64_t n, unsigned long
             mx[a] = k > mx[a] ? k : mx[a];
         }
     }
+    // one atomic of each kind to a block: the atomics of all warps, on six
+    // addresses, took most of the 21 us of 262,144 points (now 5)
+    __shared__ unsigned long long red[6][8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         for (int o = 16; o > 0; o >>= 1) {
@@ -266,12 +338,23 @@ __global__ void bbox_keys(const double *__restrict__ p, int64_t n, unsigned long
             mn[a] = x < mn[a] ? x : mn[a];
             mx[a] = y > mx[a] ? y : mx[a];
         }
-    }
-    if ((threadIdx.x & 31) == 0)
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(out + a, mn[a]);
-            atomicMax(out + 3 + a, mx[a]);
+        if (lane == 0) {
+            red[a][warp] = mn[a];
+            red[3 + a][warp] = mx[a];
         }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        unsigned long long m = red[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) {
+            const unsigned long long x = red[threadIdx.x][w];
+            m = threadIdx.x < 3 ? (x < m ? x : m) : (x > m ? x : m);
+        }
+        if (threadIdx.x < 3)
+            atomicMin(out + threadIdx.x, m);
+        else
+            atomicMax(out + threadIdx.x, m);
+    }
 }
 
 // keys back to doubles
@@ -300,9 +383,9 @@ size_t scan_scratch_bytes(int64_t n) {
 }
 
 size_t sort_scratch_bytes(int64_t n) {
-    const int64_t tile = kSortThreads * (n >= kBigSort ? 16 : 8);
-    const int64_t h = (n + tile - 1) / tile * kRadix;
-    return (size_t)(h + 1) * sizeof(int64_t) + scan_scratch_bytes(h) + 256;
+    const int64_t tile = n >= kBigSort ? kBigTile : kSmallTile;
+    const int64_t ld = ((n + tile - 1) / tile + 3) / 4 * 4;
+    return (size_t)(ld + 1) * kRadix * sizeof(uint32_t);
 }
 
 gf_status exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, void *scratch, cudaStream_t st) {
@@ -320,7 +403,7 @@ template <class K>
 gf_status radix_sort(K *keys, int32_t *vals, K *keys_alt, int32_t *vals_alt, int64_t n, int bits, void *scratch,
                      cudaStream_t st) {
     if (n <= 0) return GF_OK;
-    int64_t *hist = reinterpret_cast<int64_t *>(scratch);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(scratch);
     const int passes = sort_passes(bits);
     // odd: from keys_alt; each pass crosses over, the last one into keys
     K *ka = passes % 2 ? keys_alt : keys, *kb = passes % 2 ? keys : keys_alt;
@@ -328,9 +411,9 @@ gf_status radix_sort(K *keys, int32_t *vals, K *keys_alt, int32_t *vals_alt, int
     for (int ps = 0; ps < passes; ++ps) {
         const int32_t *vin = ps ? va : nullptr;
         if (n >= kBigSort)
-            GF_TRY((radix_pass<K, 16>(ka, vin, n, 8 * ps, hist, kb, vb, st)));
+            GF_TRY((radix_pass<K, 256, 16>(ka, vin, n, 8 * ps, hist, kb, vb, st)));
         else
-            GF_TRY((radix_pass<K, 8>(ka, vin, n, 8 * ps, hist, kb, vb, st)));
+            GF_TRY((radix_pass<K, 256, 8>(ka, vin, n, 8 * ps, hist, kb, vb, st)));
         std::swap(ka, kb);
         std::swap(va, vb);
     }
