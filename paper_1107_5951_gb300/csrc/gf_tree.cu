@@ -95,33 +95,111 @@ __global__ void obs_keys(const double *__restrict__ obs, int64_t M, Geo g, uint6
 // treat indices past the count as absent.
 __device__ __forceinline__ int64_t dev_count(const int64_t *d_n, int64_t n) { return d_n ? *d_n : n; }
 
-__global__ void mark_new(const uint64_t *__restrict__ keys, const int64_t *d_n, int64_t n, int64_t ub, int shift,
-                         int64_t *__restrict__ flags) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ub) return;
-    const int64_t cnt = dev_count(d_n, n);
-    flags[i] = (i < cnt && (i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift))) ? 1 : 0;
+// Lists written in order from counts per element (runs of equal keys, evaluation
+// items): one launch counts each tile of 1,024 elements, one ranks the elements of
+// a tile from the tiles before it (their counts summed by the block, or, from
+// kScanTiles tiles on, scanned first) and writes.  Bound by the launches: flags,
+// scan, offsets, total and the writing pass in a launch each took 18 us for the
+// leaves of 262,144 observers, now 7.
+constexpr int kListThreads = 256, kListTile = 4 * kListThreads;
+constexpr int64_t kScanTiles = 2048;
+
+// Sum over the block, to all threads (every thread, uniformly).
+__device__ __forceinline__ int64_t block_total(int64_t v) {
+    __shared__ int64_t part[kListThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int64_t t = 0;
+#pragma unroll
+    for (int w = 0; w < kListThreads / 32; ++w) t += part[w];
+    return t;
 }
 
-// After an exclusive scan of the flags: write the unique (shifted) keys, the
-// first index of each run, and the run index of every element.
-// (also: the number of runs, excl[ub], into *runs)
-__global__ void compact_runs(const uint64_t *__restrict__ keys, const int64_t *d_n, int64_t n, int64_t ub, int shift,
-                             const int64_t *__restrict__ excl, uint64_t *__restrict__ ukeys,
-                             int32_t *__restrict__ beg, int32_t *__restrict__ run_of, int64_t *__restrict__ runs) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *runs = excl[ub];
-    if (i >= dev_count(d_n, n)) return;
-    const bool nw = (i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift));
-    const int64_t e = excl[i];
-    if (nw) {
-        ukeys[e] = keys[i] >> shift;
-        if (beg) beg[e] = (int32_t)i;
+template <class F>
+__global__ void __launch_bounds__(kListThreads) list_count(F f, int64_t *__restrict__ cnts) {
+    const int64_t i0 = (int64_t)blockIdx.x * kListTile + 4 * threadIdx.x, n = f.size();
+    int c = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (i0 + e < n) c += f.count(i0 + e);
+    const int64_t t = block_total(c);
+    if (threadIdx.x == 0) cnts[blockIdx.x] = t;
+}
+
+template <class F>
+__global__ void __launch_bounds__(kListThreads) list_write(F f, const int64_t *__restrict__ cnts, int scanned) {
+    __shared__ int wsum[kListThreads / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i0 = (int64_t)blockIdx.x * kListTile + 4 * threadIdx.x, n = f.size();
+    int64_t first = 0;
+    if (scanned) {
+        first = cnts[blockIdx.x];
+    } else {
+        for (int64_t b = threadIdx.x; b < blockIdx.x; b += kListThreads) first += cnts[b];
+        first = block_total(first);
     }
-    if (run_of) run_of[i] = (int32_t)(nw ? e : e - 1);
+    int c[4], mine = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) mine += c[e] = i0 + e < n ? f.count(i0 + e) : 0;
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int64_t at = first + incl - mine;
+#pragma unroll
+    for (int w = 0; w < kListThreads / 32; ++w)
+        if (w < warp) at += wsum[w];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (i0 + e < n) f.put(i0 + e, c[e], at);
+        at += c[e];
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kListThreads - 1) f.total(at);
 }
 
-__global__ void set_last(int32_t *__restrict__ a, const int64_t *d_idx, int32_t v) { a[*d_idx] = v; }
+// f over at most ub >= 1 elements; cnts: ceil(ub / kListTile) + 1 of device memory.
+template <class F>
+gf_status write_list(const F &f, int64_t ub, int64_t *cnts, void *scratch, cudaStream_t st) {
+    const int64_t nb = (ub + kListTile - 1) / kListTile;
+    list_count<<<(unsigned)nb, kListThreads, 0, st>>>(f, cnts);
+    GF_KERNEL_DONE();
+    if (nb >= kScanTiles) GF_TRY(exclusive_scan_i64(cnts, cnts, nb, scratch, st));
+    list_write<<<(unsigned)nb, kListThreads, 0, st>>>(f, cnts, nb >= kScanTiles ? 1 : 0);
+    GF_KERNEL_DONE();
+    return GF_OK;
+}
+
+// The distinct (shifted) keys, each run's first index, and the run of every
+// element; the number of runs to *runs, and beg[runs] = the number of elements.
+struct RunList {
+    const uint64_t *keys;
+    const int64_t *d_n;
+    int64_t n;
+    int shift;
+    uint64_t *ukeys;
+    int32_t *beg, *run_of;
+    int64_t *runs;
+    __device__ int64_t size() const { return dev_count(d_n, n); }
+    __device__ int count(int64_t i) const { return i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift) ? 1 : 0; }
+    __device__ void put(int64_t i, int c, int64_t at) const {
+        if (c) {
+            ukeys[at] = keys[i] >> shift;
+            if (beg) beg[at] = (int32_t)i;
+        }
+        if (run_of) run_of[i] = (int32_t)(at + c - 1);
+    }
+    __device__ void total(int64_t t) const {
+        *runs = t;
+        if (beg) beg[t] = (int32_t)size();
+    }
+};
 
 // Every ancestor level of the leaves in one block: for l = L-1 down to 1 the
 // occupied boxes of level l are the distinct keys (child key >> 3) of the
@@ -280,24 +358,22 @@ __global__ void __launch_bounds__(kClsBlock) cls_scatter(ClsArgs a) {
     }
 }
 
-__global__ void item_counts(const int32_t *__restrict__ beg, const int64_t *d_nleaf, int64_t ub,
-                            int64_t *__restrict__ cnt) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ub) return;
-    const int64_t n = i < *d_nleaf ? beg[i + 1] - beg[i] : 0;
-    cnt[i] = (n + kItemTargets - 1) / kItemTargets;
-}
-
-// (also: the number of items, off[ub], into *nitems)
-__global__ void item_fill(const int32_t *__restrict__ beg, const int64_t *d_nleaf, int64_t ub,
-                          const int64_t *__restrict__ off, int4 *__restrict__ items, int64_t *__restrict__ nitems) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *nitems = off[ub];
-    if (i >= *d_nleaf) return;
-    const int b0 = beg[i], b1 = beg[i + 1];
-    int64_t o = off[i];
-    for (int f = b0; f < b1; f += kItemTargets) items[o++] = make_int4((int)i, f, min(kItemTargets, b1 - f), 0);
-}
+// Evaluation items: up to kItemTargets observers of a leaf; their number to *nitems.
+struct ItemList {
+    const int32_t *beg;
+    const int64_t *d_nleaf;
+    int4 *items;
+    int64_t *nitems;
+    __device__ int64_t size() const { return *d_nleaf; }
+    __device__ int count(int64_t i) const {
+        return (int)(((unsigned)(beg[i + 1] - beg[i]) + kItemTargets - 1) / kItemTargets);
+    }
+    __device__ void put(int64_t i, int, int64_t at) const {
+        const int b0 = beg[i], b1 = beg[i + 1];
+        for (int f = b0; f < b1; f += kItemTargets) items[at++] = make_int4((int)i, f, min(kItemTargets, b1 - f), 0);
+    }
+    __device__ void total(int64_t t) const { *nitems = t; }
+};
 
 // Interaction list (316 offsets, dz/dy/dx ascending, max-norm >= 2) and near
 // list (27 offsets) of observer boxes, as source box Morton keys or -1.
@@ -602,36 +678,27 @@ gf_status fmm_observer_tree(gf_plan_s *plan, const double *obs, const double oz[
     int64_t *d_cnt;   // [0, L]: boxes per level, [kMaxLevels + 1]: items, then the
                       // evaluation kernel's item queue (2 counters)
     int *d_ccnt;      // [8 (kMaxLevels + 1)]: boxes per parity class and level
-    GF_TRY(A.alloc_n(&d_cnt, kMaxLevels + 4));
-    GF_TRY(A.alloc_n(&d_ccnt, 8 * (kMaxLevels + 1)));
-    GF_CUDA(cudaMemsetAsync(d_cnt, 0, sizeof(int64_t) * (kMaxLevels + 4), st));
+    constexpr int kCounts = kMaxLevels + 4 + 4 * (kMaxLevels + 1);   // both, in 64-bit words
+    GF_TRY(A.alloc_n(&d_cnt, kCounts));
+    d_ccnt = reinterpret_cast<int *>(d_cnt + kMaxLevels + 4);
     F->eval_queue = reinterpret_cast<unsigned long long *>(d_cnt + kMaxLevels + 2);
-    GF_CUDA(cudaMemsetAsync(d_ccnt, 0, sizeof(int) * 8 * (kMaxLevels + 1), st));
+    GF_CUDA(cudaMemsetAsync(d_cnt, 0, sizeof(int64_t) * kCounts, st));
     GF_TRY(A.alloc_n(&leaf.tkey, ub[L]));
     GF_TRY(A.alloc_n(&F->leaf_beg, ub[L] + 1));
     if (M > 0) {
-        mark_new<<<ceil_div(M, 256), 256, 0, st>>>(keys, nullptr, M, M, 0, flags);
-        GF_KERNEL_DONE();
-        GF_TRY(exclusive_scan_i64(flags, flags, M, scratch, st));
-        compact_runs<<<ceil_div(M, 256), 256, 0, st>>>(keys, nullptr, M, M, 0, flags, leaf.tkey, F->leaf_beg,
-                                                      nullptr, d_cnt + L);
-        GF_KERNEL_DONE();
+        const RunList runs{keys, nullptr, M, 0, leaf.tkey, F->leaf_beg, nullptr, d_cnt + L};
+        GF_TRY(write_list(runs, M, flags, scratch, st));
+    } else {
+        GF_CUDA(cudaMemsetAsync(F->leaf_beg, 0, sizeof(int32_t), st));
     }
-    set_last<<<1, 1, 0, st>>>(F->leaf_beg, d_cnt + L, (int32_t)M);
-    GF_KERNEL_DONE();
     const bool anc_small = ub[L] <= kAncMaxLeaves;
     for (int l = L - 1; l >= 1; --l) {
         FmmLevel &ch = F->lev[l + 1], &pa = F->lev[l];
         GF_TRY(A.alloc_n(&ch.tparent, ub[l + 1]));
         GF_TRY(A.alloc_n(&pa.tkey, ub[l]));
         if (M > 0 && !anc_small) {
-            const int64_t u = ub[l + 1];
-            mark_new<<<ceil_div(u, 256), 256, 0, st>>>(ch.tkey, d_cnt + l + 1, 0, u, 3, flags);
-            GF_KERNEL_DONE();
-            GF_TRY(exclusive_scan_i64(flags, flags, u, scratch, st));
-            compact_runs<<<ceil_div(u, 256), 256, 0, st>>>(ch.tkey, d_cnt + l + 1, 0, u, 3, flags, pa.tkey, nullptr,
-                                                          ch.tparent, d_cnt + l);
-            GF_KERNEL_DONE();
+            const RunList runs{ch.tkey, d_cnt + l + 1, 0, 3, pa.tkey, nullptr, ch.tparent, d_cnt + l};
+            GF_TRY(write_list(runs, ub[l + 1], flags, scratch, st));
         }
     }
     if (M > 0 && anc_small && L >= 2) {
@@ -688,20 +755,16 @@ gf_status fmm_observer_tree(gf_plan_s *plan, const double *obs, const double oz[
     const int64_t item_ub = ub[L] + M / kItemTargets + 1;
     GF_TRY(A.alloc_n(&F->items, item_ub));
     if (M > 0) {
-        item_counts<<<ceil_div(ub[L], 256), 256, 0, st>>>(F->leaf_beg, d_cnt + L, ub[L], flags);
-        GF_KERNEL_DONE();
-        GF_TRY(exclusive_scan_i64(flags, flags, ub[L], scratch, st));
-        item_fill<<<ceil_div(ub[L], 256), 256, 0, st>>>(F->leaf_beg, d_cnt + L, ub[L], flags, F->items,
-                                                        d_cnt + kMaxLevels + 1);
-        GF_KERNEL_DONE();
+        const ItemList items{F->leaf_beg, d_cnt + L, F->items, d_cnt + kMaxLevels + 1};
+        GF_TRY(write_list(items, ub[L], flags, scratch, st));
     }
 
     // ---- the one read-back: box counts, items, class counts
-    int64_t hcnt[kMaxLevels + 2];
-    int ccnt[8 * (kMaxLevels + 1)];
+    int64_t hcnt[kCounts];
     GF_CUDA(cudaMemcpyAsync(hcnt, d_cnt, sizeof(hcnt), cudaMemcpyDeviceToHost, st));
-    GF_CUDA(cudaMemcpyAsync(ccnt, d_ccnt, sizeof(ccnt), cudaMemcpyDeviceToHost, st));
     GF_CUDA(cudaStreamSynchronize(st));
+    int ccnt[8 * (kMaxLevels + 1)];
+    memcpy(ccnt, hcnt + kMaxLevels + 4, sizeof(ccnt));
     for (int l = 1; l <= L; ++l) F->lev[l].nt = M > 0 ? hcnt[l] : 0;
     F->n_items = M > 0 ? hcnt[kMaxLevels + 1] : 0;
     for (int l = 2; l <= L; ++l) {
