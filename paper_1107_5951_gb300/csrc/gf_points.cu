@@ -493,12 +493,12 @@ __device__ __forceinline__ void ld_loc(const T *loc, int64_t i, T &x, T &y, T &z
 // Sorted masses in leaf units: m_i = rho_{c(perm_i)} v_i, [B][S].
 template <class T>
 __global__ void point_masses(const void *__restrict__ rho, int rho_f32, const int32_t *__restrict__ perm,
-                             const T *__restrict__ loc, int64_t S, int per_cell, int64_t ncell, int B,
+                             const T *__restrict__ loc, int64_t S, int per_cell, int64_t ncell,
                              T *__restrict__ m, int *__restrict__ status) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= S * B) return;
-    const int b = (int)(e / S);
-    const int64_t i = e - (int64_t)b * S;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= S) return;
+    const int b = (int)blockIdx.y;
+    const int64_t e = (int64_t)b * S + i;
     const int64_t src = (int64_t)b * ncell + perm[i] / per_cell;
     if constexpr (sizeof(T) == 4) {
         if (rho_f32) {   // one rounding of the product, without the FP64 pipe
@@ -1275,9 +1275,9 @@ gf_status points_masses(gf_plan_s *plan, const void *rho, int rho_dtype, int B, 
     FmmPlan *F = plan->fmm;
     const PointSet &P = plan->pts;
     if (P.S == 0) return GF_OK;
-    point_masses<T><<<ceil_div(P.S * B, 256), 256, 0, st>>>(rho, rho_dtype == GF_DTYPE_F32, P.perm,
-                                                           (const T *)P.loc, P.S, P.per_cell, P.ncell, B,
-                                                           (T *)F->mass, plan->d_status);
+    point_masses<T><<<dim3(ceil_div(P.S, 256), (unsigned)B), 256, 0, st>>>(rho, rho_dtype == GF_DTYPE_F32, P.perm,
+                                                                          (const T *)P.loc, P.S, P.per_cell, P.ncell,
+                                                                          (T *)F->mass, plan->d_status);
     GF_KERNEL_DONE();
     return GF_OK;
 }

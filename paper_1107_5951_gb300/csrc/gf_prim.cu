@@ -150,21 +150,24 @@ gf_status scan_rec(const int64_t *in, int64_t *out, int64_t n, int64_t *scratch,
 }
 
 // -------------------------------------------------------------- radix sort
-// Counts of a pass: hist[digit][block] (rows of ld entries, a multiple of 4).
+// Counts of a pass: hist[digit][block] (rows of ld entries, a multiple of 4).  All
+// of a thread's keys are read before the first is counted: 2^25 keys 67 -> 30 us
+// (20 us to read them); four tiles to a block, a quarter of the writes, took 78.
 template <class K, int T, int R>
 __global__ void __launch_bounds__(T)
 radix_hist(const K *__restrict__ keys, int64_t n, int shift, int64_t ld, uint32_t *__restrict__ hist) {
     __shared__ uint32_t cnt[kRadix];
-    if (threadIdx.x < kRadix) cnt[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * (T * R);
+    const int64_t base = (int64_t)blockIdx.x * (T * R) + threadIdx.x;
+    K k[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int64_t i = base + r * T + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 0xff], 1u);
-    }
+    for (int r = 0; r < R; ++r) k[r] = base + r * T < n ? keys[base + r * T] : 0;
+    cnt[threadIdx.x] = 0;
     __syncthreads();
-    if (threadIdx.x < kRadix) hist[(int64_t)threadIdx.x * ld + blockIdx.x] = cnt[threadIdx.x];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (base + r * T < n) atomicAdd(&cnt[(k[r] >> shift) & 0xff], 1u);
+    __syncthreads();
+    hist[(int64_t)threadIdx.x * ld + blockIdx.x] = cnt[threadIdx.x];
 }
 
 // Exclusive scan of each digit's row in place, its total to tot[digit]: one block
@@ -223,7 +226,7 @@ radix_rows(uint32_t *__restrict__ hist, int64_t nb, int64_t ld, uint32_t *__rest
 // the values are the indices.  Bound by the scattered writes (a tile's keys of a
 // digit are a run, 16 on average in the large tiles); ranking a block's row at a
 // time, five block barriers to 256 keys, it was bound by those: 200 us a pass over
-// 2^25 keys, now 150.
+// 2^25 (64-bit) keys, now 124 for 32-bit ones.
 template <class K, int T, int R>
 __global__ void __launch_bounds__(T)
 radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int64_t n, int shift, int64_t ld,
@@ -241,11 +244,7 @@ radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int6
 #pragma unroll
     for (int r = 0; r < R; ++r) k[r] = base + 32 * r < n ? keys[base + 32 * r] : 0;
     // thread d: where digit d's keys of this block begin
-    uint32_t mine = 0, start = 0;
-    if (threadIdx.x < kRadix) {
-        mine = tot[threadIdx.x];
-        start = offs[(int64_t)threadIdx.x * ld + blockIdx.x];
-    }
+    const uint32_t mine = tot[threadIdx.x], start = offs[(int64_t)threadIdx.x * ld + blockIdx.x];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = vals && base + 32 * r < n ? vals[base + 32 * r] : (int32_t)(base + 32 * r);
     for (int d = lane; d < kRadix; d += 32) wcnt[warp][d] = 0;
@@ -267,9 +266,9 @@ radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int6
         const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += t;
     }
-    if (threadIdx.x < kRadix && lane == 31) dsum[warp] = incl;
+    if (lane == 31) dsum[warp] = incl;
     __syncthreads();
-    if (threadIdx.x < kRadix) {   // digit threadIdx.x: its keys of the warps before, from its own start
+    {   // digit threadIdx.x: its keys of the warps before, from its own start
         uint32_t acc = start + incl - mine;
 #pragma unroll
         for (int w = 0; w < kRadix / 32; ++w)
@@ -294,6 +293,7 @@ radix_scatter(const K *__restrict__ keys, const int32_t *__restrict__ vals, int6
 template <class K, int T, int R>
 gf_status radix_pass(const K *keys, const int32_t *vals, int64_t n, int shift, uint32_t *hist, K *keys_out,
                      int32_t *vals_out, cudaStream_t st) {
+    static_assert(T == kRadix, "a thread to a digit");
     const int64_t nb = (n + T * R - 1) / (T * R), ld = (nb + 3) / 4 * 4;
     uint32_t *tot = hist + ld * kRadix;
     radix_hist<K, T, R><<<(unsigned)nb, T, 0, st>>>(keys, n, shift, ld, hist);
