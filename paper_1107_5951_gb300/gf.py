@@ -365,7 +365,7 @@ class Plan:
     observer set (see ``gf_plan_create``).
 
     obs must be a CUDA float64 tensor of shape (M, 3).  m2l="simt" runs the
-    mixed-precision M2L on the SIMT cores; m2l="tensor" runs an FP64 plan's
+    M2L on the SIMT cores in either precision; m2l="tensor" runs an FP64 plan's
     M2L on the tensor cores (FP16 parts, the rest FP64); voxels="closed_form" integrates
     every voxel exactly (SUM-AN; direct mode, FP64) instead of sampling it
     with the rule (xi, w).  flags: further GF_FLAG_* bits (testing aids)."""
