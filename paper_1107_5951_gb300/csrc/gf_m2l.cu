@@ -229,9 +229,10 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
         if (max(ma[0], max(ma[1], ma[2])) < 2) continue;
         __syncthreads();   // the previous magnitude's inputs have been used
         int any = 0;
-        if (tid < 8 * P) {
+        // (a strided loop: the block of a small degree has fewer threads than entries)
+        for (int e = tid; e < 8 * P; e += nthr) {
             // source at (s_x a, s_y b, s_z c), s = - where the bit of o is clear
-            const int c = tid >> 3, o = tid & 7;
+            const int c = e >> 3, o = e & 7;
             int64_t row = -1;
             int s[3];
             bool ok = col0 + c < L.ncol;
@@ -254,12 +255,10 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
                     if (m >= 0) row = ((int64_t)m * a.B + cmember[c]) * a.ldk;
                 }
             }
-            crow[tid] = row;
-            any = row >= 0 ? 1 << o : 0;
+            crow[e] = row;
+            any |= row >= 0;
         }
-        const int sides = tid < 32 * ((8 * P + 31) / 32) ? __reduce_or_sync(0xffffffffu, any) : 0;
-        const int has = __syncthreads_or(sides) ? 1 : 0;
-        if (!has) continue;
+        if (!__syncthreads_or(any)) continue;
         // Q inputs of one column per thread; a mirror pair with one side
         // missing throughout the column needs no additions
         for (int e = tid; e < (((K + 3) & ~3) / Q) * P; e += nthr) {
