@@ -44,24 +44,35 @@ static void keep_pool_memory(int device) {
     done.fetch_or(bit);
 }
 
+gf_status DeviceArena::take_chunk(void **chunk, size_t c) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    keep_pool_memory(dev);
+    cudaError_t e = cudaMallocAsync(chunk, c, stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        set_error("device allocation of %zu bytes failed: %s", c, cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? GF_ERR_OOM : GF_ERR_CUDA;
+    }
+    blocks.push_back(*chunk);
+    bytes += c;
+    return GF_OK;
+}
+
+gf_status DeviceArena::alloc_exact(void **p, size_t n) {
+    *p = nullptr;
+    n = (n + 255) & ~size_t(255);
+    return n <= left ? alloc(p, n) : take_chunk(p, n);
+}
+
 gf_status DeviceArena::alloc(void **p, size_t n) {
     *p = nullptr;
     if (n == 0) n = 16;
     n = (n + 255) & ~size_t(255);
     if (n > left) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        keep_pool_memory(dev);
         const size_t c = std::max(n, next);
         void *chunk = nullptr;
-        cudaError_t e = cudaMallocAsync(&chunk, c, stream);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            set_error("device allocation of %zu bytes failed: %s", c, cudaGetErrorString(e));
-            return e == cudaErrorMemoryAllocation ? GF_ERR_OOM : GF_ERR_CUDA;
-        }
-        blocks.push_back(chunk);
-        bytes += c;
+        GF_TRY(take_chunk(&chunk, c));
         cur = static_cast<unsigned char *>(chunk);
         left = c;
         if (c == next) next = std::min(next * 2, size_t(64) << 20);
@@ -301,20 +312,8 @@ static gf_status finish_create(gf_plan_s *p, gf_status s, cudaStream_t st, gf_pl
     return GF_OK;
 }
 
-}  // namespace gf
-
-using namespace gf;
-
-extern "C" {
-
-int32_t gf_version(void) { return GF_VERSION; }
-
-int64_t gf_launch_count(void) { return (int64_t)g_launches.load(); }
-
-const char *gf_last_error(void) { return get_error(); }
-
-gf_status gf_plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M,
-                        const gf_options *opt, size_t *bytes) {
+gf_status plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M, const gf_options *opt, bool tight,
+                     size_t *bytes) {
     GF_TRY(validate(grid, quad, M, opt));
     if (!bytes) {
         set_error("bytes must be non-NULL");
@@ -326,14 +325,14 @@ gf_status gf_plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M,
         if (opt->precision == GF_PREC_MIXED) b += (size_t)M * 6 * sizeof(float) + 512;
         if (opt->reserved0 & GF_FLAG_SUM_AN) b += sum_an_bytes(grid, opt->max_batch);
     } else {
-        b += fmm_bytes_estimate(grid, quad->nq, M, opt);
+        b += fmm_bytes_estimate(grid, quad->nq, M, opt, tight);
     }
     *bytes = b;
     return GF_OK;
 }
 
-gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad, const double *obs_dev,
-                         int64_t M, const gf_options *opt, void *stream, gf_plan_t *out) {
+gf_status plan_create(const gf_grid *grid, const gf_quad *quad, const double *obs_dev, int64_t M, const gf_options *opt,
+                      bool tight, cudaStream_t st, gf_plan_s **out) {
     if (!out) {
         set_error("plan output pointer is NULL");
         return GF_ERR_INVALID_ARG;
@@ -344,7 +343,6 @@ gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad, const double 
         set_error("obs_dev is NULL with M = %lld", (long long)M);
         return GF_ERR_INVALID_ARG;
     }
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     gf_plan_s *p = new (std::nothrow) gf_plan_s();
     if (!p) {
         set_error("host allocation failed");
@@ -352,6 +350,7 @@ gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad, const double 
     }
     cudaGetDevice(&p->device);
     p->arena.stream = st;
+    p->tight = tight;
     p->grid = *grid;
     p->opt = *opt;
     p->G = opt->G > 0.0 ? opt->G : 6.67428e-11;
@@ -391,6 +390,28 @@ gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad, const double 
             s = fmm_create(p, obs_dev, st);
     }
     return finish_create(p, s, st, out);
+}
+
+}  // namespace gf
+
+using namespace gf;
+
+extern "C" {
+
+int32_t gf_version(void) { return GF_VERSION; }
+
+int64_t gf_launch_count(void) { return (int64_t)g_launches.load(); }
+
+const char *gf_last_error(void) { return get_error(); }
+
+gf_status gf_plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M,
+                        const gf_options *opt, size_t *bytes) {
+    return plan_bytes(grid, quad, M, opt, false, bytes);
+}
+
+gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad, const double *obs_dev,
+                         int64_t M, const gf_options *opt, void *stream, gf_plan_t *out) {
+    return plan_create(grid, quad, obs_dev, M, opt, false, reinterpret_cast<cudaStream_t>(stream), out);
 }
 
 gf_status gf_hex_sources(const double *verts_dev, int64_t ncell, const gf_quad *quad, int32_t precision,

@@ -123,8 +123,8 @@ struct FmmPlan {
     uint32_t *tc_amax = nullptr;
     bool amax_fused = false;      // this forward's expansion writers took the M2L input maxima
     // tensor-core M2L: active offsets of the tiles (forward [0], adjoint [1]);
-    // partial rows of cut tiles, two slots for each of m2l_part_ctas CTAs, and
-    // where each CTA's units start
+    // m2l_part_rows partial rows of cut tiles, and where the units of each of up to
+    // m2l_part_ctas CTAs start
     uint32_t *m2l_mask[2] = {};
     float *m2l_part = nullptr;
     int4 *m2l_cut = nullptr;
@@ -135,6 +135,7 @@ struct FmmPlan {
     double *oz_rscale = nullptr, *oz_part = nullptr;
     void *oz_levels = nullptr;
     int64_t oz_row0[kMaxLevels + 1] = {};
+    int64_t m2l_part_rows = 0;
     int m2l_part_ctas = 0;
     // the M2L inputs of levels 2..L split into scaled FP16 high and low
     // parts: for every input row and 32-wide chunk, 64 bytes of high parts

@@ -67,11 +67,16 @@ struct DeviceArena {
     size_t next = size_t(1) << 20;
     cudaStream_t stream = nullptr;
     gf_status alloc(void **p, size_t n);
+    // a request beyond the open chunk gets memory of its own size, beside the chunk
+    gf_status alloc_exact(void **p, size_t n);
     template <class T>
     gf_status alloc_n(T **p, size_t count) {
         return alloc(reinterpret_cast<void **>(p), count * sizeof(T));
     }
     void release();
+
+  private:
+    gf_status take_chunk(void **chunk, size_t c);
 };
 
 struct FmmPlan;   // defined in gf_fmm.cuh
@@ -110,6 +115,7 @@ struct gf_plan_s {
     float *d_obs_fvox = nullptr;     // [M][3] fractional voxel coordinates (mixed)
     double *d_corner = nullptr;      // closed-form voxels: [max_batch][corners] weights
     gf::FmmPlan *fmm = nullptr;
+    bool tight = false;              // made by plan_create with tight set
     gf::PointSet pts;            // point-source plans only
     int *d_status = nullptr;     // device-side check word
     size_t device_bytes = 0;
@@ -171,7 +177,14 @@ gf_status fmm_info(const gf_plan_s *plan, gf_plan_info *info);
 gf_status fmm_work_counts(gf_plan_s *plan, cudaStream_t st);
 gf_status fmm_export_tree(gf_plan_s *plan, int level, int32_t *perm, uint64_t *keys,
                           uint64_t *box_keys, int64_t *ilist, int64_t *near_);
-size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_options *opt);
+size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_options *opt, bool tight);
+// gf_plan_bytes and gf_plan_create; tight: without the M2L's workspaces that only
+// make it faster (partial rows of cut tiles, split FP64 inputs) beyond what the
+// plan's size has room for anyway.
+gf_status plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M, const gf_options *opt, bool tight,
+                     size_t *bytes);
+gf_status plan_create(const gf_grid *grid, const gf_quad *quad, const double *obs_dev, int64_t M, const gf_options *opt,
+                      bool tight, cudaStream_t st, gf_plan_s **out);
 
 inline unsigned ceil_div(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 

@@ -416,8 +416,9 @@ struct TcArgs {
     const uint32_t *tmask;      // [ntiles][8]: 189 offset bits, [6]: how many
     int stream;                 // units dealt out over the grid (else one tile per CTA)
     int min_units;              // a CTA takes no fewer units than this (stream)
-    float *mpart;               // [2 gridDim][Npad / 4][128] float4: partial rows, slot 0 of CTA c for its
-                                // first tile, slot 1 for its last
+    float *mpart;               // [gridDim][Npad / 4][prow] float4: partial rows of CTA c's first tile, when
+                                // an earlier CTA starts it
+    int prow;                   // rows of a tile that may hold a target, at most
     int4 *mcut;                 // [gridDim + 1] (stream): CTA c's first tile, the units before it and up to its
                                 // end, G; [gridDim].x: T
     int test_stall;             // testing aid: the MMA issuer first waits on a barrier that
@@ -712,9 +713,16 @@ __device__ __forceinline__ void store4(const TcArgs &a, const TcLevel &L, int64_
     }
 }
 
-// Tiles cut between CTAs: the sum of their partial rows in CTA order.  Blocks
-// (c - 1, .) look at the boundary before CTA c and, when it is the first one
-// inside its tile, write the tile's rows, the columns split over blockIdx.y.
+__device__ __forceinline__ float4 read4(const TcArgs &a, const TcLevel &L, int64_t row, int col) {
+    if (!a.le_f64) return *reinterpret_cast<const float4 *>(L.le + row * a.ldk + col);
+    const double2 *d = reinterpret_cast<const double2 *>(reinterpret_cast<const double *>(L.le) + row * a.ldk + col);
+    return make_float4((float)d[0].x, (float)d[0].y, (float)d[1].x, (float)d[1].y);   // FP32 values
+}
+
+// Tiles cut between CTAs: the first CTA's sums, in the output rows, plus the other
+// CTAs' partial rows in CTA order.  Blocks (c - 1, .) look at the boundary before
+// CTA c and, when it is the first one inside its tile, finish the tile's rows, the
+// columns split over blockIdx.y.
 // A chain of dependent loads with little behind it: one wave of blocks.
 __global__ void __launch_bounds__(512) m2l_join(const __grid_constant__ TcArgs a) {
     const int c = (int)blockIdx.x + 1;
@@ -730,14 +738,13 @@ __global__ void __launch_bounds__(512) m2l_join(const __grid_constant__ TcArgs a
     const TcTile tile = tile_of(a, cut.x);
     const int64_t row = out_row(a, tile, 128 / a.B, r);
     if (row < 0) return;
-    const int first = (uint32_t)((uint64_t)cf * T / G) < p0 ? 1 : 0;
-    const size_t slot = (size_t)(a.Npad / 4) * 128;
+    const size_t slot = (size_t)(a.Npad / 4) * a.prow;
     const float4 *p = reinterpret_cast<const float4 *>(a.mpart) + r;
     for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < a.Npad / 4; q += 4 * (int)gridDim.y) {
-        float4 s = __ldg(p + (2 * cf + first) * slot + (size_t)q * 128);
+        float4 s = read4(a, *tile.L, row, 4 * q);
 #pragma unroll 8
         for (int e = cf + 1; e <= cl; ++e) {
-            const float4 v = __ldg(p + 2 * e * slot + (size_t)q * 128);
+            const float4 v = __ldg(p + e * slot + (size_t)q * a.prow);
             s.x += v.x;
             s.y += v.y;
             s.z += v.z;
@@ -1117,14 +1124,15 @@ m2l_tc(const __grid_constant__ TcArgs a) {
                         acc[q + 3] = acc[q + 3] * c4.w * sig_inv;
                     }
             }
-            if (a.stream && n < (int)(pref[t + 1] - pref[t])) {
-                // a cut tile: partial rows, summed by m2l_join
+            if (a.stream && pref[t] < u0) {
+                // the rest of an earlier CTA's tile: partial rows, added by m2l_join
                 const int q4 = nsum / 4;
                 float4 *mine = reinterpret_cast<float4 *>(a.mpart) +
-                               ((size_t)(2 * blockIdx.x + (pref[t] > u0 ? 1 : 0)) * (Npad / 4) + ph_half * q4) * 128 + r;
+                               ((size_t)blockIdx.x * (Npad / 4) + ph_half * q4) * a.prow + r;
 #pragma unroll
                 for (int q = 0; q < NS; q += 4)
-                    if (q < nsum) mine[(q / 4) * 128] = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
+                    if (q < nsum && r < a.prow)
+                        mine[(q / 4) * a.prow] = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
                 continue;
             }
             const int64_t row = out_row(a, tile, nbox, r);
@@ -1189,7 +1197,7 @@ struct OzArgs {
     int nb, bb;                 // batch members of the rows, and the one this launch does (t.B = 1)
     const unsigned char *img;   // [343][ngrp][nck][kSl][ng rows of 32 bytes, swizzled]
     const double *cinv;         // [ngrp ng] inverse column scales
-    double *part;               // [2 gridDim][ng][128] partial rows
+    double *part;               // [gridDim][ng][t.prow] partial rows
 };
 
 // Byte offset of 16-byte half h of row r in a slice (8-row atoms of 256 bytes).
@@ -1558,12 +1566,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) m2l_oz(const __grid_constant__ 
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const int col0 = (t % ngrp) * NG + half * nh;
-            if (a.stream && n < (int)(pref[t + 1] - pref[t])) {
-                // a cut tile: partial rows, summed by m2l_oz_join
-                double *mine = o.part + ((size_t)(2 * blockIdx.x + (pref[t] > u0 ? 1 : 0)) * NG + half * nh) * 128 + r;
+            if (a.stream && pref[t] < u0) {
+                // the rest of an earlier CTA's tile: partial rows, added by m2l_oz_join
+                double *mine = o.part + ((size_t)blockIdx.x * NG + half * nh) * a.prow + r;
 #pragma unroll
                 for (int q = 0; q < NH; ++q)
-                    if (q < nh) mine[q * 128] = acc[q];
+                    if (q < nh && r < a.prow) mine[q * a.prow] = acc[q];
                 continue;
             }
             const TcTile tile = tile_of(a, t / ngrp);
@@ -1583,7 +1591,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) m2l_oz(const __grid_constant__ 
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols));
 }
 
-// The cut (tile, group)s' partial rows, summed in CTA order (see m2l_join).
+// The cut (tile, group)s' partial rows, added in CTA order (see m2l_join; the
+// column scales are powers of two, so it does not matter when they are applied).
 __global__ void __launch_bounds__(512) m2l_oz_join(const __grid_constant__ OzArgs o) {
     const TcArgs &a = o.t;
     const int c = (int)blockIdx.x + 1;
@@ -1598,16 +1607,16 @@ __global__ void __launch_bounds__(512) m2l_oz_join(const __grid_constant__ OzArg
     const TcTile tile = tile_of(a, cut.x / o.ngrp);
     const int64_t row = out_row(a, tile, 128, r);
     if (row < 0) return;
-    const int first = (uint32_t)((uint64_t)cf * T / G) < p0 ? 1 : 0;
     const int col0 = (cut.x % o.ngrp) * o.ng;
     double *dst = reinterpret_cast<double *>(tile.L->le) + (row * o.nb + o.bb) * a.ldk + col0;
     const double *p = o.part + r;
-    const size_t slot = (size_t)o.ng * 128;
+    const size_t slot = (size_t)o.ng * a.prow;
     for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < o.ng && col0 + q < a.K; q += 4 * (int)gridDim.y) {
-        double s = __ldg(p + (2 * cf + first) * slot + (size_t)q * 128);
+        const double scale = __ldg(o.cinv + col0 + q);
+        double s = dst[q];
 #pragma unroll 8
-        for (int e = cf + 1; e <= cl; ++e) s += __ldg(p + 2 * e * slot + (size_t)q * 128);
-        dst[q] = s * __ldg(o.cinv + col0 + q);
+        for (int e = cf + 1; e <= cl; ++e) s = fma(__ldg(p + e * slot + (size_t)q * a.prow), scale, s);
+        dst[q] = s;
     }
 }
 
@@ -1757,33 +1766,76 @@ static int64_t tc_tiles(const FmmPlan *F, bool adj, int B, int *tile_begin) {
     return tiles;
 }
 
-// CTAs of a launch that deals out units: one per SM, and no more than could
-// have kMinUnits each.
+// Rows of a tile that may hold a target, at most, for batches of B.
+static int tc_tile_rows(const FmmPlan *F, bool adj, int B) {
+    const int64_t nbox = 128 / B;
+    int64_t most = 1;
+    for (int l = 2; l <= F->L; ++l)
+        for (int c = 0; c < 8; ++c) {
+            const int64_t *off = adj ? F->scls_off[l] : F->lev[l].cls_off;
+            if (adj || F->lev[l].nt > 0) most = std::max(most, std::min(nbox, off[c + 1] - off[c]));
+        }
+    return (int)(most * B);
+}
+
+// CTAs of a launch that deals out units: one per SM, no more than could have
+// kMinUnits each, and no more than the partial rows held serve; 0: whole tiles
+// (too many of them, or rows for fewer CTAs than tiles).
 constexpr int kMinUnits = 6;
-static int64_t tc_stream_ctas(int64_t tiles) {
-    return std::max<int64_t>(1, std::min<int64_t>(sm_count(), tiles * 189 / kMinUnits));
+static int64_t tc_stream_ctas(int64_t tiles, int64_t rows, int prow) {
+    if (tiles > kStreamTiles) return 0;
+    const int64_t c = std::max<int64_t>(1, std::min<int64_t>(sm_count(), tiles * 189 / kMinUnits));
+    return std::min(c, rows / prow) >= std::min<int64_t>(tiles, sm_count()) ? std::min(c, rows / prow) : 0;
 }
 
 size_t m2l_tc_bytes(int p, bool fp64) {
     const int npad = ((p + 1) * (p + 1) + 15) & ~15;
-    const size_t cuts = (size_t)(sm_count() + 1) * sizeof(int4) + 65536;
-    if (fp64) return (size_t)2 * sm_count() * 128 * kOzCols * sizeof(double) + cuts;
-    return npad > 256 ? 0 : (size_t)2 * sm_count() * 128 * npad * sizeof(float) + cuts;
+    const size_t cuts = (size_t)(sm_count() + 1) * sizeof(int4) + 4096;
+    if (fp64) return (size_t)sm_count() * 128 * kOzCols * sizeof(double) + cuts;
+    return npad > 256 ? 0 : (size_t)sm_count() * 128 * npad * sizeof(float) + cuts;
 }
 
-// Masks of the tiles and the partial rows of cut tiles, for the plan's largest batch (smaller batches have no more tiles); the
-// forward's partial rows serve the adjoint too when they suffice.
+// Bytes that the plan can still allocate within the size it was announced with
+// (gf_plan_bytes): what is left of the open chunk, or a chunk of its own
+// (alloc_exact).  Point plans, and FP64 plans with the M2L on FP16 parts, have no
+// announced size.
+static size_t announced_room(const gf_plan_s *plan) {
+    if (plan->fmm->points || plan->fmm->m2l_tc64) return SIZE_MAX;
+    const DeviceArena &A = plan->arena;
+    const size_t all = fmm_bytes_estimate(&plan->grid, plan->quad.nq, plan->M, &plan->opt, plan->tight);
+    return all > A.bytes ? std::max(A.left, all - A.bytes) : A.left;
+}
+
+// Masks of the tiles and the partial rows of cut tiles, for every batch up to the
+// plan's largest (which has the most tiles).  Only rows that hold targets are kept:
+// a 32^3 grid under a plane of stations has 16 to a tile, 1.7 MB for 152 CTAs, where
+// two whole tiles to a CTA took 27 MB.  The forward's rows serve the adjoint too when
+// they suffice.  A plan without room for them takes whole tiles.
 static gf_status m2l_tc_workspaces(gf_plan_s *plan, bool adj) {
     FmmPlan *F = plan->fmm;
     if (F->B > 128) return GF_OK;
     const int64_t tiles = tc_tiles(F, adj, F->B, nullptr);
     if (tiles == 0) return GF_OK;
     GF_TRY(plan->arena.alloc((void **)&F->m2l_mask[adj], (size_t)tiles * 8 * sizeof(uint32_t)));
-    if (tiles > kStreamTiles) return GF_OK;
-    const int64_t ctas = tc_stream_ctas(tiles);
-    if (ctas <= F->m2l_part_ctas) return GF_OK;
-    GF_TRY(plan->arena.alloc((void **)&F->m2l_cut, (size_t)(ctas + 1) * sizeof(int4)));
-    GF_TRY(plan->arena.alloc((void **)&F->m2l_part, (size_t)ctas * 2 * 128 * F->tab->tc_npad * sizeof(float)));
+    int64_t rows = 0, ctas = 0;
+    for (int B = 1; B <= F->B; ++B) {
+        const int64_t c = tc_stream_ctas(tc_tiles(F, adj, B, nullptr), INT64_MAX, 1);
+        rows = std::max(rows, c * tc_tile_rows(F, adj, B));
+        ctas = std::max(ctas, c);
+    }
+    const size_t row = F->tab->tc_npad * sizeof(float), cut = (size_t)(sm_count() + 1) * sizeof(int4) + 512;
+    if (plan->tight) {
+        const size_t room = adj ? 0 : announced_room(plan);
+        rows = room > cut ? std::min<int64_t>(rows, (int64_t)std::min<size_t>((room - cut) / row, INT64_MAX)) : 0;
+    }
+    if (rows == 0 || (rows <= F->m2l_part_rows && ctas <= F->m2l_part_ctas)) return GF_OK;
+    rows = std::max(rows, F->m2l_part_rows);
+    ctas = std::max<int64_t>(ctas, F->m2l_part_ctas);
+    unsigned char *mem = nullptr;
+    if (plan->arena.alloc_exact((void **)&mem, rows * row + cut) != GF_OK) return GF_OK;
+    F->m2l_part = (float *)mem;
+    F->m2l_cut = (int4 *)(mem + ((rows * row + 255) & ~(size_t)255));
+    F->m2l_part_rows = rows;
     F->m2l_part_ctas = (int)ctas;
     return GF_OK;
 }
@@ -2037,8 +2089,9 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
     a.mcut = F->m2l_cut;
     a.mpart = F->m2l_part;
     a.min_units = kMinUnits;
-    const int64_t ctas = tc_stream_ctas(a.ntiles);
-    a.stream = a.ntiles <= kStreamTiles && ctas <= F->m2l_part_ctas;
+    a.prow = tc_tile_rows(F, adj, B);
+    const int64_t ctas = std::min<int64_t>(F->m2l_part_ctas, tc_stream_ctas(a.ntiles, F->m2l_part_rows, a.prow));
+    a.stream = ctas > 0;
     // the largest |input| of every level, for the FP16 input scales
     {
         AmaxArgs m;
@@ -2247,19 +2300,26 @@ gf_status m2l_oz_prepare(gf_plan_s *plan) {
     const double fold_us = 0.8e-4 * K * K * (double)((cols + sms * P - 1) / (sms * P) * (sms * P));
     if (oz_us > 0.85 * fold_us) return GF_OK;
     const int64_t ctas = std::min<int64_t>(sm_count(), tiles * ngrp * 189);
-    const bool stream = tiles * ngrp <= kOzStreamTiles;
     const size_t row_bytes = (size_t)nck * kOzRowChunk;
-    const size_t need = (size_t)rows * (row_bytes + sizeof(double)) + (size_t)tiles * 8 * sizeof(uint32_t) +
-                        (F->L + 1) * sizeof(TcLevel) +
-                        (stream ? (size_t)ctas * 2 * ng * 128 * sizeof(double) + (size_t)(ctas + 1) * sizeof(int4) : 0) + 4096;
-    const size_t grows = need + 4096 > plan->arena.left ? std::max(need + 4096, plan->arena.next) : 0;
-    if (!F->points && plan->arena.bytes + grows > fmm_bytes_estimate(&plan->grid, plan->quad.nq, plan->M, &plan->opt))
+    const size_t part_bytes = (size_t)ctas * ng * tc_tile_rows(F, false, 1) * sizeof(double);
+    const size_t inputs = (size_t)rows * (row_bytes + sizeof(double)) + (size_t)tiles * 8 * sizeof(uint32_t) +
+                          (F->L + 1) * sizeof(TcLevel) + (size_t)(ctas + 1) * sizeof(int4) + 4096;
+    const size_t room = announced_room(plan);
+    if (inputs > room) return GF_OK;
+    const bool stream = tiles * ngrp <= kOzStreamTiles && inputs + part_bytes <= room;
+    // whole tiles in place of few dealt-out ones: the longest lists, rounds of blocks
+    if (!stream && tiles * ngrp <= kOzStreamTiles &&
+        F->B * ((tiles * ngrp + sms - 1) / sms * 189.0 + 2.0) * (1.2 * nck + 8.0) > 0.85 * fold_us)
         return GF_OK;
+    const size_t need = inputs + (stream ? part_bytes : 0);
     const OzTables *z = nullptr;
     GF_TRY(oz_tables(F->tab, plan->arena.stream, &z));
     if (!z) return GF_OK;
     unsigned char *mem = nullptr;
-    if (plan->arena.alloc((void **)&mem, need) != GF_OK) {   // no room: the SIMT M2L serves the plan
+    // a whole chunk where the announced size has room for it (it is then found again among the freed
+    // chunks of the plan before)
+    const bool whole = plan->arena.next >= need && room >= plan->arena.next;
+    if ((whole ? plan->arena.alloc((void **)&mem, need) : plan->arena.alloc_exact((void **)&mem, need)) != GF_OK) {
         cudaGetLastError();
         return GF_OK;
     }
@@ -2271,7 +2331,7 @@ gf_status m2l_oz_prepare(gf_plan_s *plan) {
     F->oz_split = take((size_t)rows * row_bytes);
     F->oz_rscale = (double *)take((size_t)rows * sizeof(double));
     F->m2l_mask[0] = (uint32_t *)take((size_t)tiles * 8 * sizeof(uint32_t));
-    F->oz_part = stream ? (double *)take((size_t)ctas * 2 * ng * 128 * sizeof(double)) : nullptr;
+    F->oz_part = stream ? (double *)take(part_bytes) : nullptr;
     F->m2l_cut = stream ? (int4 *)take((size_t)(ctas + 1) * sizeof(int4)) : nullptr;
     std::vector<TcLevel> h(F->L + 1);
     memset(h.data(), 0, h.size() * sizeof(TcLevel));
@@ -2319,6 +2379,7 @@ static gf_status m2l_run_oz(gf_plan_s *plan, int B, cudaStream_t st, cudaEvent_t
     a.ntiles = (int)tc_tiles(F, false, 1, a.tile_begin);
     a.tmask = F->m2l_mask[0];
     a.mcut = F->m2l_cut;
+    a.prow = tc_tile_rows(F, false, 1);
     a.min_units = 1;
     o.nb = B;
     o.ngrp = oz_groups(F->K);

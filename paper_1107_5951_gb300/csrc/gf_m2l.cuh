@@ -41,8 +41,8 @@ gf_status p2m_leaf_run(gf_plan_s *plan, int B, int64_t first, int64_t count, cud
 template <class T>
 gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaStream_t st);
 
-// Upper bound of the tensor-core M2L's own workspaces (beside the expansions
-// and their split parts; fp64: of the digit M2L).
+// Upper bound of the partial rows of the tensor-core M2L's cut tiles (fp64: of the
+// digit M2L's).
 size_t m2l_tc_bytes(int p, bool fp64);
 // Plan-time set-up of the tensor-core path (level descriptors on the device).
 gf_status m2l_tc_prepare(gf_plan_s *plan);

@@ -49,6 +49,7 @@ struct Ticket {
     gf_request req{};
     std::vector<double> xi, w, obs;   // copies of the request's host geometry
     size_t need = 0;                  // device bytes of a plan for it
+    bool tight = false;               // the plan goes without the M2L's spare workspaces
     Clock::time_point t_submit, t_done;
     bool done = false;
     gf_status status = GF_OK;
@@ -159,7 +160,7 @@ gf_status build_entry(gf_server_s *s, Ticket *t, cudaStream_t st, Entry **out) {
         delete e;
         return ce == cudaErrorMemoryAllocation ? GF_ERR_OOM : GF_ERR_CUDA;
     }
-    gf_status rc = gf_plan_create(&r.grid, &r.quad, obs_dev, r.M, &o, st, &e->plan);
+    gf_status rc = plan_create(&r.grid, &r.quad, obs_dev, r.M, &o, t->tight, st, &e->plan);
     cudaFreeAsync(obs_dev, st);
     if (rc != GF_OK) {
         cudaStreamSynchronize(st);
@@ -396,11 +397,16 @@ gf_status gf_server_submit(gf_server_t s, const gf_request *req, int64_t *ticket
     // gf_plan_bytes also validates the grid, the rule and M before anything
     // is copied
     const gf_options o = plan_options(s->opt);
-    size_t b = 0;
-    const gf_status rc = gf_plan_bytes(&req->grid, &req->quad, req->M, &o, &b);
-    if (rc != GF_OK) return rc;
-    const int64_t nvox = req->grid.n[0] * req->grid.n[1] * req->grid.n[2];
-    const size_t need = b + dtype_size(req->rho_dtype) * nvox + 4 * sizeof(double) * req->M;
+    size_t need = 0;
+    bool tight = false;
+    for (int t = 0; t < 2; ++t) {   // a request too large for the budget may fit it without the M2L's spare workspaces
+        tight = t == 1;
+        const gf_status rc = plan_bytes(&req->grid, &req->quad, req->M, &o, tight, &need);
+        if (rc != GF_OK) return rc;
+        const int64_t nvox = req->grid.n[0] * req->grid.n[1] * req->grid.n[2];
+        need += dtype_size(req->rho_dtype) * nvox + 4 * sizeof(double) * req->M;
+        if (need <= s->opt.mem_budget) break;
+    }
     if (need > s->opt.mem_budget) {
         set_error("request needs %zu device bytes, more than the server's budget of %zu", need,
                   s->opt.mem_budget);
@@ -426,6 +432,7 @@ gf_status gf_server_submit(gf_server_t s, const gf_request *req, int64_t *ticket
     t->req.obs_host = t->obs.data();
     t->srv = s;
     t->need = need;
+    t->tight = tight;
     t->t_submit = Clock::now();
     {
         std::lock_guard<std::mutex> lk(s->mu);

@@ -467,7 +467,7 @@ void il_offsets_host(int cls, signed char out[189][3]) {
             }
 }
 
-size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_options *opt) {
+size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_options *opt, bool tight) {
     const int b = opt->leaf_vox > 0 ? opt->leaf_vox : default_leaf_vox(nq);
     const int K = (opt->p + 1) * (opt->p + 1);
     const size_t rs = opt->precision == GF_PREC_MIXED ? 4 : 8;
@@ -479,7 +479,8 @@ size_t fmm_bytes_estimate(const gf_grid *grid, int nq, int64_t M, const gf_optio
     bytes += nleaf * b * b * b * rs * opt->max_batch;          // blocked densities
     if (opt->precision == GF_PREC_MIXED)                         // M2L inputs split into FP16 parts
         bytes += nsrc * ((K + 31) / 32 * 32) * 4.0 * opt->max_batch;
-    bytes += (double)m2l_tc_bytes(opt->p, opt->precision != GF_PREC_MIXED && !(opt->reserved0 & GF_FLAG_M2L_TENSOR));
+    if (!tight)
+        bytes += (double)m2l_tc_bytes(opt->p, opt->precision != GF_PREC_MIXED && !(opt->reserved0 & GF_FLAG_M2L_TENSOR));
     bytes += (double)M * (8 + 4 + 4 + 12 + 24) + ntgt * 24;       // keys, perm, locals, box tables
     bytes += (double)M * 32 + 8e6;                                // sort buffers and scratch
     return (size_t)bytes;
