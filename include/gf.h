@@ -160,7 +160,10 @@ gf_status gf_plan_create(const gf_grid *grid, const gf_quad *quad,
  *   gz_dev    : [B][M] FP64 vertical component, or NULL (not both NULL
  *               unless M = 0)
  * Enqueues on `stream` and returns; allocates nothing, so it may be captured
- * in a CUDA graph.  Direct mode sums every pair (Sec. 2.1); FMM mode runs
+ * in a CUDA graph.  Direct mode sums every pair (Sec. 2.1), the sources of a tile
+ * of observers shared by a number of blocks that depends on M: the last bits
+ * of a sum are the same for every batch size, but not for every set of
+ * observers.  FMM mode runs
  * P2M, M2M, M2L, L2L, L2P and the near-field P2P (Sec. 2.3, Fig. 3) and adds
  * near and far parts (Eq. 10).  The plan's workspaces (expansions, the M2L's
  * split inputs) serve all its calls: calls on one plan whose device work

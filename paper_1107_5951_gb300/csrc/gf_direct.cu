@@ -388,11 +388,11 @@ gf_status launch_fwd_f64(const double *obs, int64_t M, const void *rho, int rho_
     const RowSplit rs = row_split(ga.nx);
     const int64_t units = (int64_t)rs.nch * nq * ga.ny * ga.nz;
     if (M <= 32) {
-        const int c = pair_cluster(B, units);
+        const int c = pair_cluster(1, units);
         return pair_launch(direct_fwd_f64<1>, 1, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
     }
     const int64_t tiles = (M + 63) / 64;
-    const int c = pair_cluster(tiles * B, units);
+    const int c = pair_cluster(tiles, units);
     return pair_launch(direct_fwd_f64<2>, tiles, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
 }
 
@@ -401,7 +401,7 @@ gf_status launch_fwd_mixed(const float *oi, const float *of, int64_t M, const vo
                            int *status, cudaStream_t st) {
     const RowSplit rs = row_split(ga.nx);
     const int64_t tiles = (M + 63) / 64;
-    const int c = pair_cluster(tiles * B, (int64_t)rs.nch * nq * ga.ny * ga.nz);
+    const int c = pair_cluster(tiles, (int64_t)rs.nch * nq * ga.ny * ga.nz);
     return pair_launch(direct_fwd_mixed, tiles, B, c, st, oi, of, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
 }
 

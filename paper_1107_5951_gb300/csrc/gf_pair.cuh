@@ -109,7 +109,9 @@ constexpr size_t pair_smem() {
 // Blocks per cluster for `tiles` observer tiles and `units` work units per
 // tile: the size that leaves the smallest share of the SMs idle in the last
 // round of blocks (the smaller size when it is within 2% of the best), with
-// at least two units for each warp of the cluster.
+// at least two units for each warp of the cluster.  The size decides how an
+// observer's sum associates: callers count the tiles of one batch member, so that a
+// member's sums are the same bits alone and in any batch.
 inline int pair_cluster(int64_t tiles, int64_t units) {
     const int64_t sms = sm_count();
     const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kPairMaxCluster, units / (2 * kPairWarps)));

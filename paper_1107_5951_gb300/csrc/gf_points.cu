@@ -1118,7 +1118,7 @@ gf_status points_direct_forward(gf_plan_s *plan, const void *rho, int rho_dtype,
     if (M == 0) return GF_OK;
     const int f32 = rho_dtype == GF_DTYPE_F32;
     const int64_t tiles = (M + 63) / 64;
-    const int cl = pair_cluster(tiles * B, (P.S + 31) / 32);
+    const int cl = pair_cluster(tiles, (P.S + 31) / 32);
     if (plan->opt.precision == GF_PREC_FP64 || P.S == 0)
         return pair_launch(direct_points_f64, tiles, B, cl, st, plan->d_obs, M, P.x, P.a, P.S, P.per_cell, P.ncell, rho,
                            f32, plan->G, g, gz, plan->d_status);

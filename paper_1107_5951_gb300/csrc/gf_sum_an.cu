@@ -239,7 +239,7 @@ gf_status sum_an_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B,
     GF_KERNEL_DONE();
     if (plan->M == 0) return GF_OK;
     const int64_t tiles = (plan->M + 31) / 32;
-    return pair_launch(an_forward, tiles, B, pair_cluster(tiles * B, (ga.nc + kAnPiece - 1) / kAnPiece), st, plan->d_obs, plan->M,
+    return pair_launch(an_forward, tiles, B, pair_cluster(tiles, (ga.nc + kAnPiece - 1) / kAnPiece), st, plan->d_obs, plan->M,
                        plan->d_corner, ga, plan->G, g, gz);
 }
 
