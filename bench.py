@@ -312,20 +312,24 @@ def fmm_roofline(stages, info, args, peaks, workload, nvox=None, rho_bytes=4, n_
     fbytes = 4 if args.precision == "mixed" else 8
     L = int(getattr(info, "L", 0))
     work = {"eval": ("alu", FLOPS_PER_PAIR * float(info.near_pairs),
-                     "eval_kernel (near field) + eval_far_kernel (L2P, near + far, scatter)"),
+                     "near field (eval_kernel; FP64 lattices near_f64_kernel, closed form near_an_kernel) + "
+                     "L2P, near + far, scatter (eval_far_kernel; FP64 far_f64_kernel)"),
             "m2l": ("tensor" if tensor else "alu", 2.0 * K * K * float(info.m2l_pairs),
                     "m2l_tc (tcgen05 FP16 parts, 3 products, all levels)" if tensor
                     else "m2l_oz (BF16 digits) or m2l_fold (all levels)")}
     if nvox is not None and L >= 2:
         ns = {l: level_boxes(info, l) for l in range(2, L + 1)}
-        # 4^3-voxel leaves with L - 1 > 2: the P2M stage makes level L-1
-        # straight from the densities (its essential traffic: the densities
-        # once, those expansions once) and the M2M stage starts from level L-1
-        up = L - 1 > 2
+        # 4^3-voxel leaves (under a rule that is its own mirror image, as every
+        # rule here) with L - 1 > 2: the P2M stage makes level L-1 straight from
+        # the densities (its essential traffic: the densities once, those
+        # expansions once) and the M2M stage starts from level L-1; other leaves
+        # all get expansions
+        fold = int(getattr(info, "leaf_vox", 4)) == 4
+        up = fold and L - 1 > 2
         top = L - 1 if up else L
         work["p2m"] = ("hbm", float(nvox * rho_bytes + ns[top] * K * fbytes),
                        "block_rows + p2m_leaf_fold + p2m_up_quad (into level L-1 from the grid)" if up
-                       else "block_rows + p2m_leaf_fold")
+                       else "block_rows + p2m_leaf_fold" if fold else "p2m_fused")
         work["m2m"] = ("hbm", float(sum(ns[l] * K * fbytes for l in range(3, top + 1))
                                     + sum(ns[l] * K * fbytes for l in range(2, top))),
                        "fold_quad + fold_kernel (FP64 into level 2)")
