@@ -442,7 +442,7 @@ struct NearTArgs {
     const void *tloc;
     const double *r;
     int64_t M;
-    int B, nq, guard_all;
+    int B, nq;
     const int32_t *imap;       // level L window map
     int32_t mlo[3], mn[3];
     int32_t blo[3], bn[3];     // leaf source block

@@ -1840,45 +1840,48 @@ static gf_status m2l_tc_workspaces(gf_plan_s *plan, bool adj) {
     return GF_OK;
 }
 
+// The level table of the forward (or its transpose) on the device.
+static gf_status m2l_tc_levels(gf_plan_s *plan, bool adj) {
+    FmmPlan *F = plan->fmm;
+    std::vector<TcLevel> h(F->L + 1);
+    memset(h.data(), 0, h.size() * sizeof(TcLevel));
+    for (int l = 2; l <= F->L; ++l) {
+        const FmmLevel &lv = F->lev[l];
+        TcLevel &t = h[l];
+        t.le = (float *)(adj ? lv.me : lv.le);
+        t.order = lv.m2l_order;
+        t.tkey = lv.tkey;
+        t.adj = adj;
+        t.imap = F->imap[l];
+        for (int d = 0; d < 3; ++d) {
+            t.blo[d] = lv.slo[d];
+            t.bn[d] = lv.sn[d];
+            t.mlo[d] = F->mlo[l][d];
+            t.mn[d] = F->mn[l][d];
+        }
+        if (adj) {   // output: the z-slabs an interaction list reaches
+            t.blo[2] += lv.m2l_z0;
+            t.bn[2] = std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
+            t.slab0 = lv.m2l_z0 * lv.sn[0] * lv.sn[1];
+        }
+        for (int c = 0; c <= 8; ++c) t.cls_off[c] = adj ? F->scls_off[l][c] : lv.cls_off[c];
+        t.amax = F->tc_amax + (adj ? kMaxLevels + 1 : 0) + l;
+        t.split = (adj ? F->tc_split_adj : F->tc_split) + split_offset(F, adj, l);
+        t.shift = l - 2;
+    }
+    std::vector<unsigned char> &hb = adj ? F->tc_levels_adj_host : F->tc_levels_host;
+    void *&dev = adj ? F->tc_levels_adj : F->tc_levels;
+    hb.assign(reinterpret_cast<unsigned char *>(h.data()), reinterpret_cast<unsigned char *>(h.data() + h.size()));
+    GF_TRY(plan->arena.alloc(&dev, hb.size()));
+    return upload_small(dev, hb.data(), hb.size(), plan->arena.stream);
+}
+
 gf_status m2l_tc_prepare_adj(gf_plan_s *plan) {
     FmmPlan *F = plan->fmm;
     if (!F->mixed || !F->tab->m2l_tc) return GF_OK;
     GF_TRY(plan->arena.alloc((void **)&F->tc_split_adj, std::max<size_t>(16, split_offset(F, 1, F->L + 1))));
     GF_TRY(m2l_tc_workspaces(plan, true));
-    for (int adj = 1; adj < 2; ++adj) {
-        std::vector<TcLevel> h(F->L + 1);
-        memset(h.data(), 0, h.size() * sizeof(TcLevel));
-        for (int l = 2; l <= F->L; ++l) {
-            const FmmLevel &lv = F->lev[l];
-            TcLevel &t = h[l];
-            t.le = (float *)(adj ? lv.me : lv.le);
-            t.order = lv.m2l_order;
-            t.tkey = lv.tkey;
-            t.adj = adj;
-            t.imap = F->imap[l];
-            for (int d = 0; d < 3; ++d) {
-                t.blo[d] = lv.slo[d];
-                t.bn[d] = lv.sn[d];
-                t.mlo[d] = F->mlo[l][d];
-                t.mn[d] = F->mn[l][d];
-            }
-            if (adj) {   // output: the z-slabs an interaction list reaches
-                t.blo[2] += lv.m2l_z0;
-                t.bn[2] = std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
-                t.slab0 = lv.m2l_z0 * lv.sn[0] * lv.sn[1];
-            }
-            for (int c = 0; c <= 8; ++c) t.cls_off[c] = adj ? F->scls_off[l][c] : lv.cls_off[c];
-            t.amax = F->tc_amax + (adj ? kMaxLevels + 1 : 0) + l;
-            t.split = (adj ? F->tc_split_adj : F->tc_split) + split_offset(F, adj, l);
-            t.shift = l - 2;
-        }
-        std::vector<unsigned char> &hb = adj ? F->tc_levels_adj_host : F->tc_levels_host;
-        void *&dev = adj ? F->tc_levels_adj : F->tc_levels;
-        hb.assign(reinterpret_cast<unsigned char *>(h.data()), reinterpret_cast<unsigned char *>(h.data() + h.size()));
-        GF_TRY(plan->arena.alloc(&dev, hb.size()));
-        GF_TRY(upload_small(dev, hb.data(), hb.size(), plan->arena.stream));
-    }
-    return GF_OK;
+    return m2l_tc_levels(plan, true);
 }
 
 gf_status m2l_tc_prepare(gf_plan_s *plan) {
@@ -1887,40 +1890,7 @@ gf_status m2l_tc_prepare(gf_plan_s *plan) {
     GF_TRY(plan->arena.alloc((void **)&F->tc_amax, 2 * (kMaxLevels + 1) * sizeof(uint32_t)));
     GF_TRY(plan->arena.alloc((void **)&F->tc_split, std::max<size_t>(16, split_offset(F, 0, F->L + 1))));
     GF_TRY(m2l_tc_workspaces(plan, false));
-    for (int adj = 0; adj < 1; ++adj) {
-        std::vector<TcLevel> h(F->L + 1);
-        memset(h.data(), 0, h.size() * sizeof(TcLevel));
-        for (int l = 2; l <= F->L; ++l) {
-            const FmmLevel &lv = F->lev[l];
-            TcLevel &t = h[l];
-            t.le = (float *)(adj ? lv.me : lv.le);
-            t.order = lv.m2l_order;
-            t.tkey = lv.tkey;
-            t.adj = adj;
-            t.imap = F->imap[l];
-            for (int d = 0; d < 3; ++d) {
-                t.blo[d] = lv.slo[d];
-                t.bn[d] = lv.sn[d];
-                t.mlo[d] = F->mlo[l][d];
-                t.mn[d] = F->mn[l][d];
-            }
-            if (adj) {   // output: the z-slabs an interaction list reaches
-                t.blo[2] += lv.m2l_z0;
-                t.bn[2] = std::max<int64_t>(0, lv.m2l_z1 - lv.m2l_z0 + 1);
-                t.slab0 = lv.m2l_z0 * lv.sn[0] * lv.sn[1];
-            }
-            for (int c = 0; c <= 8; ++c) t.cls_off[c] = adj ? F->scls_off[l][c] : lv.cls_off[c];
-            t.amax = F->tc_amax + (adj ? kMaxLevels + 1 : 0) + l;
-            t.split = (adj ? F->tc_split_adj : F->tc_split) + split_offset(F, adj, l);
-            t.shift = l - 2;
-        }
-        std::vector<unsigned char> &hb = adj ? F->tc_levels_adj_host : F->tc_levels_host;
-        void *&dev = adj ? F->tc_levels_adj : F->tc_levels;
-        hb.assign(reinterpret_cast<unsigned char *>(h.data()), reinterpret_cast<unsigned char *>(h.data() + h.size()));
-        GF_TRY(plan->arena.alloc(&dev, hb.size()));
-        GF_TRY(upload_small(dev, hb.data(), hb.size(), plan->arena.stream));
-    }
-    return GF_OK;
+    return m2l_tc_levels(plan, false);
 }
 
 namespace {

@@ -135,13 +135,9 @@ gf_status scan_rec(const int64_t *in, int64_t *out, int64_t n, int64_t *scratch,
     int64_t *offs = scratch + nb;       // [nb + 1]
     scan_tiles<<<(unsigned)nb, kScanThreads, 0, st>>>(in, out, n, sums);
     GF_KERNEL_DONE();
-    if (nb > 1) {
-        GF_TRY(scan_rec(sums, offs, nb, scratch + 2 * nb + 1, st, false));
-        add_tile_offsets<<<ceil_div(n, 256), 256, 0, st>>>(out, n, offs);
-        GF_KERNEL_DONE();
-    } else {
-        GF_CUDA(cudaMemsetAsync(offs, 0, sizeof(int64_t), st));
-    }
+    GF_TRY(scan_rec(sums, offs, nb, scratch + 2 * nb + 1, st, false));
+    add_tile_offsets<<<ceil_div(n, 256), 256, 0, st>>>(out, n, offs);
+    GF_KERNEL_DONE();
     if (write_tot) {
         write_total<<<1, 1, 0, st>>>(out, n, offs, sums, nb);
         GF_KERNEL_DONE();
