@@ -2,7 +2,8 @@
 20 MB in mixed precision (the M2L's partial rows take what the targets need, not
 whole tiles for every SM), and a server whose budget holds such a request's
 expansions, buffers and scratch (20 MB; FP64 25 MB) takes it, with the same field
-to rounding."""
+to rounding; so does one whose budget is some MB short of a small grid's with
+observers throughout, which then deals its M2L out to fewer blocks, or not at all."""
 import numpy as np
 import pytest
 
@@ -36,4 +37,19 @@ def test_small_request_fits(precision, p, dtype, budget, bar):
         srv.register(1, *geo, obs)
         _, g, _ = srv.wait(srv.submit(1, rho, want_g=True))
         assert srv.stats()["resident_bytes"] <= budget
+    assert rel_l2(g, want) <= bar
+
+
+@pytest.mark.parametrize("short", [1e6, 6e6, 9e6])
+@pytest.mark.parametrize("precision,p,dtype,bar", [("mixed", 12, np.float32, 2e-6), ("fp64", 10, np.float64, 1e-13)])
+def test_short_budget(precision, p, dtype, bar, short):
+    wk = wl.random_small(750, n=(44, 40, 41), n_obs=6000, h=(1.0, 1.0, 1.0), origin=(-3.0, 2.0, -30.0), obs_pad=1.0)
+    geo = (wk.grid.n, wk.grid.origin, wk.grid.h, wk.xi, wk.w)
+    rho = wk.rho.astype(dtype)
+    with pkg.Plan(*geo, torch.tensor(wk.obs, device=DEV), mode="fmm", precision=precision, p=p) as plan:
+        want = plan.forward(torch.tensor(rho, device=DEV))[0].cpu().numpy()
+    need = pkg.plan_bytes(*geo, len(wk.obs), mode="fmm", precision=precision, p=p) + rho.nbytes + 32 * len(wk.obs)
+    with pkg.Server(slots=1, precision=precision, p=p, mem_budget=int(need - short)) as srv:
+        srv.register(1, *geo, wk.obs)
+        _, g, _ = srv.wait(srv.submit(1, rho, want_g=True))
     assert rel_l2(g, want) <= bar
