@@ -76,8 +76,9 @@ typedef struct {
 enum { GF_MODE_DIRECT = 0, GF_MODE_FMM = 1 };
 /* GF_PREC_FP64: every stage in FP64 (the forward M2L on the FP64 units or, where
  * that is faster and the plan's announced size has room for its inputs, on the
- * tensor cores from seven base-256 digits per value with exact sums: the error
- * of FP64 additions).  GF_PREC_MIXED: FP32 near field with
+ * tensor cores from seven base-256 digits per value, relative to the largest of
+ * its row, with sums that are exact where they count: the error of FP64 additions
+ * of the largest terms).  GF_PREC_MIXED: FP32 near field with
  * compensated accumulation; tensor-core M2L on FP16 high/low parts of
  * power-of-two-scaled operands (three products, FP32 accumulation) and
  * P2M/M2M/L2L in FP32 folded by mirror symmetry; FP64 for the top-level
@@ -311,10 +312,11 @@ gf_status gf_plan_set_source_part(gf_plan_t plan, int32_t part, int32_t nparts, 
  *               sits at reference coordinates (2i - 1, 2j - 1, 2k - 1)
  *   quad      : nq nodes in [-1, 1]^3 and positive weights (host)
  *   precision : GF_PREC_FP64: every step in FP64.  GF_PREC_MIXED (for
- *               mixed-precision plans): the corners as 64-bit fixed point,
- *               the image relative to the cell's first corner and the
- *               Jacobian in FP32 -- positions within about 1e-6 of the
- *               cell's extent, weights within about 1e-6 relative.
+ *               mixed-precision plans): the corners' FP64 differences to the
+ *               cell's first corner rounded to FP32, the image relative to
+ *               that corner and the Jacobian in FP32 -- positions within
+ *               about 1e-6 of the cell's extent, weights within about 1e-6
+ *               relative.
  *   x_dev     : [ncell * nq][3] FP64 output, the trilinear image of node q
  *               of cell c at source s = c * nq + q
  *   a_dev     : [ncell * nq] FP64 output, the volume weight
@@ -343,7 +345,8 @@ gf_status gf_hex_sources(const double *verts_dev, int64_t ncell, const gf_quad *
  *             apply (GF_ERR_UNSUPPORTED for the flag)
  * Direct mode sums every pair (FP64 with compensated sums, or mixed:
  * positions split into an exact integer number of quanta of 2^-22 of the
- * joint extent plus an FP32 fraction, FP32 pair terms, FP64 tile sums).
+ * joint extent plus an FP32 fraction, FP32 pair terms, compensated FP32 sums
+ * of each warp's share, FP64 beyond).
  * FMM mode builds a uniform octree whose leaf side makes about 48 sources
  * per leaf of the sources' extent; the sources are sorted by leaf, their
  * multipole expansions come from the points themselves, and the near field
@@ -367,8 +370,11 @@ gf_status gf_plan_check(gf_plan_t plan, void *stream);
 /* One-line message describing the calling thread's last failure. */
 const char *gf_last_error(void);
 
-/* Device bytes a plan with these inputs would hold (upper bound), without
- * allocating; used for admission by memory footprint. */
+/* Device bytes a plan with these inputs would hold (upper bound, but for what
+ * its allocation in chunks rounds up), without allocating; used for admission by
+ * memory footprint.  Not counted: what all plans of a device and degree share for
+ * the life of the process -- the operator tables, and for FP64 plans whose M2L
+ * runs on the tensor cores the operators' digits (295 MB at p = 14, 467 MB at 16). */
 gf_status gf_plan_bytes(const gf_grid *grid, const gf_quad *quad, int64_t M,
                         const gf_options *opt, size_t *bytes);
 

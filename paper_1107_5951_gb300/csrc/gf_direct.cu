@@ -130,7 +130,7 @@ __device__ __forceinline__ const void *rho_of(const void *rho, int f32, int64_t 
 
 // Bound by the FP64 pipe: 11 instructions a pair and about 20 a piece of
 // R x 16 pairs.  16^3 voxels, 2x2x2 rule, 4096 stations (134 M pairs):
-// 41.6 -> 4.07 ms (16 blocks of 256 threads before; 3.0 ms at two FP64
+// 41.6 -> 4.07 ms (16 blocks of 256 threads before; 2.5 ms at two FP64
 // instructions a clock and SM).
 template <int R>
 __global__ void __launch_bounds__(kPairThreads)

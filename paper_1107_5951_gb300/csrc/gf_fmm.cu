@@ -995,7 +995,7 @@ eval_kernel(EvalArgs a) {
 // leaf, which the warp holding the item before it covers.
 // Bound by the FP32 pipe.  With the real recursion of l2p_sum2 (nine operations a
 // term; the complex one took twelve) 2.1 M observers in 128^3 283 -> 227 us,
-// 464 x 464 x 16 with 512 x 512 stations 130 -> 101 us.
+// 1024 x 1024 stations over 464^3 130 -> 101 us.
 constexpr int kFarWarps = 4;
 constexpr int kFarTargets = 128;
 static_assert(kFarTargets == 2 * kTPL * 32, "two evaluation items per far item");
@@ -1095,7 +1095,7 @@ __global__ void __launch_bounds__(kFarWarps * 32, 5) eval_far_kernel(EvalArgs a,
 }
 
 // Near field in FP64 of rules whose sources form a 4^3 lattice per leaf: the sums
-// of eval_kernel's mode 1.  The FP64 pipe takes two instructions a clock and SM,
+// that eval_kernel makes.  The FP64 pipe takes two instructions a clock and SM,
 // so their number is what counts: with the lattice sums of the FP32 form (|d|^2
 // from the squared plane distances, rows added up before they are weighted) and
 // inv_r3's seven, 10.3 per pair of observer and source against 23.  A block takes
@@ -1325,8 +1325,8 @@ __global__ void __launch_bounds__(kFar64Warps * 32) far_f64_kernel(EvalArgs a) {
 constexpr int kAnNb = 12;                          // voxels per axis of the 27-leaf block of closed-form voxels
 constexpr int kAnBlock = kAnNb * kAnNb * kAnNb;
 
-// Near field of closed-form voxels (SUM-AN in the FMM) in FP32: the sums of
-// eval_kernel's mode 1, the far field following as for quadrature voxels.  One
+// Near field of closed-form voxels (SUM-AN in the FMM) in FP32: the sums that
+// eval_kernel makes, the far field following as for quadrature voxels.  One
 // warp per half work item, an observer per lane; the densities of the item's 27
 // neighbour leaves (a 12^3 voxel block, 4^3-voxel leaves) are staged in the
 // warp's shared-memory slice.  The sums are those of an_near_block with radius 2:
@@ -1345,8 +1345,8 @@ constexpr int kAnBlock = kAnNb * kAnNb * kAnNb;
 // divisions in one kernel, took 1,690 us for 512 x 512 stations over 128^3 voxels;
 // now 600 us and 40 us of far field.
 //
-// Quotients and roots from the approximate reciprocals, refined by their
-// residual (in the last place); operands are normal numbers here.
+// Quotients and roots from the approximate reciprocals, refined by one Newton
+// step on the residual (in the last place); operands are normal numbers here.
 __device__ __forceinline__ float an_quot(float n, float d) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
@@ -1360,8 +1360,8 @@ __device__ __forceinline__ float an_root(float x) {
 
 // atan(n / d), d != 0, as the angle of the smaller to the larger of |n| and |d|:
 // one division for both ranges.  On [0, 1] t + t s q(s), s = t^2, q of degree 8
-// fitted to the smallest largest relative error (2.4e-9; evaluated, 1.2 units in
-// the last place).
+// fitted to the smallest largest relative error (1.1e-8 in this form; evaluated in
+// FP32, 1.2 units in the last place).
 __device__ __forceinline__ float an_angle(float n, float d) {
     const float an = fabsf(n), ad = fabsf(d);
     const float t = an_quot(fminf(an, ad), fmaxf(an, ad)), s = t * t;

@@ -1,8 +1,10 @@
 // gf_m2l.cu -- M2L over the interaction list, as a batched dense contraction:
-// on the tensor cores in mixed precision (tiles of 128 columns of one parity
-// class, offset by offset), on the SIMT cores otherwise (columns folded by
-// mirror symmetry).  Sources outside the source block contribute zeros.  Each
-// output is written once, so the result is deterministic.
+// on the tensor cores (tiles of 128 columns of one parity class, offset by
+// offset) from FP16 parts in mixed precision and from BF16 digits in FP64, or on
+// the SIMT cores (columns folded by mirror symmetry): small FP64 plans, the FP64
+// transpose, and where a plan asks for it.  Sources outside the source block
+// contribute zeros.  Every sum is made in an order that the plan fixes, so the
+// result is deterministic.
 #include <cuda_fp16.h>
 #include <string.h>
 
@@ -376,8 +378,8 @@ m2l_fold(const __grid_constant__ FoldM2LArgs a) {
 // refill (wake-up, 16 copies a thread, L2) takes longer than another stage's MMAs.
 // One pipeline took 5,800 cycles an offset; two, each hiding the other's, 5,000.
 // Measured against one CTA, or two, per tile and producers that waited for their
-// copies: 16 tiles' worth of a 32^3 grid 260 -> 33 us + 6 us to join; 156 tiles of
-// 464 x 464 x 16 (K = 121) 327 -> 127 + 14; 16 grids of 128^3 846 -> 397; a 2^25-point
+// copies: the 8 tiles of a 32^3 grid under a plane of stations 260 -> 33 us + 6 us to
+// join; the 156 of a 464^3 grid (K = 121) 327 -> 127 + 14; 16 grids of 128^3 846 -> 397; a 2^25-point
 // set 1,050 -> 522; 128^3 with observers throughout 1,236 -> 1,011.  (A gather by TMA
 // of the rows took 20 cycles a row, three times as long in all.)
 // Every wait is bounded and watches an abort
@@ -1158,12 +1160,16 @@ m2l_tc(const __grid_constant__ TcArgs a) {
 // own, and both are written as kSl = 7 digits in base 256, -128..128, exact in
 // BF16 (56 bits); powers of two per input component, taken from the operators,
 // balance the orders first.  Digit products of equal weight, i + j = d <= 6, add
-// up in one FP32 accumulator, d of them for up to 304 inputs of at most 2^14:
-// below 2^24 for d <= 3, so exact, and beyond it only where the weight is 2^-32 and
-// less of the first digits'.  (The splitting into exactly multipliable slices is
-// Ozaki, Ogita, Oishi and Rump's, 2012.)  What is left out, d >= 7, and the last
-// place of the digits are some 2^-54 of a row's largest term, as much as FP64
-// rounds away in one of its additions.
+// up in one FP32 accumulator: d + 1 products of at most 2^14 for each of up to 289
+// inputs.  That is at most 2^24, so exact whatever the digits, for d <= 3 up to
+// p = 15 and for d <= 2 at p = 16.  A later sum passes 2^24 only if nearly all its
+// products agree in sign and are of the largest size (of random digits it is
+// some 2^18), and then loses units of its own weight, 2^-24 (p = 16, d = 3) or
+// 2^-32 and less of the first digits'.  (The splitting into exactly multipliable
+// slices is Ozaki, Ogita, Oishi and Rump's, 2012.)  What is left out, d >= 7, and the
+// last place of the digits are some 2^-54 of a row's largest term, as much as FP64
+// rounds away in one of its additions; a component far below its row's largest has
+// fewer than 53 bits.
 //
 // The pipeline is m2l_tc's: tiles of 128 targets, units of one (tile, column
 // group, offset) dealt out over the grid, chunks of 16 inputs in a ring of stages
@@ -1550,8 +1556,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) m2l_oz(const __grid_constant__ 
                             int v[kSl];
 #pragma unroll
                             for (int i = 0; i < kSl; ++i) v[i] = __float2int_rn(__uint_as_float(d[i][c]));
-                            // in units of 256^-5 of the first digits' products; |d_0| <= 304 2^14 and so on:
-                            // below 2^62
+                            // in units of 256^-5 of the first digits' products; |d_0| <= 289 2^14 and so on:
+                            // below 2^63
                             long long x = (long long)(v[0] * 256 + v[1]) * 65536 + (long long)v[2] * 256 + v[3];
                             x = x * 65536 + (long long)v[4] * 256 + v[5] + v[6] / 256;
                             acc[c0 + c] = fma(i64_to_f64(x), sc, acc[c0 + c]);

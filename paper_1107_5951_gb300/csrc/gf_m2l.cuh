@@ -11,7 +11,8 @@ gf_status m2l_prepare_tables(Tables *T, cudaStream_t st);
 // LE_l[t] = sum over the interaction list of box t of T_o * ME_l[t + o],
 // for every observer box t of every level (overwrites each LE_l).  Mixed
 // precision runs on the tensor cores (tcgen05, FP16 parts) unless the plan asks
-// for the SIMT kernel; FP64 runs on the SIMT kernel.
+// for the SIMT kernel; FP64 forwards run on the tensor cores from BF16 digits
+// where m2l_oz_prepare chose so, the rest of FP64 on the SIMT kernel.
 // adj: the transpose, MEdual_l[s] = sum_{o in IL(class of s)} T_{-o}^T LEdual_l[s + o]
 // over every source box s (observer boxes found through the level's map).
 // fork: when non-null, recorded on st right before the M2L kernels are
