@@ -1104,6 +1104,8 @@ __global__ void __launch_bounds__(kFarWarps * 32, 5) eval_far_kernel(EvalArgs a,
 // items are enough to keep many SMs busy (a warp per item left 16 of 152 busy for
 // 0.8 ms under 64 x 64 stations).  65,536 observers over 128^3: 3,000 -> 1,715 us.
 constexpr int kNear64Warps = 8;
+// static shared memory: lattice planes, weights, voxels; masses and sums of each warp
+constexpr size_t kNear64Static = 12 * 8 + 64 * 8 + 64 * 4 + kNear64Warps * (64 * 8 + 96 * 16);
 
 __global__ void __launch_bounds__(kNear64Warps * 32) near_f64_kernel(EvalArgs a) {
     __shared__ double lat[3][4];                          // lattice planes from the leaf's centre (voxel units)
@@ -1923,15 +1925,32 @@ int eval_setup(gf_plan_s *plan, int B, double *g, double *gz, EvalArgs &a) {
     return lattice_of(plan->quad, F->b, a);
 }
 
+// Dynamic shared memory, at least shm, with which no more blocks of a launch fit one
+// SM than an even spread over the SMs puts there (`stat`: the kernel's static part).
+// The near field of a small model is a few dozen blocks that start as the M2L on
+// the tensor cores leaves the SMs, and the first SMs to come free took as many as
+// fitted while the others stood idle: 64^3 voxels under 128^2 stations, 2x2x2 rule in 4^3-voxel leaves,
+// 798 us where the same launches in line took 441; closed form 394 against 272; FP64
+// 38.1 ms against 12.4; now 387, 213 us and 12.3 ms.  (Beside an M2L on the SIMT cores
+// nothing is in the way, and an FP64 near field on every SM slows it.)
+size_t spread_smem(bool spread, unsigned blocks, size_t shm, size_t stat) {
+    if (!spread) return shm;
+    constexpr size_t kSM = 228 * 1024, kBlock = 1024;   // an SM's; what a block takes beside its own
+    const size_t per = (blocks + (unsigned)sm_count() - 1) / (unsigned)sm_count();
+    const size_t want = (kSM / (per + 1) + 128) & ~(size_t)127;
+    return std::max(shm, want > kBlock + stat ? want - kBlock - stat : 0);
+}
+
 // One evaluation kernel (mode 1: near field, 2: far field).  FP64 rules of a 4^3
 // lattice per leaf and closed-form voxels have near fields of their own; the
 // queued kernels run on the blocks that fit the device at once.
 template <class T>
 gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_t st) {
     const FmmPlan *F = plan->fmm;
-    const size_t shm = kSrcTable * (sizeof(Vec4<T>) + sizeof(int)) +
-                       sizeof(T) * kEvalWarps * eval_slice((int)sizeof(T));
+    const bool spread = mode == 1 && m2l_fills_sms(plan, a.B);
     const unsigned grid = (unsigned)std::min<int64_t>((F->n_items + kEvalWarps - 1) / kEvalWarps, 152 * 64);
+    const size_t shm = spread_smem(spread, grid, kSrcTable * (sizeof(Vec4<T>) + sizeof(int)) +
+                                             sizeof(T) * kEvalWarps * eval_slice((int)sizeof(T)), 0);
     if (sizeof(T) == 4 && mode == 2) {
         const size_t fshm = sizeof(float) * kFarWarps * far_slice(F->p * F->p);
         GF_TRY((ensure_smem(eval_far_kernel, fshm)));
@@ -1943,11 +1962,14 @@ gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_
         const unsigned fg = (unsigned)std::min<int64_t>((2 * F->n_items + kFar64Warps - 1) / kFar64Warps, 152 * 64);
         far_f64_kernel<<<fg, kFar64Warps * 32, fshm, st>>>(a);
     } else if (sizeof(T) == 8 && n1 == 4) {
-        near_f64_kernel<<<(unsigned)std::min<int64_t>(2 * F->n_items, 152 * 64), kNear64Warps * 32, 0, st>>>(a);
+        const unsigned ng = (unsigned)std::min<int64_t>(2 * F->n_items, 152 * 64);
+        const size_t nshm = spread_smem(spread, ng, 0, kNear64Static);
+        GF_TRY((ensure_smem(near_f64_kernel, nshm)));
+        near_f64_kernel<<<ng, kNear64Warps * 32, nshm, st>>>(a);
     } else if (sizeof(T) == 4 && (plan->opt.reserved0 & GF_FLAG_SUM_AN)) {
-        const size_t ashm = sizeof(float) * kAnWarps * near_an_slice();
-        GF_TRY((ensure_smem(near_an_kernel, ashm)));
         const unsigned ag = (unsigned)std::min<int64_t>((2 * F->n_items + kAnWarps - 1) / kAnWarps, 152 * 64);
+        const size_t ashm = spread_smem(spread, ag, sizeof(float) * kAnWarps * near_an_slice(), 0);
+        GF_TRY((ensure_smem(near_an_kernel, ashm)));
         near_an_kernel<<<std::min<unsigned>(ag, resident_blocks(near_an_kernel, kAnWarps * 32, ashm)), kAnWarps * 32, ashm,
                          st>>>(a);
     } else if (sizeof(T) == 4 && n1 == 4) {

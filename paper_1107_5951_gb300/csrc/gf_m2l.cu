@@ -2403,13 +2403,19 @@ static gf_status m2l_run_oz(gf_plan_s *plan, int B, cudaStream_t st, cudaEvent_t
     return GF_OK;
 }
 
+// Whether the M2L runs from FP16 parts on the tensor cores.
+static bool m2l_on_f16(const gf_plan_s *plan, int B, bool adj) {
+    const FmmPlan *F = plan->fmm;
+    return (F->mixed || (F->m2l_tc64 && !adj)) && F->tab->m2l_tc && (adj ? F->tc_levels_adj : F->tc_levels) &&
+           !(plan->opt.reserved0 & GF_FLAG_M2L_SIMT) && B <= 128 && tc_stages(F->tab->tc_npad) >= 2;
+}
+
+bool m2l_fills_sms(const gf_plan_s *plan, int B) { return m2l_on_f16(plan, B, false) || plan->fmm->oz; }
+
 template <class T>
 gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t fork) {
     FmmPlan *F = plan->fmm;
-    const bool tc = (sizeof(T) == 4 || (F->m2l_tc64 && !adj)) && F->tab->m2l_tc && (adj ? F->tc_levels_adj : F->tc_levels) &&
-                    !(plan->opt.reserved0 & GF_FLAG_M2L_SIMT) && B <= 128 &&
-                    tc_stages(F->tab->tc_npad) >= 2;
-    if (tc) return m2l_run_tc(plan, B, adj, st, fork);
+    if (m2l_on_f16(plan, B, adj)) return m2l_run_tc(plan, B, adj, st, fork);
     if (sizeof(T) == 8 && !adj && F->oz) return m2l_run_oz(plan, B, st, fork);
     if (!adj) stage_mark(plan, 4, st);   // no input split on this path
     if (fork) GF_CUDA(cudaEventRecord(fork, st));

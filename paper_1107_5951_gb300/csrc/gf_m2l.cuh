@@ -19,6 +19,9 @@ gf_status m2l_prepare_tables(Tables *T, cudaStream_t st);
 // launched (after the input split).
 template <class T>
 gf_status m2l_run(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEvent_t fork = nullptr);
+// Whether a block of the forward M2L leaves no room for others on its SM (tensor
+// cores: its shared memory).
+bool m2l_fills_sms(const gf_plan_s *plan, int B);
 
 // Translations between levels (gf_xlate.cu; Ts = storage, Tc = arithmetic):
 //   kind 0  M2M into `level` from level + 1 (store)
