@@ -1812,6 +1812,15 @@ static size_t announced_room(const gf_plan_s *plan) {
     return all > A.bytes ? std::max(A.left, all - A.bytes) : A.left;
 }
 
+// Scratch of n bytes, `room` at most: of its own size in a small plan, whose chunks
+// would multiply what it holds; from a chunk in a plan of 64 MB or more, because a
+// piece of another size splits a chunk that the pool holds for the next plan
+// (creating one took 200 us longer).
+static gf_status take_scratch(gf_plan_s *plan, void **p, size_t n, size_t room) {
+    DeviceArena &A = plan->arena;
+    return A.next >= ((size_t)32 << 20) && A.next >= n && room >= A.next ? A.alloc(p, n) : A.alloc_exact(p, n);
+}
+
 // Masks of the tiles and the partial rows of cut tiles, for every batch up to the
 // plan's largest (which has the most tiles).  Only rows that hold targets are kept:
 // a 32^3 grid under a plane of stations has 16 to a tile, 1.7 MB for 152 CTAs, where
@@ -1830,15 +1839,16 @@ static gf_status m2l_tc_workspaces(gf_plan_s *plan, bool adj) {
         ctas = std::max(ctas, c);
     }
     const size_t row = F->tab->tc_npad * sizeof(float), cut = (size_t)(sm_count() + 1) * sizeof(int4) + 512;
+    size_t room = SIZE_MAX;
     if (plan->tight) {
-        const size_t room = adj ? 0 : announced_room(plan);
+        room = adj ? 0 : announced_room(plan);
         rows = room > cut ? std::min<int64_t>(rows, (int64_t)std::min<size_t>((room - cut) / row, INT64_MAX)) : 0;
     }
     if (rows == 0 || (rows <= F->m2l_part_rows && ctas <= F->m2l_part_ctas)) return GF_OK;
     rows = std::max(rows, F->m2l_part_rows);
     ctas = std::max<int64_t>(ctas, F->m2l_part_ctas);
     unsigned char *mem = nullptr;
-    if (plan->arena.alloc_exact((void **)&mem, rows * row + cut) != GF_OK) return GF_OK;
+    if (take_scratch(plan, (void **)&mem, rows * row + cut, room) != GF_OK) return GF_OK;
     F->m2l_part = (float *)mem;
     F->m2l_cut = (int4 *)(mem + ((rows * row + 255) & ~(size_t)255));
     F->m2l_part_rows = rows;
@@ -2292,10 +2302,7 @@ gf_status m2l_oz_prepare(gf_plan_s *plan) {
     GF_TRY(oz_tables(F->tab, plan->arena.stream, &z));
     if (!z) return GF_OK;
     unsigned char *mem = nullptr;
-    // a whole chunk where the announced size has room for it (it is then found again among the freed
-    // chunks of the plan before)
-    const bool whole = plan->arena.next >= need && room >= plan->arena.next;
-    if ((whole ? plan->arena.alloc((void **)&mem, need) : plan->arena.alloc_exact((void **)&mem, need)) != GF_OK) {
+    if (take_scratch(plan, (void **)&mem, need, room) != GF_OK) {   // no room: the SIMT M2L serves the plan
         cudaGetLastError();
         return GF_OK;
     }
