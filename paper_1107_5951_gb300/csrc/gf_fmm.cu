@@ -136,6 +136,30 @@ __global__ void compose_p2m_up(const double *__restrict__ P, const double *__res
     }
 }
 
+// Shift of an expansion by a rule's nodes, for a leaf (block 0) and its parent
+// (block 1): S[c][k] = sum_q wn_q T_q[c][k], T_q the M2M by node q's offset from the
+// voxel's centre without the M2M's change of scale (2^-degree of the input).
+__global__ void build_shift(int p, int K, int b, const QuadRule *__restrict__ qr, LogFact lf, double *__restrict__ sd,
+                            float *__restrict__ sf) {
+    extern __shared__ double sh[];
+    const double unit = 0.5 / ((double)b * (blockIdx.x + 1));
+    const int nt = (p + 1) * (p + 2) / 2;
+    double *re = sh, *im = sh + nt;
+    double *out = sd + (size_t)blockIdx.x * K * K;
+    for (int e = threadIdx.x; e < K * K; e += blockDim.x) out[e] = 0.0;
+    for (int q = 0; q < qr->nq; ++q) {
+        __syncthreads();
+        if (threadIdx.x == 0)
+            regular_harmonics<double>(p, unit * qr->xi[q][0], unit * qr->xi[q][1], unit * qr->xi[q][2], re, im);
+        __syncthreads();
+        for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
+            const int c = e / K;
+            out[e] += qr->wn[q] * ldexp(op_entry(OP_M2M, p, e - c * K, c, re, im, lf.v), (int)sqrt(c + 0.5));
+        }
+    }
+    for (int e = threadIdx.x; e < K * K; e += blockDim.x) sf[(size_t)blockIdx.x * K * K + e] = (float)out[e];
+}
+
 // The P2M matrices of position 7 transposed for the adjoint, rows in class
 // order: ut[c][v] = Q[v][perm_c], lt[c][v] = P[octant voxel v][perm_c] (zeros for
 // perm_c = -1).  One block per row.
@@ -1741,6 +1765,11 @@ struct P2MEntry {
     float *uf = nullptr, *uq = nullptr;   // FP32 copy, and in quad order
     double *utd = nullptr, *ltd = nullptr;   // transposes in class order [K][64], [K][8]
     float *utf = nullptr, *ltf = nullptr;
+    // rules that do not mirror: the shift by their nodes (leaf, parent) in FP64 and
+    // FP32, in quad order, and the matrices of the voxel centres
+    double *sd = nullptr;
+    float *sf = nullptr, *sq[2] = {};
+    P2MEntry *centre = nullptr;
 };
 std::mutex g_p2m_mu;
 std::vector<P2MEntry *> g_p2m;
@@ -1748,35 +1777,53 @@ std::vector<P2MEntry *> g_p2m;
 static void use_p2m(FmmPlan *F, const P2MEntry *e) {
     F->p2m_d = e->pd;
     F->p2m_f = e->pf;
-    F->p2m_up_d = e->ud;
-    F->p2m_up_f = e->uf;
-    F->p2m_up_q = e->uq;
     F->p2m_upt_d = e->utd;
     F->p2m_upt_f = e->utf;
     F->p2m_leaft_d = e->ltd;
     F->p2m_leaft_f = e->ltf;
+    // the split inputs hold the centres' expansions until the M2L's input split
+    const bool shift = e->centre && F->mixed && F->tab->m2l_tc;
+    for (int i = 0; i < 2; ++i) {
+        F->shift_f[i] = shift ? e->sf + (size_t)i * F->K * F->K : nullptr;
+        F->shift_q[i] = shift ? e->sq[i] : nullptr;
+    }
+    if (shift) {
+        e = e->centre;
+        F->p2m_c_f = e->pf;
+    }
+    F->p2m_up_d = e->ud;
+    F->p2m_up_f = e->uf;
+    F->p2m_up_q = e->uq;
 }
 
-gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
-    FmmPlan *F = plan->fmm;
-    const QuadRule &q = plan->quad;
-    std::lock_guard<std::mutex> lk(g_p2m_mu);
-    const int exact = (plan->opt.reserved0 & GF_FLAG_SUM_AN) ? 1 : 0;
+// The cached matrices of a rule, made when they are not there (qr: the rule on the
+// device; null: the voxel's centre).  Called with g_p2m_mu held.
+static gf_status find_p2m(const FmmPlan *F, int device, const QuadRule &q, const QuadRule *qr, int exact, cudaStream_t st,
+                          P2MEntry **out) {
     for (P2MEntry *e : g_p2m)
-        if (e->device == plan->device && e->p == F->p && e->b == F->b && e->nq == q.nq && e->exact == exact &&
+        if (e->device == device && e->p == F->p && e->b == F->b && e->nq == q.nq && e->exact == exact &&
             !memcmp(e->xi, q.xi, sizeof(double) * 3 * q.nq) && !memcmp(e->wn, q.wn, sizeof(double) * q.nq)) {
-            use_p2m(F, e);
+            *out = e;
             return GF_OK;
         }
+    const int b3 = F->b * F->b * F->b, K = F->K, KP = F->tab->cls_off[8];
+    P2MEntry *centre = nullptr;
+    if (F->b == 4 && !exact && !rule_mirrors(q)) {
+        QuadRule c;
+        memset(&c, 0, sizeof(c));
+        c.nq = 1;
+        c.wn[0] = 1.0;
+        GF_TRY(find_p2m(F, device, c, nullptr, 0, st, &centre));
+    }
     P2MEntry *e = new P2MEntry();
-    e->device = plan->device;
+    e->device = device;
     e->p = F->p;
     e->b = F->b;
     e->nq = q.nq;
     e->exact = exact;
+    e->centre = centre;
     memcpy(e->xi, q.xi, sizeof(double) * 3 * q.nq);
     memcpy(e->wn, q.wn, sizeof(double) * q.nq);
-    const int b3 = F->b * F->b * F->b, K = F->K, KP = F->tab->cls_off[8];
     if (cudaMalloc(&e->pd, sizeof(double) * b3 * K) != cudaSuccess ||
         cudaMalloc(&e->pf, sizeof(float) * b3 * K) != cudaSuccess ||
         (F->b == 4 && (cudaMalloc(&e->ud, sizeof(double) * b3 * K) != cudaSuccess ||
@@ -1784,21 +1831,23 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
                        cudaMalloc(&e->utd, sizeof(double) * b3 * KP) != cudaSuccess ||
                        cudaMalloc(&e->utf, sizeof(float) * b3 * KP) != cudaSuccess ||
                        cudaMalloc(&e->ltd, sizeof(double) * 8 * KP) != cudaSuccess ||
-                       cudaMalloc(&e->ltf, sizeof(float) * 8 * KP) != cudaSuccess))) {
+                       cudaMalloc(&e->ltf, sizeof(float) * 8 * KP) != cudaSuccess)) ||
+        (centre && (cudaMalloc(&e->sd, sizeof(double) * 2 * K * K) != cudaSuccess ||
+                    cudaMalloc(&e->sf, sizeof(float) * 2 * K * K) != cudaSuccess))) {
         cudaGetLastError();
         for (void *m : {(void *)e->pd, (void *)e->pf, (void *)e->ud, (void *)e->uf, (void *)e->utd, (void *)e->utf,
-                        (void *)e->ltd, (void *)e->ltf})
+                        (void *)e->ltd, (void *)e->ltf, (void *)e->sd, (void *)e->sf})
             cudaFree(m);
         delete e;
         set_error("cannot allocate the P2M matrix");
         return GF_ERR_OOM;
     }
     const size_t shm = sizeof(double) * ((F->p + 1) * (F->p + 2) + K);
-    if (exact) {
-        // degree <= p exactly: ceil((p + 1) / 2) nodes per axis
-        build_p2m_exact<<<b3, 128, shm, st>>>(F->p, K, F->b, gauss_legendre((F->p + 2) / 2), e->pd, e->pf);
+    if (exact || !qr) {
+        // exact: degree <= p, ceil((p + 1) / 2) nodes per axis
+        build_p2m_exact<<<b3, 128, shm, st>>>(F->p, K, F->b, gauss_legendre(exact ? (F->p + 2) / 2 : 1), e->pd, e->pf);
     } else {
-        build_p2m<<<b3, 128, shm, st>>>(F->p, K, F->b, quad_device(plan), e->pd, e->pf);
+        build_p2m<<<b3, 128, shm, st>>>(F->p, K, F->b, qr, e->pd, e->pf);
     }
     GF_KERNEL_DONE();
     if (e->ud) {
@@ -1808,9 +1857,23 @@ gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
         transpose_p2m<<<KP, 64, 0, st>>>(e->pd, e->ud, F->tab->cls_perm, K, e->utd, e->utf, e->ltd, e->ltf);
         GF_KERNEL_DONE();
     }
+    if (centre) {
+        build_shift<<<2, 256, shm, st>>>(F->p, K, F->b, qr, host_logfact(), e->sd, e->sf);
+        GF_KERNEL_DONE();
+        for (int i = 0; i < 2; ++i) GF_TRY(xlate_quad_table(F->tab, e->sf + (size_t)i * K * K, K, &e->sq[i], st));
+    }
     GF_CUDA(cudaStreamSynchronize(st));   // other streams may use the cached matrix next
     g_p2m.push_back(e);
-    use_p2m(F, e);
+    *out = e;
+    return GF_OK;
+}
+
+gf_status get_p2m(gf_plan_s *plan, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(g_p2m_mu);
+    P2MEntry *e = nullptr;
+    GF_TRY(find_p2m(plan->fmm, plan->device, plan->quad, quad_device(plan),
+                    (plan->opt.reserved0 & GF_FLAG_SUM_AN) ? 1 : 0, st, &e));
+    use_p2m(plan->fmm, e);
     return GF_OK;
 }
 
@@ -1994,8 +2057,10 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
     const bool pts = F->points;
     const bool fused = !pts && p2m_fused_ok<T>(F);
     const Block3 lb = block_of(F->lev[L]);
-    // 4^3-voxel leaves under a mirror-symmetric rule: the folded P2M kernels
-    const bool fold = !pts && p2m_fold_ok(plan) && lb.n[1] * 4 <= 65535 && lb.n[2] * 4 * B <= 65535;
+    // 4^3-voxel leaves: the folded P2M kernels, where the rule does not mirror on the
+    // voxel centres with its shift after them
+    const bool shift = F->shift_f[0] != nullptr;
+    const bool fold = !pts && (p2m_fold_ok(plan) || shift) && lb.n[1] * 4 <= 65535 && lb.n[2] * 4 * B <= 65535;
     bool up = false;   // level L-1 expansions made straight from the density grid
     // the kernels that write each level's expansions (folded, or the points'
     // P2M) also take the largest |input| of the slabs its M2L reads, in place of a pass over
@@ -2021,6 +2086,10 @@ gf_status run_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B, do
         GF_TRY((launch_blocking<T, 4>(plan, rho, rho_dtype == GF_DTYPE_F32, B, z0, nz, st)));
         GF_TRY(p2m_leaf_run<T>(plan, B, z0 * slab, nz * slab, st));
         if (up) GF_TRY(p2m_up_run<T>(plan, rho, rho_dtype == GF_DTYPE_F32, B, st));
+        if (shift) {
+            GF_TRY(p2m_shift_run(plan, B, L, z0 * slab, nz * slab, st));
+            if (up) GF_TRY(p2m_shift_run(plan, B, L - 1, 0, F->lev[L - 1].ns, st));
+        }
     } else if (fused) {
         stage_mark(plan, 1, st);
         GF_TRY(launch_p2m_fused<T>(plan, rho, rho_dtype == GF_DTYPE_F32, B, st));

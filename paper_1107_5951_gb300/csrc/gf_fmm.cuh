@@ -111,6 +111,11 @@ struct FmmPlan {
     double *p2m_up_d = nullptr;
     float *p2m_up_f = nullptr;
     float *p2m_up_q = nullptr;    // the FP32 matrix in quad order [64][quad][4]
+    // 4^3-voxel leaves under a rule that is not its own mirror image, mixed
+    // precision: the matrices above are those of the voxel centres, p2m_c_f the
+    // leaf's, and the expansions made from them (in tc_split, which is free until the
+    // M2L) are shifted by the rule's nodes, shift_f (leaf, parent), also in quad order
+    const float *p2m_c_f = nullptr, *shift_f[2] = {}, *shift_q[2] = {};
     // the transposes for the adjoint, rows in class order (zeros where it has
     // none): [cls_off[8]][64] (up) and [..][8] (the leaf's octant at position 7)
     double *p2m_upt_d = nullptr, *p2m_leaft_d = nullptr;

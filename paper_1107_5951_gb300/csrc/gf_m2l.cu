@@ -1756,6 +1756,10 @@ static size_t split_offset(const FmmPlan *F, int adj, int l) {
     return off;
 }
 
+float *tc_split_rows(const FmmPlan *F, int level) {
+    return reinterpret_cast<float *>(F->tc_split + split_offset(F, 0, level));
+}
+
 // Tiles of the M2L (adj: of its transpose) for batches of B.
 static int64_t tc_tiles(const FmmPlan *F, bool adj, int B, int *tile_begin) {
     const int nbox = 128 / B;

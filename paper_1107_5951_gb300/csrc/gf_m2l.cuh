@@ -40,10 +40,16 @@ gf_status xlate_quad_table(const Tables *T, const float *src, int rows, float **
 // leaves [first, first + count) from their leaf-blocked masses, and every box
 // of level L - 1 straight from the density grid.
 bool p2m_fold_ok(const gf_plan_s *plan);
+bool rule_mirrors(const QuadRule &q);
 template <class T>
 gf_status p2m_leaf_run(gf_plan_s *plan, int B, int64_t first, int64_t count, cudaStream_t st);
 template <class T>
 gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaStream_t st);
+// Plans with shift tables: the expansions that the two above left in tc_split, of
+// boxes [first, first + count) of a level, shifted by the rule's nodes into ME.
+gf_status p2m_shift_run(gf_plan_s *plan, int B, int level, int64_t first, int64_t count, cudaStream_t st);
+// The rows of a level in the M2L's split inputs, as FP32 rows (mixed precision).
+float *tc_split_rows(const FmmPlan *F, int level);
 
 // Upper bound of the partial rows of the tensor-core M2L's cut tiles (fp64: of the
 // digit M2L's).

@@ -107,10 +107,13 @@ __device__ __forceinline__ int64_t child_row(const XArgs &a, uint32_t col, int o
     return ch >= 0 ? ((int64_t)ch * a.B + bb) * a.ldk : -1;
 }
 
-// Parent row and the child's position for column `col` of L2L / M2M^T.
+// Parent row and the child's position for column `col` of L2L / M2M^T (kShift: the
+// column's own row, no signs).
+template <bool kShift>
 __device__ __forceinline__ int64_t parent_row(const XArgs &a, uint32_t col, int &o) {
-    o = 0;
+    o = kShift ? 7 : 0;
     if (col >= a.ncol) return -1;
+    if constexpr (kShift) return (int64_t)col * a.ldk;
     const uint32_t box = col / (uint32_t)a.B, bb = col - box * a.B;
     if (a.kind == 1) {
         o = (int)(a.tkey[box] & 7);
@@ -221,7 +224,8 @@ __global__ void __launch_bounds__(xlate_max<Tc>()) fold_kernel(XArgs a) {
 // positions, thread (i, y) as above; the child's signs are applied to the
 // staged parent expansion and to the result, so every column uses the same
 // operator.
-template <class Ts, class Tc, int P>
+// kShift: the shift of a box's own expansion, stored (p2m_shift_run).
+template <class Ts, class Tc, int P, bool kShift = false>
 __global__ void __launch_bounds__(xlate_max<Tc>()) spread_kernel(XArgs a) {
     extern __shared__ __align__(16) unsigned char shraw[];
     Tc *xs = reinterpret_cast<Tc *>(shraw);   // [K rounded up to 4][P], then the partial sums
@@ -229,23 +233,29 @@ __global__ void __launch_bounds__(xlate_max<Tc>()) spread_kernel(XArgs a) {
     __shared__ int poct[P];
     const int K = a.K, tid = threadIdx.y * blockDim.x + threadIdx.x, nthr = blockDim.x * blockDim.y;
     const uint32_t col0 = blockIdx.x * P;
-    if (tid < P) prow[tid] = parent_row(a, col0 + tid, poct[tid]);
+    if (tid < P) prow[tid] = parent_row<kShift>(a, col0 + tid, poct[tid]);
     __syncthreads();
     stage_spread<Ts, Tc, P>(a, prow, poct, xs, tid, nthr);
     __syncthreads();
     const int i = threadIdx.x, ic = min(i, K - 1);
     const int cls = parity_of(ic);
-    // the warp's lowest degree: the first input it takes (zero before a thread's own)
-    const int n = degree_of(min(K - 1, i & ~31));
+    // the warp's inputs: from its lowest degree on (zero before a thread's own); kShift:
+    // up to its highest
+    const int n = kShift ? 0 : degree_of(min(K - 1, i & ~31));
+    int jend = K;
+    if constexpr (kShift) {
+        const int top = degree_of(min(K - 1, i | 31)) + 1;
+        jend = top * top;
+    }
     const Tc *t = reinterpret_cast<const Tc *>(a.tab) + ic;
     Acc<Tc, P> acc;
     acc.zero();
     constexpr int G = Lay<Tc, P>::G, NG = Lay<Tc, P>::NG;
 #pragma unroll 2
-    for (int g = ((n * n) >> 2) + threadIdx.y; 4 * g < K; g += blockDim.y) {
+    for (int g = ((n * n) >> 2) + threadIdx.y; 4 * g < jend; g += blockDim.y) {
         Tc tv[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tv[q] = 4 * g + q < K ? __ldg(t + (size_t)(4 * g + q) * K) : Tc(0);
+        for (int q = 0; q < 4; ++q) tv[q] = 4 * g + q < jend ? __ldg(t + (size_t)(4 * g + q) * K) : Tc(0);
 #pragma unroll
         for (int u = 0; u < NG; ++u) {
             const Tc *x = xs + (size_t)4 * g * P + u * G;
@@ -255,11 +265,21 @@ __global__ void __launch_bounds__(xlate_max<Tc>()) spread_kernel(XArgs a) {
     }
     __syncthreads();   // the staged inputs have been used
     Ts *out = reinterpret_cast<Ts *>(a.out);
+    float am = 0.f;
     merge_parts<Tc, P>(acc, xs, [&](int k, int c, Tc sum) {
-        if (k >= K || col0 + c >= a.ncol) return;
-        Ts *o = out + (int64_t)(col0 + c) * a.ldk + k;
-        *o = (Ts)((Tc)*o + (mirror_neg(cls, poct[c]) ? -sum : sum));
+        if constexpr (kShift) {
+            const uint32_t col = col0 + c;
+            if (k >= a.ldk || col >= a.ncol) return;
+            out[(int64_t)col * a.ldk + k] = k < K ? (Ts)sum : Ts(0);
+            if (a.amax && k < K && col >= a.alo && col < a.ahi) am = fmaxf(am, fabsf((float)sum));
+        } else {
+            if (k >= K || col0 + c >= a.ncol) return;
+            Ts *o = out + (int64_t)(col0 + c) * a.ldk + k;
+            *o = (Ts)((Tc)*o + (mirror_neg(cls, poct[c]) ? -sum : sum));
+        }
     });
+    if constexpr (kShift)
+        if (a.amax) amax_merge(a.amax, am);
 }
 
 // Parents to all their children (M2M^T) in FP64: with the inputs' classes kept
@@ -453,6 +473,7 @@ __global__ void __launch_bounds__(160) fold_quad(XArgs a, QuadArgs q) {
     rows_out(xs, reinterpret_cast<float *>(a.out), col0, a.ncol, kFoldCols, a.K, a.ldk, a.amax, a.alo, a.ahi);
 }
 
+template <bool kShift>
 __global__ void __launch_bounds__(320) spread_quad(XArgs a, QuadArgs q) {
     extern __shared__ __align__(16) unsigned char shraw[];
     float *xs = reinterpret_cast<float *>(shraw);   // [K rounded up to 4][kSpreadCols], then the rows
@@ -460,17 +481,25 @@ __global__ void __launch_bounds__(320) spread_quad(XArgs a, QuadArgs q) {
     __shared__ int poct[kSpreadCols];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const uint32_t col0 = blockIdx.x * kSpreadCols;
-    if (tid < kSpreadCols) prow[tid] = parent_row(a, col0 + tid, poct[tid]);
+    if (tid < kSpreadCols) prow[tid] = parent_row<kShift>(a, col0 + tid, poct[tid]);
     __syncthreads();
     stage_spread<float, float, kSpreadCols>(a, prow, poct, xs, tid, nthr);
     __syncthreads();
     const int on = tid < q.nq * (kSpreadCols / 8), cg = on ? tid / q.nq : 0, quad = on ? tid - cg * q.nq : 0;
     const int info = q.info[quad], cls = info & 0xff;
-    const int nmin = __reduce_min_sync(0xffffffffu, (info >> 8) & 0xff);
+    // inputs from the lowest output's degree on (kShift: up to the highest's)
+    int g0 = 0, jend = a.K;
+    if constexpr (kShift) {
+        const int nmax = __reduce_max_sync(0xffffffffu, info >> 16);
+        jend = (nmax + 1) * (nmax + 1);
+    } else {
+        const int nmin = __reduce_min_sync(0xffffffffu, (info >> 8) & 0xff);
+        g0 = (nmin * nmin) >> 2;
+    }
     uint64_t acc[4][4] = {};
     const float4 *t = reinterpret_cast<const float4 *>(q.tq) + quad;
 #pragma unroll 2
-    for (int g = (nmin * nmin) >> 2; 4 * g < a.K; ++g) {
+    for (int g = g0; 4 * g < jend; ++g) {
         const float *x = xs + 4 * g * kSpreadCols + 8 * cg;
 #pragma unroll
         for (int u = 0; u < 4; ++u) quad_fma<8>(acc, __ldg(t + (4 * g + u) * q.nq), x + u * kSpreadCols, 4);
@@ -478,6 +507,10 @@ __global__ void __launch_bounds__(320) spread_quad(XArgs a, QuadArgs q) {
     __syncthreads();   // the staged inputs have been used
     if (on) quad_store<8>(acc, q.qk + 4 * quad, xs, 8 * cg, a.ldk, [&](int c) { return mirror_neg(cls, poct[c]); });
     __syncthreads();
+    if constexpr (kShift) {
+        rows_out(xs, reinterpret_cast<float *>(a.out), col0, a.ncol, kSpreadCols, a.K, a.ldk, a.amax, a.alo, a.ahi);
+        return;
+    }
     // rows added to the children's, 16 bytes a thread
     float *out = reinterpret_cast<float *>(a.out) + (int64_t)col0 * a.ldk;
     const int n4 = a.ldk >> 2, nv = (int)min((uint32_t)kSpreadCols, a.ncol - col0) * n4;
@@ -772,10 +805,11 @@ gf_status launch_fold_quad(const XArgs &a, const QuadArgs &q, cudaStream_t st) {
     return GF_OK;
 }
 
+template <bool kShift>
 gf_status launch_spread_quad(const XArgs &a, const QuadArgs &q, cudaStream_t st) {
     const size_t shm = sizeof(float) * kSpreadCols * std::max((a.K + 3) & ~3, a.ldk);
-    GF_TRY(ensure_smem(spread_quad, shm));
-    spread_quad<<<ceil_div((int64_t)a.ncol, kSpreadCols), (q.nq * (kSpreadCols / 8) + 31) & ~31, shm, st>>>(a, q);
+    GF_TRY(ensure_smem(spread_quad<kShift>, shm));
+    spread_quad<kShift><<<ceil_div((int64_t)a.ncol, kSpreadCols), (q.nq * (kSpreadCols / 8) + 31) & ~31, shm, st>>>(a, q);
     GF_KERNEL_DONE();
     return GF_OK;
 }
@@ -790,12 +824,12 @@ gf_status launch_fold(const XArgs &a, cudaStream_t st) {
     return GF_OK;
 }
 
-template <class Ts, class Tc, int P>
+template <class Ts, class Tc, int P, bool kShift = false>
 gf_status launch_spread(const XArgs &a, cudaStream_t st) {
     const dim3 blk = xlate_block<Tc>(a.K, a.ldk);
     const size_t shm = xlate_smem<Tc>((a.K + 3) & ~3, P, blk);
-    GF_TRY((ensure_smem(spread_kernel<Ts, Tc, P>, shm)));
-    spread_kernel<Ts, Tc, P><<<ceil_div((int64_t)a.ncol, P), blk, shm, st>>>(a);
+    GF_TRY((ensure_smem(spread_kernel<Ts, Tc, P, kShift>, shm)));
+    spread_kernel<Ts, Tc, P, kShift><<<ceil_div((int64_t)a.ncol, P), blk, shm, st>>>(a);
     GF_KERNEL_DONE();
     return GF_OK;
 }
@@ -953,7 +987,7 @@ gf_status translate_run(gf_plan_s *plan, int level, int kind, int B, cudaStream_
     }
     if (sizeof(Ts) == 4 && sizeof(Tc) == 4 && many_columns(ncol)) {
         const QuadArgs q = quad_args(T, T->quad_f[kind]);
-        return kind == 0 || kind == 3 ? launch_fold_quad(a, q, st) : launch_spread_quad(a, q, st);
+        return kind == 0 || kind == 3 ? launch_fold_quad(a, q, st) : launch_spread_quad<false>(a, q, st);
     }
     if (kind == 2 && sizeof(Tc) == 8) {   // by parents: every child of the dense blocks is updated
         const int64_t np = up.ns * B;
@@ -984,8 +1018,10 @@ template gf_status translate_run<double, double>(gf_plan_s *, int, int, int, cud
 bool p2m_fold_ok(const gf_plan_s *plan) {
     const FmmPlan *F = plan->fmm;
     if (F->points || F->b != 4 || !F->p2m_up_d) return false;
-    if (plan->opt.reserved0 & GF_FLAG_SUM_AN) return true;   // exact voxel moments
-    const QuadRule &q = plan->quad;
+    return (plan->opt.reserved0 & GF_FLAG_SUM_AN) || rule_mirrors(plan->quad);   // (SUM-AN: exact voxel moments)
+}
+
+bool rule_mirrors(const QuadRule &q) {
     for (int a = 0; a < 3; ++a)   // the rule mirrored across axis a is the same set of nodes and weights
         for (int s = 0; s < q.nq; ++s) {
             bool found = false;
@@ -1007,6 +1043,10 @@ static P2MArgs p2m_args(gf_plan_s *plan, int B, int level, int64_t first) {
     a.ldk = F->KS;
     a.me = F->lev[level].me;
     amax_range(F, level, B, first, a.amax, a.alo, a.ahi);
+    if (F->shift_f[0]) {   // p2m_shift_run makes the expansions
+        a.me = tc_split_rows(F, level);
+        a.amax = nullptr;
+    }
     a.status = plan->d_status;
     return a;
 }
@@ -1020,7 +1060,7 @@ gf_status p2m_leaf_run(gf_plan_s *plan, int B, int64_t first, int64_t count, cud
     a.first = first;
     GF_TRY(check_columns(count * B, F->L));
     a.ncol = (uint32_t)(count * B);
-    a.tab = sizeof(T) == 8 ? (const void *)F->p2m_d : (const void *)F->p2m_f;
+    a.tab = sizeof(T) == 8 ? (const void *)F->p2m_d : (const void *)(F->shift_f[0] ? F->p2m_c_f : F->p2m_f);
     p2m_leaf_fold<T><<<ceil_div(a.ncol, kLeafCols), xlate_threads(a.K, a.ldk), 0, st>>>(a);
     GF_KERNEL_DONE();
     return GF_OK;
@@ -1071,6 +1111,38 @@ gf_status p2m_up_run(gf_plan_s *plan, const void *rho, int rho_f32, int B, cudaS
 #undef GF_UP_LAUNCH
     GF_KERNEL_DONE();
     return GF_OK;
+}
+
+// A source moved by d moves its expansion by a triangular operator of d alone (the
+// M2M without the change of scale), and every voxel moves by the same nodes: so the
+// expansions of any rule are those of the voxel centres, which mirror, times one
+// matrix, the nodes' weighted sum.  One node off the centre, 464^3, p = 10: the forward
+// 3,022 us with the leaf P2M of every leaf (1,458 with a P2M on the tensor cores), now
+// 1,463; 232^3 646 (543), now 460.
+gf_status p2m_shift_run(gf_plan_s *plan, int B, int level, int64_t first, int64_t count, cudaStream_t st) {
+    FmmPlan *F = plan->fmm;
+    if (count <= 0) return GF_OK;
+    const int which = level == F->L ? 0 : 1;
+    const int64_t at = first * B * F->KS;
+    XArgs a;
+    memset(&a, 0, sizeof(a));
+    a.in = tc_split_rows(F, level) + at;
+    a.out = (float *)F->lev[level].me + at;
+    a.tab = F->shift_f[which];
+    a.K = F->K;
+    a.ldk = F->KS;
+    a.B = B;
+    GF_TRY(check_columns(count * B, level));
+    a.ncol = (uint32_t)(count * B);
+    amax_range(F, level, B, first, a.amax, a.alo, a.ahi);
+    if (many_columns(a.ncol)) return launch_spread_quad<true>(a, quad_args(F->tab, F->shift_q[which]), st);
+    switch (cols_per_block(a.ncol, 16)) {
+        case 1: return launch_spread<float, float, 1, true>(a, st);
+        case 2: return launch_spread<float, float, 2, true>(a, st);
+        case 4: return launch_spread<float, float, 4, true>(a, st);
+        case 8: return launch_spread<float, float, 8, true>(a, st);
+        default: return launch_spread<float, float, 16, true>(a, st);
+    }
 }
 
 template gf_status p2m_leaf_run<float>(gf_plan_s *, int, int64_t, int64_t, cudaStream_t);
