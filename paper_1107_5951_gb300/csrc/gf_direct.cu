@@ -76,13 +76,35 @@ __device__ __forceinline__ double node_coord(double o, double h, int64_t i, doub
 constexpr int kRow = 30;   // lanes 30 and 31 form the row's y and z
 
 struct RowSplit {
-    int clen, nch;   // voxels per piece, pieces per row
+    int clen, nch;       // voxels per piece, pieces per row
+    int ax[3];           // the axes of a row, j and k
+    int n[3];            // their voxels
+    int64_t stride[3];   // and strides in the density array
+    double o[3], h[3];   // the grid's origin and voxel size along them
 };
 
-inline RowSplit row_split(int64_t nx) {
+// Rows run along x, unless its pieces would be less than half as long as another
+// axis's (a column of voxels: 20 instructions for every voxel's own row).
+inline RowSplit row_split(const GridArgs &ga) {
+    const int64_t n[3] = {ga.nx, ga.ny, ga.nz}, stride[3] = {1, ga.nx, ga.nx * ga.ny};
+    const double o[3] = {ga.ox, ga.oy, ga.oz}, h[3] = {ga.hx, ga.hy, ga.hz};
+    auto clen = [&](int a) {
+        const int64_t nch = (n[a] + kRow - 1) / kRow;
+        return (int)((n[a] + nch - 1) / nch);
+    };
+    int row = 0;
+    for (int a = 1; a < 3; ++a)
+        if (clen(a) > 2 * clen(0) && clen(a) > clen(row)) row = a;
     RowSplit r;
-    r.nch = (int)((nx + kRow - 1) / kRow);
-    r.clen = (int)((nx + r.nch - 1) / r.nch);
+    r.nch = (int)((n[row] + kRow - 1) / kRow);
+    r.clen = clen(row);
+    for (int d = 0; d < 3; ++d) {
+        r.ax[d] = d == 0 ? row : (d - 1 < row ? d - 1 : d);
+        r.n[d] = (int)n[r.ax[d]];
+        r.stride[d] = stride[r.ax[d]];
+        r.o[d] = o[r.ax[d]];
+        r.h[d] = h[r.ax[d]];
+    }
     return r;
 }
 
@@ -132,15 +154,15 @@ __device__ __forceinline__ const void *rho_of(const void *rho, int f32, int64_t 
 // R x 16 pairs.  16^3 voxels, 2x2x2 rule, 4096 stations (134 M pairs):
 // 41.6 -> 4.07 ms (16 blocks of 256 threads before; 2.5 ms at two FP64
 // instructions a clock and SM).
-template <int R>
-__global__ void __launch_bounds__(kPairThreads)
+template <int R, bool kSolo>
+__global__ void __launch_bounds__(kSolo ? 32 : kPairThreads)
 direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict__ rho, int rho_f32, GridArgs ga,
                RowSplit rs, const QuadRule *__restrict__ qr, double G, double *__restrict__ g,
                double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ double2 red[(kPairWarps + 1) * 3 * R * 32];
-    __shared__ __align__(16) double2 row_s[kPairWarps][32];   // (x, mass) of the piece; entries 30, 31: y, z
-    const int C = (int)cooperative_groups::this_cluster().num_blocks();
-    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    __shared__ double2 red[kSolo ? 1 : (kPairWarps + 1) * 3 * R * 32];
+    __shared__ __align__(16) double2 row_s[kSolo ? 1 : kPairWarps][32];   // (x, mass) of the piece; entries 30, 31: y, z
+    const int C = kSolo ? 1 : (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = kSolo ? 0 : (int)cooperative_groups::this_cluster().block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int64_t tile = blockIdx.x / C;
@@ -149,33 +171,33 @@ direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         const int64_t j = (tile * R + u) * 32 + lane;
-        rx[u] = j < M ? obs[3 * j + 0] : 0.0;
-        ry[u] = j < M ? obs[3 * j + 1] : 0.0;
-        rz[u] = j < M ? obs[3 * j + 2] : 0.0;
+        rx[u] = j < M ? obs[3 * j + rs.ax[0]] : 0.0;
+        ry[u] = j < M ? obs[3 * j + rs.ax[1]] : 0.0;
+        rz[u] = j < M ? obs[3 * j + rs.ax[2]] : 0.0;
     }
 #pragma unroll
     for (int v = 0; v < 3 * R; ++v) s[v] = c[v] = a[v] = 0.0;
     const void *rho_b = rho_of(rho, rho_f32, b * ga.nvox);
     double2 *row = row_s[warp];
     bool bad = false;   // a non-finite density (reported through status[0])
-    RowIter it(rank * kPairWarps + warp, (int64_t)C * kPairWarps, rs.nch, qr->nq, (int)ga.ny);
+    RowIter it(rank * kPairWarps + warp, kSolo ? 1 : (int64_t)C * kPairWarps, rs.nch, qr->nq, rs.n[1]);
     auto fetch = [&](double &rv) {
         const int64_t i = (int64_t)it.ch * rs.clen + lane;
         rv = 0.0;
-        if (it.k < ga.nz && lane < rs.clen && i < ga.nx)
-            rv = load_rho(rho_b, rho_f32, ((int64_t)it.k * ga.ny + it.j) * ga.nx + i);
+        if (it.k < rs.n[2] && lane < rs.clen && i < rs.n[0])
+            rv = load_rho(rho_b, rho_f32, it.k * rs.stride[2] + it.j * rs.stride[1] + i * rs.stride[0]);
     };
     double rv;
     fetch(rv);
     int since = 0;   // sources summed since the last merge into (s, c)
-    while (it.k < ga.nz) {
+    while (it.k < rs.n[2]) {
         const int i0 = it.ch * rs.clen;
-        const int cnt = min(rs.clen, (int)ga.nx - i0);
+        const int cnt = min(rs.clen, rs.n[0] - i0);
         // one node coordinate per lane: x of the piece's voxels, y (lane 30), z (lane 31)
         const int ax = lane < kRow ? 0 : lane - (kRow - 1);
-        const double co = ax == 0 ? ga.ox : ax == 1 ? ga.oy : ga.oz, ch = ax == 0 ? ga.hx : ax == 1 ? ga.hy : ga.hz;
-        const int ci = ax == 0 ? i0 + lane : ax == 1 ? it.j : it.k;
-        const double x = node_coord(co, ch, ci, qr->xi[it.q][ax]);
+        const double co = ax == 0 ? rs.o[0] : ax == 1 ? rs.o[1] : rs.o[2], ch = ax == 0 ? rs.h[0] : ax == 1 ? rs.h[1] : rs.h[2];
+        const int ci = ax == 0 ? i0 + lane : ax == 1 ? it.j : it.k, da = ax == 0 ? rs.ax[0] : ax == 1 ? rs.ax[1] : rs.ax[2];
+        const double x = node_coord(co, ch, ci, qr->xi[it.q][da]);
         bad |= !isfinite(rv);
         const double m = __dmul_rn(__dmul_rn(rv, ga.vol), qr->wn[it.q]);
         __syncwarp();
@@ -222,17 +244,23 @@ direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict
 #pragma unroll
     for (int v = 0; v < 3 * R; ++v) two_sum_d(s[v], c[v], a[v]);
     if (bad && status && tile == 0) atomicOr(status, 1);
-    const double tot = cluster_total<3 * R>(s, c, red);
-    const int t = threadIdx.x;
-    if (rank == 0 && t < 3 * R * 32) {
-        const int v = t >> 5, u = v / 3, d = v - 3 * u;
-        const int64_t j = (tile * R + u) * 32 + (t & 31);
+    auto put = [&](int v, int l, double tot) {
+        const int u = v / 3, d = v - 3 * u, da = d == 0 ? rs.ax[0] : d == 1 ? rs.ax[1] : rs.ax[2];
+        const int64_t j = (tile * R + u) * 32 + l;
         if (j < M) {
-            if (g) g[((int64_t)b * M + j) * 3 + d] = G * tot;
-            if (gz && d == 2) gz[(int64_t)b * M + j] = G * tot;
+            if (g) g[((int64_t)b * M + j) * 3 + da] = G * tot;
+            if (gz && da == 2) gz[(int64_t)b * M + j] = G * tot;
         }
+    };
+    if constexpr (kSolo) {
+#pragma unroll
+        for (int v = 0; v < 3 * R; ++v) put(v, lane, s[v] + c[v]);
+    } else {
+        const double tot = cluster_total<3 * R>(s, c, red);
+        if (rank == 0 && threadIdx.x < 3 * R * 32) put(threadIdx.x >> 5, lane, tot);
     }
 }
+
 
 // Mixed precision: positions in voxel units split into an integer part
 // (held exactly in FP32, |i| < 2^24) and a fraction; the pair separation is
@@ -247,15 +275,16 @@ direct_fwd_f64(const double *__restrict__ obs, int64_t M, const void *__restrict
 // hundred stations by latency.  40 x 40 x 32 voxels, 2x2x2 rule, 6000 stations
 // (2.5e9 pairs): 29.3 -> 1.33 ms; 12 x 10 x 9 voxels, 300 stations: 625 -> 46 us,
 // most of it the host.
-__global__ void __launch_bounds__(kPairThreads)
+template <bool kSolo>
+__global__ void __launch_bounds__(kSolo ? 32 : kPairThreads)
 direct_fwd_mixed(const float *__restrict__ obs_i, const float *__restrict__ obs_f, int64_t M,
                  const void *__restrict__ rho, int rho_f32, GridArgs ga, RowSplit rs,
                  const QuadRule *__restrict__ qr, double G, double *__restrict__ g, double *__restrict__ gz,
                  int *__restrict__ status) {
-    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
-    __shared__ __align__(16) float2 row_s[kPairWarps][32];   // masses as duplicated pairs
-    const int C = (int)cooperative_groups::this_cluster().num_blocks();
-    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    __shared__ double2 red[kSolo ? 1 : (kPairWarps + 1) * 6 * 32];
+    __shared__ __align__(16) float2 row_s[kSolo ? 1 : kPairWarps][32];   // masses as duplicated pairs
+    const int C = kSolo ? 1 : (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = kSolo ? 0 : (int)cooperative_groups::this_cluster().block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int64_t tile = blockIdx.x / C;
@@ -264,21 +293,22 @@ direct_fwd_mixed(const float *__restrict__ obs_i, const float *__restrict__ obs_
         const int64_t j0 = tile * 64 + lane, j1 = j0 + 32;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            RI[d] = pk2(j0 < M ? obs_i[3 * j0 + d] : 0.f, j1 < M ? obs_i[3 * j1 + d] : 0.f);
-            RF[d] = pk2(j0 < M ? obs_f[3 * j0 + d] : 0.f, j1 < M ? obs_f[3 * j1 + d] : 0.f);
+            const int da = rs.ax[d];
+            RI[d] = pk2(j0 < M ? obs_i[3 * j0 + da] : 0.f, j1 < M ? obs_i[3 * j1 + da] : 0.f);
+            RF[d] = pk2(j0 < M ? obs_f[3 * j0 + da] : 0.f, j1 < M ? obs_f[3 * j1 + da] : 0.f);
         }
     }
-    const float fx = (float)ga.hx, fy = (float)ga.hy, fz = (float)ga.hz;
+    const float fx = (float)rs.h[0], fy = (float)rs.h[1], fz = (float)rs.h[2];
     const uint64_t HX = pk2(fx, fx), HY = pk2(fy, fy), HZ = pk2(fz, fz), NEG1 = pk2(-1.f, -1.f);
     const void *rho_b = rho_of(rho, rho_f32, b * ga.nvox);
     float2 *row = row_s[warp];
     uint64_t A[3] = {0, 0, 0}, H[3] = {0, 0, 0}, L[3] = {0, 0, 0};
     bool bad = false;   // a non-finite density (reported through status[0])
-    RowIter it(rank * kPairWarps + warp, (int64_t)C * kPairWarps, rs.nch, qr->nq, (int)ga.ny);
+    RowIter it(rank * kPairWarps + warp, kSolo ? 1 : (int64_t)C * kPairWarps, rs.nch, qr->nq, rs.n[1]);
     auto fetch = [&]() -> float {
         const int64_t i = (int64_t)it.ch * rs.clen + lane;
-        if (it.k < ga.nz && lane < rs.clen && i < ga.nx) {
-            const int64_t idx = ((int64_t)it.k * ga.ny + it.j) * ga.nx + i;
+        if (it.k < rs.n[2] && lane < rs.clen && i < rs.n[0]) {
+            const int64_t idx = it.k * rs.stride[2] + it.j * rs.stride[1] + i * rs.stride[0];
             if (rho_f32) {
                 const float v = __ldg((const float *)rho_b + idx);
                 bad |= !isfinite(v);
@@ -302,11 +332,11 @@ direct_fwd_mixed(const float *__restrict__ obs_i, const float *__restrict__ obs_
     };
     float rv = fetch();
     int since = 0;   // sources summed since the last merge
-    while (it.k < ga.nz) {
+    while (it.k < rs.n[2]) {
         const int i0 = it.ch * rs.clen;
-        const int cnt = min(rs.clen, (int)ga.nx - i0);
+        const int cnt = min(rs.clen, rs.n[0] - i0);
         const float *of = qr->offf[it.q];
-        const float sx = of[0], sy = of[1], sz = of[2], wq = qr->wnf[it.q];
+        const float sx = of[rs.ax[0]], sy = of[rs.ax[1]], sz = of[rs.ax[2]], wq = qr->wnf[it.q];
         const float cj = (float)it.j, ck = (float)it.k, ci = (float)(i0 - 1);
         __syncwarp();
         row[lane] = make_float2(rv, rv);
@@ -369,40 +399,50 @@ direct_fwd_mixed(const float *__restrict__ obs_i, const float *__restrict__ obs_
         s[3 + d] = (double)h1;
         c[3 + d] = (double)l1;
     }
-    const double tot = cluster_total<6>(s, c, red);
     const double scale = G * ga.vol;
-    const int t = threadIdx.x;
-    if (rank == 0 && t < 6 * 32) {
-        const int v = t >> 5, u = v / 3, d = v - 3 * u;
-        const int64_t j = tile * 64 + u * 32 + (t & 31);
+    auto put = [&](int v, int l, double tot) {
+        const int u = v / 3, d = v - 3 * u, da = d == 0 ? rs.ax[0] : d == 1 ? rs.ax[1] : rs.ax[2];
+        const int64_t j = tile * 64 + u * 32 + l;
         if (j < M) {
-            if (g) g[((int64_t)b * M + j) * 3 + d] = scale * tot;
-            if (gz && d == 2) gz[(int64_t)b * M + j] = scale * tot;
+            if (g) g[((int64_t)b * M + j) * 3 + da] = scale * tot;
+            if (gz && da == 2) gz[(int64_t)b * M + j] = scale * tot;
         }
+    };
+    if constexpr (kSolo) {
+#pragma unroll
+        for (int v = 0; v < 6; ++v) put(v, lane, s[v] + c[v]);
+    } else {
+        const double tot = cluster_total<6>(s, c, red);
+        if (rank == 0 && threadIdx.x < 6 * 32) put(threadIdx.x >> 5, lane, tot);
     }
 }
 
-// Tiles of 64 observers (two per lane), or of 32 when there are no more.
+// Tiles of 64 observers (two per lane), or of 32 when there are no more.  An FP64
+// instruction of a warp takes 16 clocks of its SM.
 gf_status launch_fwd_f64(const double *obs, int64_t M, const void *rho, int rho_f32, const GridArgs &ga, int nq,
                          const QuadRule *qr, int B, double G, double *g, double *gz, int *status, cudaStream_t st) {
-    const RowSplit rs = row_split(ga.nx);
-    const int64_t units = (int64_t)rs.nch * nq * ga.ny * ga.nz;
+    const RowSplit rs = row_split(ga);
+    const int64_t units = (int64_t)rs.nch * nq * rs.n[1] * rs.n[2];
     if (M <= 32) {
-        const int c = pair_cluster(1, units);
-        return pair_launch(direct_fwd_f64<1>, 1, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+        const int c = std::max(1, pair_cluster(1, units, {(11.0 * rs.clen + 30.0) * 16.0 / 2070.0, 4.0, 4.0}));
+        return pair_launch(direct_fwd_f64<1, false>, 1, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
     }
     const int64_t tiles = (M + 63) / 64;
-    const int c = pair_cluster(tiles, units);
-    return pair_launch(direct_fwd_f64<2>, tiles, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+    const int c = pair_cluster(tiles, units, {(22.0 * rs.clen + 30.0) * 16.0 / 2070.0, 8.0, 4.0});
+    if (c == 0)
+        return pair_launch_solo(direct_fwd_f64<2, true>, tiles, B, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+    return pair_launch(direct_fwd_f64<2, false>, tiles, B, c, st, obs, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
 }
 
 gf_status launch_fwd_mixed(const float *oi, const float *of, int64_t M, const void *rho, int rho_f32,
                            const GridArgs &ga, int nq, const QuadRule *qr, int B, double G, double *g, double *gz,
                            int *status, cudaStream_t st) {
-    const RowSplit rs = row_split(ga.nx);
+    const RowSplit rs = row_split(ga);
     const int64_t tiles = (M + 63) / 64;
-    const int c = pair_cluster(tiles, (int64_t)rs.nch * nq * ga.ny * ga.nz);
-    return pair_launch(direct_fwd_mixed, tiles, B, c, st, oi, of, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+    const int c = pair_cluster(tiles, (int64_t)rs.nch * nq * rs.n[1] * rs.n[2], {(12.0 * rs.clen + 40.0) / 2070.0, 5.0, 8.0});
+    if (c == 0)
+        return pair_launch_solo(direct_fwd_mixed<true>, tiles, B, st, oi, of, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
+    return pair_launch(direct_fwd_mixed<false>, tiles, B, c, st, oi, of, M, rho, rho_f32, ga, rs, qr, G, g, gz, status);
 }
 
 // Transpose: one thread per voxel, observers (with their weights) staged in

@@ -10,7 +10,9 @@
 // of a cluster takes a share of the sources for the whole tile, and the
 // partial sums meet in shared memory (the block's 8 warps) and then over the
 // cluster's distributed shared memory, in a fixed order: no workspace, and
-// the same result on every run.
+// the same result on every run.  Few sources over many observers need no sharing, and
+// adding up the shares would take longer than the sums: there a warp takes a tile by
+// itself (kSolo; pair_cluster chooses).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -106,26 +108,48 @@ constexpr size_t pair_smem() {
     return sizeof(double2) * (kPairWarps + 1) * NV * 32;
 }
 
-// Blocks per cluster for `tiles` observer tiles and `units` work units per
-// tile: the size that leaves the smallest share of the SMs idle in the last
-// round of blocks (the smaller size when it is within 2% of the best), with
-// at least two units for each warp of the cluster.  The size decides how an
-// observer's sum associates: callers count the tiles of one batch member, so that a
-// member's sums are the same bits alone and in any batch.
-inline int pair_cluster(int64_t tiles, int64_t units) {
+// How one SM's time goes in a direct sum, in microseconds: a work unit of one tile,
+// a block's start and its cluster_total, and how much longer a warp alone on an SM
+// takes over a unit than warps that fill it take on average.
+struct PairCost {
+    double unit, block, alone;
+};
+
+// Blocks per cluster for `tiles` observer tiles and `units` work units per tile, or
+// 0: a warp alone to a tile, without partial sums to add up.  The size with the
+// least time for the SM with the most blocks (the smaller size when it is within 2%
+// of the best), with at least two units for each warp of a cluster.  A tile's
+// cluster_total is some 400 FP64 instructions, 5 to 8 us of an SM.  A million observers
+// of one voxel 557 us (mixed) and 868 (FP64) with it, 40 and 108 a warp to a tile (a
+// thread per observer before either: 38 and 103); of 4^3 voxels 617 and 2,405, now 74
+// and 1,753 (82 and 2,179); of 8^3 882, now 285 (515), FP64 12.6 ms (17.0).  The size
+// decides how an observer's sum associates: callers count the tiles of one batch
+// member, so that a member's sums are the same bits alone and in any batch.
+inline int pair_cluster(int64_t tiles, int64_t units, PairCost cost) {
     const int64_t sms = sm_count();
     const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kPairMaxCluster, units / (2 * kPairWarps)));
-    int best = 1;
-    double beff = 0.0;
+    // a warp to a tile (a tenth slower a unit than warps that share a block)
+    double best_us = 1.1 * (double)units * cost.unit * std::max((double)((tiles + sms - 1) / sms), cost.alone);
+    int best = 0;
     for (int64_t c = 1; c <= most; ++c) {
-        const int64_t n = tiles * c;
-        const double eff = (double)n / (double)((n + sms - 1) / sms * sms);
-        if (eff > 1.02 * beff) {
-            beff = eff;
+        const int64_t rounds = (tiles * c + sms - 1) / sms;
+        // the warps of a block that have no unit do not help
+        const double share = std::max(1.0 / (double)c, cost.alone / (double)std::max<int64_t>(1, units));
+        const double us = (double)rounds * (cost.block + (double)units * cost.unit * share);
+        if (us < 0.98 * best_us) {
+            best_us = us;
             best = (int)c;
         }
     }
     return best;
+}
+
+// Launch of `kernel` on tiles x batch warps.
+template <class... A, class... B>
+gf_status pair_launch_solo(void (*kernel)(A...), int64_t tiles, int batch, cudaStream_t st, B &&...args) {
+    kernel<<<dim3((unsigned)tiles, (unsigned)batch), 32, 0, st>>>(std::forward<B>(args)...);
+    GF_KERNEL_DONE();
+    return GF_OK;
 }
 
 // Launch of `kernel` on tiles x batch clusters of `cluster` blocks.

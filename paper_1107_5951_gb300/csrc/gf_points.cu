@@ -174,14 +174,15 @@ __device__ __forceinline__ double load_rho_p(const void *rho, int f32, int64_t i
 // sources 32 at a time (gf_pair.cuh), each lane staging one with its mass
 // rho_{c(s)} a_s of batch member blockIdx.y.  16 FP64 instructions a pair,
 // bound by the FP64 pipe.
-__global__ void __launch_bounds__(kPairThreads)
+template <bool kSolo>
+__global__ void __launch_bounds__(kSolo ? 32 : kPairThreads)
 direct_points_f64(const double *__restrict__ obs, int64_t M, const double *__restrict__ src,
                   const double *__restrict__ wt, int64_t S, int per_cell, int64_t ncell, const void *__restrict__ rho,
                   int rho_f32, double G, double *__restrict__ g, double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
-    __shared__ __align__(16) double2 stage[kPairWarps][32][2];   // (x, y), (z, mass)
-    const int C = (int)cooperative_groups::this_cluster().num_blocks();
-    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    __shared__ double2 red[kSolo ? 1 : (kPairWarps + 1) * 6 * 32];
+    __shared__ __align__(16) double2 stage[kSolo ? 1 : kPairWarps][32][2];   // (x, y), (z, mass)
+    const int C = kSolo ? 1 : (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = kSolo ? 0 : (int)cooperative_groups::this_cluster().block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int64_t tile = blockIdx.x / C;
@@ -195,7 +196,7 @@ direct_points_f64(const double *__restrict__ obs, int64_t M, const double *__res
     bool bad = false;
     double2(*st)[2] = stage[warp];
     int since = 0;
-    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += (int64_t)C * kPairThreads) {
+    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += kSolo ? 32 : (int64_t)C * kPairThreads) {
         const int64_t i = t0 + lane;
         __syncwarp();
         if (i < S) {
@@ -231,15 +232,19 @@ direct_points_f64(const double *__restrict__ obs, int64_t M, const double *__res
 #pragma unroll
     for (int v = 0; v < 6; ++v) two_sum_d(s[v], c[v], a[v]);
     if (bad && status && tile == 0) atomicOr(status, 1);
-    const double tot = cluster_total<6>(s, c, red);
-    const int t = threadIdx.x;
-    if (rank == 0 && t < 6 * 32) {
-        const int v = t >> 5;
-        const int64_t j = tile * 64 + (v / 3) * 32 + (t & 31);
+    auto put = [&](int v, int l, double tot) {
+        const int64_t j = tile * 64 + (v / 3) * 32 + l;
         if (j < M) {
             if (g) g[((int64_t)b * M + j) * 3 + v % 3] = G * tot;
             if (gz && v % 3 == 2) gz[(int64_t)b * M + j] = G * tot;
         }
+    };
+    if constexpr (kSolo) {
+#pragma unroll
+        for (int v = 0; v < 6; ++v) put(v, lane, s[v] + c[v]);
+    } else {
+        const double tot = cluster_total<6>(s, c, red);
+        if (rank == 0 && threadIdx.x < 6 * 32) put(threadIdx.x >> 5, lane, tot);
     }
 }
 
@@ -262,16 +267,17 @@ __global__ void split_points(const double *__restrict__ x, int64_t n, double lo0
 // integer difference plus one rounding; FP32 pair terms, compensated FP32
 // sums of about 256 sources, FP64 beyond.  Sources are staged as packed pairs
 // (f32x2), so one instruction does two pairs of an observer.
-__global__ void __launch_bounds__(kPairThreads)
+template <bool kSolo>
+__global__ void __launch_bounds__(kSolo ? 32 : kPairThreads)
 direct_points_mixed(const float *__restrict__ oi, const float *__restrict__ of, int64_t M,
                     const float *__restrict__ si, const float *__restrict__ sf, const double *__restrict__ wt,
                     int64_t S, int per_cell, int64_t ncell, const void *__restrict__ rho, int rho_f32, float q,
                     double Gq, double *__restrict__ g, double *__restrict__ gz, int *__restrict__ status) {
-    __shared__ double2 red[(kPairWarps + 1) * 6 * 32];
+    __shared__ double2 red[kSolo ? 1 : (kPairWarps + 1) * 6 * 32];
     // per pair of sources: integer parts {x0,x1, y0,y1}, {z0,z1, m0,m1}, fractions {x, y}, {z, -}
-    __shared__ __align__(16) float stage[kPairWarps][16 * 16];
-    const int C = (int)cooperative_groups::this_cluster().num_blocks();
-    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    __shared__ __align__(16) float stage[kSolo ? 1 : kPairWarps][16 * 16];
+    const int C = kSolo ? 1 : (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = kSolo ? 0 : (int)cooperative_groups::this_cluster().block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int64_t tile = blockIdx.x / C;
@@ -299,7 +305,7 @@ direct_points_mixed(const float *__restrict__ oi, const float *__restrict__ of, 
         }
     };
     int since = 0;
-    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += (int64_t)C * kPairThreads) {
+    for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * 32; t0 < S; t0 += kSolo ? 32 : (int64_t)C * kPairThreads) {
         const int64_t i = t0 + lane;
         __syncwarp();
         {
@@ -358,15 +364,19 @@ direct_points_mixed(const float *__restrict__ oi, const float *__restrict__ of, 
         s[v] = (double)h[v];
         c[v] = (double)l[v];
     }
-    const double tot = cluster_total<6>(s, c, red);
-    const int t = threadIdx.x;
-    if (rank == 0 && t < 6 * 32) {
-        const int v = t >> 5;
-        const int64_t j = tile * 64 + (v / 3) * 32 + (t & 31);
+    auto put = [&](int v, int l, double tot) {
+        const int64_t j = tile * 64 + (v / 3) * 32 + l;
         if (j < M) {
             if (g) g[((int64_t)b * M + j) * 3 + v % 3] = Gq * tot;
             if (gz && v % 3 == 2) gz[(int64_t)b * M + j] = Gq * tot;
         }
+    };
+    if constexpr (kSolo) {
+#pragma unroll
+        for (int v = 0; v < 6; ++v) put(v, lane, s[v] + c[v]);
+    } else {
+        const double tot = cluster_total<6>(s, c, red);
+        if (rank == 0 && threadIdx.x < 6 * 32) put(threadIdx.x >> 5, lane, tot);
     }
 }
 
@@ -1118,13 +1128,21 @@ gf_status points_direct_forward(gf_plan_s *plan, const void *rho, int rho_dtype,
     if (M == 0) return GF_OK;
     const int f32 = rho_dtype == GF_DTYPE_F32;
     const int64_t tiles = (M + 63) / 64;
-    const int cl = pair_cluster(tiles, (P.S + 31) / 32);
-    if (plan->opt.precision == GF_PREC_FP64 || P.S == 0)
-        return pair_launch(direct_points_f64, tiles, B, cl, st, plan->d_obs, M, P.x, P.a, P.S, P.per_cell, P.ncell, rho,
-                           f32, plan->G, g, gz, plan->d_status);
+    const bool f64 = plan->opt.precision == GF_PREC_FP64 || P.S == 0;
+    const int cl = pair_cluster(tiles, (P.S + 31) / 32, f64 ? PairCost{8.0, 8.0, 4.0} : PairCost{0.25, 5.0, 8.0});
+    if (f64) {
+        if (cl == 0)
+            return pair_launch_solo(direct_points_f64<true>, tiles, B, st, plan->d_obs, M, P.x, P.a, P.S, P.per_cell,
+                                    P.ncell, rho, f32, plan->G, g, gz, plan->d_status);
+        return pair_launch(direct_points_f64<false>, tiles, B, cl, st, plan->d_obs, M, P.x, P.a, P.S, P.per_cell, P.ncell,
+                           rho, f32, plan->G, g, gz, plan->d_status);
+    }
     // mass and separations in quanta: g = G / q^2 * (quantum-unit sum)
-    return pair_launch(direct_points_mixed, tiles, B, cl, st, P.oi, P.of, M, P.xi, P.xf, P.a, P.S, P.per_cell, P.ncell,
-                       rho, f32, (float)P.q, plan->G * P.q, g, gz, plan->d_status);
+    if (cl == 0)
+        return pair_launch_solo(direct_points_mixed<true>, tiles, B, st, P.oi, P.of, M, P.xi, P.xf, P.a, P.S, P.per_cell,
+                                P.ncell, rho, f32, (float)P.q, plan->G * P.q, g, gz, plan->d_status);
+    return pair_launch(direct_points_mixed<false>, tiles, B, cl, st, P.oi, P.of, M, P.xi, P.xf, P.a, P.S, P.per_cell,
+                       P.ncell, rho, f32, (float)P.q, plan->G * P.q, g, gz, plan->d_status);
 }
 
 gf_status points_fmm_create(gf_plan_s *plan, const double *src, const double *wt, const double *obs,

@@ -105,12 +105,13 @@ __global__ void an_corner_weights(const void *__restrict__ rho, int rho_f32, AnG
 // the FP64 pipe (a square root, three logarithms, three arctangents and their
 // quotients per corner and observer).  17^3 corners, 4096 stations:
 // 60.8 -> 14.9 ms; 9^3 corners, 200 stations: 8.97 -> 0.32 ms.
-__global__ void __launch_bounds__(kPairThreads)
+template <bool kSolo>
+__global__ void __launch_bounds__(kSolo ? 32 : kPairThreads)
 an_forward(const double *__restrict__ obs, int64_t M, const double *__restrict__ D, AnGrid g, double G,
            double *__restrict__ gout, double *__restrict__ gz) {
-    __shared__ double2 red[(kPairWarps + 1) * 3 * 32];
-    const int C = (int)cooperative_groups::this_cluster().num_blocks();
-    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    __shared__ double2 red[kSolo ? 1 : (kPairWarps + 1) * 3 * 32];
+    const int C = kSolo ? 1 : (int)cooperative_groups::this_cluster().num_blocks();
+    const int rank = kSolo ? 0 : (int)cooperative_groups::this_cluster().block_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int64_t tile = blockIdx.x / C, j = tile * 32 + lane;
@@ -119,7 +120,7 @@ an_forward(const double *__restrict__ obs, int64_t M, const double *__restrict__
     const double *Db = D + (int64_t)b * g.nc;
     double s[3] = {0.0, 0.0, 0.0}, c[3] = {0.0, 0.0, 0.0};
     for (int64_t t0 = (int64_t)(rank * kPairWarps + warp) * kAnPiece; t0 < g.nc;
-         t0 += (int64_t)C * kPairWarps * kAnPiece) {
+         t0 += (kSolo ? 1 : (int64_t)C * kPairWarps) * kAnPiece) {
         const double dl = lane < kAnPiece && t0 + lane < g.nc ? Db[t0 + lane] : 0.0;
         unsigned todo = __ballot_sync(0xffffffffu, dl != 0.0);   // corners of zero weight are skipped
         double px = 0, py = 0, pz = 0;
@@ -140,15 +141,18 @@ an_forward(const double *__restrict__ obs, int64_t M, const double *__restrict__
         two_sum_d(s[1], c[1], py);
         two_sum_d(s[2], c[2], pz);
     }
-    const double tot = cluster_total<3>(s, c, red);
-    const int t = threadIdx.x;
-    if (rank == 0 && t < 3 * 32) {
-        const int v = t >> 5;
-        const int64_t jo = tile * 32 + (t & 31);
-        if (jo < M) {
-            if (gout) gout[((int64_t)b * M + jo) * 3 + v] = G * tot;
-            if (gz && v == 2) gz[(int64_t)b * M + jo] = G * tot;
+    auto put = [&](int v, double tot) {
+        if (j < M) {
+            if (gout) gout[((int64_t)b * M + j) * 3 + v] = G * tot;
+            if (gz && v == 2) gz[(int64_t)b * M + j] = G * tot;
         }
+    };
+    if constexpr (kSolo) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) put(v, s[v] + c[v]);
+    } else {
+        const double tot = cluster_total<3>(s, c, red);
+        if (rank == 0 && threadIdx.x < 3 * 32) put(threadIdx.x >> 5, tot);
     }
 }
 
@@ -239,8 +243,10 @@ gf_status sum_an_forward(gf_plan_s *plan, const void *rho, int rho_dtype, int B,
     GF_KERNEL_DONE();
     if (plan->M == 0) return GF_OK;
     const int64_t tiles = (plan->M + 31) / 32;
-    return pair_launch(an_forward, tiles, B, pair_cluster(tiles, (ga.nc + kAnPiece - 1) / kAnPiece), st, plan->d_obs, plan->M,
-                       plan->d_corner, ga, plan->G, g, gz);
+    const int cl = pair_cluster(tiles, (ga.nc + kAnPiece - 1) / kAnPiece, {kAnPiece * 3.1, 4.0, 4.0});
+    if (cl == 0)
+        return pair_launch_solo(an_forward<true>, tiles, B, st, plan->d_obs, plan->M, plan->d_corner, ga, plan->G, g, gz);
+    return pair_launch(an_forward<false>, tiles, B, cl, st, plan->d_obs, plan->M, plan->d_corner, ga, plan->G, g, gz);
 }
 
 gf_status sum_an_adjoint(gf_plan_s *plan, const double *r, int ncomp, int B, double *grad, cudaStream_t st) {
