@@ -1992,10 +1992,11 @@ int eval_setup(gf_plan_s *plan, int B, double *g, double *gz, EvalArgs &a) {
 // SM than an even spread over the SMs puts there (`stat`: the kernel's static part).
 // The near field of a small model is a few dozen blocks that start as the M2L on
 // the tensor cores leaves the SMs, and the first SMs to come free took as many as
-// fitted while the others stood idle: 64^3 voxels under 128^2 stations, 2x2x2 rule in 4^3-voxel leaves,
-// 798 us where the same launches in line took 441; closed form 394 against 272; FP64
-// 38.1 ms against 12.4; now 387, 213 us and 12.3 ms.  (Beside an M2L on the SIMT cores
-// nothing is in the way, and an FP64 near field on every SM slows it.)
+// fitted while the others stood idle: 64^3 voxels under 128^2 stations, a 2x2x2 rule
+// in 4^3-voxel leaves, 798 us where the same launches in line took 441; closed form
+// 394 against 272; FP64 38.1 ms against 12.4; now 387, 213 us and 12.3 ms.  (Beside an
+// M2L on the SIMT cores nothing is in the way, and an FP64 near field on every SM
+// slows it.)
 size_t spread_smem(bool spread, unsigned blocks, size_t shm, size_t stat) {
     if (!spread) return shm;
     constexpr size_t kSM = 228 * 1024, kBlock = 1024;   // an SM's; what a block takes beside its own

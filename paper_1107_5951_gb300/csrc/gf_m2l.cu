@@ -2250,7 +2250,9 @@ gf_status oz_tables(const Tables *T, cudaStream_t st, const OzTables **out) {
             cudaFree(img);
             cudaGetLastError();
             *out = nullptr;   // no room: the SIMT M2L serves the plan
-            return err == cudaErrorMemoryAllocation ? GF_OK : GF_ERR_CUDA;
+            if (err == cudaErrorMemoryAllocation) return GF_OK;
+            set_error("cannot make the digit M2L's operators: %s", cudaGetErrorString(err));
+            return GF_ERR_CUDA;
         }
     }
     *out = &z;
