@@ -2028,7 +2028,7 @@ gf_status eval_launch(gf_plan_s *plan, EvalArgs a, int n1, int mode, cudaStream_
     } else if (sizeof(T) == 8 && n1 == 4) {
         const unsigned ng = (unsigned)std::min<int64_t>(2 * F->n_items, 152 * 64);
         const size_t nshm = spread_smem(spread, ng, 0, kNear64Static);
-        GF_TRY((ensure_smem(near_f64_kernel, nshm)));
+        GF_TRY((ensure_smem(near_f64_kernel, nshm, kNear64Static)));
         near_f64_kernel<<<ng, kNear64Warps * 32, nshm, st>>>(a);
     } else if (sizeof(T) == 4 && (plan->opt.reserved0 & GF_FLAG_SUM_AN)) {
         const unsigned ag = (unsigned)std::min<int64_t>((2 * F->n_items + kAnWarps - 1) / kAnWarps, 152 * 64);

@@ -217,10 +217,10 @@ __host__ __device__ __forceinline__ bool in_source_part(int64_t X, int64_t Y, in
     return c >= lo && c < hi;
 }
 
-// Opt a kernel in to more than 48 KB of shared memory (up to 1 KB of it static).
+// Opt a kernel in to more than 48 KB of shared memory, `stat` bytes of it static.
 template <class Kern>
-inline gf_status ensure_smem(Kern kernel, size_t bytes) {
-    if (bytes > 47 * 1024) {
+inline gf_status ensure_smem(Kern kernel, size_t bytes, size_t stat = 1024) {
+    if (bytes + stat > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) {
             set_error("cannot reserve %zu bytes of shared memory: %s", bytes, cudaGetErrorString(e));
