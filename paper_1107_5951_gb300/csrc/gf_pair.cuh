@@ -124,8 +124,9 @@ struct PairCost {
 // thread per observer before either: 38 and 103); of 4^3 voxels 617 and 2,405, now 74
 // and 1,753 (82 and 2,179); of 8^3 882, now 285 (515), FP64 12.6 ms (17.0).  The size
 // decides how an observer's sum associates: callers count the tiles of one batch
-// member, so that a member's sums are the same bits alone and in any batch.
-inline int pair_cluster(int64_t tiles, int64_t units, PairCost cost) {
+// member, so that a member's sums are the same bits alone and in any batch.  *time:
+// the SM's time, in microseconds.
+inline int pair_cluster(int64_t tiles, int64_t units, PairCost cost, double *time = nullptr) {
     const int64_t sms = sm_count();
     const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kPairMaxCluster, units / (2 * kPairWarps)));
     // a warp to a tile (a tenth slower a unit than warps that share a block)
@@ -141,6 +142,7 @@ inline int pair_cluster(int64_t tiles, int64_t units, PairCost cost) {
             best = (int)c;
         }
     }
+    if (time) *time = best_us;
     return best;
 }
 
