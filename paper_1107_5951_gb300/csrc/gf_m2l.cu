@@ -725,12 +725,14 @@ __device__ __forceinline__ float4 read4(const TcArgs &a, const TcLevel &L, int64
 // CTAs' partial rows in CTA order.  Blocks (c - 1, .) look at the boundary before
 // CTA c and, when it is the first one inside its tile, finish the tile's rows, the
 // columns split over blockIdx.y.
-// A chain of dependent loads with little behind it: one wave of blocks, kJoin partial
-// rows on their way before the first CTA's sum is asked for.  (That sum first, a
-// column at a time: 44^3 voxels under 256^2 stations, p = 8, 111.5 us a forward, now
-// 107.5; 84 x 84 x 42 of a 2x2x2 rule 312.4, now 311.3.)
-constexpr int kJoin = 8;
-__global__ void __launch_bounds__(512) m2l_join(const __grid_constant__ TcArgs a) {
+// A chain of dependent loads with little behind it: kJoin partial rows are on their way
+// before the first CTA's sum is asked for, and the blocks are small, to start beside
+// those of the near field.  44^3 voxels under 256^2 stations, p = 8: 111.0 us a forward
+// (that sum first, a column at a time, blocks of 512), now 108.6; 45 x 182 x 28, p = 13:
+// 242.7, 237.4; 179^3, p = 10: 250.9, 246.4; 49^3 under 98^2 with their volume too,
+// p = 12: 334.1, 324.3.
+constexpr int kJoin = 4;
+__global__ void __launch_bounds__(256) m2l_join(const __grid_constant__ TcArgs a) {
     const int c = (int)blockIdx.x + 1;
     const int4 cut = a.mcut[c];
     const uint32_t G = (uint32_t)cut.w, T = a.mcut[gridDim.x + 1].x;
@@ -746,7 +748,7 @@ __global__ void __launch_bounds__(512) m2l_join(const __grid_constant__ TcArgs a
     if (row < 0) return;
     const size_t slot = (size_t)(a.Npad / 4) * a.prow;
     const float4 *p = reinterpret_cast<const float4 *>(a.mpart) + r;
-    for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < a.Npad / 4; q += 4 * (int)gridDim.y) {
+    for (int q = 2 * (int)blockIdx.y + (threadIdx.x >> 7); q < a.Npad / 4; q += 2 * (int)gridDim.y) {
         float4 s;
         for (int e = cf + 1; e <= cl; e += kJoin) {
             float4 v[kJoin];
@@ -1613,6 +1615,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) m2l_oz(const __grid_constant__ 
 // 128^3 voxels 3,889 -> 3,884 us a forward, 83^3 1,272 -> 1,267, of the loads' order
 // and of 8 blocks to a boundary in place of 2.
 __global__ void __launch_bounds__(512) m2l_oz_join(const __grid_constant__ OzArgs o) {
+    constexpr int kRows = 8;   // partial rows on their way
     const TcArgs &a = o.t;
     const int c = (int)blockIdx.x + 1;
     const int4 cut = a.mcut[c];
@@ -1632,17 +1635,17 @@ __global__ void __launch_bounds__(512) m2l_oz_join(const __grid_constant__ OzArg
     const size_t slot = (size_t)o.ng * a.prow;
     for (int q = 4 * (int)blockIdx.y + (threadIdx.x >> 7); q < o.ng && col0 + q < a.K; q += 4 * (int)gridDim.y) {
         double s = 0.0, scale = 0.0;
-        for (int e = cf + 1; e <= cl; e += kJoin) {
-            double v[kJoin];
+        for (int e = cf + 1; e <= cl; e += kRows) {
+            double v[kRows];
 #pragma unroll
-            for (int i = 0; i < kJoin; ++i)
+            for (int i = 0; i < kRows; ++i)
                 if (e + i <= cl) v[i] = __ldg(p + (e + i) * slot + (size_t)q * a.prow);
             if (e == cf + 1) {
                 scale = __ldg(o.cinv + col0 + q);
                 s = dst[q];
             }
 #pragma unroll
-            for (int i = 0; i < kJoin; ++i)
+            for (int i = 0; i < kRows; ++i)
                 if (e + i <= cl) s = fma(v[i], scale, s);
         }
         dst[q] = s;
@@ -2150,7 +2153,7 @@ gf_status m2l_run_tc(gf_plan_s *plan, int B, bool adj, cudaStream_t st, cudaEven
     if (fork) GF_CUDA(cudaEventRecord(fork, st));
     GF_TRY(tc_launch(a, a.stream ? (int)ctas : a.ntiles, st));
     if (a.stream && ctas > 1) {
-        m2l_join<<<dim3((unsigned)ctas - 1, 4), 512, 0, st>>>(a);
+        m2l_join<<<dim3((unsigned)ctas - 1, 8), 256, 0, st>>>(a);
         GF_KERNEL_DONE();
     }
     return GF_OK;
