@@ -59,14 +59,15 @@ MUFU_RSQRT_PROBE = 4.63e12
 # interaction-list box pairs for the M2L.
 NCU_TRAFFIC = {
     # evaluation: near-field and far-field kernels of one forward, scaled by the pairs
-    ("eval", "layered_scale_464^3", 10): (round((7902720 + 0 + 23410176 + 0) * 596922624 / 280629504),
+    ("eval", "layered_scale_464^3", 10): (round((14610688 + 0 + 45617664 + 18688) * 596922624 / 593799424),
                                           ("paper_1107_5951_gb300/csrc/gf_fmm.cu",
                                            "paper_1107_5951_gb300/csrc/gf_simd.cuh",
                                            "paper_1107_5951_gb300/csrc/fmm_math.cuh"),
-                                          "e6e19973d3feff22bec7f445f4c523b35d9d346b"),
-    ("m2l", "layered_scale_464^3", 10): (round((19061248 + 0) * 1125279 / 510295),
+                                          "f423990353ab0a22c9ff0c5eb4310be03fef8c00"),
+    # M2L: the units' kernel and the join
+    ("m2l", "layered_scale_464^3", 10): (round((19039488 + 0 + 12231168 + 0) * 1125279 / 510295),
                                          ("paper_1107_5951_gb300/csrc/gf_m2l.cu",),
-                                         "06e97124d0ebb1d513f65faa28dd3a3ea34f260c"),
+                                         "1410370df846165051c54dd1e0ee3a9c8d185472"),
 }
 
 
